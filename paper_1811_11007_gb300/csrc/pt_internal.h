@@ -108,6 +108,17 @@ struct ClvGroup {
     void* clv_lo;
 };
 
+// Element f = state * C + category of the vector at site p of a slot of ld
+// sites: 16-byte chunks of V consecutive elements, [chunk][site][V].  (Element 0
+// of a slot is on a 16-byte boundary, and so is every chunk.)
+#ifdef __CUDACC__
+template <typename R>
+__device__ __forceinline__ size_t vec_index(int ld, int p, int f) {
+    constexpr int V = 16 / (int)sizeof(R);
+    return ((size_t)(f / V) * ld + p) * V + f % V;
+}
+#endif
+
 // Work item of the proposal kernel: frontier tree, internal edge node, swap,
 // visited-table slot.
 struct Item {

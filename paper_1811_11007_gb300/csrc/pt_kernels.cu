@@ -1,9 +1,13 @@
 // CUDA kernels of the PT hot path (sm_103a).
 //
-// Layout in HBM (per group of trees): partial-likelihood vectors
-// [slot][site][category][state] in FP32 (mixed precision) or FP64, one 4C-wide
-// record per site so a thread owning a site reads it with 128-bit loads;
-// per-site power-of-two scaler counts [slot][site] int32.  Slots of a tree:
+// Layout in HBM (per group of trees): partial-likelihood vectors in FP32 (mixed
+// precision) or FP64.  A site's 4C values are ordered [state][category] and cut
+// into 16-byte chunks, stored [slot][chunk][site][values of the chunk]
+// (vec_index), so the 32 lanes of a warp read each chunk as one contiguous run,
+// and in FP32 with four categories a chunk is one state's four categories: two
+// register pairs that the packed FP32 instructions take as they are.
+// Transition matrices are ordered [from][to][category] to match.
+// Per-site power-of-two scaler counts [slot][site] int32.  Slots of a tree:
 // D_v (the subtree below inner node v, at v) for every inner v, then U_v (the
 // rest of the tree, at v's parent) for every inner v but the first.
 //
@@ -773,7 +777,7 @@ __global__ void k_lengths_to_input(int n, int count, TreeSet ts, double* lengths
 // P_r(t)[i][j] = isqpi_i * sum_k R_ik exp(lam_k r t) R_jk * sqpi_j, one row
 // (4 entries) per call, exponentials in FP64.
 template <typename R>
-__device__ __forceinline__ void pmat_row(const Model& M, double rt, int i, R* row) {
+__device__ __forceinline__ void pmat_row(const Model& M, double rt, int i, R* row, int stride = 1) {
     double e[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) e[k] = exp(M.lam[k] * rt);
@@ -782,11 +786,48 @@ __device__ __forceinline__ void pmat_row(const Model& M, double rt, int i, R* ro
         double acc = 0.0;
 #pragma unroll
         for (int k = 0; k < 4; ++k) acc += M.R[i * 4 + k] * e[k] * M.R[j * 4 + k];
-        row[j] = (R)(acc * M.isqpi[i] * M.sqpi[j]);
+        row[j * stride] = (R)(acc * M.isqpi[i] * M.sqpi[j]);
     }
 }
 
-// Source of a 4C-wide vector at a site: a tip (code lookup) or a stored slot.
+// ---------------------------------------------------------------- packed FP32
+// Blackwell's FP32 pipe takes two FP32 operations per lane in one instruction
+// (fma / mul / add .f32x2 on 64-bit register pairs, each half rounded as the
+// scalar instruction rounds it).  With four categories every vector operation
+// here runs on pairs of categories: the issue slots of the 4 x 4 products halve
+// and every result keeps its bits.
+using f32x2 = float2;
+__device__ __forceinline__ unsigned long long& b64(f32x2& x) { return reinterpret_cast<unsigned long long&>(x); }
+__device__ __forceinline__ unsigned long long b64c(f32x2 x) {
+    return reinterpret_cast<const unsigned long long&>(x);
+}
+__device__ __forceinline__ f32x2 pmul(f32x2 a, f32x2 b) {
+    f32x2 d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(b64(d)) : "l"(b64c(a)), "l"(b64c(b)));
+    return d;
+}
+__device__ __forceinline__ f32x2 padd(f32x2 a, f32x2 b) {
+    f32x2 d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(b64(d)) : "l"(b64c(a)), "l"(b64c(b)));
+    return d;
+}
+__device__ __forceinline__ f32x2 pfma(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(b64(d)) : "l"(b64c(a)), "l"(b64c(b)), "l"(b64c(c)));
+    return d;
+}
+__device__ __forceinline__ f32x2 pneg(f32x2 a) { return make_float2(-a.x, -a.y); }
+// a - b as one packed instruction (b * -1 is exact)
+__device__ __forceinline__ f32x2 psub(f32x2 a, f32x2 b) { return pfma(b, make_float2(-1.f, -1.f), a); }
+__device__ __forceinline__ float pmul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float padd(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float pfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ float pneg(float a) { return -a; }
+__device__ __forceinline__ float psub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ f32x2 pair(const float* x) { return make_float2(x[0], x[1]); }
+
+// Source of a 4C-wide vector at a site: a tip (code lookup) or a stored slot
+// (its sites `ld` apart per chunk, see vec_index).
 template <typename R, int C>
 struct Src {
     const R* clv;      // slot base (nullptr for a tip)
@@ -794,96 +835,136 @@ struct Src {
     const uint8_t* tip;  // tip codes of the leaf (nullptr for a slot)
 };
 
+// A stored vector at site p of a slot of ld sites, x[state * C + category].
 template <typename R, int C>
-__device__ __forceinline__ void load_raw(const Src<R, C>& s, int p, R* x, int& cnt) {
+__device__ __forceinline__ void load_vec(const R* src, int ld, int p, R* x) {
+    if constexpr (sizeof(R) == 4) {
+#pragma unroll
+        for (int q = 0; q < C; ++q) {
+            const float4 v = reinterpret_cast<const float4*>(src)[(size_t)q * ld + p];
+            x[4 * q] = v.x; x[4 * q + 1] = v.y; x[4 * q + 2] = v.z; x[4 * q + 3] = v.w;
+        }
+    } else {
+#pragma unroll
+        for (int q = 0; q < 2 * C; ++q) {
+            const double2 v = reinterpret_cast<const double2*>(src)[(size_t)q * ld + p];
+            x[2 * q] = v.x; x[2 * q + 1] = v.y;
+        }
+    }
+}
+
+template <typename R, int C>
+__device__ __forceinline__ void load_raw(const Src<R, C>& s, int ld, int p, R* x, int& cnt) {
     if (s.tip) {
         int code = s.tip[p];
 #pragma unroll
-        for (int r = 0; r < C; ++r)
+        for (int i = 0; i < 4; ++i)
 #pragma unroll
-            for (int i = 0; i < 4; ++i) x[r * 4 + i] = (code >= 4 || code == i) ? R(1) : R(0);
+            for (int r = 0; r < C; ++r) x[i * C + r] = (code >= 4 || code == i) ? R(1) : R(0);
         cnt = 0;
     } else {
-        const R* src = s.clv + (size_t)p * 4 * C;
-        if constexpr (sizeof(R) == 4) {
-#pragma unroll
-            for (int q = 0; q < C; ++q) {
-                float4 v = reinterpret_cast<const float4*>(src)[q];
-                x[4 * q] = v.x; x[4 * q + 1] = v.y; x[4 * q + 2] = v.z; x[4 * q + 3] = v.w;
-            }
-        } else {
-#pragma unroll
-            for (int q = 0; q < 2 * C; ++q) {
-                double2 v = reinterpret_cast<const double2*>(src)[q];
-                x[2 * q] = v.x; x[2 * q + 1] = v.y;
-            }
-        }
+        load_vec<R, C>(s.clv, ld, p, x);
         cnt = s.scl[p];
     }
 }
 
-// Row i of P_r from a [C][16] row-major block as one 16-byte load (FP32) or two
-// (FP64); every P block starts on a 16-byte boundary.
-template <typename R>
-__device__ __forceinline__ void pm_row(const R* Pm, int r, int i, R* w) {
-    if constexpr (sizeof(R) == 4) {
-        const float4 v = reinterpret_cast<const float4*>(Pm)[r * 4 + i];
-        w[0] = v.x; w[1] = v.y; w[2] = v.z; w[3] = v.w;
+// y_r = P_r x_r, P [16][C] ([from * 4 + to][category]), x and y [state][category].
+template <typename R, int C>
+__device__ __forceinline__ void apply_p_reg(const R* Pm, const R* x, R* y) {
+    if constexpr (sizeof(R) == 4 && C == 4) {
+        const float4* P4 = reinterpret_cast<const float4*>(Pm);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            float4 w = P4[i * 4];
+            f32x2 lo = pmul(make_float2(w.x, w.y), pair(x)), hi = pmul(make_float2(w.z, w.w), pair(x + 2));
+#pragma unroll
+            for (int j = 1; j < 4; ++j) {
+                w = P4[i * 4 + j];
+                lo = pfma(make_float2(w.x, w.y), pair(x + 4 * j), lo);
+                hi = pfma(make_float2(w.z, w.w), pair(x + 4 * j + 2), hi);
+            }
+            y[4 * i] = lo.x; y[4 * i + 1] = lo.y; y[4 * i + 2] = hi.x; y[4 * i + 3] = hi.y;
+        }
     } else {
-        const double2 a = reinterpret_cast<const double2*>(Pm)[(r * 4 + i) * 2];
-        const double2 b = reinterpret_cast<const double2*>(Pm)[(r * 4 + i) * 2 + 1];
-        w[0] = a.x; w[1] = a.y; w[2] = b.x; w[3] = b.y;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            R w[4 * C];  // row i of every category: 4C consecutive values on a 16-byte boundary
+#pragma unroll
+            for (int q = 0; q < 4 * C * (int)sizeof(R) / 16; ++q) {
+                if constexpr (sizeof(R) == 4) {
+                    const float4 v = reinterpret_cast<const float4*>(Pm)[i * C + q];
+                    w[4 * q] = v.x; w[4 * q + 1] = v.y; w[4 * q + 2] = v.z; w[4 * q + 3] = v.w;
+                } else {
+                    const double2 v = reinterpret_cast<const double2*>(Pm)[i * 2 * C + q];
+                    w[2 * q] = v.x; w[2 * q + 1] = v.y;
+                }
+            }
+#pragma unroll
+            for (int r = 0; r < C; ++r) {
+                R acc = w[r] * x[r];
+#pragma unroll
+                for (int j = 1; j < 4; ++j) acc = fma(w[j * C + r], x[j * C + r], acc);
+                y[i * C + r] = acc;
+            }
+        }
     }
 }
 
+// y_r = P_r x_r of a source; for a tip the product is a column of P (or all
+// ones for a gap).
 template <typename R, int C>
-__device__ __forceinline__ void apply_p_reg(const R* Pm, const R* x, R* y) {
-#pragma unroll
-    for (int r = 0; r < C; ++r)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            R w[4];
-            pm_row<R>(Pm, r, i, w);
-            R acc = w[0] * x[r * 4];
-#pragma unroll
-            for (int j = 1; j < 4; ++j) acc = fma(w[j], x[r * 4 + j], acc);
-            y[r * 4 + i] = acc;
-        }
-}
-
-// y_r = P_r x_r (Pm: [C][16] row-major); for a tip the product is a column
-// of P (or all ones for a gap).
-template <typename R, int C>
-__device__ __forceinline__ void apply_p(const R* Pm, const Src<R, C>& s, int p, R* y, int& cnt) {
+__device__ __forceinline__ void apply_p(const R* Pm, const Src<R, C>& s, int ld, int p, R* y, int& cnt) {
     if (s.tip) {
         int code = s.tip[p];
         cnt = 0;
         if (code >= 4) {
 #pragma unroll
             for (int q = 0; q < 4 * C; ++q) y[q] = R(1);
+        } else if constexpr (sizeof(R) == 4 && C == 4) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float4 v = reinterpret_cast<const float4*>(Pm)[i * 4 + code];
+                y[4 * i] = v.x; y[4 * i + 1] = v.y; y[4 * i + 2] = v.z; y[4 * i + 3] = v.w;
+            }
         } else {
 #pragma unroll
-            for (int r = 0; r < C; ++r)
+            for (int i = 0; i < 4; ++i)
 #pragma unroll
-                for (int i = 0; i < 4; ++i) y[r * 4 + i] = Pm[r * 16 + i * 4 + code];
+                for (int r = 0; r < C; ++r) y[i * C + r] = Pm[(i * 4 + code) * C + r];
         }
         return;
     }
     R x[4 * C];
-    load_raw<R, C>(s, p, x, cnt);
+    load_raw<R, C>(s, ld, p, x, cnt);
     apply_p_reg<R, C>(Pm, x, y);
 }
 
+// y *= z, elementwise
 template <typename R, int C>
-__device__ __forceinline__ void store_vec(R* dst, int p, const R* y) {
-    R* d = dst + (size_t)p * 4 * C;
+__device__ __forceinline__ void mul_vec(R* y, const R* z) {
+    if constexpr (sizeof(R) == 4) {
+#pragma unroll
+        for (int q = 0; q < 4 * C; q += 2) {
+            const f32x2 t = pmul(pair(y + q), pair(z + q));
+            y[q] = t.x; y[q + 1] = t.y;
+        }
+    } else {
+#pragma unroll
+        for (int q = 0; q < 4 * C; ++q) y[q] *= z[q];
+    }
+}
+
+template <typename R, int C>
+__device__ __forceinline__ void store_vec(R* dst, int ld, int p, const R* y) {
     if constexpr (sizeof(R) == 4) {
 #pragma unroll
         for (int q = 0; q < C; ++q)
-            reinterpret_cast<float4*>(d)[q] = make_float4(y[4 * q], y[4 * q + 1], y[4 * q + 2], y[4 * q + 3]);
+            reinterpret_cast<float4*>(dst)[(size_t)q * ld + p] =
+                make_float4(y[4 * q], y[4 * q + 1], y[4 * q + 2], y[4 * q + 3]);
     } else {
 #pragma unroll
-        for (int q = 0; q < 2 * C; ++q) reinterpret_cast<double2*>(d)[q] = make_double2(y[2 * q], y[2 * q + 1]);
+        for (int q = 0; q < 2 * C; ++q)
+            reinterpret_cast<double2*>(dst)[(size_t)q * ld + p] = make_double2(y[2 * q], y[2 * q + 1]);
     }
 }
 
@@ -925,88 +1006,122 @@ __device__ __forceinline__ F2 f2_of(double x) {
     return F2{h, (float)(x - (double)h)};
 }
 
-// y_r = P_r x_r for pairs: P as (Ph, Pl) [C][16] row-major, x and y as (h, l)
-// [4C].  Every term is non-negative (probabilities times likelihoods); the
-// exact products Ph x_h are summed by two-sums, the small terms (product
-// errors, Ph x_l, Pl x_h, the sums' errors) in a plain FP32 correction.
-template <int C>
-__device__ __forceinline__ void f2_apply(const float* Ph, const float* Pl, const float* xh, const float* xl, float* yh,
-                                         float* yl) {
-#pragma unroll
-    for (int r = 0; r < C; ++r)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const float* ph = Ph + r * 16 + i * 4;
-            const float* pl = Pl + r * 16 + i * 4;
-            float s = __fmul_rn(ph[0], xh[r * 4]);
-            float c = __fmaf_rn(ph[0], xh[r * 4], -s);
-            c = __fmaf_rn(ph[0], xl[r * 4], c);
-            c = __fmaf_rn(pl[0], xh[r * 4], c);
-#pragma unroll
-            for (int j = 1; j < 4; ++j) {
-                const float p = __fmul_rn(ph[j], xh[r * 4 + j]);
-                c = __fadd_rn(c, __fmaf_rn(ph[j], xh[r * 4 + j], -p));
-                c = __fmaf_rn(ph[j], xl[r * 4 + j], c);
-                c = __fmaf_rn(pl[j], xh[r * 4 + j], c);
-                const F2 t = f2_two_sum(s, p);
-                s = t.h;
-                c = __fadd_rn(c, t.l);
-            }
-            const F2 y = f2_norm(s, c);
-            yh[r * 4 + i] = y.h;
-            yl[r * 4 + i] = y.l;
-        }
+// The pair operations on T = float, or T = f32x2: two categories at once.
+template <typename T>
+struct F2T {
+    T h, l;
+};
+template <typename T>
+__device__ __forceinline__ F2T<T> t2_norm(T h, T l) {  // f2_norm
+    const T s = padd(h, l);
+    return F2T<T>{s, psub(l, psub(s, h))};
 }
+template <typename T>
+__device__ __forceinline__ F2T<T> t2_mul(F2T<T> a, F2T<T> b) {  // f2_mul
+    const T p = pmul(a.h, b.h);
+    T e = pfma(a.h, b.h, pneg(p));
+    e = pfma(a.h, b.l, e);
+    e = pfma(a.l, b.h, e);
+    return t2_norm<T>(p, e);
+}
+// The lanes of a C-category vector: pairs of categories, or the one category.
+template <int C>
+struct Lanes {
+    using T = f32x2;
+    static constexpr int n = C / 2, w = 2;
+};
+template <>
+struct Lanes<1> {
+    using T = float;
+    static constexpr int n = 1, w = 1;
+};
+__device__ __forceinline__ void lane_get(const float* p, float& x) { x = *p; }
+__device__ __forceinline__ void lane_get(const float* p, f32x2& x) { x = *reinterpret_cast<const f32x2*>(p); }
+template <typename T>
+__device__ __forceinline__ T lane_all(float x);
+template <>
+__device__ __forceinline__ float lane_all<float>(float x) { return x; }
+template <>
+__device__ __forceinline__ f32x2 lane_all<f32x2>(float x) { return make_float2(x, x); }
 
-// One category of f2_apply: y = P x with P as (Ph, Pl) [16] row-major.
-__device__ __forceinline__ void f2_apply4(const float* ph, const float* pl, const float* xh, const float* xl, float* yh,
-                                          float* yl) {
+// y = P x for pairs on lane group g of the categories: P as (ph, pl) [16][C],
+// x and y [4].  Every term is non-negative (probabilities times likelihoods);
+// the exact products ph x_h are summed by two-sums, the small terms (product
+// errors, ph x_l, pl x_h, the sums' errors) in a plain FP32 correction, kept
+// negated (cn) so that each product's error takes one instruction.
+template <int C>
+__device__ __forceinline__ void f2_apply4(const float* ph, const float* pl, int g,
+                                          const F2T<typename Lanes<C>::T>* x, F2T<typename Lanes<C>::T>* y) {
+    using T = typename Lanes<C>::T;
+    T nh[4], nl[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        nh[j] = pneg(x[j].h);
+        nl[j] = pneg(x[j].l);
+    }
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        float s = __fmul_rn(ph[i * 4], xh[0]);
-        float c = __fmaf_rn(ph[i * 4], xh[0], -s);
-        c = __fmaf_rn(ph[i * 4], xl[0], c);
-        c = __fmaf_rn(pl[i * 4], xh[0], c);
+        T s{}, cn{};
 #pragma unroll
-        for (int j = 1; j < 4; ++j) {
-            const float p = __fmul_rn(ph[i * 4 + j], xh[j]);
-            c = __fadd_rn(c, __fmaf_rn(ph[i * 4 + j], xh[j], -p));
-            c = __fmaf_rn(ph[i * 4 + j], xl[j], c);
-            c = __fmaf_rn(pl[i * 4 + j], xh[j], c);
-            const F2 t = f2_two_sum(s, p);
-            s = t.h;
-            c = __fadd_rn(c, t.l);
+        for (int j = 0; j < 4; ++j) {
+            T a, b;
+            lane_get(ph + (i * 4 + j) * C + g * Lanes<C>::w, a);
+            lane_get(pl + (i * 4 + j) * C + g * Lanes<C>::w, b);
+            const T p = pmul(a, x[j].h);
+            const T e = pfma(a, nh[j], p);
+            cn = j == 0 ? e : padd(cn, e);
+            cn = pfma(a, nl[j], cn);
+            cn = pfma(b, nh[j], cn);
+            if (j == 0) {
+                s = p;
+            } else {
+                const T t = padd(s, p), bb = psub(t, s);
+                cn = padd(cn, padd(psub(psub(t, bb), s), psub(bb, p)));
+                s = t;
+            }
         }
-        const F2 y = f2_norm(s, c);
-        yh[i] = y.h;
-        yl[i] = y.l;
+        const T t = psub(s, cn);
+        y[i] = F2T<T>{t, psub(psub(s, t), cn)};
     }
 }
 
 // x *= y for 4 pairs
-__device__ __forceinline__ void f2_mul4(float* xh, float* xl, const float* yh, const float* yl) {
+template <typename T>
+__device__ __forceinline__ void f2_mul4(F2T<T>* x, const F2T<T>* y) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const F2 t = f2_mul(F2{xh[i], xl[i]}, F2{yh[i], yl[i]});
-        xh[i] = t.h;
-        xl[i] = t.l;
-    }
+    for (int i = 0; i < 4; ++i) x[i] = t2_mul<T>(x[i], y[i]);
 }
 
-// exact power-of-two scaling of 4 pairs to max h in [1, 2); the exponent removed
-__device__ __forceinline__ int f2_normalise4(float* h, float* l) {
-    const float mx = fmaxf(fmaxf(h[0], h[1]), fmaxf(h[2], h[3]));
-    if (!(mx > 0.f)) return 0;
-    int e = ((__float_as_int(mx) >> 23) & 0xff) - 127;
+__device__ __forceinline__ float lane_max(float x) { return x; }
+__device__ __forceinline__ float lane_max(f32x2 x) { return fmaxf(x.x, x.y); }
+// exact power-of-two scaling of 4 pairs to max h in [1, 2), each category on its
+// own; the exponents removed, one per category
+__device__ __forceinline__ float pow2_norm(float mx, int& e) {
+    if (!(mx > 0.f)) { e = 0; return 1.f; }
+    e = ((__float_as_int(mx) >> 23) & 0xff) - 127;
     if (e < -125) e = -125;
-    const float m = __int_as_float((127 - e) << 23);
+    return __int_as_float((127 - e) << 23);
+}
+__device__ __forceinline__ void f2_normalise4(F2T<float>* x, int* e) {
+    const float m = pow2_norm(fmaxf(fmaxf(x[0].h, x[1].h), fmaxf(x[2].h, x[3].h)), e[0]);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        h[i] *= m;
-        l[i] *= m;
+        x[i].h *= m;
+        x[i].l *= m;
     }
-    return e;
 }
+__device__ __forceinline__ void f2_normalise4(F2T<f32x2>* x, int* e) {
+    f32x2 m;
+    m.x = pow2_norm(fmaxf(fmaxf(x[0].h.x, x[1].h.x), fmaxf(x[2].h.x, x[3].h.x)), e[0]);
+    m.y = pow2_norm(fmaxf(fmaxf(x[0].h.y, x[1].h.y), fmaxf(x[2].h.y, x[3].h.y)), e[1]);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        x[i].h = pmul(x[i].h, m);
+        x[i].l = pmul(x[i].l, m);
+    }
+}
+__device__ __forceinline__ F2 lane_of(F2T<float> x, int) { return F2{x.h, x.l}; }
+__device__ __forceinline__ F2 lane_of(F2T<f32x2> x, int k) { return k ? F2{x.h.y, x.l.y} : F2{x.h.x, x.l.x}; }
 
 // x * 2^-d for d >= 0 (0 when far below the FP32 range: negligible next to the other term)
 __device__ __forceinline__ F2 f2_down(F2 x, int d) {
@@ -1033,121 +1148,78 @@ struct Src2 {
     const uint8_t* tip;
 };
 
-// y = P x for a pair source at site p; cnt = its scaler count.
+// Lane group g of y = P x for a pair source at site p (P: [16][C] pairs, slots
+// of ld sites).
 template <int C>
-__device__ __forceinline__ void f2_apply_src(const float* Ph, const float* Pl, const Src2<C>& s, int p, float* yh,
-                                             float* yl, int& cnt) {
-    if (s.tip) {
-        const int code = s.tip[p];
-        cnt = 0;
-#pragma unroll
-        for (int r = 0; r < C; ++r)
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                yh[r * 4 + i] = code >= 4 ? 1.f : Ph[r * 16 + i * 4 + (code & 3)];
-                yl[r * 4 + i] = code >= 4 ? 0.f : Pl[r * 16 + i * 4 + (code & 3)];
-            }
-        return;
-    }
-    float xh[4 * C], xl[4 * C];
-    const float4* a = reinterpret_cast<const float4*>(s.h + (size_t)p * 4 * C);
-    const float4* b = reinterpret_cast<const float4*>(s.l + (size_t)p * 4 * C);
-#pragma unroll
-    for (int q = 0; q < C; ++q) {
-        const float4 u = a[q], v = b[q];
-        xh[4 * q] = u.x; xh[4 * q + 1] = u.y; xh[4 * q + 2] = u.z; xh[4 * q + 3] = u.w;
-        xl[4 * q] = v.x; xl[4 * q + 1] = v.y; xl[4 * q + 2] = v.z; xl[4 * q + 3] = v.w;
-    }
-    cnt = s.scl[p];
-    f2_apply<C>(Ph, Pl, xh, xl, yh, yl);
-}
-
-// Category r of y = P_r x for a pair source at site p (P: [C][16] pairs).
-template <int C>
-__device__ __forceinline__ void f2_apply_src4(const float* Ph, const float* Pl, const Src2<C>& s, int p, int r, float* yh,
-                                              float* yl) {
+__device__ __forceinline__ void f2_apply_src4(const float* Ph, const float* Pl, const Src2<C>& s, int ld, int p, int g,
+                                              F2T<typename Lanes<C>::T>* y) {
+    using T = typename Lanes<C>::T;
+    constexpr int w = Lanes<C>::w;
     if (s.tip) {
         const int code = s.tip[p];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            yh[i] = code >= 4 ? 1.f : Ph[r * 16 + i * 4 + (code & 3)];
-            yl[i] = code >= 4 ? 0.f : Pl[r * 16 + i * 4 + (code & 3)];
+            T a, b;
+            lane_get(Ph + (i * 4 + (code & 3)) * C + g * w, a);
+            lane_get(Pl + (i * 4 + (code & 3)) * C + g * w, b);
+            y[i] = code >= 4 ? F2T<T>{lane_all<T>(1.f), lane_all<T>(0.f)} : F2T<T>{a, b};
         }
         return;
     }
-    const float4 u = reinterpret_cast<const float4*>(s.h + (size_t)p * 4 * C)[r];
-    const float4 v = reinterpret_cast<const float4*>(s.l + (size_t)p * 4 * C)[r];
-    const float xh[4] = {u.x, u.y, u.z, u.w}, xl[4] = {v.x, v.y, v.z, v.w};
-    f2_apply4(Ph + r * 16, Pl + r * 16, xh, xl, yh, yl);
-}
-
-// y0 *= y1 elementwise (pairs)
-template <int C>
-__device__ __forceinline__ void f2_mul_vec(float* ah, float* al, const float* bh, const float* bl) {
+    F2T<T> x[4];
 #pragma unroll
-    for (int q = 0; q < 4 * C; ++q) {
-        const F2 t = f2_mul(F2{ah[q], al[q]}, F2{bh[q], bl[q]});
-        ah[q] = t.h;
-        al[q] = t.l;
+    for (int j = 0; j < 4; ++j) {
+        lane_get(s.h + vec_index<float>(ld, p, j * C + g * w), x[j].h);
+        lane_get(s.l + vec_index<float>(ld, p, j * C + g * w), x[j].l);
     }
+    f2_apply4<C>(Ph, Pl, g, x, y);
 }
 
-// exact power-of-two scaling of a pair vector to max h in [1, 2); returns the exponent removed
+// One site of a stored pair vector: the join of two sources under P_a and P_b,
+// rescaled by 2^32 when every h is below 2^-32 (as rescale()), and its scaler count.
 template <int C>
-__device__ __forceinline__ int f2_normalise(float* h, float* l) {
-    float mx = h[0];
+__device__ __forceinline__ void f2_join(const float* Pah, const float* Pal, const Src2<C>& a, const float* Pbh,
+                                        const float* Pbl, const Src2<C>& b, int ld, int p, float* dh, float* dl,
+                                        int32_t* ds) {
+    using T = typename Lanes<C>::T;
+    constexpr int n = Lanes<C>::n, w = Lanes<C>::w;
+    int kk = (a.tip ? 0 : a.scl[p]) + (b.tip ? 0 : b.scl[p]);
+    F2T<T> y[n][4];
+    float mx = 0.f;
 #pragma unroll
-    for (int q = 1; q < 4 * C; ++q) mx = fmaxf(mx, h[q]);
-    if (!(mx > 0.f)) return 0;
-    int e = ((__float_as_int(mx) >> 23) & 0xff) - 127;
-    if (e < -125) e = -125;
-    const float m = __int_as_float((127 - e) << 23);
+    for (int g = 0; g < n; ++g) {
+        F2T<T> z[4];
+        f2_apply_src4<C>(Pah, Pal, a, ld, p, g, y[g]);
+        f2_apply_src4<C>(Pbh, Pbl, b, ld, p, g, z);
+        f2_mul4<T>(y[g], z);
 #pragma unroll
-    for (int q = 0; q < 4 * C; ++q) {
-        h[q] *= m;
-        l[q] *= m;
+        for (int i = 0; i < 4; ++i) mx = fmaxf(mx, lane_max(y[g][i].h));
     }
-    return e;
-}
-
-// threshold rescale of a stored pair vector (as rescale(): by 2^32 when every h < 2^-32)
-template <int C>
-__device__ __forceinline__ int f2_rescale(float* h, float* l) {
-    float mx = h[0];
-#pragma unroll
-    for (int q = 1; q < 4 * C; ++q) mx = fmaxf(mx, h[q]);
     if (mx < Prec<float>::thresh()) {
+        const T m = lane_all<T>(Prec<float>::mult());
 #pragma unroll
-        for (int q = 0; q < 4 * C; ++q) {
-            h[q] *= Prec<float>::mult();
-            l[q] *= Prec<float>::mult();
-        }
-        return 1;
-    }
-    return 0;
-}
-
-template <int C>
-__device__ __forceinline__ void f2_store(float* dh, float* dl, int p, const float* h, const float* l) {
+        for (int g = 0; g < n; ++g)
 #pragma unroll
-    for (int q = 0; q < C; ++q) {
-        reinterpret_cast<float4*>(dh + (size_t)p * 4 * C)[q] = make_float4(h[4 * q], h[4 * q + 1], h[4 * q + 2], h[4 * q + 3]);
-        reinterpret_cast<float4*>(dl + (size_t)p * 4 * C)[q] = make_float4(l[4 * q], l[4 * q + 1], l[4 * q + 2], l[4 * q + 3]);
+            for (int i = 0; i < 4; ++i) {
+                y[g][i].h = pmul(y[g][i].h, m);
+                y[g][i].l = pmul(y[g][i].l, m);
+            }
+        ++kk;
     }
-}
-
-// Site likelihood across a branch as a pair: L = (1/C) sum_r sum_i pi_i X_ri Z_ri
-// with Z = P Y (P of the branch), X and Y normalised.  pi as pairs (pih, pil).
-template <int C>
-__device__ __forceinline__ F2 f2_site_lik(const float* pih, const float* pil, const float* Xh, const float* Xl,
-                                          const float* Zh, const float* Zl) {
-    F2 acc{0.f, 0.f};
+    float h[4 * C], l[4 * C];
 #pragma unroll
-    for (int q = 0; q < 4 * C; ++q) {
-        const F2 t = f2_mul(f2_mul(F2{Xh[q], Xl[q]}, F2{Zh[q], Zl[q]}), F2{pih[q & 3], pil[q & 3]});
-        acc = f2_add(acc, t);
-    }
-    return F2{acc.h * (1.0f / C), acc.l * (1.0f / C)};  // 1/C is a power of two for C = 1, 2, 4
+    for (int g = 0; g < n; ++g)
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int k = 0; k < w; ++k) {
+                const F2 v = lane_of(y[g][i], k);
+                h[i * C + g * w + k] = v.h;
+                l[i * C + g * w + k] = v.l;
+            }
+    store_vec<float, C>(dh, ld, p, h);
+    store_vec<float, C>(dl, ld, p, l);
+    ds[p] = kk;
 }
 
 // ln of a pair site likelihood times 2^E, in FP64
@@ -1155,13 +1227,14 @@ __device__ __forceinline__ double f2_log(F2 L, int E) {
     return log((double)L.h + (double)L.l) + (double)E * kLn2;
 }
 
-// Entry q (< 16C) of P_r(t) of a branch as a pair (FP64 sum, split once):
-// W[(i*4+j)*4+k] = isqpi_i sqpi_j R_ik R_jk, ex[r*4+k] = exp(lam_k rate_r t).
+// Entry q (< 16C, [16][C]) of P_r(t) of a branch as a pair (FP64 sum, split once):
+// W[(i*4+j)*4+k] = isqpi_i sqpi_j R_ik R_jk, ex[k*C+r] = exp(lam_k rate_r t).
+template <int C>
 __device__ __forceinline__ void f2_pmat_entry(const double* W, const double* ex, int q, float* Ph, float* Pl) {
-    const int r = q >> 4, ij = q & 15;
+    const int r = q % C, ij = q / C;
     double acc = 0.0;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) acc += W[ij * 4 + k] * ex[r * 4 + k];
+    for (int k = 0; k < 4; ++k) acc += W[ij * 4 + k] * ex[k * C + r];
     const F2 v = f2_of(acc);
     Ph[q] = v.h;
     Pl[q] = v.l;
@@ -1221,23 +1294,48 @@ __device__ __forceinline__ int normalise(R* y) {
 // a form without the cancellation of the plain spectral sum at short branches
 // (which costs FP32 its accuracy).  Stored: s_{r,0} = sum_i pi_i X_i Y_i,
 // s_{r,k} = x_k y_k for k >= 1.
+// X, Y [state][category], s [k][category].
 template <typename R, int C>
 __device__ __forceinline__ void sumtable(const R* Mt, const R* pi, const R* X, const R* Y, R* s) {
+    if constexpr (sizeof(R) == 4 && C == 4) {
 #pragma unroll
-    for (int r = 0; r < C; ++r) {
-        R s0 = pi[0] * X[r * 4] * Y[r * 4];
+        for (int g = 0; g < 4; g += 2) {
+            f32x2 s0 = pmul(pmul(make_float2(pi[0], pi[0]), pair(X + g)), pair(Y + g));
 #pragma unroll
-        for (int i = 1; i < 4; ++i) s0 = fma(pi[i] * X[r * 4 + i], Y[r * 4 + i], s0);
-        s[r * 4] = s0;
+            for (int i = 1; i < 4; ++i)
+                s0 = pfma(pmul(make_float2(pi[i], pi[i]), pair(X + 4 * i + g)), pair(Y + 4 * i + g), s0);
+            s[g] = s0.x; s[g + 1] = s0.y;
 #pragma unroll
-        for (int k = 1; k < 4; ++k) {
-            R x = Mt[k] * X[r * 4], y = Mt[k] * Y[r * 4];
+            for (int k = 1; k < 4; ++k) {
+                f32x2 m = make_float2(Mt[k], Mt[k]);
+                f32x2 x = pmul(m, pair(X + g)), y = pmul(m, pair(Y + g));
 #pragma unroll
-            for (int i = 1; i < 4; ++i) {
-                x = fma(Mt[i * 4 + k], X[r * 4 + i], x);
-                y = fma(Mt[i * 4 + k], Y[r * 4 + i], y);
+                for (int i = 1; i < 4; ++i) {
+                    m = make_float2(Mt[i * 4 + k], Mt[i * 4 + k]);
+                    x = pfma(m, pair(X + 4 * i + g), x);
+                    y = pfma(m, pair(Y + 4 * i + g), y);
+                }
+                x = pmul(x, y);
+                s[4 * k + g] = x.x; s[4 * k + g + 1] = x.y;
             }
-            s[r * 4 + k] = x * y;
+        }
+    } else {
+#pragma unroll
+        for (int r = 0; r < C; ++r) {
+            R s0 = pi[0] * X[r] * Y[r];
+#pragma unroll
+            for (int i = 1; i < 4; ++i) s0 = fma(pi[i] * X[i * C + r], Y[i * C + r], s0);
+            s[r] = s0;
+#pragma unroll
+            for (int k = 1; k < 4; ++k) {
+                R x = Mt[k] * X[r], y = Mt[k] * Y[r];
+#pragma unroll
+                for (int i = 1; i < 4; ++i) {
+                    x = fma(Mt[i * 4 + k], X[i * C + r], x);
+                    y = fma(Mt[i * 4 + k], Y[i * C + r], y);
+                }
+                s[k * C + r] = x * y;
+            }
         }
     }
 }
@@ -1351,7 +1449,7 @@ struct NewtonSmem {
     R egh[3][4 * C];       // coefficients on the sum-table for L, dL/dt, d2L/dt2
     double red[32][2];     // per-warp partial sums
     float redf[32][4];     // per-warp partial sums as FP32 pairs (hi, lo) x (d1, d2)
-    double lr[4 * C];      // lam_k * rate_r
+    double lr[4 * C];      // lam_k * rate_r, [k][r] (as every 4C array here)
     float lrf[4 * C];      // the same in FP32 (coefficients of the Newton derivatives)
     double ex[4 * C];      // exp(lam_k r t) for a P-matrix refresh
     double W[64];          // W[(i*4+j)*4+k] = isqpi_i sqpi_j R_ik R_jk: P_ij = sum_k W_ijk exp(lam_k r t)
@@ -1476,7 +1574,7 @@ __device__ __forceinline__ void init_newton_smem(const Model& M, NewtonSmem<R, C
         ns.leader = lead;
     }
     for (int q = threadIdx.x; q < 4 * C; q += blockDim.x) {
-        ns.lr[q] = M.lam[q & 3] * rates[q >> 2];
+        ns.lr[q] = M.lam[q / C] * rates[q % C];
         ns.lrf[q] = (float)ns.lr[q];
     }
 }
@@ -1490,8 +1588,7 @@ template <typename R, int C>
 __device__ __forceinline__ void put_egh(const Model& M, double t, NewtonSmem<R, C>& ns, bool exact,
                                         int q = threadIdx.x) {
     if (q < 4 * C) {
-        const int k = q & 3;
-        if (k == 0) {
+        if (q < C) {
             ns.egh[0][q] = (R)(1.0 / C);
             ns.egh[1][q] = R(0);
             ns.egh[2][q] = R(0);
@@ -1516,7 +1613,7 @@ __device__ __forceinline__ void put_egh(const Model& M, double t, NewtonSmem<R, 
 template <typename R, int C>
 __device__ __forceinline__ void put_egh_f(float t, NewtonSmem<R, C>& ns, int q) {
     if (q < 4 * C) {
-        if ((q & 3) == 0) {
+        if (q < C) {
             ns.egh[0][q] = (R)(1.0f / C);
             ns.egh[1][q] = R(0);
             ns.egh[2][q] = R(0);
@@ -1644,7 +1741,10 @@ __device__ double eval_lnl(const Model& M, const STab<R, C>& st, int P, double t
             st.get(p, s);
             R L = e[0] * s[0];
 #pragma unroll
-            for (int q = 1; q < 4 * C; ++q) L = fma(e[q], s[q], L);
+            for (int z = 1; z < 4 * C; ++z) {
+                const int q = (z & 3) * C + (z >> 2);  // categories outermost
+                L = fma(e[q], s[q], L);
+            }
             int b = __float_as_int(L), ex = ((b >> 23) & 0xff) - 127;
             float m = __int_as_float((b & 0x007fffff) | 0x3f800000);
             if (ex == -127) {  // subnormal: rescale exactly by 2^23 first
@@ -1666,7 +1766,10 @@ __device__ double eval_lnl(const Model& M, const STab<R, C>& st, int P, double t
             st.get(p, s);
             R L = e[0] * s[0];
 #pragma unroll
-            for (int q = 1; q < 4 * C; ++q) L = fma(e[q], s[q], L);
+            for (int z = 1; z < 4 * C; ++z) {
+                const int q = (z & 3) * C + (z >> 2);  // categories outermost
+                L = fma(e[q], s[q], L);
+            }
             acc += (double)st.ew[st.pcap + p] * (log_split(L) + (double)st.ew[p] * kLn2);
         }
     }
@@ -1692,11 +1795,12 @@ __device__ __forceinline__ void newton_site(const STab<R, C>& st, int p, const R
                                             R& wt) {
     R s[4 * C];
     st.get(p, s);
-    R L = e[0] * s[0], L1 = g[1] * s[1], L2 = h[1] * s[1];
+    R L = e[0] * s[0], L1 = g[C] * s[C], L2 = h[C] * s[C];
 #pragma unroll
-    for (int q = 1; q < 4 * C; ++q) {
+    for (int z = 1; z < 4 * C; ++z) {
+        const int q = (z & 3) * C + (z >> 2);  // categories outermost
         L = fma(e[q], s[q], L);
-        if ((q & 3) != 0 && q != 1) {
+        if ((z & 3) != 0 && z != 1) {
             L1 = fma(g[q], s[q], L1);
             L2 = fma(h[q], s[q], L2);
         }
@@ -1914,10 +2018,10 @@ __device__ double newton_solve(const Model& M, const Cfg& cfg, const STab<R, C>&
             // over the first warps so their FP64 work runs on several schedulers
             converged = ns.done == 1;
             for (int x = threadIdx.x; x < 16 * C; x += blockDim.x) {
-                const int r = x >> 4, ij = x & 15;
+                const int r = x % C, ij = x / C;
                 double acc = 0.0;
 #pragma unroll
-                for (int k = 0; k < 4; ++k) acc += ns.W[ij * 4 + k] * ns.ex[r * 4 + k];
+                for (int k = 0; k < 4; ++k) acc += ns.W[ij * 4 + k] * ns.ex[k * C + r];
                 Pdst[x] = (R)acc;
             }
             __syncthreads();
@@ -1944,12 +2048,13 @@ __device__ __forceinline__ double block_sum(double acc, double (*red)[2]) {
 }
 
 // Proposal: the four members A, X2 (at u) and B, Y2 (at v) around the new
-// edge, P matrices of the five final lengths as pairs (Ph/Pl [5][C*16]: central,
-// A, B, C, D; mbr = each member's branch); L_p across the central branch.
+// edge (slots of ld sites), P matrices of the five final lengths as pairs (Ph/Pl
+// [5][16*C]: central, A, B, C, D; mbr = each member's branch); L_p across the
+// central branch.
 template <int C, int K = 1>
 __device__ __noinline__ double propose_score_f2(const Src2<C>* mem, const int* mbr, const float* Ph, const float* Pl,
-                                                const double* pi, const int32_t* w, int p0, int p1, double (*red)[2],
-                                                double (*cx)[3], int* cseq) {
+                                                const double* pi, const int32_t* w, int ld, int p0, int p1,
+                                                double (*red)[2], double (*cx)[3], int* cseq) {
     float pih[4], pil[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -1964,21 +2069,29 @@ __device__ __noinline__ double propose_score_f2(const Src2<C>* mem, const int* m
         for (int m = 0; m < 4; ++m) kk += mem[m].tip ? 0 : mem[m].scl[p];
         F2 L{0.f, 0.f};
         int E = 0;
-        for (int r = 0; r < C; ++r) {
-            float xh[4], xl[4], yh[4], yl[4], th[4], tl[4];
-            f2_apply_src4<C>(Ph + mbr[0] * C * 16, Pl + mbr[0] * C * 16, mem[0], p, r, xh, xl);
-            f2_apply_src4<C>(Ph + mbr[1] * C * 16, Pl + mbr[1] * C * 16, mem[1], p, r, th, tl);
-            f2_mul4(xh, xl, th, tl);
-            f2_apply_src4<C>(Ph + mbr[2] * C * 16, Pl + mbr[2] * C * 16, mem[2], p, r, yh, yl);
-            f2_apply_src4<C>(Ph + mbr[3] * C * 16, Pl + mbr[3] * C * 16, mem[3], p, r, th, tl);
-            f2_mul4(yh, yl, th, tl);
-            const int e = f2_normalise4(xh, xl) + f2_normalise4(yh, yl);
-            f2_apply4(Ph + r * 16, Pl + r * 16, yh, yl, th, tl);  // across the central branch (branch 0)
-            F2 Lr{0.f, 0.f};
+        using T = typename Lanes<C>::T;
+#pragma unroll 1
+        for (int g = 0; g < Lanes<C>::n; ++g) {
+            F2T<T> x[4], y[4], t[4];
+            f2_apply_src4<C>(Ph + mbr[0] * C * 16, Pl + mbr[0] * C * 16, mem[0], ld, p, g, x);
+            f2_apply_src4<C>(Ph + mbr[1] * C * 16, Pl + mbr[1] * C * 16, mem[1], ld, p, g, t);
+            f2_mul4<T>(x, t);
+            f2_apply_src4<C>(Ph + mbr[2] * C * 16, Pl + mbr[2] * C * 16, mem[2], ld, p, g, y);
+            f2_apply_src4<C>(Ph + mbr[3] * C * 16, Pl + mbr[3] * C * 16, mem[3], ld, p, g, t);
+            f2_mul4<T>(y, t);
+            int ex[Lanes<C>::w], ey[Lanes<C>::w];
+            f2_normalise4(x, ex);
+            f2_normalise4(y, ey);
+            f2_apply4<C>(Ph, Pl, g, y, t);  // across the central branch (branch 0)
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
-                Lr = f2_add(Lr, f2_mul(f2_mul(F2{xh[i], xl[i]}, F2{th[i], tl[i]}), F2{pih[i], pil[i]}));
-            f2_merge(L, E, Lr, e);
+            for (int i = 0; i < 4; ++i) x[i] = t2_mul<T>(x[i], t[i]);
+#pragma unroll
+            for (int k = 0; k < Lanes<C>::w; ++k) {
+                F2 Lr{0.f, 0.f};
+#pragma unroll
+                for (int i = 0; i < 4; ++i) Lr = f2_add(Lr, f2_mul(lane_of(x[i], k), F2{pih[i], pil[i]}));
+                f2_merge(L, E, Lr, ex[k] + ey[k]);
+            }
         }
         L = F2{L.h * (1.0f / C), L.l * (1.0f / C)};  // 1/C is a power of two for C = 1, 2, 4
         acc += (double)w[p] * f2_log(L, E - Prec<float>::kScaleExp * kk);
@@ -2031,40 +2144,37 @@ __device__ __noinline__ double fullopt_score_f2(int n, const int32_t* ch, const 
         __syncthreads();
         for (int z = threadIdx.x; z < nm * 16 * C; z += blockDim.x) {
             const int k = z / (16 * C), q = z % (16 * C);
-            f2_pmat_entry(W, exf + k * 4 * C, q, Pf + k * 16 * C, Pfl + k * 16 * C);
+            f2_pmat_entry<C>(W, exf + k * 4 * C, q, Pf + k * 16 * C, Pfl + k * 16 * C);
         }
         __syncthreads();
         const Src2<C> s0 = src(c0), s1 = src(c1);
         for (int p = threadIdx.x; p < Pl; p += blockDim.x) {
-            const int kk = (s0.tip ? 0 : s0.scl[p]) + (s1.tip ? 0 : s1.scl[p]);
             if (v > n) {
-                float dh[4 * C], dl[4 * C];
-#pragma unroll
-                for (int r = 0; r < C; ++r) {
-                    float th[4], tl[4];
-                    f2_apply_src4<C>(Pf, Pfl, s0, p, r, dh + 4 * r, dl + 4 * r);
-                    f2_apply_src4<C>(Pf + 16 * C, Pfl + 16 * C, s1, p, r, th, tl);
-                    f2_mul4(dh + 4 * r, dl + 4 * r, th, tl);
-                }
-                const int sc = f2_rescale<C>(dh, dl);
-                f2_store<C>(clv + (size_t)(v - n) * sstride, clv + (size_t)(n - 2 + (v - n - 1)) * sstride, p, dh, dl);
-                scl[(size_t)(v - n) * Ps + p] = kk + sc;
+                f2_join<C>(Pf, Pfl, s0, Pf + 16 * C, Pfl + 16 * C, s1, Ps, p, clv + (size_t)(v - n) * sstride,
+                           clv + (size_t)(n - 2 + (v - n - 1)) * sstride, scl + (size_t)(v - n) * Ps);
             } else {
+                const int kk = (s0.tip ? 0 : s0.scl[p]) + (s1.tip ? 0 : s1.scl[p]);
                 const int code = tips0[p];  // leaf 0
                 F2 L{0.f, 0.f};
                 int E = 0;
-                for (int r = 0; r < C; ++r) {
-                    float dh[4], dl[4], th[4], tl[4];
-                    f2_apply_src4<C>(Pf, Pfl, s0, p, r, dh, dl);
-                    f2_apply_src4<C>(Pf + 16 * C, Pfl + 16 * C, s1, p, r, th, tl);
-                    f2_mul4(dh, dl, th, tl);
-                    const int e = f2_normalise4(dh, dl);
-                    f2_apply4(Pf + 32 * C + 16 * r, Pfl + 32 * C + 16 * r, dh, dl, th, tl);
-                    F2 Lr{0.f, 0.f};
+                using T = typename Lanes<C>::T;
+#pragma unroll 1
+                for (int g = 0; g < Lanes<C>::n; ++g) {
+                    F2T<T> d[4], t[4];
+                    int e[Lanes<C>::w];
+                    f2_apply_src4<C>(Pf, Pfl, s0, Ps, p, g, d);
+                    f2_apply_src4<C>(Pf + 16 * C, Pfl + 16 * C, s1, Ps, p, g, t);
+                    f2_mul4<T>(d, t);
+                    f2_normalise4(d, e);
+                    f2_apply4<C>(Pf + 32 * C, Pfl + 32 * C, g, d, t);
 #pragma unroll
-                    for (int i = 0; i < 4; ++i)
-                        if (code >= 4 || code == i) Lr = f2_add(Lr, f2_mul(F2{th[i], tl[i]}, F2{pih[i], pil[i]}));
-                    f2_merge(L, E, Lr, e);
+                    for (int k = 0; k < Lanes<C>::w; ++k) {
+                        F2 Lr{0.f, 0.f};
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                            if (code >= 4 || code == i) Lr = f2_add(Lr, f2_mul(lane_of(t[i], k), F2{pih[i], pil[i]}));
+                        f2_merge(L, E, Lr, e[k]);
+                    }
                 }
                 L = F2{L.h * (1.0f / C), L.l * (1.0f / C)};
                 acc += (double)w0[p] * f2_log(L, E - Prec<float>::kScaleExp * kk);
@@ -2080,7 +2190,7 @@ __device__ __noinline__ double fullopt_score_f2(int n, const int32_t* ch, const 
 }
 
 // ---------------------------------------------------------------- P matrices of tree sets
-// Pm[tree][v][r][16] for v = 1..NN-1 (edge (v, up v)); row per thread.
+// Pm[tree][v][16][C] for v = 1..NN-1 (edge (v, up v)); a row of one category per thread.
 // Pm_lo (FP32 only, may be null): the rounding residuals, P - Pm (pairs for the scores).
 template <typename R>
 __global__ void k_pmats(Model M, TreeSet ts, int first, DCount cnt, R* Pm, const double* rates, float* Pm_lo) {
@@ -2096,18 +2206,18 @@ __global__ void k_pmats(Model M, TreeSet ts, int first, DCount cnt, R* Pm, const
         int t = (int)(y / NN);
         double l = ts.len[(size_t)(first + t) * NN + v];
         const double rr = rates ? rates[(size_t)(first + t) * kMaxCat + r] : M.rates[r];
-        const size_t o = (((size_t)t * NN + v) * C + r) * 16 + i * 4;
+        const size_t o = ((size_t)t * NN + v) * C * 16 + i * 4 * C + r;
         if (Pm_lo) {
             double row[4];
             pmat_row<double>(M, l * rr, i, row);
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const F2 x = f2_of(row[j]);
-                Pm[o + j] = (R)x.h;
-                Pm_lo[o + j] = x.l;
+                Pm[o + j * C] = (R)x.h;
+                Pm_lo[o + j * C] = x.l;
             }
         } else {
-            pmat_row<R>(M, l * rr, i, Pm + o);
+            pmat_row<R>(M, l * rr, i, Pm + o, C);
         }
     }
 }
@@ -2142,12 +2252,11 @@ __global__ void k_partials(Model M, Aln A, TreeSet ts, int first, DCount cnt, Cl
         R y0[4 * C], y1[4 * C];
         int c0cnt, c1cnt;
         int c0 = ch[2 * v], c1 = ch[2 * v + 1];
-        apply_p<R, C>(Pm + (size_t)c0 * C * 16, srcD(c0), p, y0, c0cnt);
-        apply_p<R, C>(Pm + (size_t)c1 * C * 16, srcD(c1), p, y1, c1cnt);
-#pragma unroll
-        for (int q = 0; q < 4 * C; ++q) y0[q] *= y1[q];
+        apply_p<R, C>(Pm + (size_t)c0 * C * 16, srcD(c0), P, p, y0, c0cnt);
+        apply_p<R, C>(Pm + (size_t)c1 * C * 16, srcD(c1), P, p, y1, c1cnt);
+        mul_vec<R, C>(y0, y1);
         int sc = rescale<R, C>(y0);
-        store_vec<R, C>(clv + (size_t)(v - n) * sstride, p, y0);
+        store_vec<R, C>(clv + (size_t)(v - n) * sstride, P, p, y0);
         scl[(size_t)(v - n) * P + p] = c0cnt + c1cnt + sc;
     }
     if (!with_up) return;
@@ -2159,13 +2268,12 @@ __global__ void k_partials(Model M, Aln A, TreeSet ts, int first, DCount cnt, Cl
         else { a.clv = clv + (size_t)(n - 2 + u - n - 1) * sstride; a.scl = scl + (size_t)(n - 2 + u - n - 1) * P; a.tip = nullptr; }
         R y0[4 * C], y1[4 * C];
         int cs, ca;
-        apply_p<R, C>(Pm + (size_t)sib * C * 16, srcD(sib), p, y0, cs);
-        apply_p<R, C>(Pm + (size_t)u * C * 16, a, p, y1, ca);
-#pragma unroll
-        for (int q = 0; q < 4 * C; ++q) y0[q] *= y1[q];
+        apply_p<R, C>(Pm + (size_t)sib * C * 16, srcD(sib), P, p, y0, cs);
+        apply_p<R, C>(Pm + (size_t)u * C * 16, a, P, p, y1, ca);
+        mul_vec<R, C>(y0, y1);
         int sc = rescale<R, C>(y0);
         const int slot = n - 2 + (v - n - 1);
-        store_vec<R, C>(clv + (size_t)slot * sstride, p, y0);
+        store_vec<R, C>(clv + (size_t)slot * sstride, P, p, y0);
         scl[(size_t)slot * P + p] = cs + ca + sc;
     }
 }
@@ -2203,14 +2311,8 @@ __global__ void k_partials_f2(Model M, Aln A, TreeSet ts, int first, DCount cnt,
         return v < n ? Src2<C>{nullptr, nullptr, nullptr, A.tips + (size_t)v * P} : slot_src(v - n);
     };
     auto make = [&](int slot, int a, const Src2<C>& sa, int b, const Src2<C>& sb) {
-        float yh[4 * C], yl[4 * C], zh[4 * C], zl[4 * C];
-        int ka, kb;
-        f2_apply_src<C>(Ph + (size_t)a * C * 16, Pl + (size_t)a * C * 16, sa, p, yh, yl, ka);
-        f2_apply_src<C>(Ph + (size_t)b * C * 16, Pl + (size_t)b * C * 16, sb, p, zh, zl, kb);
-        f2_mul_vec<C>(yh, yl, zh, zl);
-        const int sc = f2_rescale<C>(yh, yl);
-        f2_store<C>(clv + (size_t)slot * sstride, clo + (size_t)slot * sstride, p, yh, yl);
-        scl[(size_t)slot * P + p] = ka + kb + sc;
+        f2_join<C>(Ph + (size_t)a * C * 16, Pl + (size_t)a * C * 16, sa, Ph + (size_t)b * C * 16, Pl + (size_t)b * C * 16,
+                   sb, P, p, clv + (size_t)slot * sstride, clo + (size_t)slot * sstride, scl + (size_t)slot * P);
     };
     for (int v = NN - 1; v >= n; --v) make(v - n, ch[2 * v], srcD(ch[2 * v]), ch[2 * v + 1], srcD(ch[2 * v + 1]));
     if (!with_up) return;
@@ -2364,15 +2466,15 @@ __global__ void __launch_bounds__(512) k_propose(const PropGroup* __restrict__ g
         if (G.init) {  // P matrices at the learned starting lengths (the others are the parent's)
             for (int z = threadIdx.x; z < 5 * 4 * C; z += blockDim.x) {
                 const int b = z / (4 * C), q = z % (4 * C);
-                if (sm.warm[b]) sm.ex5[b][q] = exp(M.lam[q & 3] * rr[q >> 2] * sm.T[b]);
+                if (sm.warm[b]) sm.ex5[b][q] = exp(M.lam[q / C] * rr[q % C] * sm.T[b]);
             }
             __syncthreads();
             for (int z = threadIdx.x; z < 5 * 16 * C; z += blockDim.x) {
-                const int b = z / (16 * C), q = z % (16 * C), r = q >> 4, ij = q & 15;
+                const int b = z / (16 * C), q = z % (16 * C), r = q % C, ij = q / C;
                 if (!sm.warm[b]) continue;
                 double acc = 0.0;
 #pragma unroll
-                for (int k = 0; k < 4; ++k) acc += sm.ns.W[ij * 4 + k] * sm.ex5[b][r * 4 + k];
+                for (int k = 0; k < 4; ++k) acc += sm.ns.W[ij * 4 + k] * sm.ex5[b][k * C + r];
                 sm.Pm[b][q] = (R)acc;
             }
             __syncthreads();
@@ -2400,23 +2502,20 @@ __global__ void __launch_bounds__(512) k_propose(const PropGroup* __restrict__ g
                     const int p = p0 + pl;
                     R X[4 * C], Y[4 * C], t0[4 * C], t1[4 * C];
                     int k0, k1, k2, k3;
-                    apply_p<R, C>(P0, a0, p, t0, k0);
-                    apply_p<R, C>(P1, a1, p, t1, k1);
-#pragma unroll
-                    for (int q = 0; q < 4 * C; ++q) t0[q] *= t1[q];
+                    apply_p<R, C>(P0, a0, P, p, t0, k0);
+                    apply_p<R, C>(P1, a1, P, p, t1, k1);
+                    mul_vec<R, C>(t0, t1);
                     if (b == 0) {
 #pragma unroll
                         for (int q = 0; q < 4 * C; ++q) X[q] = t0[q];
-                        apply_p<R, C>(P2, a2, p, t0, k2);
-                        apply_p<R, C>(P3, a3, p, t1, k3);
-#pragma unroll
-                        for (int q = 0; q < 4 * C; ++q) Y[q] = t0[q] * t1[q];
+                        apply_p<R, C>(P2, a2, P, p, Y, k2);
+                        apply_p<R, C>(P3, a3, P, p, t1, k3);
+                        mul_vec<R, C>(Y, t1);
                     } else {
                         apply_p_reg<R, C>(sm.Pm[0], t0, X);  // X used as scratch for the far side
-                        apply_p<R, C>(P2, a2, p, t1, k2);
-#pragma unroll
-                        for (int q = 0; q < 4 * C; ++q) Y[q] = t1[q] * X[q];
-                        load_raw<R, C>(a3, p, X, k3);
+                        apply_p<R, C>(P2, a2, P, p, Y, k2);
+                        mul_vec<R, C>(Y, X);
+                        load_raw<R, C>(a3, P, p, X, k3);
                     }
                     // b > 0: X is the member's stored vector (kept above 2^-kScaleExp by the
                     // rescaling) or a tip, so it needs no normalisation: its scale multiplies
@@ -2454,7 +2553,7 @@ __global__ void __launch_bounds__(512) k_propose(const PropGroup* __restrict__ g
                 __syncthreads();
                 for (int z = threadIdx.x; z < 5 * 16 * C; z += blockDim.x) {
                     const int b = z / (16 * C), q = z % (16 * C);
-                    f2_pmat_entry(sm.ns.W, sm.ex5[b], q, reinterpret_cast<float*>(sm.Pm[b]), sm.Plo[b]);
+                    f2_pmat_entry<C>(sm.ns.W, sm.ex5[b], q, reinterpret_cast<float*>(sm.Pm[b]), sm.Plo[b]);
                 }
                 __syncthreads();
                 Src2<C> mem[4];
@@ -2463,7 +2562,7 @@ __global__ void __launch_bounds__(512) k_propose(const PropGroup* __restrict__ g
                     mem[m] = Src2<C>{reinterpret_cast<const float*>(sm.msrc[m].clv), sm.mlo[m], sm.msrc[m].scl,
                                      sm.msrc[m].tip};
                 f1 = propose_score_f2<C, K>(mem, sm.mbr, reinterpret_cast<const float*>(sm.Pm), &sm.Plo[0][0], M.pi,
-                                            G.A.w, p0, p1, sm.ns.red, sm.ns.cx, &cseq);
+                                            G.A.w, P, p0, p1, sm.ns.red, sm.ns.cx, &cseq);
             } else {
                 f1 = eval_lnl<R, C, K>(M, st, Pl, tlast, sm.ns, &cseq);
             }
@@ -2616,7 +2715,7 @@ __global__ void __launch_bounds__(512) k_fullopt(const FullGroup* __restrict__ g
         __syncthreads();
         for (int z = threadIdx.x; z < NN * C * 4; z += blockDim.x) {
             const int v = z / (C * 4), r = (z / 4) % C, i = z & 3;
-            if (v > 0) pmat_row<R>(M, len[v] * rr[r], i, Pm + ((size_t)v * C + r) * 16 + i * 4);
+            if (v > 0) pmat_row<R>(M, len[v] * rr[r], i, Pm + (size_t)v * C * 16 + i * 4 * C + r, C);
         }
         __syncthreads();
         auto srcD = [&](int v) {
@@ -2636,12 +2735,11 @@ __global__ void __launch_bounds__(512) k_fullopt(const FullGroup* __restrict__ g
             for (int p = threadIdx.x; p < Pl; p += blockDim.x) {
                 R y0[4 * C], y1[4 * C];
                 int k0, k1;
-                apply_p<R, C>(Pm + (size_t)c0 * C * 16, srcD(c0), p, y0, k0);
-                apply_p<R, C>(Pm + (size_t)c1 * C * 16, srcD(c1), p, y1, k1);
-#pragma unroll
-                for (int q = 0; q < 4 * C; ++q) y0[q] *= y1[q];
+                apply_p<R, C>(Pm + (size_t)c0 * C * 16, srcD(c0), Ps, p, y0, k0);
+                apply_p<R, C>(Pm + (size_t)c1 * C * 16, srcD(c1), Ps, p, y1, k1);
+                mul_vec<R, C>(y0, y1);
                 const int sc = rescale<R, C>(y0);
-                store_vec<R, C>(clv + (size_t)(v - n) * sstride, p, y0);
+                store_vec<R, C>(clv + (size_t)(v - n) * sstride, Ps, p, y0);
                 scl[(size_t)(v - n) * Ps + p] = k0 + k1 + sc;
             }
         };
@@ -2653,23 +2751,22 @@ __global__ void __launch_bounds__(512) k_fullopt(const FullGroup* __restrict__ g
                 int cx, cy;
                 // D_v first: its load then overlaps the two below instead of waiting
                 // behind the store of U_v (the same array, so it could not be hoisted)
-                load_raw<R, C>(srcD(v), p, Y, cy);
+                load_raw<R, C>(srcD(v), Ps, p, Y, cy);
                 if (v == n) {
-                    load_raw<R, C>(tip0, p, X, cx);
+                    load_raw<R, C>(tip0, Ps, p, X, cx);
                 } else {
                     const int u = up[v];
                     const int sib = ch[2 * u] == v ? ch[2 * u + 1] : ch[2 * u];
                     R y1[4 * C];
                     int k0, k1;
-                    apply_p<R, C>(Pm + (size_t)sib * C * 16, srcD(sib), p, X, k0);
-                    apply_p<R, C>(Pm + (size_t)u * C * 16, u == n ? tip0 : srcU(u), p, y1, k1);
-#pragma unroll
-                    for (int q = 0; q < 4 * C; ++q) X[q] *= y1[q];
+                    apply_p<R, C>(Pm + (size_t)sib * C * 16, srcD(sib), Ps, p, X, k0);
+                    apply_p<R, C>(Pm + (size_t)u * C * 16, u == n ? tip0 : srcU(u), Ps, p, y1, k1);
+                    mul_vec<R, C>(X, y1);
                     const int sc = rescale<R, C>(X);
                     cx = k0 + k1 + sc;
                     if (v >= n) {
                         const int slot = n - 2 + (v - n - 1);
-                        store_vec<R, C>(clv + (size_t)slot * sstride, p, X);
+                        store_vec<R, C>(clv + (size_t)slot * sstride, Ps, p, X);
                         scl[(size_t)slot * Ps + p] = cx;
                     }
                 }

@@ -404,7 +404,10 @@ __global__ void k_slot_summary(Aln A, ClvGroup g, DCount ntrees, int nslot, floa
     for (int p = threadIdx.x; p < A.P; p += blockDim.x) {
         float v[4 * C], s = 0.f;
 #pragma unroll
-        for (int q = 0; q < 4 * C; ++q) { v[q] = (float)base[(size_t)p * 4 * C + q]; s += v[q]; }
+        for (int q = 0; q < 4 * C; ++q) {  // [category][state], as the features are
+            v[q] = (float)base[vec_index<R>(A.P, p, (q & 3) * C + (q >> 2))];
+            s += v[q];
+        }
         const float w = (float)A.w[p], f = s > 0.f ? w / s : 0.f;
 #pragma unroll
         for (int q = 0; q < 4 * C; ++q) acc[q] += v[q] * f;
