@@ -8,6 +8,8 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <array>
+#include <climits>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -86,6 +88,7 @@ struct Ctx {
     bool autotune = false;
     std::string tune_path;
     std::map<std::string, Tune> tune;
+    std::map<std::array<int, 8>, int> occ;  // resident CTAs by launch shape (see occupancy)
     // learned warm start: FP32 master weights, gradients, Adam moments, BF16 copies
     float* mlp_w = nullptr;
     float* mlp_g = nullptr;
@@ -439,35 +442,113 @@ std::string tune_key(int prec, int C, int n, int P) {
 const int kTuneThreads[] = {64, 96, 128, 192, 256, 384, 512};
 const int kTuneClusterThreads[] = {128, 256, 512};
 const int kClusters[] = {2, 4, 8};
+size_t nn_pmat(int n, int C) { return ((size_t)(2 * n - 2) * C * 16 * 4 + 15) & ~size_t(15); }
+// Occupancy queries cost microseconds each: kept per context by their arguments.
+template <typename F>
+int occupancy(Ctx& c, const std::array<int, 8>& key, F query) {
+    auto it = c.occ.find(key);
+    if (it == c.occ.end()) it = c.occ.emplace(key, query()).first;
+    return it->second;
+}
 
-// CTAs per proposal when not tuned: one while the whole sum-table fits in a
-// CTA's shared memory; else the smallest cluster whose share leaves room for
-// two CTAs per SM (the sum-table would otherwise stream through L2/HBM at
-// every Newton evaluation).
-// Default CTAs per item of an untuned launch: one CTA when its sum-table fits in
-// shared memory; else the smallest thread-block cluster whose shares leave room
-// for two CTAs per SM (a resident grid of at least 1.9 x the SMs), the shape
-// the tuner picks at 128 taxa x 5908 patterns; failing that, the smallest
-// cluster that launches at all.
-template <typename Grid>
-int pick_cluster(const Ctx& c, int prec, int C, Grid grid) {
+// Default summation geometry (Geo: shares per item, virtual threads per share) of an
+// untuned launch: one share when its sum-table, with 72 bytes per site, fits in a
+// CTA's shared memory; else the smallest number of shares whose CTAs fit two to an
+// SM (a resident grid of at least 1.9 x the SMs); failing that, the smallest that
+// launches at all.  The byte counts are constants of this rule, not of the
+// kernels: the geometry fixes the rounding of the Newton sums, so it must not move
+// when a kernel's shared memory does.  How the geometry is spread over the GPU is
+// pick_shape's choice.
+size_t geometry_bytes(bool full, int prec, int C, int n, int P) {
+    const size_t rs = prec == PT_PREC_FP64 ? 8 : 4, nn = (size_t)(2 * n - 2);
+    const size_t fixed = full ? 6240 + ((nn * 8 + 15) & ~size_t(15)) : 7744;
+    return fixed + (4 * (size_t)C + 2) * rs * (size_t)((P + 3) & ~3) + 16;
+}
+int default_shares(Ctx& c, bool full, int prec, int C, int n, int P, int threads) {
+    if (prec != PT_PREC_MIXED || C != 4) return 1;
+    size_t one = geometry_bytes(full, prec, C, n, P);
+    const size_t pb = nn_pmat(n, C);
+    if (full && threads >= 512 && one + pb <= (size_t)227 * 1024) one += pb;
+    if (one <= c.smem_optin) return 1;
     int any = 0;
     for (int K : kClusters) {
-        if (!propose_cluster_ok(prec, C, K)) continue;
-        const int g = grid(K);
+        if (K * ((threads + 31) / 32) > 64) continue;
+        size_t b = geometry_bytes(full, prec, C, n, cluster_sites(P, K));
+        if (full && threads >= 512 && b + pb <= (size_t)227 * 1024) b += pb;
+        const int g = b > (size_t)227 * 1024 ? 0 : occupancy(c, {4, full, K, threads, (int)b, 0, 0, 0}, [&] {
+            return geometry_resident(prec, C, full, K, threads, b, c.sm_count);
+        });
         if (g <= 0) continue;
         if (!any) any = K;
         if (10 * g >= 19 * c.sm_count) return K;
     }
     return any ? any : 1;
 }
-int default_cluster(const Ctx& c, int prec, int C, int P, int threads) {
-    if (propose_smem_bytes(prec, C, P, true, threads) <= c.smem_optin) return 1;
-    return pick_cluster(c, prec, C, [&](int K) { return propose_cluster_grid(prec, C, K, threads, P); });
+
+// A launch shape and the CTAs of it that are resident at once.
+struct ShapeFit {
+    Shape h;
+    int resident;
+};
+// The shapes of a summation geometry (vt virtual threads, vk shares), by increasing
+// cluster size: vk CTAs per item, then 2, 4, 8 as long as the lanes of a virtual
+// thread each get a site.
+std::vector<ShapeFit> shapes_of(Ctx& c, bool full, int prec, int C, int maxN, int maxP, int vt, int vk) {
+    std::vector<ShapeFit> v;
+    auto fit = [&](const Shape& h) {
+        return occupancy(c, {full, prec, C, maxN, maxP, h.geo.vt, h.geo.vk * 64 + h.kp, h.smem_tab}, [&] {
+            return full ? fullopt_resident(prec, C, h, maxN, maxP, c.sm_count)
+                        : propose_resident(prec, C, h, maxP, c.sm_count);
+        });
+    };
+    const int J = (cluster_sites(maxP, vk) + vt - 1) / vt;  // sites per virtual thread
+    for (int lanes = 1; vk * lanes <= 8 && (lanes == 1 || lanes < 2 * J); lanes *= 2) {
+        const Shape h{Geo{vt, vk, lanes}, vk * lanes, 1};
+        const int r = fit(h);
+        if (r > 0) v.push_back({h, r});
+    }
+    if (v.empty() && vk > 1) return shapes_of(c, full, prec, C, maxN, maxP, vt, 1);  // not launchable as clusters
+    if (v.empty()) {  // a sum-table too large for shared memory in every form
+        const Shape h{Geo{vt, 1, 1}, 1, 0};
+        v.push_back({h, std::max(fit(h), c.sm_count)});
+    }
+    return v;
 }
-int default_full_cluster(const Ctx& c, int prec, int C, int maxN, int P, int threads) {
-    if (fullopt_smem_bytes(prec, C, maxN, P, true, threads) <= c.smem_optin) return 1;
-    return pick_cluster(c, prec, C, [&](int K) { return fullopt_cluster_grid(prec, C, K, threads, maxN, P); });
+// The shape for more items than are resident at once: the smallest cluster with
+// (nearly) the most resident threads.
+const ShapeFit& full_load(const std::vector<ShapeFit>& v) {
+    int most = 0;
+    for (const ShapeFit& x : v) most = std::max(most, x.resident);
+    for (const ShapeFit& x : v)
+        if (10 * x.resident >= 9 * most) return x;
+    return v.back();
+}
+// The shape for `total` items: the largest clusters that are all resident at once
+// (an item's time falls with the lanes and SMs it gets while the rest of the GPU
+// would idle), else full_load.
+const ShapeFit& pick_shape(const std::vector<ShapeFit>& v, long long total) {
+    for (size_t i = v.size(); i-- > 0;)
+        if (total * v[i].h.kp <= v[i].resident) return v[i];
+    return full_load(v);
+}
+// The shapes of a launch whose number of items is only known on the device (at
+// most cap): each with the counts (lo, hi] it is launched for, as pick_shape picks.
+struct ShapeRange {
+    ShapeFit f;
+    int lo, hi;
+};
+std::vector<ShapeRange> shape_ranges(const std::vector<ShapeFit>& v, int cap) {
+    std::vector<ShapeRange> out;
+    int lo = 0;
+    for (size_t i = v.size(); i-- > 0 && lo < cap;) {
+        const int hi = v[i].resident / v[i].h.kp;
+        if (hi > lo) {
+            out.push_back({v[i], lo, hi});
+            lo = hi;
+        }
+    }
+    if (lo < cap) out.push_back({full_load(v), lo, INT_MAX});
+    return out;
 }
 
 void save_tune(Ctx& c) {
@@ -577,7 +658,6 @@ void run_full_jobs(Ctx& c, std::vector<FullJob> jobs, bool allow_tune = true) {
         std::vector<int> counts;
         int maxN = 3, maxP = 1;
         const int C = jobs[0].a->M.C;
-        size_t slab_stride = 0;
         for (const FullJob& j : jobs) {
             AlnState& a = *j.a;
             if (a.M.C != C) fail(c, PT_ERR_INVALID_ARG, "alignments of one batch must share the number of categories");
@@ -595,42 +675,31 @@ void run_full_jobs(Ctx& c, std::vector<FullJob> jobs, bool allow_tune = true) {
             counts.push_back(j.count);
             maxN = std::max(maxN, a.n);
             maxP = std::max(maxP, a.P);
-            slab_stride = std::max(slab_stride, fullopt_slab_bytes(prec, C, a.n, a.P));
         }
         int total = 0;
         for (int x : counts) total += x;
         const int* gstart;
         int* counter;
         const FullGroup* dg = upload_groups(c, "full", groups, counts, &gstart, &counter);
-        // one launch at a given CTA size and number of CTAs per tree (a cluster
-        // of K shares each tree's sites); returns its device time when timed
+        // one launch of a summation geometry (threads, K shares per tree) in the shape
+        // that suits the number of trees; returns its device time when timed
         auto run = [&](int threads, int K, unsigned long long* stats, bool timed) {
-            const bool smem_tab = fullopt_smem_bytes(prec, C, maxN, maxP, true, threads) <= c.smem_optin;
-            int grid = 0;
+            const std::vector<ShapeFit> shapes = shapes_of(c, true, prec, C, maxN, maxP, threads, K);
+            const ShapeFit& f = pick_shape(shapes, total);
+            const int grid = (int)std::min<long long>((long long)total * f.h.kp, f.resident) / f.h.kp * f.h.kp;
             void* scratch = nullptr;
-            size_t spc = 0, sl = slab_stride;
-            if (K > 1) {
-                const int cgr = fullopt_cluster_grid(prec, C, K, threads, maxN, maxP);
-                grid = std::min(total * K, cgr) / K * K;
-                if (grid == 0) K = 1;
-                sl = 0;
-                for (const FullJob& j : jobs)
-                    sl = std::max(sl, fullopt_slab_bytes(prec, C, j.a->n, cluster_sites(j.a->P, K)));
+            size_t spc = 0, sl = 0;
+            if (!f.h.smem_tab) {
+                spc = (sumtable_bytes(prec, C, maxP) + 255) & ~size_t(255);
+                scratch = buf<unsigned char>(c, "full.scratch", spc * grid);
             }
-            if (K == 1) {
-                sl = slab_stride;
-                const int bps = std::max(1, fullopt_blocks_per_sm(prec, C, threads, smem_tab, maxN, maxP));
-                grid = std::min(total, bps * c.sm_count);
-                if (!smem_tab) {
-                    spc = (sumtable_bytes(prec, C, maxP) + 255) & ~size_t(255);
-                    scratch = buf<unsigned char>(c, "full.scratch", spc * grid);
-                }
-            }
+            for (const FullJob& j : jobs)
+                sl = std::max(sl, fullopt_slab_bytes(prec, C, j.a->n, geo_local(j.a->P, f.h.geo, threads)));
             unsigned char* slab = buf<unsigned char>(c, "full.slab", sl * grid);
             ck(c, cudaMemsetAsync(counter, 0, sizeof(int), c.stream), "counter");
             size_t e0 = timed ? ev_record(c) : 0;
-            launch_fullopt(c.stream, prec, C, dg, gstart, (int)groups.size(), counter, maxN, maxP, kcfg(c), stats,
-                           threads, grid, scratch, spc, slab, sl, K);
+            launch_fullopt(c.stream, prec, C, dg, gstart, (int)groups.size(), counter, maxN, maxP, kcfg(c), stats, f.h,
+                           grid, scratch, spc, slab, sl);
             ck(c, cudaGetLastError(), "full optimisation launch");
             float ms = 0.f;
             if (timed) {
@@ -641,7 +710,7 @@ void run_full_jobs(Ctx& c, std::vector<FullJob> jobs, bool allow_tune = true) {
             return (double)ms;
         };
         const std::string key = tune_key(prec, C, maxN, maxP);
-        int threads = threads_for(c, maxP), K = default_full_cluster(c, prec, C, maxN, maxP, threads_for(c, maxP));
+        int threads = threads_for(c, maxP), K = default_shares(c, true, prec, C, maxN, maxP, threads_for(c, maxP));
         const int dK = K;
         auto it = c.tune.find(key);
         const bool have = it != c.tune.end() && it->second.full_threads;
@@ -678,9 +747,9 @@ void run_full_jobs(Ctx& c, std::vector<FullJob> jobs, bool allow_tune = true) {
             std::vector<std::pair<int, int>> cands;
             for (int t : kTuneThreads) cands.push_back({t, 1});
             for (int k : kClusters)
-                if (propose_cluster_ok(prec, C, k) && (maxP + k - 1) / k >= 64)
+                if (prec == PT_PREC_MIXED && C == 4 && (maxP + k - 1) / k >= 64)
                     for (int t : kTuneClusterThreads)
-                        if (fullopt_cluster_grid(prec, C, k, t, maxN, maxP) > 0) cands.push_back({t, k});
+                        if (shapes_of(c, true, prec, C, maxN, maxP, t, k)[0].h.geo.vk == k) cands.push_back({t, k});
             int bt = threads, bK = K;
             for (auto [ct, kc] : cands) {
                 double ms = 1e30;
@@ -1156,27 +1225,19 @@ void expand_batch(Ctx& c, const std::vector<RoundIn>& ins, std::vector<RoundOut>
         int* counter;
         const PropGroup* dg = upload_groups(c, "prop", groups, counts, &gstart, &counter);
         auto run = [&](int threads, int K, unsigned long long* stats, bool timed) {
-            const bool smem_tab = propose_smem_bytes(prec, C, maxP, true, threads) <= c.smem_optin;
-            int grid = 0;
+            const std::vector<ShapeFit> shapes = shapes_of(c, false, prec, C, 3, maxP, threads, K);
+            const ShapeFit& f = pick_shape(shapes, tot);
+            const int grid = (int)std::min<long long>((long long)tot * f.h.kp, f.resident) / f.h.kp * f.h.kp;
             void* scratch = nullptr;
             size_t spc = 0;
-            if (K > 1) {  // clusters of K CTAs, each CTA a share of the sites
-                const int cgr = propose_cluster_grid(prec, C, K, threads, maxP);
-                grid = std::min(tot * K, cgr) / K * K;
-                if (grid == 0) K = 1;
-            }
-            if (K == 1) {
-                const int bps = std::max(1, propose_blocks_per_sm(prec, C, threads, smem_tab, maxP));
-                grid = std::min(tot, bps * c.sm_count);
-                if (!smem_tab) {
-                    spc = (sumtable_bytes(prec, C, maxP) + 255) & ~size_t(255);
-                    scratch = buf<unsigned char>(c, "prop.scratch", spc * grid);
-                }
+            if (!f.h.smem_tab) {
+                spc = (sumtable_bytes(prec, C, maxP) + 255) & ~size_t(255);
+                scratch = buf<unsigned char>(c, "prop.scratch", spc * grid);
             }
             ck(c, cudaMemsetAsync(counter, 0, sizeof(int), c.stream), "counter");
             size_t e0 = timed ? ev_record(c) : 0;
-            launch_propose(c.stream, prec, C, dg, gstart, (int)groups.size(), counter, kcfg(c), stats, threads, grid,
-                           scratch, spc, maxP, K);
+            launch_propose(c.stream, prec, C, dg, gstart, (int)groups.size(), counter, kcfg(c), stats, f.h, grid,
+                           scratch, spc, maxP);
             ck(c, cudaGetLastError(), "propose launch");
             float ms = 0.f;
             if (timed) {
@@ -1188,7 +1249,7 @@ void expand_batch(Ctx& c, const std::vector<RoundIn>& ins, std::vector<RoundOut>
         };
         const std::string key = tune_key(prec, C, maxN, maxP);
         int threads = threads_for(c, maxP);
-        int K = default_cluster(c, prec, C, maxP, threads);
+        int K = default_shares(c, false, prec, C, 3, maxP, threads);
         auto tt = c.tune.find(key);
         const bool have = tt != c.tune.end() && tt->second.prop_threads;
         if (have) {
@@ -1204,14 +1265,14 @@ void expand_batch(Ctx& c, const std::vector<RoundIn>& ins, std::vector<RoundOut>
             // in a cluster of K CTAs); single CTAs whose sum-table does not fit in shared
             // memory are tried at the default size only
             std::vector<std::pair<int, int>> cands;
-            const bool fits = propose_smem_bytes(prec, C, maxP, true, threads_for(c, maxP)) <= c.smem_optin;
+            const bool fits = shapes_of(c, false, prec, C, 3, maxP, threads_for(c, maxP), 1)[0].h.smem_tab;
             if (fits) for (int t : kTuneThreads) cands.push_back({t, 1});
             else cands.push_back({threads_for(c, maxP), 1});
             for (int k : kClusters)
-                if (propose_cluster_ok(prec, C, k) && (maxP + k - 1) / k >= 64)
+                if (prec == PT_PREC_MIXED && C == 4 && (maxP + k - 1) / k >= 64)
                     for (int t : kTuneClusterThreads)
-                        if (propose_cluster_grid(prec, C, k, t, maxP) > 0) cands.push_back({t, k});
-            const int dK = default_cluster(c, prec, C, maxP, threads_for(c, maxP));
+                        if (shapes_of(c, false, prec, C, 3, maxP, t, k)[0].h.geo.vk == k) cands.push_back({t, k});
+            const int dK = default_shares(c, false, prec, C, 3, maxP, threads_for(c, maxP));
             int bt = threads, bK = K;
             for (auto [ct, kc] : cands) {
                 double ms = 1e30;
@@ -1609,9 +1670,20 @@ void graph_free(Ctx& c, GraphRound* g) {
     delete g;
 }
 
+// CTAs of a recorded launch, and the slab of each of its full-optimisation CTAs.
+int range_grid(const ShapeRange& x) {
+    return (int)std::min<long long>((long long)x.hi * x.f.h.kp, x.f.resident) / x.f.h.kp * x.f.h.kp;
+}
+size_t graph_slab(const Ctx& c, const GraphRound& g, const ShapeRange& x) {
+    size_t b = 0;
+    for (const GraphAln& a : g.a)
+        b = std::max(b, fullopt_slab_bytes(c.cfg.precision, c.alns[a.aln].M.C, a.n, geo_local(a.P, x.f.h.geo, x.f.h.geo.vt)));
+    return b;
+}
+
 // The launch sequence of one graph round on stream s (recorded under capture).
-void graph_record(Ctx& c, GraphRound& g, cudaStream_t s, int C, int maxN, int maxP, int pgrid, size_t pspc,
-                  int fgrid, size_t fspc, size_t slab_stride) {
+void graph_record(Ctx& c, GraphRound& g, cudaStream_t s, int C, int maxN, int maxP,
+                  const std::vector<ShapeRange>& ps, size_t pspc, const std::vector<ShapeRange>& fs, size_t fspc) {
     const int na = g.na, prec = c.cfg.precision;
     int* di = g.di;
     for (GraphAln& x : g.a) {  // flags past the device counts must read as zero in the scans
@@ -1649,8 +1721,9 @@ void graph_record(Ctx& c, GraphRound& g, cudaStream_t s, int C, int maxN, int ma
     }
     launch_prefix_counts(s, na, di + g.oW(), di + g.oPerm(), di + g.oGSP());
     cudaMemsetAsync(di + g.oCP(), 0, sizeof(int), s);
-    launch_propose(s, prec, C, g.dpg, di + g.oGSP(), na, di + g.oCP(), kcfg(c), c.d_stats, g.prop_threads, pgrid,
-                   g.prop_scratch, pspc, maxP, g.prop_cluster);
+    for (const ShapeRange& x : ps)  // one of them runs, by the number of items
+        launch_propose(s, prec, C, g.dpg, di + g.oGSP(), na, di + g.oCP(), kcfg(c), c.d_stats, x.f.h, range_grid(x),
+                       g.prop_scratch, pspc, maxP, x.lo, x.hi);
     if (g.mlp)  // the judges take this round's proposals
         for (int k = 0; k < na; ++k) {
             GraphAln& x = g.a[k];
@@ -1668,8 +1741,9 @@ void graph_record(Ctx& c, GraphRound& g, cudaStream_t s, int C, int maxN, int ma
     }
     launch_prefix_counts(s, na, di + g.oK(), di + g.oPerm(), di + g.oGSF());
     cudaMemsetAsync(di + g.oCF(), 0, sizeof(int), s);
-    launch_fullopt(s, prec, C, g.dfg, di + g.oGSF(), na, di + g.oCF(), maxN, maxP, kcfg(c), c.d_stats,
-                   g.full_threads, fgrid, g.full_scratch, fspc, g.slab, slab_stride, g.full_cluster);
+    for (const ShapeRange& x : fs)
+        launch_fullopt(s, prec, C, g.dfg, di + g.oGSF(), na, di + g.oCF(), maxN, maxP, kcfg(c), c.d_stats, x.f.h,
+                       range_grid(x), g.full_scratch, fspc, g.slab, graph_slab(c, g, x), x.lo, x.hi);
     for (int k = 0; k < na; ++k) {
         GraphAln& x = g.a[k];
         AlnState& A = c.alns[x.aln];
@@ -1693,8 +1767,7 @@ GraphRound* graph_create(Ctx& c, const std::vector<int>& ids, const std::vector<
     GraphRound& g = *own;
     g.na = na;
     g.a.resize(na);
-    int C = -1, maxN = 3, maxP = 1, maxCap = 1;
-    size_t slab_stride = 0;
+    int C = -1, maxN = 3, maxP = 1, maxCap = 1, totCap = 0;
     for (int k = 0; k < na; ++k) {
         AlnState& A = aln_of(c, ids[k]);
         if (C < 0) C = A.M.C;
@@ -1717,7 +1790,7 @@ GraphRound* graph_create(Ctx& c, const std::vector<int>& ids, const std::vector<
         maxN = std::max(maxN, A.n);
         maxP = std::max(maxP, A.P);
         maxCap = std::max(maxCap, x.cap);
-        slab_stride = std::max(slab_stride, fullopt_slab_bytes(prec, C, A.n, A.P));
+        totCap = (int)std::min<long long>((long long)totCap + x.cap, INT_MAX);
     }
     if (c.cfg.propose_mode == PT_PROPOSE_FULL)
         fail(c, PT_ERR_INVALID_ARG, "graph rounds take five-branch or central proposals (not full radius)");
@@ -1727,8 +1800,8 @@ GraphRound* graph_create(Ctx& c, const std::vector<int>& ids, const std::vector<
     // CTA sizes: the autotuned ones of this problem bucket when known
     const std::string key = tune_key(prec, C, maxN, maxP);
     g.prop_threads = g.full_threads = threads_for(c, maxP);
-    g.prop_cluster = default_cluster(c, prec, C, maxP, g.prop_threads);
-    g.full_cluster = default_full_cluster(c, prec, C, maxN, maxP, g.full_threads);
+    g.prop_cluster = default_shares(c, false, prec, C, 3, maxP, g.prop_threads);
+    g.full_cluster = default_shares(c, true, prec, C, maxN, maxP, g.full_threads);
     auto tt = c.tune.find(key);
     if (tt != c.tune.end()) {
         if (tt->second.prop_threads) g.prop_threads = tt->second.prop_threads;
@@ -1736,36 +1809,17 @@ GraphRound* graph_create(Ctx& c, const std::vector<int>& ids, const std::vector<
         if (tt->second.full_threads) g.full_threads = tt->second.full_threads;
         if (tt->second.full_cluster) g.full_cluster = tt->second.full_cluster;
     }
-    bool ptab = propose_smem_bytes(prec, C, maxP, true, g.prop_threads) <= c.smem_optin;
-    const bool ftab = fullopt_smem_bytes(prec, C, maxN, maxP, true, g.full_threads) <= c.smem_optin;
-    int pgrid = std::max(1, propose_blocks_per_sm(prec, C, g.prop_threads, ptab, maxP)) * c.sm_count;
-    if (g.prop_cluster > 1) {  // clusters: every CTA's sum-table share in shared memory
-        const int cgrid = propose_cluster_grid(prec, C, g.prop_cluster, g.prop_threads, maxP);
-        if (cgrid > 0) {
-            pgrid = cgrid;
-            ptab = true;
-        } else {
-            g.prop_cluster = 1;
-        }
-    }
-    int fgrid = std::max(1, fullopt_blocks_per_sm(prec, C, g.full_threads, ftab, maxN, maxP)) * c.sm_count;
-    bool ftab2 = ftab;
-    if (g.full_cluster > 1) {  // the tuned cluster form of the visits, as pt_expand_batch runs them
-        const int cgrid = fullopt_cluster_grid(prec, C, g.full_cluster, g.full_threads, maxN, maxP);
-        if (cgrid > 0) {
-            fgrid = cgrid;
-            ftab2 = true;
-            slab_stride = 0;
-            for (int k = 0; k < na; ++k) {
-                const AlnState& A = c.alns[ids[k]];
-                slab_stride = std::max(slab_stride, fullopt_slab_bytes(prec, C, A.n, cluster_sites(A.P, g.full_cluster)));
-            }
-        } else {
-            g.full_cluster = 1;
-        }
-    }
+    const std::vector<ShapeRange>
+        ps = shape_ranges(shapes_of(c, false, prec, C, 3, maxP, g.prop_threads, g.prop_cluster), totCap),
+        fs = shape_ranges(shapes_of(c, true, prec, C, maxN, maxP, g.full_threads, g.full_cluster), totCap);
     const size_t tabb = (sumtable_bytes(prec, C, maxP) + 255) & ~size_t(255);
-    const size_t pspc = ptab ? 0 : tabb, fspc = ftab2 ? 0 : tabb;
+    size_t pscratch = 0, fscratch = 0, slab = 0;
+    for (const ShapeRange& x : ps)
+        if (!x.f.h.smem_tab) pscratch = std::max(pscratch, tabb * range_grid(x));
+    for (const ShapeRange& x : fs) {
+        if (!x.f.h.smem_tab) fscratch = std::max(fscratch, tabb * range_grid(x));
+        slab = std::max(slab, graph_slab(c, g, x) * range_grid(x));
+    }
     Arena ar;
     for (GraphAln& x : g.a) {
         const int n = x.n, E = x.E, cap = x.cap, F = x.F_cap;
@@ -1825,9 +1879,9 @@ GraphRound* graph_create(Ctx& c, const std::vector<int>& ids, const std::vector<
     ar.add(g.dpg, na);
     ar.add(g.dfg, na);
     ar.add(g.scan_tmp, (size_t)(maxCap + 1023) / 1024 + 2);
-    if (pspc) ar.addv(g.prop_scratch, pspc * pgrid);
-    if (fspc) ar.addv(g.full_scratch, fspc * fgrid);
-    ar.add(g.slab, slab_stride * fgrid);
+    if (pscratch) ar.addv(g.prop_scratch, pscratch);
+    if (fscratch) ar.addv(g.full_scratch, fscratch);
+    ar.add(g.slab, slab);
     dev_alloc(c, &g.mem, ar.total(), "allocating the graph round's buffers");
     ar.carve(g.mem);
     ck(c, cudaHostAlloc(reinterpret_cast<void**>(&g.hi), sizeof(int) * g.nints(), cudaHostAllocDefault), "pinned");
@@ -1898,7 +1952,7 @@ GraphRound* graph_create(Ctx& c, const std::vector<int>& ids, const std::vector<
     ck(c, cudaStreamCreateWithFlags(&g.cs, cudaStreamNonBlocking), "graph stream");
     ck(c, cudaStreamBeginCapture(g.cs, cudaStreamCaptureModeRelaxed), "begin capture");
     const long long k0 = launch_count();
-    graph_record(c, g, g.cs, C, maxN, maxP, pgrid, pspc, fgrid, fspc, slab_stride);
+    graph_record(c, g, g.cs, C, maxN, maxP, ps, tabb, fs, tabb);
     g.kernels = launch_count() - k0;
     cudaGraph_t graph = nullptr;
     ck(c, cudaStreamEndCapture(g.cs, &graph), "end capture");

@@ -99,8 +99,7 @@ enum {
 // start at clv + g * tree_stride (R elements), scalers at scl + g * scl_stride.
 // Slots: D_v (v inner, n-2 of them) then U_v (v inner except the first, n-3).
 // Mixed precision: clv_lo (same layout as clv) holds the FP32 residuals of
-// the partials, clv + clv_lo being the pair form the scores use; null when
-// absent (FP64 path, or partials made by the full optimisation itself).
+// the partials, clv + clv_lo being the pair form the scores use; null in FP64.
 struct ClvGroup {
     void* clv;
     int32_t* scl;
@@ -118,6 +117,35 @@ __device__ __forceinline__ size_t vec_index(int ld, int p, int f) {
     return ((size_t)(f / V) * ld + p) * V + f % V;
 }
 #endif
+
+// Sites per share when K shares split P sites (a multiple of 4).
+#ifdef __CUDACC__
+#define PT_INLINE __host__ __device__ inline
+#else
+#define PT_INLINE inline
+#endif
+PT_INLINE int cluster_sites(int P, int K) { return K > 1 ? ((P + K - 1) / K + 3) & ~3 : P; }
+
+// How an item's sites are summed, and spread over threads.  Summation geometry:
+// vk shares of cluster_sites(P, vk) consecutive sites, vt virtual threads per
+// share (it fixes the rounding of the FP32 Newton sums, so results depend on it
+// and on nothing else of a launch shape); lanes: lanes per virtual thread.
+struct Geo {
+    int vt, vk, lanes;
+};
+// A launch shape of the persistent kernels: clusters of kp = vk * lanes CTAs of
+// geo.vt threads per item; smem_tab 0: one CTA with its sum-table in global scratch.
+struct Shape {
+    Geo geo;
+    int kp, smem_tab;
+};
+// Local sites of one CTA of `threads` threads (its sum-table's and slab's capacity).
+PT_INLINE int geo_local(int P, const Geo& g, int threads) {
+    const int Ps = cluster_sites(P, g.vk), step = g.vt * g.lanes;
+    return g.lanes == 1 ? Ps : (Ps + step - 1) / step * threads;
+}
+// Warps of a cluster whose Newton sums one CTA receives: shapes above it are not offered.
+constexpr int kMaxTeamWarps = 128;
 
 // Work item of the proposal kernel: frontier tree, internal edge node, swap,
 // visited-table slot.
@@ -239,7 +267,7 @@ void launch_lengths_to_input(cudaStream_t s, int n, int count, TreeSet ts, doubl
 
 // Partials of a group of trees (all D_v, and U_v when with_up).
 // pm: P-matrix buffer of pmat_bytes(prec, C, n, count) bytes; launch_propose reads it for the same group.
-// Mixed precision with g.clv_lo set: the partials are made as pairs (h in clv, l in clv_lo).
+// Mixed precision: the partials are made as pairs (h in clv, l in clv_lo).
 size_t pmat_bytes(int prec, int C, int n, int count);
 // rates (may be null: the model's): per-tree category rates [tree][kMaxCat], indexed like ts.
 void launch_partials(cudaStream_t s, int prec, const Model& M, Aln A, TreeSet ts, int first, DCount count, ClvGroup g,
@@ -282,38 +310,31 @@ struct FullGroup {
 };
 // Batched launches over groups: gstart [ngroups + 1] is the prefix sum of the
 // groups' item (tree) counts (device); counter (device, zeroed) hands out the
-// items dynamically, in order, to the persistent CTAs.
-// cluster > 1 (FP32, 4 categories; 2, 4 or 8): thread-block clusters of that many CTAs
-// share each item, each CTA a contiguous share of the sites with its sum-table in
-// shared memory (scratch unused); grid is then a multiple of cluster.
+// items dynamically, in order, to the persistent CTAs (or clusters: grid is a
+// multiple of h.kp).  A launch does nothing unless its number of items is in
+// (lo, hi]: a recorded round, whose counts are only known on the device, issues
+// one launch per shape with the counts that shape is for.
+// scratch: sum-tables of scratch_per_cta bytes per CTA when h.smem_tab is 0.
 void launch_propose(cudaStream_t s, int prec, int C, const PropGroup* groups, const int* gstart, int ngroups,
-                    int* counter, Cfg cfg, unsigned long long* stats, int threads, int grid, void* scratch,
-                    size_t scratch_per_cta, int maxP, int cluster = 1);
-// Whether the proposal kernel has a cluster form for (precision, categories, cluster size).
-bool propose_cluster_ok(int prec, int C, int K);
-// Resident CTAs of the cluster form on the whole GPU (a multiple of K; 0 when it cannot run).
-int propose_cluster_grid(int prec, int C, int K, int threads, int maxP);
-// cluster > 1 (slab mode, FP32, 4 categories): clusters of that many CTAs share each tree,
-// each CTA a share of the sites (cluster_sites(P, cluster)) with its own slab of
-// slab_per_cta = fullopt_slab_bytes of the share; grid a multiple of cluster.
+                    int* counter, Cfg cfg, unsigned long long* stats, const Shape& h, int grid, void* scratch,
+                    size_t scratch_per_cta, int maxP, int lo = 0, int hi = 0x7fffffff);
+// slab: slab_per_cta = fullopt_slab_bytes of a CTA's local sites (geo_local) per CTA.
 void launch_fullopt(cudaStream_t s, int prec, int C, const FullGroup* groups, const int* gstart, int ngroups,
-                    int* counter, int maxN, int maxP, Cfg cfg, unsigned long long* stats, int threads, int grid,
-                    void* scratch, size_t scratch_per_cta, void* slab = nullptr, size_t slab_per_cta = 0,
-                    int cluster = 1);
-// Resident CTAs of the full optimisation's cluster form (a multiple of K; 0: cannot run).
-int fullopt_cluster_grid(int prec, int C, int K, int threads, int maxN, int maxP);
-// Sites per CTA when K CTAs share P sites (a multiple of 4).
-inline int cluster_sites(int P, int K) { return K > 1 ? ((P + K - 1) / K + 3) & ~3 : P; }
+                    int* counter, int maxN, int maxP, Cfg cfg, unsigned long long* stats, const Shape& h, int grid,
+                    void* scratch, size_t scratch_per_cta, void* slab, size_t slab_per_cta, int lo = 0,
+                    int hi = 0x7fffffff);
+// Resident CTAs of a shape on a GPU of sms SMs (a multiple of h.kp; 0: cannot run).
+int propose_resident(int prec, int C, const Shape& h, int maxP, int sms);
+int fullopt_resident(int prec, int C, const Shape& h, int maxN, int maxP, int sms);
+// Resident CTAs of the cluster kernels (FP32, 4 categories; else 0) at a given amount of
+// shared memory, for the default geometry's rule.
+int geometry_resident(int prec, int C, bool full, int K, int threads, size_t smem, int sms);
 // Bytes of one CTA's slab for trees of n taxa and P patterns (a multiple of 256): partials,
 // scalers and the P matrices of every edge.  Every full-optimisation launch passes slabs.
 size_t fullopt_slab_bytes(int prec, int C, int n, int P);
 
 // GTR+Gamma model set-up on the host (pt_api.cu); false on invalid parameters.
 bool host_build_model(const double exch[6], const double freqs[4], double alpha, int C, Model& M);
-
-// Resident CTAs per SM of the two persistent kernels at a given CTA size (occupancy API).
-int propose_blocks_per_sm(int prec, int C, int threads, bool smem_tab, int maxP);
-int fullopt_blocks_per_sm(int prec, int C, int threads, bool smem_tab, int maxN, int maxP);
 
 // Kernels launched so far by this process (all contexts).
 long long launch_count();
@@ -359,9 +380,9 @@ void launch_judge(cudaStream_t s, DCount count, const int32_t* evals, Judge* jud
 void launch_log_pairs(cudaStream_t s, const Item* items, int i0, int i1, const float* Xf, const double* len5, float* LX,
                       float* LT, unsigned long long* count, size_t cap);
 
-// Shared-memory sizing helpers for the host.
-size_t propose_smem_bytes(int prec, int C, int P, bool table_in_smem, int threads);
-size_t fullopt_smem_bytes(int prec, int C, int n, int P, bool table_in_smem, int threads);
-size_t sumtable_bytes(int prec, int C, int P);
+// Shared-memory sizing helpers for the host (ld: local sites of the sum-table; 0: none).
+size_t propose_smem_bytes(int prec, int C, int ld);
+size_t fullopt_smem_bytes(int prec, int C, int n, int ld, int threads);
+size_t sumtable_bytes(int prec, int C, int ld);
 
 }  // namespace pt

@@ -22,9 +22,11 @@
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <cstdint>
+#include <type_traits>
 
 namespace pt {
 
@@ -45,6 +47,7 @@ template <> struct Prec<float> {
     __device__ static float ex(float x) { return expf(x); }
     __device__ static float lg(float x) { return logf(x); }
     __device__ static float rcp(float x) { return __frcp_rn(x); }
+    __device__ static float mul(float x, float y) { return __fmul_rn(x, y); }  // never part of an FMA
 };
 template <> struct Prec<double> {
     static constexpr int kScaleExp = 256;
@@ -53,6 +56,7 @@ template <> struct Prec<double> {
     __device__ static double ex(double x) { return exp(x); }
     __device__ static double lg(double x) { return log(x); }
     __device__ static double rcp(double x) { return 1.0 / x; }
+    __device__ static double mul(double x, double y) { return __dmul_rn(x, y); }
 };
 
 // ---------------------------------------------------------------- hashing
@@ -826,8 +830,8 @@ __device__ __forceinline__ float pneg(float a) { return -a; }
 __device__ __forceinline__ float psub(float a, float b) { return __fsub_rn(a, b); }
 __device__ __forceinline__ f32x2 pair(const float* x) { return make_float2(x[0], x[1]); }
 
-// Source of a 4C-wide vector at a site: a tip (code lookup) or a stored slot
-// (its sites `ld` apart per chunk, see vec_index).
+// Source of a 4C-wide vector at a site: a tip (code lookup, by the site pg) or a
+// stored slot (`ld` sites per chunk, see vec_index; by the slot's index p).
 template <typename R, int C>
 struct Src {
     const R* clv;      // slot base (nullptr for a tip)
@@ -854,9 +858,9 @@ __device__ __forceinline__ void load_vec(const R* src, int ld, int p, R* x) {
 }
 
 template <typename R, int C>
-__device__ __forceinline__ void load_raw(const Src<R, C>& s, int ld, int p, R* x, int& cnt) {
+__device__ __forceinline__ void load_raw(const Src<R, C>& s, int ld, int p, int pg, R* x, int& cnt) {
     if (s.tip) {
-        int code = s.tip[p];
+        int code = s.tip[pg];
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
@@ -913,9 +917,9 @@ __device__ __forceinline__ void apply_p_reg(const R* Pm, const R* x, R* y) {
 // y_r = P_r x_r of a source; for a tip the product is a column of P (or all
 // ones for a gap).
 template <typename R, int C>
-__device__ __forceinline__ void apply_p(const R* Pm, const Src<R, C>& s, int ld, int p, R* y, int& cnt) {
+__device__ __forceinline__ void apply_p(const R* Pm, const Src<R, C>& s, int ld, int p, int pg, R* y, int& cnt) {
     if (s.tip) {
-        int code = s.tip[p];
+        int code = s.tip[pg];
         cnt = 0;
         if (code >= 4) {
 #pragma unroll
@@ -935,7 +939,7 @@ __device__ __forceinline__ void apply_p(const R* Pm, const Src<R, C>& s, int ld,
         return;
     }
     R x[4 * C];
-    load_raw<R, C>(s, ld, p, x, cnt);
+    load_raw<R, C>(s, ld, p, pg, x, cnt);
     apply_p_reg<R, C>(Pm, x, y);
 }
 
@@ -1148,15 +1152,15 @@ struct Src2 {
     const uint8_t* tip;
 };
 
-// Lane group g of y = P x for a pair source at site p (P: [16][C] pairs, slots
-// of ld sites).
+// Lane group g of y = P x for a pair source (P: [16][C] pairs): slot index p of
+// slots of ld sites, site pg of a tip row.
 template <int C>
-__device__ __forceinline__ void f2_apply_src4(const float* Ph, const float* Pl, const Src2<C>& s, int ld, int p, int g,
+__device__ __forceinline__ void f2_apply_src4(const float* Ph, const float* Pl, const Src2<C>& s, int ld, int p, int pg, int g,
                                               F2T<typename Lanes<C>::T>* y) {
     using T = typename Lanes<C>::T;
     constexpr int w = Lanes<C>::w;
     if (s.tip) {
-        const int code = s.tip[p];
+        const int code = s.tip[pg];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             T a, b;
@@ -1179,7 +1183,7 @@ __device__ __forceinline__ void f2_apply_src4(const float* Ph, const float* Pl, 
 // rescaled by 2^32 when every h is below 2^-32 (as rescale()), and its scaler count.
 template <int C>
 __device__ __forceinline__ void f2_join(const float* Pah, const float* Pal, const Src2<C>& a, const float* Pbh,
-                                        const float* Pbl, const Src2<C>& b, int ld, int p, float* dh, float* dl,
+                                        const float* Pbl, const Src2<C>& b, int ld, int p, int pg, float* dh, float* dl,
                                         int32_t* ds) {
     using T = typename Lanes<C>::T;
     constexpr int n = Lanes<C>::n, w = Lanes<C>::w;
@@ -1189,8 +1193,8 @@ __device__ __forceinline__ void f2_join(const float* Pah, const float* Pal, cons
 #pragma unroll
     for (int g = 0; g < n; ++g) {
         F2T<T> z[4];
-        f2_apply_src4<C>(Pah, Pal, a, ld, p, g, y[g]);
-        f2_apply_src4<C>(Pbh, Pbl, b, ld, p, g, z);
+        f2_apply_src4<C>(Pah, Pal, a, ld, p, pg, g, y[g]);
+        f2_apply_src4<C>(Pbh, Pbl, b, ld, p, pg, g, z);
         f2_mul4<T>(y[g], z);
 #pragma unroll
         for (int i = 0; i < 4; ++i) mx = fmaxf(mx, lane_max(y[g][i].h));
@@ -1238,14 +1242,6 @@ __device__ __forceinline__ void f2_pmat_entry(const double* W, const double* ex,
     const F2 v = f2_of(acc);
     Ph[q] = v.h;
     Pl[q] = v.l;
-}
-
-// L2 prefetch hint for [p, p + bytes): the block's threads request its
-// 128-byte lines in turn (every address lies inside the range).
-__device__ __forceinline__ void prefetch_l2(const void* p, size_t bytes) {
-    const char* c = static_cast<const char*>(p);
-    for (size_t o = (size_t)threadIdx.x * 128; o < bytes; o += (size_t)blockDim.x * 128)
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(c + o));
 }
 
 // threshold rescale of a stored vector
@@ -1340,14 +1336,61 @@ __device__ __forceinline__ void sumtable(const R* Mt, const R* pi, const R* X, c
     }
 }
 
-// Sum-table storage: chunk q (4 values for FP32 / 2 for FP64) of site p at
-// index q * pcap + p, so consecutive threads touch consecutive 16 bytes.
+// The sites of a CTA's threads.  Their FP32 Newton sums are rounded, so the sum
+// over the sites is defined by a launch-independent geometry: vk shares of
+// consecutive sites (cluster_sites), vt virtual threads per share, virtual
+// thread t of a share adding its sites t, t + vt, t + 2 vt, ... in that order,
+// and the virtual threads' sums added by one binary tree over their linear index
+// (neighbours first).  A launch spreads the vk * vt virtual threads over a cluster
+// of kp CTAs, each virtual thread over `lanes` neighbouring lanes that take its
+// sites in turn: the same sums, bit for bit, with as many SMs per item as the
+// number of items leaves room for.
+struct Sites {
+    int p0, step;    // site m of this thread: p0 + m * step,
+    int pl0, pstep;  // stored at local index pl0 + m * pstep
+    int cnt;         // this thread's sites
+    int M;           // the largest cnt of any thread
+    int lanes, jj;   // lanes per virtual thread, this thread's among them
+    int nt;          // sites of the virtual thread
+    int ld;          // local capacity
+};
+__device__ __forceinline__ Sites make_sites(int P, const Geo& g, int rank, int kp) {
+    Sites x;
+    const int Ps = cluster_sites(P, g.vk), pt = blockDim.x;
+    const int gv = (rank * pt + (int)threadIdx.x) / g.lanes, jj = (int)threadIdx.x % g.lanes;
+    const int vr = gv / g.vt, vt = gv - vr * g.vt;
+    const int start = min(P, vr * Ps), len = min(P, start + Ps) - start;
+    const int i0 = vt + g.vt * jj;
+    x.step = g.vt * g.lanes;
+    x.p0 = start + i0;
+    x.cnt = i0 < len ? (len - i0 + x.step - 1) / x.step : 0;
+    x.M = (Ps + x.step - 1) / x.step;
+    x.pl0 = threadIdx.x;
+    x.pstep = pt;
+    x.lanes = g.lanes;
+    x.jj = jj;
+    x.nt = vt < len ? (len - vt + g.vt - 1) / g.vt : 0;
+    x.ld = geo_local(P, g, pt);
+    return x;
+}
+
+// Sum-table storage: chunk q (16 bytes: 4 values in FP32, 2 in FP64) of local
+// site p at index q * pcap + p, so consecutive threads touch consecutive 16
+// bytes; then the site weights, and in FP64 the rows' exponents (the mixed path
+// scores from pairs, and its Newton ratios do not see a row's power of two).
 template <typename R, int C>
 struct STab {
     R* s;          // [nchunk][pcap] vec
-    R* ew;         // [2][pcap]: exponent, weight
+    R* w;          // [pcap] site weights, set once per item
+    R* e;          // [pcap] exponents (FP64)
     int pcap;
-    __device__ __forceinline__ void put(int p, const R* v, R E, R w) const {
+    __device__ __forceinline__ void init(unsigned char* base, int ld) {
+        pcap = (ld + 3) & ~3;
+        s = reinterpret_cast<R*>(base);
+        w = s + (size_t)4 * C * pcap;
+        e = w + pcap;
+    }
+    __device__ __forceinline__ void put(int p, const R* v, int E) const {
         if constexpr (sizeof(R) == 4) {
 #pragma unroll
             for (int q = 0; q < C; ++q)
@@ -1356,9 +1399,8 @@ struct STab {
 #pragma unroll
             for (int q = 0; q < 2 * C; ++q)
                 reinterpret_cast<double2*>(s)[(size_t)q * pcap + p] = make_double2(v[2 * q], v[2 * q + 1]);
+            e[p] = (R)E;
         }
-        ew[p] = E;
-        ew[pcap + p] = w;
     }
     __device__ __forceinline__ void get(int p, R* v) const {
         if constexpr (sizeof(R) == 4) {
@@ -1377,9 +1419,9 @@ struct STab {
     }
 };
 
-// Warps of one thread-block cluster whose Newton sums one CTA receives (K x warps
-// per CTA); launch shapes above it are not offered.
-constexpr int kMaxClusterWarps = 64;
+// Warps of one thread-block cluster whose Newton sums one CTA receives (CTAs x
+// warps per CTA); launch shapes above it are not offered.
+constexpr int kMaxClusterWarps = kMaxTeamWarps;
 // A CTA gives up waiting for its cluster's Newton sums after this many cycles
 // (about 2 s); the kernel then reports PT_ERR_TIMEOUT through its statistics.
 constexpr long long kExchangeWaitCycles = 1ll << 32;
@@ -1431,6 +1473,11 @@ __device__ __forceinline__ unsigned cluster_rank() {
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
     return r;
 }
+__device__ __forceinline__ unsigned cluster_ctas() {
+    unsigned r;
+    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+    return r;
+}
 // Sets up the two exchange barriers of a cluster CTA (once per launch, before its
 // first cluster barrier; thread 0): each phase takes one arrival per warp of the
 // CTA (its local entry) and one from the leader, which arms the remote bytes.
@@ -1446,9 +1493,8 @@ __device__ __forceinline__ void cluster_exchange_init(NS& ns) {
 // Block-wide context for the Newton machinery.
 template <typename R, int C>
 struct NewtonSmem {
-    R egh[3][4 * C];       // coefficients on the sum-table for L, dL/dt, d2L/dt2
-    double red[32][2];     // per-warp partial sums
-    float redf[32][4];     // per-warp partial sums as FP32 pairs (hi, lo) x (d1, d2)
+    alignas(16) R egh[3][4 * C];  // coefficients on the sum-table for L, dL/dt, d2L/dt2
+    double red[2][32];     // per-warp partial sums of scores, two alternating slots
     double lr[4 * C];      // lam_k * rate_r, [k][r] (as every 4C array here)
     float lrf[4 * C];      // the same in FP32 (coefficients of the Newton derivatives)
     double ex[4 * C];      // exp(lam_k r t) for a P-matrix refresh
@@ -1456,101 +1502,50 @@ struct NewtonSmem {
     double tb;             // broadcast of the current length
     int done;
     int leader;            // the warp that takes the Newton steps
-    double cx[2][3];       // cluster exchange: this CTA's partial sums, two alternating slots
-    alignas(16) float cxf[2][4];  // the same for FP32 pairs (d1 hi, lo, d2 hi, lo), read as float4
-    // Newton sums of a cluster (K > 1, FP32 pairs): every warp of every CTA pushes its
-    // (d1 h, l, d2 h, l) into entry rank * nw + warp of every CTA's slot, two
-    // alternating slots, each with an mbarrier that counts the bytes it received
+    // Newton sums: each warp's (d1 h, l, d2 h, l) in FP32 or (d1, d2) in FP64; in a
+    // cluster every warp of every CTA pushes its entry into entry rank * nw + warp of
+    // every CTA's slot, two alternating slots, each with an mbarrier that counts the
+    // bytes it received
     alignas(16) float cxr[2][kMaxClusterWarps][4];
     alignas(8) unsigned long long mbx[2];
     int abort_;            // a wait on mbx ran out: later waits are skipped (reported by the kernel)
 };
 
-// Sums of up to three values held by one thread (`writer`) of each CTA of a
-// thread-block cluster of K CTAs, returned to every thread of every CTA.  The
-// K partials are added in rank order, so every CTA gets the same bits (the
-// CTAs of a cluster then take identical Newton steps).  Every thread of every
-// CTA must call it the same number of times; `seq` (a per-thread count,
-// equal in all threads) alternates the slot, so a CTA writes a slot only
-// after every CTA has passed the barrier of the exchange that last read it.
-template <int K>
-__device__ __forceinline__ void cluster_sum(bool writer, double (*cx)[3], int& seq, double& a, double& b, double& c) {
-    namespace cg = cooperative_groups;
-    cg::cluster_group cl = cg::this_cluster();
-    const int s = seq & 1;
-    ++seq;
-    if (writer) {
-        cx[s][0] = a;
-        cx[s][1] = b;
-        cx[s][2] = c;
-    }
-    cl.sync();
-    double x = 0.0, y = 0.0, z = 0.0;
-#pragma unroll
-    for (int r = 0; r < K; ++r) {
-        const double* q = cl.map_shared_rank(&cx[s][0], r);
-        x += q[0];
-        y += q[1];
-        z += q[2];
-    }
-    a = x;
-    b = y;
-    c = z;
-}
+// A CTA's place in its cluster (the CTAs that share one item): kp CTAs, and the
+// exchanges made so far (equal in every thread of the cluster).
+struct Team {
+    int kp, rank;
+    int cseq, nseq;
+};
 
-// cluster_sum for two values held as FP32 pairs (h, l): the K CTAs' pairs are
-// added in rank order with two-sums (every CTA gets the same bits).
-template <int K>
-__device__ __forceinline__ void cluster_sum_f2(bool writer, float (*cx)[4], int& seq, float& ah, float& al, float& bh,
-                                               float& bl) {
-    namespace cg = cooperative_groups;
-    cg::cluster_group cl = cg::this_cluster();
-    const int s = seq & 1;
-    ++seq;
-    if (writer) {
-        cx[s][0] = ah;
-        cx[s][1] = al;
-        cx[s][2] = bh;
-        cx[s][3] = bl;
-    }
-    cl.sync();
-    float xh = 0.f, xl = 0.f, yh = 0.f, yl = 0.f;
-#pragma unroll
-    for (int r = 0; r < K; ++r) {
-        const float4 q = *reinterpret_cast<const float4*>(cl.map_shared_rank(&cx[s][0], r));
-        const F2 u = f2_two_sum(xh, q.x), v = f2_two_sum(yh, q.z);
-        xh = u.h;
-        xl = __fadd_rn(__fadd_rn(xl, q.y), u.l);
-        yh = v.h;
-        yl = __fadd_rn(__fadd_rn(yl, q.w), v.l);
-    }
-    ah = xh;
-    al = xl;
-    bh = yh;
-    bl = yl;
-}
+// The entries of the binary tree that one warp finishes: entry i of ne at
+// index i of the linear order; lane j takes its `per` neighbouring entries, then
+// the lanes are added neighbours first (entries past ne count as zero, exactly).
+__device__ __forceinline__ int tree_per(int ne) { return ne > 64 ? 4 : ne > 32 ? 2 : 1; }
 
-__device__ __forceinline__ double warp_sum(double x) {
-    for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+// Compensated warp sums of two FP32 partials (two-sums over the virtual threads of
+// the warp, which lie `lanes` apart; neighbours first): every lane ends with both
+// sums as unevaluated pairs (d1 h, l, d2 h, l), with no FP64 instruction.
+__device__ __forceinline__ float4 warp_sum_comp(float x, float y, int lanes) {
+    float s = x, c = 0.f, s2 = y, c2 = 0.f;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        if (o < lanes) continue;
+        const float os = __shfl_xor_sync(0xffffffffu, s, o), oc = __shfl_xor_sync(0xffffffffu, c, o);
+        const float os2 = __shfl_xor_sync(0xffffffffu, s2, o), oc2 = __shfl_xor_sync(0xffffffffu, c2, o);
+        const F2 u = f2_two_sum(s, os), v = f2_two_sum(s2, os2);
+        s = u.h;
+        c = __fadd_rn(__fadd_rn(c, oc), u.l);
+        s2 = v.h;
+        c2 = __fadd_rn(__fadd_rn(c2, oc2), v.l);
+    }
+    return make_float4(s, c, s2, c2);
+}
+__device__ __forceinline__ double warp_sum(double x, int lanes) {
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1)
+        if (o >= lanes) x += __shfl_xor_sync(0xffffffffu, x, o);
     return x;
-}
-
-// Warp sum of per-lane FP32 partials with a compensated (two-sum) tree, so
-// the cross-lane additions lose nothing beyond FP32 rounding of the running
-// error; FP64 partials are summed directly.
-// Compensated warp sum of FP32 partials: lane 0 ends with the sum as an
-// unevaluated pair s + c (no FP64 instruction in the calling warps).
-__device__ __forceinline__ float2 warp_sum_comp(float x) {
-    float s = x, c = 0.f;
-    for (int o = 16; o; o >>= 1) {
-        float os = __shfl_down_sync(0xffffffffu, s, o), oc = __shfl_down_sync(0xffffffffu, c, o);
-        float t = __fadd_rn(s, os);
-        float bp = __fsub_rn(t, s);
-        float err = __fadd_rn(__fsub_rn(s, __fsub_rn(t, bp)), __fsub_rn(os, bp));
-        s = t;
-        c = __fadd_rn(__fadd_rn(c, oc), err);
-    }
-    return make_float2(s, c);
 }
 
 template <typename R, int C>
@@ -1717,82 +1712,79 @@ __device__ __forceinline__ bool newton_step_f2(F2& t, F2& lo, F2& hi, F2 d1, F2 
     return conv;
 }
 
-// ln x of an FP64 site likelihood.
-__device__ __forceinline__ double log_split(double x) { return log(x); }
+// Sum of the virtual threads' scores over the item, the same in every thread
+// whatever the launch shape: the warps' sums in shared memory (red), then the
+// cluster's kp x nw of them by the tree.  Every thread of every CTA must call it
+// the same number of times; cseq alternates the slot, so a CTA writes one only
+// after every CTA has passed the barrier of the exchange that last read it.
+template <bool kClus>
+__device__ __forceinline__ double team_sum(double acc, double (*red)[32], Team& tm, int lanes) {
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5, sl = tm.cseq++ & 1;
+    acc = warp_sum(acc, lanes);
+    if (lane == 0) red[sl][w] = acc;
+    if constexpr (kClus) cooperative_groups::this_cluster().sync();
+    else __syncthreads();
+    const int ne = tm.kp * nw, per = tree_per(ne);
+    double e[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int i = lane * per + k;
+        if (k < per && i < ne) {
+            if constexpr (kClus) e[k] = cooperative_groups::this_cluster().map_shared_rank(&red[sl][0], i / nw)[i % nw];
+            else e[k] = red[sl][i];
+        }
+    }
+    return warp_sum((e[0] + e[1]) + (e[2] + e[3]), 1);
+}
+// One site's score, added to the virtual thread's sum in site order; term of the
+// lane's own site (0 where it has none this round).
+__device__ __forceinline__ void add_score(double& acc, double term, int lanes) {
+    if (lanes == 1) {
+        acc = __dadd_rn(acc, term);
+        return;
+    }
+    const int base = (threadIdx.x & 31) & ~(lanes - 1);
+    for (int j = 0; j < lanes; ++j) acc = __dadd_rn(acc, __shfl_sync(0xffffffffu, term, base + j));
+}
 
-// lnL of the current sum-table at length t: sum_p w_p (ln L_p + E_p ln 2), FP64 accumulation.
-// K > 1: the CTA's sites are its share of a cluster's; the result is the cluster's sum.
-template <typename R, int C, int K = 1>
-__device__ double eval_lnl(const Model& M, const STab<R, C>& st, int P, double t, NewtonSmem<R, C>& ns,
-                           int* cseq = nullptr) {
-    put_egh<R, C>(M, t, ns, true);
+// lnL of the current sum-table at length t: sum_p w_p (ln L_p + E_p ln 2) (FP64;
+// the mixed path scores from pairs).
+template <int C, bool kClus>
+__device__ double eval_lnl(const Model& M, const STab<double, C>& st, const Sites& sx, double t,
+                           NewtonSmem<double, C>& ns, Team& tm) {
+    put_egh<double, C>(M, t, ns, true);
     __syncthreads();
-    R e[4 * C];
+    double e[4 * C];
 #pragma unroll
     for (int q = 0; q < 4 * C; ++q) e[q] = ns.egh[0][q];
     double acc = 0.0;
-    if constexpr (sizeof(R) == 4) {
-        // sum_p w_p ln L_p = sum_p w_p ln m_p + ln 2 * sum_p w_p (e_p + E_p), L_p = 2^e_p m_p:
-        // the exponent part is an exact integer sum, the mantissa logs a compensated FP32 sum
-        long long ie = 0;
-        float am = 0.f, ac = 0.f;
-        for (int p = threadIdx.x; p < P; p += blockDim.x) {
-            R s[4 * C];
-            st.get(p, s);
-            R L = e[0] * s[0];
+    for (int m = 0; m < sx.M; ++m) {
+        double term = 0.0;
+        if (m < sx.cnt) {
+            const int pl = sx.pl0 + m * sx.pstep;
+            double s[4 * C];
+            st.get(pl, s);
+            double L = e[0] * s[0];
 #pragma unroll
             for (int z = 1; z < 4 * C; ++z) {
                 const int q = (z & 3) * C + (z >> 2);  // categories outermost
                 L = fma(e[q], s[q], L);
             }
-            int b = __float_as_int(L), ex = ((b >> 23) & 0xff) - 127;
-            float m = __int_as_float((b & 0x007fffff) | 0x3f800000);
-            if (ex == -127) {  // subnormal: rescale exactly by 2^23 first
-                const int b2 = __float_as_int(L * 8388608.0f);
-                ex = ((b2 >> 23) & 0xff) - 127 - 23;
-                m = __int_as_float((b2 & 0x007fffff) | 0x3f800000);
-            }
-            const int wi = (int)st.ew[st.pcap + p];
-            ie += (long long)wi * (ex + (int)st.ew[p]);
-            float y = __fsub_rn(__fmul_rn((float)wi, logf(m)), ac);
-            float t = __fadd_rn(am, y);
-            ac = __fsub_rn(__fsub_rn(t, am), y);
-            am = t;
+            term = __dmul_rn(st.w[pl], log(L) + st.e[pl] * kLn2);
         }
-        acc = ((double)am - (double)ac) + (double)ie * kLn2;
-    } else {
-        for (int p = threadIdx.x; p < P; p += blockDim.x) {
-            R s[4 * C];
-            st.get(p, s);
-            R L = e[0] * s[0];
-#pragma unroll
-            for (int z = 1; z < 4 * C; ++z) {
-                const int q = (z & 3) * C + (z >> 2);  // categories outermost
-                L = fma(e[q], s[q], L);
-            }
-            acc += (double)st.ew[st.pcap + p] * (log_split(L) + (double)st.ew[p] * kLn2);
-        }
+        add_score(acc, term, sx.lanes);
     }
-    acc = warp_sum(acc);
-    const int w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-    if ((threadIdx.x & 31) == 0) ns.red[w][0] = acc;
-    __syncthreads();
-    double tot = 0.0;
-    for (int i = 0; i < nw; ++i) tot += ns.red[i][0];
-    __syncthreads();
-    if constexpr (K > 1) {
-        double b = 0.0, c = 0.0;
-        cluster_sum<K>(threadIdx.x == 0, ns.cx, *cseq, tot, b, c);
-    }
-    return tot;
+    return team_sum<kClus>(acc, ns.red, tm, sx.lanes);
 }
 
-// One site's terms of the Newton sums: a = L'/L, b = L''/L and the site weight,
-// from the sum-table at the coefficients e, g, h (the stationary slots, k = 0,
-// have zero derivative coefficients).
+// One site's terms of the Newton sums: a = L'/L, c = L''/L - (L'/L)^2 and the site
+// weight, from the sum-table at the coefficients e, g, h (the stationary slots,
+// k = 0, have zero derivative coefficients).  A virtual thread takes its sites in
+// pairs; the two of a pair (and a last single one) round c in the forms they have
+// always had: first of a pair fma(-a, a, L''/L), else fma(L'', 1/L, -a a).
 template <typename R, int C>
-__device__ __forceinline__ void newton_site(const STab<R, C>& st, int p, const R* e, const R* g, const R* h, R& a, R& b,
-                                            R& wt) {
+__device__ __forceinline__ void newton_site(const STab<R, C>& st, int p, const R* e, const R* g, const R* h, bool first,
+                                            R& a, R& c, R& wt) {
     R s[4 * C];
     st.get(p, s);
     R L = e[0] * s[0], L1 = g[C] * s[C], L2 = h[C] * s[C];
@@ -1806,28 +1798,26 @@ __device__ __forceinline__ void newton_site(const STab<R, C>& st, int p, const R
         }
     }
     const R inv = Prec<R>::rcp(L);
-    a = L1 * inv;
-    b = L2 * inv;
-    wt = st.ew[st.pcap + p];
+    a = Prec<R>::mul(L1, inv);
+    c = first ? fma(-a, a, Prec<R>::mul(L2, inv)) : fma(L2, inv, -Prec<R>::mul(a, a));
+    wt = st.w[p];
 }
 
 // Newton solve on the current sum-table from t0.  Per evaluation: every
 // thread sums w L'/L and w (L''/L - (L'/L)^2) over its sites, the warps
-// reduce, and warp 0 alone takes the FP64 step and writes the coefficients
-// of the next length; after the last step warp 0 also writes P_r(t) of the
-// final length into Pdst [C][16] (visible when the call returns).  Returns
+// reduce, and one warp alone takes the step and writes the coefficients
+// of the next length; after the last step it also writes P_r(t) of the
+// final length into Pdst [16][C] (visible when the call returns).  Returns
 // the final length (in every thread).
-// K > 1: the sum-table holds this CTA's share of a cluster's sites; each
-// evaluation's derivative sums are reduced over the cluster (cluster_sum), and
-// every CTA takes the same step.
-template <typename R, int C, int K = 1>
-__device__ double newton_solve(const Model& M, const Cfg& cfg, const STab<R, C>& st, int P, double t0,
-                               NewtonSmem<R, C>& ns, int& evals, bool& converged, R* Pdst, int* cseq = nullptr,
-                               int* nseq = nullptr) {
+// kClus: the sum-table holds this CTA's share of a cluster's sites; each
+// evaluation's derivative sums are exchanged over the cluster, and every CTA
+// takes the same step.
+template <typename R, int C, bool kClus>
+__device__ double newton_solve(const Model& M, const Cfg& cfg, const STab<R, C>& st, const Sites& sx, double t0,
+                               NewtonSmem<R, C>& ns, int& evals, bool& converged, R* Pdst, Team& tm) {
     double lo = cfg.tmin, hi = cfg.tmax;
     double t = fmin(fmax(t0, lo), hi);
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5;
-    const int top = nw > 8 ? 8 : nw > 4 ? 4 : nw > 2 ? 2 : 1;  // first butterfly offset
     const bool prior = __double_as_longlong(cfg.prior_rate) != 0;
     put_egh<R, C>(M, t, ns, false);
     if (threadIdx.x == 0) ns.tb = t;
@@ -1849,168 +1839,145 @@ __device__ double newton_solve(const Model& M, const Cfg& cfg, const STab<R, C>&
 #pragma unroll
         for (int q = 0; q < 4 * C; ++q) { e[q] = ns.egh[0][q]; g[q] = ns.egh[1][q]; h[q] = ns.egh[2][q]; }
         R a1 = R(0), a2 = R(0);
-        // two sites per pass (their chains interleave), added in site order
-        const int bd = blockDim.x;
-        int p = threadIdx.x;
-        for (; p + bd < P; p += 2 * bd) {
-            R a, b, wt, a_, b_, wt_;
-            newton_site<R, C>(st, p, e, g, h, a, b, wt);
-            newton_site<R, C>(st, p + bd, e, g, h, a_, b_, wt_);
-            a1 = fma(wt, a, a1);
-            a2 = fma(wt, b - a * a, a2);
-            a1 = fma(wt_, a_, a1);
-            a2 = fma(wt_, b_ - a_ * a_, a2);
-        }
-        if (p < P) {
-            R a, b, wt;
-            newton_site<R, C>(st, p, e, g, h, a, b, wt);
-            a1 = fma(wt, a, a1);
-            a2 = fma(wt, b - a * a, a2);
-        }
-        // the per-warp sums: to this CTA's shared memory, or (FP32 pairs in a cluster)
-        // pushed into every CTA of the cluster, where the leader waits for them
-        bool pub = false;  // pushed to the cluster (slot cs of exchange xe)
-        int cs = 0, xe = 0;
-        if constexpr (sizeof(R) == 4) {
-            const float2 d1 = warp_sum_comp(a1), d2 = warp_sum_comp(a2);
-            if constexpr (K > 1) {
-                // Slot cs is free in every CTA: a warp pushes exchange xe only after its
-                // CTA's leader received all of exchange xe - 1, which every CTA pushed
-                // after its own leader had read exchange xe - 2 (the last use of cs).
-                xe = *nseq;
-                cs = xe & 1;
-                ++*nseq;
-                if (lane == 0) {
-                    const float4 v = make_float4(d1.x, d1.y, d2.x, d2.y);
-                    const unsigned me = cluster_rank();
-                    float* slot = &ns.cxr[cs][me * nw + w][0];
-#pragma unroll
-                    for (int r = 0; r < K; ++r)
-                        if ((unsigned)r != me) cluster_push16(slot, &ns.mbx[cs], (unsigned)r, v);
-                    *reinterpret_cast<float4*>(slot) = v;  // this CTA's own copy
-                    mbar_arrive(&ns.mbx[cs]);
-                }
-                pub = true;  // no block barrier here: only the leader needs the sums
-            } else if (lane == 0) {
-                ns.redf[w][0] = d1.x; ns.redf[w][1] = d1.y; ns.redf[w][2] = d2.x; ns.redf[w][3] = d2.y;
+        if (sx.lanes == 1) {
+            // two sites per pass (their chains interleave), added in site order
+            int m = 0, p = sx.pl0;
+            for (; m + 1 < sx.cnt; m += 2, p += 2 * sx.pstep) {
+                R a, c, wt, a_, c_, wt_;
+                newton_site<R, C>(st, p, e, g, h, true, a, c, wt);
+                newton_site<R, C>(st, p + sx.pstep, e, g, h, false, a_, c_, wt_);
+                a1 = fma(wt, a, a1);
+                a2 = fma(wt, c, a2);
+                a1 = fma(wt_, a_, a1);
+                a2 = fma(wt_, c_, a2);
+            }
+            if (m < sx.cnt) {
+                R a, c, wt;
+                newton_site<R, C>(st, p, e, g, h, false, a, c, wt);
+                a1 = fma(wt, a, a1);
+                a2 = fma(wt, c, a2);
             }
         } else {
-            const double d1 = warp_sum(a1), d2 = warp_sum(a2);
-            if (lane == 0) { ns.red[w][0] = d1; ns.red[w][1] = d2; }
-        }
-        if (!pub) __syncthreads();
-        ++evals;
-        double D1 = 0.0, D2 = 0.0;
-        float D2f = 0.f;
-        if constexpr (sizeof(R) == 4) {
-            // Both derivative sums as FP32 pairs in one compensated butterfly: lane
-            // j < nw holds warp j's d1 pair, lane 16 + j its d2 pair; offsets below 16
-            // keep the halves apart.  Two-sums carry the pairs exactly enough (~48
-            // bits) that FP64 is needed only to convert the totals for the step.
-            float h = 0.f, l = 0.f;
-            if constexpr (K > 1) {
-                if (w == ld) {
-                    // wait (bounded) until the slot holds all K x nw pushes of this exchange
-                    if (lane == 0) mbar_arrive_expect(&ns.mbx[cs], (unsigned)((K - 1) * nw * 16));
-                    bool ok = ns.abort_ != 0;  // after a wait ran out, none is waited for again
-                    const long long tw = clock64();
-                    while (!ok) {
-                        ok = mbar_try_wait(&ns.mbx[cs], (unsigned)(xe >> 1) & 1u);
-                        if (!ok && clock64() - tw > kExchangeWaitCycles) break;
-                    }
-                    if (__any_sync(0xffffffffu, !ok) && lane == 0) ns.abort_ = 1;
-                    // the cluster's K x nw warp pairs: lane j takes pairs j, j + 32, ...
-                    // (CTA j / nw, warp j % nw) in a fixed order, then a 32-lane
-                    // butterfly: every CTA adds the same numbers in the same order
-                    float h2 = 0.f, l2 = 0.f;
-                    for (int j = lane; j < K * nw; j += 32) {
-                        const float4 q = *reinterpret_cast<const float4*>(&ns.cxr[cs][j][0]);
-                        const F2 u = f2_two_sum(h, q.x), v = f2_two_sum(h2, q.z);
-                        h = u.h;
-                        l = __fadd_rn(__fadd_rn(l, q.y), u.l);
-                        h2 = v.h;
-                        l2 = __fadd_rn(__fadd_rn(l2, q.w), v.l);
-                    }
-                    for (int o = 16; o; o >>= 1) {
-                        const float oh = __shfl_xor_sync(0xffffffffu, h, o), ol = __shfl_xor_sync(0xffffffffu, l, o);
-                        const float oh2 = __shfl_xor_sync(0xffffffffu, h2, o), ol2 = __shfl_xor_sync(0xffffffffu, l2, o);
-                        const F2 u = f2_two_sum(h, oh), v = f2_two_sum(h2, oh2);
-                        h = u.h;
-                        l = __fadd_rn(__fadd_rn(l, ol), u.l);
-                        h2 = v.h;
-                        l2 = __fadd_rn(__fadd_rn(l2, ol2), v.l);
-                    }
-                    if (lane >= 16) {  // lanes < 16: d1, the others d2 (as below)
-                        h = h2;
-                        l = l2;
-                    }
-                }
-            } else if (w == ld) {
-                const int src = lane & 15, half = lane >> 4;
-                if (src < nw) {
-                    h = ns.redf[src][2 * half];
-                    l = ns.redf[src][2 * half + 1];
-                }
-                for (int o = top; o; o >>= 1) {
-                    const float oh = __shfl_xor_sync(0xffffffffu, h, o), ol = __shfl_xor_sync(0xffffffffu, l, o);
-                    const F2 t2 = f2_two_sum(h, oh);
-                    h = t2.h;
-                    l = __fadd_rn(__fadd_rn(l, ol), t2.l);
+            // the virtual thread's sites of this round lie in its lanes, in order:
+            // every lane of the group adds all of them (the same sum as one thread's)
+            const int base = lane & ~(sx.lanes - 1);
+            for (int m = 0; m < sx.M; ++m) {
+                R a = R(0), c = R(0), wt = R(0);
+                const int k = sx.jj + m * sx.lanes;  // this lane's site among the virtual thread's
+                if (m < sx.cnt)
+                    newton_site<R, C>(st, sx.pl0 + m * sx.pstep, e, g, h, !(k & 1) && k + 1 < sx.nt, a, c, wt);
+                for (int j = 0; j < sx.lanes; ++j) {
+                    const R aj = __shfl_sync(0xffffffffu, a, base + j), cj = __shfl_sync(0xffffffffu, c, base + j),
+                            wj = __shfl_sync(0xffffffffu, wt, base + j);
+                    a1 = fma(wj, aj, a1);
+                    a2 = fma(wj, cj, a2);
                 }
             }
-            if (w == ld) {  // lanes < 16 hold d1, the others d2
+        }
+        // the per-warp sums, one 16-byte entry each: to this CTA's shared memory, or
+        // pushed into every CTA of the cluster, where the leader waits for them
+        const int xe = tm.nseq++, cs = kClus ? xe & 1 : 0;
+        float4 v;
+        if constexpr (sizeof(R) == 4) {
+            v = warp_sum_comp(a1, a2, sx.lanes);
+        } else {
+            const double2 d = make_double2(warp_sum(a1, sx.lanes), warp_sum(a2, sx.lanes));
+            v = reinterpret_cast<const float4&>(d);
+        }
+        if constexpr (kClus) {
+            // Slot cs is free in every CTA: a warp pushes exchange xe only after its
+            // CTA's leader received all of exchange xe - 1, which every CTA pushed
+            // after its own leader had read exchange xe - 2 (the last use of cs).
+            if (lane == 0) {
+                float* slot = &ns.cxr[cs][tm.rank * nw + w][0];
+                for (int r = 0; r < tm.kp; ++r)
+                    if (r != tm.rank) cluster_push16(slot, &ns.mbx[cs], (unsigned)r, v);
+                *reinterpret_cast<float4*>(slot) = v;  // this CTA's own copy
+                mbar_arrive(&ns.mbx[cs]);
+            }
+            // no block barrier here: only the leader needs the sums
+        } else {
+            if (lane == 0) *reinterpret_cast<float4*>(&ns.cxr[0][w][0]) = v;
+            __syncthreads();
+        }
+        ++evals;
+        if (w == ld) {
+            if constexpr (kClus) {
+                // wait (bounded) until the slot holds all kp x nw pushes of this exchange
+                if (lane == 0) mbar_arrive_expect(&ns.mbx[cs], (unsigned)((tm.kp - 1) * nw * 16));
+                bool ok = ns.abort_ != 0;  // after a wait ran out, none is waited for again
+                const long long tw = clock64();
+                while (!ok) {
+                    ok = mbar_try_wait(&ns.mbx[cs], (unsigned)(xe >> 1) & 1u);
+                    if (!ok && clock64() - tw > kExchangeWaitCycles) break;
+                }
+                if (__any_sync(0xffffffffu, !ok) && lane == 0) ns.abort_ = 1;
+            }
+            // the rest of the tree over the kp x nw warp entries: every CTA adds the same
+            // numbers in the same order
+            const int ne = tm.kp * nw, per = tree_per(ne);
+            bool done;
+            if constexpr (sizeof(R) == 4) {
+                // FP32 pairs, added by two-sums (~48 bits)
+                auto entry = [&](int k) {
+                    const int i = lane * per + k;
+                    return k < per && i < ne ? *reinterpret_cast<const float4*>(&ns.cxr[cs][i][0])
+                                             : make_float4(0.f, 0.f, 0.f, 0.f);
+                };
+                auto add = [](float4 x, float4 y) {
+                    const F2 u = f2_two_sum(x.x, y.x), z = f2_two_sum(x.z, y.z);
+                    return make_float4(u.h, __fadd_rn(__fadd_rn(x.y, y.y), u.l), z.h,
+                                       __fadd_rn(__fadd_rn(x.w, y.w), z.l));
+                };
+                float4 q = entry(0);
+                if (per > 1) q = add(q, entry(1));
+                if (per > 2) q = add(q, add(entry(2), entry(3)));
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    if (o >= ne) break;  // only zeros from here on
+                    q = add(q, make_float4(__shfl_xor_sync(0xffffffffu, q.x, o), __shfl_xor_sync(0xffffffffu, q.y, o),
+                                           __shfl_xor_sync(0xffffffffu, q.z, o), __shfl_xor_sync(0xffffffffu, q.w, o)));
+                }
                 // the butterfly leaves (h, l) unnormalised (l can reach a sizeable
                 // fraction of h after cancellation): renormalise, so that the
                 // quotient's reciprocal seed is taken from the rounded total
-                F2 d1p = f2_two_sum(__shfl_sync(0xffffffffu, h, 0), __shfl_sync(0xffffffffu, l, 0));
-                const F2 d2p = f2_two_sum(__shfl_sync(0xffffffffu, h, 16), __shfl_sync(0xffffffffu, l, 16));
+                F2 d1p = f2_two_sum(__shfl_sync(0xffffffffu, q.x, 0), __shfl_sync(0xffffffffu, q.y, 0));
+                const F2 d2p = f2_two_sum(__shfl_sync(0xffffffffu, q.z, 0), __shfl_sync(0xffffffffu, q.w, 0));
                 if (prior) d1p = f2_sub(d1p, prp);  // MAP: the prior's slope
-                const bool done = newton_step_f2(tp, lop, hip, d1p, d2p, tolp);
-                const bool last = done || it + 1 == cfg.newton_maxit;
-                if (!last) {
-                    put_egh_f<R, C>(tp.h, ns, lane);
-                } else {
-                    t = (double)tp.h + (double)tp.l;
-                    if (lane < 4 * C) ns.ex[lane] = exp(ns.lr[lane] * t);  // for the P matrices below
+                done = newton_step_f2(tp, lop, hip, d1p, d2p, tolp);
+            } else {
+                auto entry = [&](int k) {
+                    const int i = lane * per + k;
+                    return k < per && i < ne ? *reinterpret_cast<const double2*>(&ns.cxr[cs][i][0]) : make_double2(0.0, 0.0);
+                };
+                double2 q = entry(0);
+                if (per > 1) {
+                    const double2 x = entry(1), y = entry(2), z = entry(3);
+                    q = make_double2((q.x + x.x) + (y.x + z.x), (q.y + x.y) + (y.y + z.y));
                 }
-                if (lane == 0) {
-                    if (last) ns.tb = t;
-                    ns.done = last ? (done ? 1 : 2) : 0;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    if (o >= ne) break;
+                    q.x += __shfl_xor_sync(0xffffffffu, q.x, o);
+                    q.y += __shfl_xor_sync(0xffffffffu, q.y, o);
                 }
+                double D1 = __shfl_sync(0xffffffffu, q.x, 0);
+                const double D2 = __shfl_sync(0xffffffffu, q.y, 0);
+                if (prior) D1 -= cfg.prior_rate;  // MAP: the prior's slope
+                done = newton_step(t, lo, hi, D1, D2, (float)D2, cfg.newton_tol);
             }
-        } else {
-            if (w == ld) {
-                // Both derivative sums in one FP64 butterfly: lane j < nw holds warp j's
-                // d1 partial, lane 16 + j its d2 partial; offsets below 16 keep the halves
-                // apart.  An FP32 sum of the same words runs alongside (reciprocal seed).
-                const int src = lane & 15, half = lane >> 4;
-                double D = 0.0;
-                float Df = 0.f;
-                if (src < nw) {
-                    D = ns.red[src][half];
-                    Df = (float)D;
-                }
-                for (int o = top; o; o >>= 1) {
-                    D += __shfl_xor_sync(0xffffffffu, D, o);
-                    Df += __shfl_xor_sync(0xffffffffu, Df, o);
-                }
-                D1 = __shfl_sync(0xffffffffu, D, 0);
-                D2 = __shfl_sync(0xffffffffu, D, 16);
-                D2f = __shfl_sync(0xffffffffu, Df, 16);
-            }
-            if constexpr (K > 1) {  // the cluster's sums (every thread takes part in the exchange)
-                double d2f = D2f;
-                cluster_sum<K>(w == ld && lane == 0, ns.cx, *cseq, D1, D2, d2f);
-                D2f = (float)d2f;
-            }
-        }
-        if (sizeof(R) == 8 && w == ld) {
-            if (prior) D1 -= cfg.prior_rate;  // MAP: the prior's slope
-            const bool done = newton_step(t, lo, hi, D1, D2, D2f, cfg.newton_tol);
             const bool last = done || it + 1 == cfg.newton_maxit;
-            if (!last) put_egh<R, C>(M, t, ns, false, lane);
-            else if (lane < 4 * C) ns.ex[lane] = exp(ns.lr[lane] * t);  // for the P matrices below
-            if (lane == 0) { ns.tb = t; ns.done = last ? (done ? 1 : 2) : 0; }
+            if (!last) {
+                if constexpr (sizeof(R) == 4) put_egh_f<R, C>(tp.h, ns, lane);
+                else put_egh<R, C>(M, t, ns, false, lane);
+            } else {
+                if (sizeof(R) == 4) t = (double)tp.h + (double)tp.l;
+                if (lane < 4 * C) ns.ex[lane] = exp(ns.lr[lane] * t);  // for the P matrices below
+            }
+            if (lane == 0) {
+                if (last) ns.tb = t;
+                ns.done = last ? (done ? 1 : 2) : 0;
+            }
         }
         __syncthreads();
         if (ns.done) {
@@ -2037,24 +2004,15 @@ __device__ double newton_solve(const Model& M, const Cfg& cfg, const STab<R, C>&
 // sum over the calling block's sites of w_p ln L_p, reduced over the block
 // into red[32] (FP64) and returned in every thread.  Kept out of line so the
 // FP32 Newton loops around them keep their registers.
-__device__ __forceinline__ double block_sum(double acc, double (*red)[2]) {
-    acc = warp_sum(acc);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][0] = acc;
-    __syncthreads();
-    double tot = 0.0;
-    for (int i = 0; i < (int)((blockDim.x + 31) >> 5); ++i) tot += red[i][0];
-    __syncthreads();
-    return tot;
-}
 
 // Proposal: the four members A, X2 (at u) and B, Y2 (at v) around the new
 // edge (slots of ld sites), P matrices of the five final lengths as pairs (Ph/Pl
 // [5][16*C]: central, A, B, C, D; mbr = each member's branch); L_p across the
 // central branch.
-template <int C, int K = 1>
+template <int C, bool kClus>
 __device__ __noinline__ double propose_score_f2(const Src2<C>* mem, const int* mbr, const float* Ph, const float* Pl,
-                                                const double* pi, const int32_t* w, int ld, int p0, int p1,
-                                                double (*red)[2], double (*cx)[3], int* cseq) {
+                                                const double* pi, const int32_t* w, int ld, const Sites& sx,
+                                                double (*red)[32], Team& tm) {
     float pih[4], pil[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -2063,21 +2021,21 @@ __device__ __noinline__ double propose_score_f2(const Src2<C>* mem, const int* m
         pil[i] = x.l;
     }
     double acc = 0.0;
-    for (int p = p0 + threadIdx.x; p < p1; p += blockDim.x) {
+    auto site = [&](int p) {
         int kk = 0;
 #pragma unroll
-        for (int m = 0; m < 4; ++m) kk += mem[m].tip ? 0 : mem[m].scl[p];
+        for (int b = 0; b < 4; ++b) kk += mem[b].tip ? 0 : mem[b].scl[p];
         F2 L{0.f, 0.f};
         int E = 0;
         using T = typename Lanes<C>::T;
 #pragma unroll 1
         for (int g = 0; g < Lanes<C>::n; ++g) {
             F2T<T> x[4], y[4], t[4];
-            f2_apply_src4<C>(Ph + mbr[0] * C * 16, Pl + mbr[0] * C * 16, mem[0], ld, p, g, x);
-            f2_apply_src4<C>(Ph + mbr[1] * C * 16, Pl + mbr[1] * C * 16, mem[1], ld, p, g, t);
+            f2_apply_src4<C>(Ph + mbr[0] * C * 16, Pl + mbr[0] * C * 16, mem[0], ld, p, p, g, x);
+            f2_apply_src4<C>(Ph + mbr[1] * C * 16, Pl + mbr[1] * C * 16, mem[1], ld, p, p, g, t);
             f2_mul4<T>(x, t);
-            f2_apply_src4<C>(Ph + mbr[2] * C * 16, Pl + mbr[2] * C * 16, mem[2], ld, p, g, y);
-            f2_apply_src4<C>(Ph + mbr[3] * C * 16, Pl + mbr[3] * C * 16, mem[3], ld, p, g, t);
+            f2_apply_src4<C>(Ph + mbr[2] * C * 16, Pl + mbr[2] * C * 16, mem[2], ld, p, p, g, y);
+            f2_apply_src4<C>(Ph + mbr[3] * C * 16, Pl + mbr[3] * C * 16, mem[3], ld, p, p, g, t);
             f2_mul4<T>(y, t);
             int ex[Lanes<C>::w], ey[Lanes<C>::w];
             f2_normalise4(x, ex);
@@ -2094,14 +2052,10 @@ __device__ __noinline__ double propose_score_f2(const Src2<C>* mem, const int* m
             }
         }
         L = F2{L.h * (1.0f / C), L.l * (1.0f / C)};  // 1/C is a power of two for C = 1, 2, 4
-        acc += (double)w[p] * f2_log(L, E - Prec<float>::kScaleExp * kk);
-    }
-    double tot = block_sum(acc, red);
-    if constexpr (K > 1) {
-        double b = 0.0, c = 0.0;
-        cluster_sum<K>(threadIdx.x == 0, cx, *cseq, tot, b, c);
-    }
-    return tot;
+        return __dmul_rn((double)w[p], f2_log(L, E - Prec<float>::kScaleExp * kk));
+    };
+    for (int m = 0; m < sx.M; ++m) add_score(acc, m < sx.cnt ? site(sx.p0 + m * sx.step) : 0.0, sx.lanes);
+    return team_sum<kClus>(acc, red, tm, sx.lanes);
 }
 
 // Visit: a pruning pass in pairs over one tree's partials buffer.  D_v of
@@ -2110,15 +2064,14 @@ __device__ __noinline__ double propose_score_f2(const Src2<C>* mem, const int* m
 // combined with leaf 0 across the edge of n.  The block computes each node's
 // P pairs (its two children, and n's own edge at the root) into Pf/Pfl from
 // W and lr (as NewtonSmem) at the lengths len.
-// Sites: tips0 / w0 are the alignment's tip rows (row stride A.P) and weights
-// offset to this CTA's first site, Pl sites of them, stored vectors of Ps
-// sites per slot; with K > 1 the result is summed over the cluster.
-template <int C, int K = 1>
-__device__ __noinline__ double fullopt_score_f2(int n, const int32_t* ch, const double* len, Aln A, const uint8_t* tips0,
-                                                const int32_t* w0, int Pl, int Ps, float* clv, int32_t* scl,
-                                                const double* W, const double* lr, float* Pf, float* Pfl, double* exf,
-                                                const double* pi, double (*red)[2], double (*cx)[3], int* cseq) {
-    const int NN = 2 * n - 2, P = A.P;
+// Stored vectors are indexed by the local site (sx.ld per slot), tips and
+// weights by the site; in a cluster the result is summed over it.
+template <int C, bool kClus>
+__device__ __noinline__ double fullopt_score_f2(int n, const uint8_t* ch, const double* len, const Aln& A,
+                                                const Sites& sx, float* clv, int32_t* scl, const double* W,
+                                                const double* lr, float* Pf, float* Pfl, double* exf, const double* pi,
+                                                double (*red)[32], Team& tm) {
+    const int NN = 2 * n - 2, Ps = sx.ld;
     const size_t sstride = (size_t)Ps * 4 * C;
     float pih[4], pil[4];
 #pragma unroll
@@ -2128,7 +2081,7 @@ __device__ __noinline__ double fullopt_score_f2(int n, const int32_t* ch, const 
         pil[i] = x.l;
     }
     auto src = [&](int v) {
-        if (v < n) return Src2<C>{nullptr, nullptr, nullptr, tips0 + (size_t)v * P};
+        if (v < n) return Src2<C>{nullptr, nullptr, nullptr, A.tips + (size_t)v * A.P};
         return Src2<C>{clv + (size_t)(v - n) * sstride, clv + (size_t)(n - 2 + (v - n - 1)) * sstride,
                        scl + (size_t)(v - n) * Ps, nullptr};
     };
@@ -2148,45 +2101,44 @@ __device__ __noinline__ double fullopt_score_f2(int n, const int32_t* ch, const 
         }
         __syncthreads();
         const Src2<C> s0 = src(c0), s1 = src(c1);
-        for (int p = threadIdx.x; p < Pl; p += blockDim.x) {
-            if (v > n) {
-                f2_join<C>(Pf, Pfl, s0, Pf + 16 * C, Pfl + 16 * C, s1, Ps, p, clv + (size_t)(v - n) * sstride,
-                           clv + (size_t)(n - 2 + (v - n - 1)) * sstride, scl + (size_t)(v - n) * Ps);
-            } else {
-                const int kk = (s0.tip ? 0 : s0.scl[p]) + (s1.tip ? 0 : s1.scl[p]);
-                const int code = tips0[p];  // leaf 0
-                F2 L{0.f, 0.f};
-                int E = 0;
-                using T = typename Lanes<C>::T;
-#pragma unroll 1
-                for (int g = 0; g < Lanes<C>::n; ++g) {
-                    F2T<T> d[4], t[4];
-                    int e[Lanes<C>::w];
-                    f2_apply_src4<C>(Pf, Pfl, s0, Ps, p, g, d);
-                    f2_apply_src4<C>(Pf + 16 * C, Pfl + 16 * C, s1, Ps, p, g, t);
-                    f2_mul4<T>(d, t);
-                    f2_normalise4(d, e);
-                    f2_apply4<C>(Pf + 32 * C, Pfl + 32 * C, g, d, t);
-#pragma unroll
-                    for (int k = 0; k < Lanes<C>::w; ++k) {
-                        F2 Lr{0.f, 0.f};
-#pragma unroll
-                        for (int i = 0; i < 4; ++i)
-                            if (code >= 4 || code == i) Lr = f2_add(Lr, f2_mul(lane_of(t[i], k), F2{pih[i], pil[i]}));
-                        f2_merge(L, E, Lr, e[k]);
-                    }
-                }
-                L = F2{L.h * (1.0f / C), L.l * (1.0f / C)};
-                acc += (double)w0[p] * f2_log(L, E - Prec<float>::kScaleExp * kk);
-            }
+        if (v > n) {
+            for (int m = 0; m < sx.cnt; ++m)
+                f2_join<C>(Pf, Pfl, s0, Pf + 16 * C, Pfl + 16 * C, s1, Ps, sx.pl0 + m * sx.pstep, sx.p0 + m * sx.step,
+                           clv + (size_t)(v - n) * sstride, clv + (size_t)(n - 2 + (v - n - 1)) * sstride,
+                           scl + (size_t)(v - n) * Ps);
+            continue;
         }
+        auto site = [&](int p, int pg) {
+            const int kk = (s0.tip ? 0 : s0.scl[p]) + (s1.tip ? 0 : s1.scl[p]);
+            const int code = A.tips[pg];  // leaf 0
+            F2 L{0.f, 0.f};
+            int E = 0;
+            using T = typename Lanes<C>::T;
+#pragma unroll 1
+            for (int g = 0; g < Lanes<C>::n; ++g) {
+                F2T<T> d[4], t[4];
+                int e[Lanes<C>::w];
+                f2_apply_src4<C>(Pf, Pfl, s0, Ps, p, pg, g, d);
+                f2_apply_src4<C>(Pf + 16 * C, Pfl + 16 * C, s1, Ps, p, pg, g, t);
+                f2_mul4<T>(d, t);
+                f2_normalise4(d, e);
+                f2_apply4<C>(Pf + 32 * C, Pfl + 32 * C, g, d, t);
+#pragma unroll
+                for (int k = 0; k < Lanes<C>::w; ++k) {
+                    F2 Lr{0.f, 0.f};
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        if (code >= 4 || code == i) Lr = f2_add(Lr, f2_mul(lane_of(t[i], k), F2{pih[i], pil[i]}));
+                    f2_merge(L, E, Lr, e[k]);
+                }
+            }
+            L = F2{L.h * (1.0f / C), L.l * (1.0f / C)};
+            return __dmul_rn((double)A.w[pg], f2_log(L, E - Prec<float>::kScaleExp * kk));
+        };
+        for (int m = 0; m < sx.M; ++m)
+            add_score(acc, m < sx.cnt ? site(sx.pl0 + m * sx.pstep, sx.p0 + m * sx.step) : 0.0, sx.lanes);
     }
-    double tot = block_sum(acc, red);
-    if constexpr (K > 1) {
-        double b = 0.0, c = 0.0;
-        cluster_sum<K>(threadIdx.x == 0, cx, *cseq, tot, b, c);
-    }
-    return tot;
+    return team_sum<kClus>(acc, red, tm, sx.lanes);
 }
 
 // ---------------------------------------------------------------- P matrices of tree sets
@@ -2252,8 +2204,8 @@ __global__ void k_partials(Model M, Aln A, TreeSet ts, int first, DCount cnt, Cl
         R y0[4 * C], y1[4 * C];
         int c0cnt, c1cnt;
         int c0 = ch[2 * v], c1 = ch[2 * v + 1];
-        apply_p<R, C>(Pm + (size_t)c0 * C * 16, srcD(c0), P, p, y0, c0cnt);
-        apply_p<R, C>(Pm + (size_t)c1 * C * 16, srcD(c1), P, p, y1, c1cnt);
+        apply_p<R, C>(Pm + (size_t)c0 * C * 16, srcD(c0), P, p, p, y0, c0cnt);
+        apply_p<R, C>(Pm + (size_t)c1 * C * 16, srcD(c1), P, p, p, y1, c1cnt);
         mul_vec<R, C>(y0, y1);
         int sc = rescale<R, C>(y0);
         store_vec<R, C>(clv + (size_t)(v - n) * sstride, P, p, y0);
@@ -2268,8 +2220,8 @@ __global__ void k_partials(Model M, Aln A, TreeSet ts, int first, DCount cnt, Cl
         else { a.clv = clv + (size_t)(n - 2 + u - n - 1) * sstride; a.scl = scl + (size_t)(n - 2 + u - n - 1) * P; a.tip = nullptr; }
         R y0[4 * C], y1[4 * C];
         int cs, ca;
-        apply_p<R, C>(Pm + (size_t)sib * C * 16, srcD(sib), P, p, y0, cs);
-        apply_p<R, C>(Pm + (size_t)u * C * 16, a, P, p, y1, ca);
+        apply_p<R, C>(Pm + (size_t)sib * C * 16, srcD(sib), P, p, p, y0, cs);
+        apply_p<R, C>(Pm + (size_t)u * C * 16, a, P, p, p, y1, ca);
         mul_vec<R, C>(y0, y1);
         int sc = rescale<R, C>(y0);
         const int slot = n - 2 + (v - n - 1);
@@ -2312,7 +2264,7 @@ __global__ void k_partials_f2(Model M, Aln A, TreeSet ts, int first, DCount cnt,
     };
     auto make = [&](int slot, int a, const Src2<C>& sa, int b, const Src2<C>& sb) {
         f2_join<C>(Ph + (size_t)a * C * 16, Pl + (size_t)a * C * 16, sa, Ph + (size_t)b * C * 16, Pl + (size_t)b * C * 16,
-                   sb, P, p, clv + (size_t)slot * sstride, clo + (size_t)slot * sstride, scl + (size_t)slot * P);
+                   sb, P, p, p, clv + (size_t)slot * sstride, clo + (size_t)slot * sstride, scl + (size_t)slot * P);
     };
     for (int v = NN - 1; v >= n; --v) make(v - n, ch[2 * v], srcD(ch[2 * v]), ch[2 * v + 1], srcD(ch[2 * v + 1]));
     if (!with_up) return;
@@ -2348,35 +2300,36 @@ struct ProposeSmem {
     NewtonSmem<R, C> ns;
 };
 
-// K > 1: launched as clusters of K CTAs; the CTAs of a cluster work on the
-// same item, each on a contiguous share of the sites (its sum-table in shared
+// kClus: launched as clusters of CTAs; the CTAs of a cluster work on the same
+// item, each on its share of the sites (make_sites; its sum-table in shared
 // memory), with the Newton sums and scores reduced over the cluster.
-template <typename R, int C, bool kSmemTab, int K = 1>
+template <typename R, int C, bool kSmemTab, bool kClus>
 __global__ void __launch_bounds__(512) k_propose(const PropGroup* __restrict__ groups, const int* __restrict__ gstart,
                                                  int ngroups, int* counter, Cfg cfg, unsigned long long* stats,
-                                                 unsigned char* scratch, size_t scratch_per_cta) {
+                                                 unsigned char* scratch, size_t scratch_per_cta, Geo geo, int lo,
+                                                 int hi) {
     extern __shared__ __align__(16) unsigned char smraw[];
+    const int total = gstart[ngroups];
+    if (total <= lo || total > hi) return;  // another launch shape's number of items
     ProposeSmem<R, C>& sm = *reinterpret_cast<ProposeSmem<R, C>*>(smraw);
     unsigned char* const tab_base = kSmemTab ? smraw + ((sizeof(ProposeSmem<R, C>) + 15) & ~size_t(15))
                                              : scratch + (size_t)blockIdx.x * scratch_per_cta;
-    const int total = gstart[ngroups];
     const int nb = cfg.propose_mode == 1 ? 1 : 5;
     unsigned long long evals_total = 0, sweeps_total = 0, nonconv = 0;
-    int cseq = 0;  // cluster exchanges so far (equal in every thread of the cluster)
-    int nseq = 0;  // pushed Newton exchanges so far (the same)
-    const int rank = K > 1 ? (int)cooperative_groups::this_cluster().block_rank() : 0;
-    if (K > 1 && threadIdx.x == 0) cluster_exchange_init(sm.ns);  // before the first cluster barrier
+    Team tm{kClus ? (int)cluster_ctas() : 1, kClus ? (int)cluster_rank() : 0, 0, 0};
+    const int rank = tm.rank;
+    if (kClus && threadIdx.x == 0) cluster_exchange_init(sm.ns);  // before the first cluster barrier
     while (true) {
         // previous item done with shared memory (in every CTA of the cluster: rank 0 writes theirs)
-        if constexpr (K > 1) cooperative_groups::this_cluster().sync();
+        if constexpr (kClus) cooperative_groups::this_cluster().sync();
         else __syncthreads();
         if (threadIdx.x == 0 && rank == 0) {
             const int x = atomicAdd(counter, 1);
             int k = 0;
             while (k + 1 < ngroups && gstart[k + 1] <= x) ++k;
-            if constexpr (K > 1) {
+            if constexpr (kClus) {
                 cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
-                for (int r = 0; r < K; ++r) {
+                for (int r = 0; r < tm.kp; ++r) {
                     *cl.map_shared_rank(&sm.next, r) = x;
                     *cl.map_shared_rank(&sm.grp, r) = k;
                 }
@@ -2385,7 +2338,7 @@ __global__ void __launch_bounds__(512) k_propose(const PropGroup* __restrict__ g
                 sm.grp = k;
             }
         }
-        if constexpr (K > 1) cooperative_groups::this_cluster().sync();
+        if constexpr (kClus) cooperative_groups::this_cluster().sync();
         else __syncthreads();
         const int x = sm.next;
         if (x >= total) break;
@@ -2393,13 +2346,10 @@ __global__ void __launch_bounds__(512) k_propose(const PropGroup* __restrict__ g
         const int o = x - gstart[sm.grp];
         const Model& M = G.M;
         const int n = G.fr.n, NN = 2 * n - 2, P = G.A.P;
-        // this CTA's sites [p0, p1) (all of them when K = 1)
-        const int S = K > 1 ? (((P + K - 1) / K + 3) & ~3) : P;
-        const int p0 = min(P, rank * S), p1 = min(P, p0 + S), Pl = p1 - p0;
+        const Sites sx = make_sites(P, geo, rank, tm.kp);
         STab<R, C> st;
-        st.pcap = (S + 3) & ~3;
-        st.s = reinterpret_cast<R*>(tab_base);
-        st.ew = st.s + (size_t)4 * C * st.pcap;
+        st.init(tab_base, sx.ld);
+        for (int m = 0; m < sx.cnt; ++m) st.w[sx.pl0 + m * sx.pstep] = (R)G.A.w[sx.p0 + m * sx.step];
         const size_t sstride = (size_t)P * 4 * C;
         const Item it = G.items[o];
         const int gi = it.tree - G.first;
@@ -2425,7 +2375,7 @@ __global__ void __launch_bounds__(512) k_propose(const PropGroup* __restrict__ g
             const int node[4] = {u, it.swap == 0 ? c0 : c1, sib, it.swap == 0 ? c1 : c0};
             const int brn[4] = {1, it.swap == 0 ? 3 : 4, 2, it.swap == 0 ? 4 : 3};
             sm.bmem[0] = -1;
-            const float* clo = reinterpret_cast<const float*>(G.g.clv_lo);
+            const float* clo = reinterpret_cast<const float*>(G.g.clv_lo);  // mixed precision only
             if (clo) clo += (size_t)gi * G.g.tree_stride;
             for (int m = 0; m < 4; ++m) {
                 Src<R, C> y;
@@ -2498,24 +2448,24 @@ __global__ void __launch_bounds__(512) k_propose(const PropGroup* __restrict__ g
                 const R* P1 = sm.Pm[sm.mbr[i1m]];
                 const R* P2 = sm.Pm[sm.mbr[i2m]];
                 const R* P3 = sm.Pm[sm.mbr[i3m]];
-                for (int pl = threadIdx.x; pl < Pl; pl += blockDim.x) {
-                    const int p = p0 + pl;
+                for (int m = 0; m < sx.cnt; ++m) {
+                    const int pl = sx.pl0 + m * sx.pstep, p = sx.p0 + m * sx.step;
                     R X[4 * C], Y[4 * C], t0[4 * C], t1[4 * C];
                     int k0, k1, k2, k3;
-                    apply_p<R, C>(P0, a0, P, p, t0, k0);
-                    apply_p<R, C>(P1, a1, P, p, t1, k1);
+                    apply_p<R, C>(P0, a0, P, p, p, t0, k0);
+                    apply_p<R, C>(P1, a1, P, p, p, t1, k1);
                     mul_vec<R, C>(t0, t1);
                     if (b == 0) {
 #pragma unroll
                         for (int q = 0; q < 4 * C; ++q) X[q] = t0[q];
-                        apply_p<R, C>(P2, a2, P, p, Y, k2);
-                        apply_p<R, C>(P3, a3, P, p, t1, k3);
+                        apply_p<R, C>(P2, a2, P, p, p, Y, k2);
+                        apply_p<R, C>(P3, a3, P, p, p, t1, k3);
                         mul_vec<R, C>(Y, t1);
                     } else {
                         apply_p_reg<R, C>(sm.Pm[0], t0, X);  // X used as scratch for the far side
-                        apply_p<R, C>(P2, a2, P, p, Y, k2);
+                        apply_p<R, C>(P2, a2, P, p, p, Y, k2);
                         mul_vec<R, C>(Y, X);
-                        load_raw<R, C>(a3, P, p, X, k3);
+                        load_raw<R, C>(a3, P, p, p, X, k3);
                     }
                     // b > 0: X is the member's stored vector (kept above 2^-kScaleExp by the
                     // rescaling) or a tip, so it needs no normalisation: its scale multiplies
@@ -2524,13 +2474,13 @@ __global__ void __launch_bounds__(512) k_propose(const PropGroup* __restrict__ g
                     int ex = b == 0 ? normalise<R, C>(X) : 0, ey = normalise<R, C>(Y);
                     R s4[4 * C];
                     sumtable<R, C>(sm.Mt, sm.pi, X, Y, s4);
-                    st.put(pl, s4, (R)(ex + ey - Prec<R>::kScaleExp * (k0 + k1 + k2 + k3)), (R)G.A.w[p]);
+                    st.put(pl, s4, ex + ey - Prec<R>::kScaleExp * (k0 + k1 + k2 + k3));
                 }
                 const double told = sm.T[b];
                 int ev;
                 bool conv;
                 // new length; the solve leaves P matrices of branch b at it in sm.Pm[b]
-                const double t = newton_solve<R, C, K>(M, cfg, st, Pl, told, sm.ns, ev, conv, sm.Pm[b], &cseq, &nseq);
+                const double t = newton_solve<R, C, kClus>(M, cfg, st, sx, told, sm.ns, ev, conv, sm.Pm[b], tm);
                 moved = fmax(moved, fabs(t - told));
                 evals_total += ev;
                 item_evals += ev;
@@ -2544,30 +2494,26 @@ __global__ void __launch_bounds__(512) k_propose(const PropGroup* __restrict__ g
         // in mixed precision, the pair form of the four members around the new edge
         double f1;
         if constexpr (sizeof(R) == 4) {
-            if (G.g.clv_lo) {
-                __syncthreads();  // the last solve is done with sm.Pm
-                for (int z = threadIdx.x; z < 5 * 4 * C; z += blockDim.x) {
-                    const int b = z / (4 * C), q = z % (4 * C);
-                    sm.ex5[b][q] = exp(sm.ns.lr[q] * sm.T[b]);
-                }
-                __syncthreads();
-                for (int z = threadIdx.x; z < 5 * 16 * C; z += blockDim.x) {
-                    const int b = z / (16 * C), q = z % (16 * C);
-                    f2_pmat_entry<C>(sm.ns.W, sm.ex5[b], q, reinterpret_cast<float*>(sm.Pm[b]), sm.Plo[b]);
-                }
-                __syncthreads();
-                Src2<C> mem[4];
-#pragma unroll
-                for (int m = 0; m < 4; ++m)
-                    mem[m] = Src2<C>{reinterpret_cast<const float*>(sm.msrc[m].clv), sm.mlo[m], sm.msrc[m].scl,
-                                     sm.msrc[m].tip};
-                f1 = propose_score_f2<C, K>(mem, sm.mbr, reinterpret_cast<const float*>(sm.Pm), &sm.Plo[0][0], M.pi,
-                                            G.A.w, P, p0, p1, sm.ns.red, sm.ns.cx, &cseq);
-            } else {
-                f1 = eval_lnl<R, C, K>(M, st, Pl, tlast, sm.ns, &cseq);
+            __syncthreads();  // the last solve is done with sm.Pm
+            for (int z = threadIdx.x; z < 5 * 4 * C; z += blockDim.x) {
+                const int b = z / (4 * C), q = z % (4 * C);
+                sm.ex5[b][q] = exp(sm.ns.lr[q] * sm.T[b]);
             }
+            __syncthreads();
+            for (int z = threadIdx.x; z < 5 * 16 * C; z += blockDim.x) {
+                const int b = z / (16 * C), q = z % (16 * C);
+                f2_pmat_entry<C>(sm.ns.W, sm.ex5[b], q, reinterpret_cast<float*>(sm.Pm[b]), sm.Plo[b]);
+            }
+            __syncthreads();
+            Src2<C> mem[4];
+#pragma unroll
+            for (int m = 0; m < 4; ++m)
+                mem[m] = Src2<C>{reinterpret_cast<const float*>(sm.msrc[m].clv), sm.mlo[m], sm.msrc[m].scl,
+                                 sm.msrc[m].tip};
+            f1 = propose_score_f2<C, kClus>(mem, sm.mbr, reinterpret_cast<const float*>(sm.Pm), &sm.Plo[0][0], M.pi,
+                                            G.A.w, P, sx, sm.ns.red, tm);
         } else {
-            f1 = eval_lnl<R, C, K>(M, st, Pl, tlast, sm.ns, &cseq);
+            f1 = eval_lnl<C, kClus>(M, st, sx, tlast, sm.ns, tm);
         }
         sweeps_total += sweeps;
         if (threadIdx.x == 0 && rank == 0) {
@@ -2599,8 +2545,8 @@ __global__ void __launch_bounds__(512) k_propose(const PropGroup* __restrict__ g
         atomicAdd(&stats[kStPropSweeps], sweeps_total);
         atomicAdd(&stats[kStNonconv], nonconv);
     }
-    if (K > 1 && threadIdx.x == 0 && sm.ns.abort_) atomicAdd(&stats[kStTimeout], 1ull);
-    if constexpr (K > 1) cooperative_groups::this_cluster().sync();  // no CTA leaves while others may read it
+    if (kClus && threadIdx.x == 0 && sm.ns.abort_) atomicAdd(&stats[kStTimeout], 1ull);
+    if constexpr (kClus) cooperative_groups::this_cluster().sync();  // no CTA leaves while others may read it
 }
 
 // ---------------------------------------------------------------- full optimisation (K7)
@@ -2613,38 +2559,56 @@ struct FullSmem {
     R Mt[16];
     R pi[4];
     int next, grp;
+    alignas(16) R Pst[2][C * 16];         // the current operation's P matrices, when the tree's stay in the slab
     float Pf[3][C * 16], Pfl[3][C * 16];  // pair P matrices of the score pass (two children, the node)
     double exf[3][4 * C];
     NewtonSmem<R, C> ns;
 };
+// Shared memory after FullSmem: lengths, the tree (parents and children as
+// bytes, the schedule), then the P matrices (p_smem), then the sum-table.
+__host__ __device__ inline size_t full_meta_bytes(int nn) {
+    const int n = (nn + 2) / 2;
+    return (size_t)nn * 8 + (((size_t)3 * nn + 2 * 3 * n + 15) & ~size_t(15));
+}
+constexpr unsigned short kUpd16 = 0x8000;  // kUpd in a 16-bit schedule entry
 
-// K > 1: launched as clusters of K CTAs working on the same tree, each on a
-// contiguous share of the sites (partials slab and sum-table of its share),
-// Newton sums and scores reduced over the cluster; slab mode only.
-template <typename R, int C, bool kSmemTab, int K = 1>
+// kClus: launched as clusters of CTAs working on the same tree, each on its share
+// of the sites (make_sites: partials slab and sum-table of its share), Newton
+// sums and scores reduced over the cluster.
+//
+// A launch is bound by the latency of its 2n - 3 solves per sweep, which follow one
+// another; what shortens them: the schedule and the tree in shared memory (they
+// were chains of three or four global loads before each operation), the P matrices
+// of an operation there too (read through L1 they were evicted by the vectors that
+// stream past), and as many lanes and CTAs per tree as the number of trees leaves
+// room for (Sites).
+template <typename R, int C, bool kSmemTab, bool kClus>
 __global__ void __launch_bounds__(512) k_fullopt(const FullGroup* __restrict__ groups, const int* __restrict__ gstart,
                                                  int ngroups, int* counter, int nn_max, Cfg cfg,
                                                  unsigned long long* stats, unsigned char* scratch,
                                                  size_t scratch_per_cta, unsigned char* slab, size_t slab_per_cta,
-                                                 int p_smem) {
+                                                 int p_smem, Geo geo, int lo, int hi) {
     extern __shared__ __align__(16) unsigned char smraw[];
+    const int total = gstart[ngroups];
+    if (total <= lo || total > hi) return;  // another launch shape's number of trees
     FullSmem<R, C>& sm = *reinterpret_cast<FullSmem<R, C>*>(smraw);
     size_t off = (sizeof(FullSmem<R, C>) + 15) & ~size_t(15);
     double* len = reinterpret_cast<double*>(smraw + off);
-    off += ((size_t)nn_max * sizeof(double) + 15) & ~size_t(15);
+    uint16_t* const sched = reinterpret_cast<uint16_t*>(len + nn_max);
+    uint8_t* const up = reinterpret_cast<uint8_t*>(sched + 3 * ((nn_max + 2) / 2));
+    uint8_t* const ch = up + nn_max;
+    off += full_meta_bytes(nn_max);
     R* const Psm = reinterpret_cast<R*>(smraw + off);  // P matrices here when p_smem
-    if (p_smem) off += ((size_t)nn_max * C * 16 * sizeof(R) + 15) & ~size_t(15);
+    if (p_smem) off += (size_t)nn_max * C * 16 * sizeof(R);
     unsigned char* const tab_base = kSmemTab ? smraw + off : scratch + (size_t)blockIdx.x * scratch_per_cta;
-    const int total = gstart[ngroups];
     unsigned long long evals_total = 0, sweeps_total = 0, nonconv = 0;
-    int cseq = 0;  // cluster exchanges so far (equal in every thread of the cluster)
-    int nseq = 0;  // pushed Newton exchanges so far (the same)
-    const int rank = K > 1 ? (int)cooperative_groups::this_cluster().block_rank() : 0;
-    if (K > 1 && threadIdx.x == 0) cluster_exchange_init(sm.ns);  // before the first cluster barrier
+    Team tm{kClus ? (int)cluster_ctas() : 1, kClus ? (int)cluster_rank() : 0, 0, 0};
+    const int rank = tm.rank;
+    if (kClus && threadIdx.x == 0) cluster_exchange_init(sm.ns);  // before the first cluster barrier
     bool first = true;  // thread 0: this CTA (cluster) has not taken a tree yet
     while (true) {
         // previous tree done with shared memory (in every CTA of the cluster: rank 0 writes theirs)
-        if constexpr (K > 1) cooperative_groups::this_cluster().sync();
+        if constexpr (kClus) cooperative_groups::this_cluster().sync();
         else __syncthreads();
         if (threadIdx.x == 0 && rank == 0) {
             // Cluster c's first tree is tree c (the costliest trees come first, and clusters
@@ -2652,14 +2616,14 @@ __global__ void __launch_bounds__(512) k_fullopt(const FullGroup* __restrict__ g
             // after the grid's first trees.  With fewer trees than clusters, taking the
             // first trees from the counter let two CTAs of one SM win trees while other SMs
             // stayed idle (a capacity-sized graph launch).
-            const int nclus = (int)(gridDim.x / K);
-            const int x = first ? (int)(blockIdx.x / K) : nclus + atomicAdd(counter, 1);
+            const int nclus = (int)gridDim.x / tm.kp;
+            const int x = first ? (int)blockIdx.x / tm.kp : nclus + atomicAdd(counter, 1);
             first = false;
             int k = 0;
             while (k + 1 < ngroups && gstart[k + 1] <= x) ++k;
-            if constexpr (K > 1) {
+            if constexpr (kClus) {
                 cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
-                for (int r = 0; r < K; ++r) {
+                for (int r = 0; r < tm.kp; ++r) {
                     *cl.map_shared_rank(&sm.next, r) = x;
                     *cl.map_shared_rank(&sm.grp, r) = k;
                 }
@@ -2668,7 +2632,7 @@ __global__ void __launch_bounds__(512) k_fullopt(const FullGroup* __restrict__ g
                 sm.grp = k;
             }
         }
-        if constexpr (K > 1) cooperative_groups::this_cluster().sync();
+        if constexpr (kClus) cooperative_groups::this_cluster().sync();
         else __syncthreads();
         const int x = sm.next;
         if (x >= total) break;
@@ -2676,27 +2640,19 @@ __global__ void __launch_bounds__(512) k_fullopt(const FullGroup* __restrict__ g
         const int gi = G.order ? G.order[x - gstart[sm.grp]] : x - gstart[sm.grp];
         const Model& M = G.M;
         const Aln& A = G.A;
-        const int n = G.ts.n, NN = 2 * n - 2, P = A.P;
-        // this CTA's sites [p0, p0 + Pl) of the tree's P (all of them when K = 1); its
-        // stored vectors hold Ps sites per slot; tip rows keep the stride P
-        const int Ps = K > 1 ? (((P + K - 1) / K + 3) & ~3) : P;
-        const int p0 = min(P, rank * Ps), Pl = min(P, p0 + Ps) - p0;
-        const uint8_t* tips0 = A.tips + p0;
-        const int32_t* w0 = A.w + p0;
+        const int n = G.ts.n, NN = 2 * n - 2, P = A.P, nsched = 3 * n - 5;
+        const Sites sx = make_sites(P, geo, rank, tm.kp);
+        const int Ps = sx.ld;
         STab<R, C> st;
-        st.pcap = (Ps + 3) & ~3;
-        st.s = reinterpret_cast<R*>(tab_base);
-        st.ew = st.s + (size_t)4 * C * st.pcap;
+        st.init(tab_base, Ps);
+        for (int m = 0; m < sx.cnt; ++m) st.w[sx.pl0 + m * sx.pstep] = (R)A.w[sx.p0 + m * sx.step];
         const size_t sstride = (size_t)Ps * 4 * C;
         const int tree = G.first + gi;
-        const int32_t* up = G.ts.up + (size_t)tree * NN;
-        const int32_t* ch = G.ts.ch + (size_t)tree * NN * 2;
-        const int32_t* sched = G.ts.sched + (size_t)tree * 3 * n;
         double* glen = G.ts.len + (size_t)tree * NN;
         // this CTA's own slab, reused tree after tree: partials, scalers and the P
         // matrices of every edge; the P matrices move to shared memory when the
-        // launch shape leaves it free (p_smem, see full_p_smem), else they are read
-        // from the slab through L1 and the shared memory holds the sum-table share
+        // launch shape leaves it free (p_smem, see full_p_smem), else an operation
+        // copies the two it reads
         unsigned char* const b = slab + (size_t)blockIdx.x * slab_per_cta;
         const size_t clv_bytes = ((size_t)(2 * n - 5) * Ps * 4 * C * sizeof(R) + 255) & ~size_t(255);
         const size_t scl_bytes = ((size_t)(2 * n - 5) * Ps * 4 + 255) & ~size_t(255);
@@ -2711,7 +2667,16 @@ __global__ void __launch_bounds__(512) k_fullopt(const FullGroup* __restrict__ g
         // per-tree category rates (a visit that re-optimises the Gamma shape), else the model's
         const double* rr = G.rates ? G.rates + (size_t)gi * kMaxCat : M.rates;
         init_newton_smem<R, C>(M, sm.ns, rr);
-        for (int v = threadIdx.x; v < NN; v += blockDim.x) len[v] = glen[v];
+        for (int v = threadIdx.x; v < NN; v += blockDim.x) {
+            len[v] = glen[v];
+            up[v] = (uint8_t)G.ts.up[(size_t)tree * NN + v];
+            ch[2 * v] = (uint8_t)G.ts.ch[((size_t)tree * NN + v) * 2];
+            ch[2 * v + 1] = (uint8_t)G.ts.ch[((size_t)tree * NN + v) * 2 + 1];
+        }
+        for (int k = threadIdx.x; k < nsched; k += blockDim.x) {
+            const int op = G.ts.sched[(size_t)tree * 3 * n + k];
+            sched[k] = (uint16_t)((op & 0xff) | (op & kUpd ? kUpd16 : 0));
+        }
         __syncthreads();
         for (int z = threadIdx.x; z < NN * C * 4; z += blockDim.x) {
             const int v = z / (C * 4), r = (z / 4) % C, i = z & 3;
@@ -2720,23 +2685,40 @@ __global__ void __launch_bounds__(512) k_fullopt(const FullGroup* __restrict__ g
         __syncthreads();
         auto srcD = [&](int v) {
             Src<R, C> y;
-            if (v < n) { y.clv = nullptr; y.scl = nullptr; y.tip = tips0 + (size_t)v * P; }
+            if (v < n) { y.clv = nullptr; y.scl = nullptr; y.tip = A.tips + (size_t)v * P; }
             else { y.clv = clv + (size_t)(v - n) * sstride; y.scl = scl + (size_t)(v - n) * Ps; y.tip = nullptr; }
             return y;
         };
-        auto srcU = [&](int v) {  // the vector at up[v] without v's subtree, for inner v != n
+        auto srcU = [&](int v) {  // the vector at up[v] without v's subtree, for inner v != n; leaf 0 for n
             Src<R, C> y;
             const int slot = n - 2 + (v - n - 1);
             y.clv = clv + (size_t)slot * sstride; y.scl = scl + (size_t)slot * Ps; y.tip = nullptr;
+            if (v == n) { y.clv = nullptr; y.scl = nullptr; y.tip = A.tips; }
             return y;
+        };
+        // the P matrices of edges a and b for the operation that follows
+        const R *Pa = sm.Pst[0], *Pb = sm.Pst[1];
+        auto stage_p = [&](int a, int b) {
+            if (p_smem) {
+                Pa = Psm + (size_t)a * C * 16;
+                Pb = Psm + (size_t)b * C * 16;
+                return;
+            }
+            __syncthreads();  // the operation before is done with the staged pair
+            for (int z = threadIdx.x; z < 2 * C * 16; z += blockDim.x)
+                (&sm.Pst[0][0])[z] = Pm[(size_t)(z < C * 16 ? a : b) * C * 16 + z % (C * 16)];
+            __syncthreads();
         };
         auto refreshD = [&](int v) {
             const int c0 = ch[2 * v], c1 = ch[2 * v + 1];
-            for (int p = threadIdx.x; p < Pl; p += blockDim.x) {
+            stage_p(c0, c1);
+            const Src<R, C> s0 = srcD(c0), s1 = srcD(c1);
+            for (int m = 0; m < sx.cnt; ++m) {
+                const int p = sx.pl0 + m * sx.pstep, pg = sx.p0 + m * sx.step;
                 R y0[4 * C], y1[4 * C];
                 int k0, k1;
-                apply_p<R, C>(Pm + (size_t)c0 * C * 16, srcD(c0), Ps, p, y0, k0);
-                apply_p<R, C>(Pm + (size_t)c1 * C * 16, srcD(c1), Ps, p, y1, k1);
+                apply_p<R, C>(Pa, s0, Ps, p, pg, y0, k0);
+                apply_p<R, C>(Pb, s1, Ps, p, pg, y1, k1);
                 mul_vec<R, C>(y0, y1);
                 const int sc = rescale<R, C>(y0);
                 store_vec<R, C>(clv + (size_t)(v - n) * sstride, Ps, p, y0);
@@ -2745,22 +2727,23 @@ __global__ void __launch_bounds__(512) k_fullopt(const FullGroup* __restrict__ g
         };
         // builds the sum-table of edge (v, up v), storing U_v for inner v
         auto visit_build = [&](int v) {
-            const Src<R, C> tip0 = {nullptr, nullptr, tips0};
-            for (int p = threadIdx.x; p < Pl; p += blockDim.x) {
+            const int u = up[v], sib = ch[2 * u] == v ? ch[2 * u + 1] : ch[2 * u];
+            if (v != n) stage_p(sib, u);
+            const Src<R, C> sv = srcD(v), ss = v == n ? srcU(n) : srcD(sib), su = srcU(v == n ? n : u);
+            for (int m = 0; m < sx.cnt; ++m) {
+                const int p = sx.pl0 + m * sx.pstep, pg = sx.p0 + m * sx.step;
                 R X[4 * C], Y[4 * C];
                 int cx, cy;
                 // D_v first: its load then overlaps the two below instead of waiting
                 // behind the store of U_v (the same array, so it could not be hoisted)
-                load_raw<R, C>(srcD(v), Ps, p, Y, cy);
+                load_raw<R, C>(sv, Ps, p, pg, Y, cy);
                 if (v == n) {
-                    load_raw<R, C>(tip0, Ps, p, X, cx);
+                    load_raw<R, C>(su, Ps, p, pg, X, cx);
                 } else {
-                    const int u = up[v];
-                    const int sib = ch[2 * u] == v ? ch[2 * u + 1] : ch[2 * u];
                     R y1[4 * C];
                     int k0, k1;
-                    apply_p<R, C>(Pm + (size_t)sib * C * 16, srcD(sib), Ps, p, X, k0);
-                    apply_p<R, C>(Pm + (size_t)u * C * 16, u == n ? tip0 : srcU(u), Ps, p, y1, k1);
+                    apply_p<R, C>(Pa, ss, Ps, p, pg, X, k0);
+                    apply_p<R, C>(Pb, su, Ps, p, pg, y1, k1);
                     mul_vec<R, C>(X, y1);
                     const int sc = rescale<R, C>(X);
                     cx = k0 + k1 + sc;
@@ -2772,22 +2755,23 @@ __global__ void __launch_bounds__(512) k_fullopt(const FullGroup* __restrict__ g
                 }
                 // Y is D_v as stored (kept above 2^-kScaleExp by the rescaling) or a tip:
                 // no normalisation needed (an exact power-of-two scale of the row)
-                const int ex = normalise<R, C>(X), ey = 0;
+                const int ex = normalise<R, C>(X);
                 R s4[4 * C];
                 sumtable<R, C>(sm.Mt, sm.pi, X, Y, s4);
-                st.put(p, s4, (R)(ex + ey - Prec<R>::kScaleExp * (cx + cy)), (R)w0[p]);
+                st.put(p, s4, ex - Prec<R>::kScaleExp * (cx + cy));
             }
         };
         // the stored vectors an operation of the schedule reads, requested into L2
-        // while the operation before it runs (its Newton iterations touch no HBM)
+        // while the operation before it runs (its Newton iterations touch no HBM): a
+        // slot is one run of memory, so one thread asks for it in one instruction
         auto prefetch_op = [&](int op) {
-            const size_t vb = (size_t)Pl * 4 * C * sizeof(R);
             auto slot = [&](int sl) {
-                prefetch_l2(clv + (size_t)sl * sstride, vb);
-                prefetch_l2(scl + (size_t)sl * Ps, (size_t)Pl * 4);
+                asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(clv + (size_t)sl * sstride),
+                             "r"((unsigned)(sstride * sizeof(R)))
+                             : "memory");
             };
-            if (op & kUpd) {
-                const int w = op & (kUpd - 1);
+            if (op & kUpd16) {
+                const int w = op & 0xff;
                 if (ch[2 * w] >= n) slot(ch[2 * w] - n);
                 if (ch[2 * w + 1] >= n) slot(ch[2 * w + 1] - n);
                 return;
@@ -2806,34 +2790,32 @@ __global__ void __launch_bounds__(512) k_fullopt(const FullGroup* __restrict__ g
         // bottom-up D pass
         if (!(pair_score && G.max_sweeps == 0))
             for (int v = NN - 1; v >= n; --v) refreshD(v);
-        int sweeps = 0, last = n;
+        int sweeps = 0;
         double tlast = 0.0;
-        const int nsched = 3 * n - 5;
         if (G.max_sweeps == 0 && !pair_score) visit_build(n);
         for (int sw = 0; sw < G.max_sweeps; ++sw) {
             ++sweeps;
             double moved = 0.0;
             for (int k = 0; k < nsched; ++k) {
                 const int op = sched[k];
-                if (op & kUpd) {
-                    if (k + 1 < nsched) prefetch_op(sched[k + 1]);
-                    refreshD(op & (kUpd - 1));
+                if (op & kUpd16) {
+                    if (threadIdx.x == 0 && k + 1 < nsched) prefetch_op(sched[k + 1]);
+                    refreshD(op & 0xff);
                     continue;
                 }
                 const int v = op;
                 visit_build(v);
-                if (k + 1 < nsched) prefetch_op(sched[k + 1]);
+                if (threadIdx.x == 0 && k + 1 < nsched) prefetch_op(sched[k + 1]);
                 const double told = len[v];
                 int ev;
                 bool conv;
                 // the solve leaves the P matrices of edge v at its new length in Pm
-                const double t = newton_solve<R, C, K>(M, cfg, st, Pl, told, sm.ns, ev, conv, Pm + (size_t)v * C * 16,
-                                                       &cseq, &nseq);
+                const double t = newton_solve<R, C, kClus>(M, cfg, st, sx, told, sm.ns, ev, conv,
+                                                           Pm + (size_t)v * C * 16, tm);
                 moved = fmax(moved, fabs(t - told));
                 evals_total += ev;
                 if (!conv) ++nonconv;
                 if (threadIdx.x == 0) len[v] = t;  // read again only after later barriers
-                last = v;
                 tlast = t;
             }
             if (moved <= cfg.sweep_tol) break;
@@ -2844,11 +2826,10 @@ __global__ void __launch_bounds__(512) k_fullopt(const FullGroup* __restrict__ g
         // free after the sweeps), the first inner node's combined at the root
         double f1;
         if constexpr (sizeof(R) == 4) {
-            f1 = fullopt_score_f2<C, K>(n, ch, len, A, tips0, w0, Pl, Ps, reinterpret_cast<float*>(clv), scl, sm.ns.W,
-                                        sm.ns.lr, &sm.Pf[0][0], &sm.Pfl[0][0], &sm.exf[0][0], M.pi, sm.ns.red,
-                                        sm.ns.cx, &cseq);
+            f1 = fullopt_score_f2<C, kClus>(n, ch, len, A, sx, reinterpret_cast<float*>(clv), scl, sm.ns.W, sm.ns.lr,
+                                            &sm.Pf[0][0], &sm.Pfl[0][0], &sm.exf[0][0], M.pi, sm.ns.red, tm);
         } else {
-            f1 = eval_lnl<R, C, K>(M, st, Pl, G.max_sweeps == 0 ? len[n] : tlast, sm.ns, &cseq);
+            f1 = eval_lnl<C, kClus>(M, st, sx, G.max_sweeps == 0 ? len[n] : tlast, sm.ns, tm);
         }
         sweeps_total += sweeps;
         __syncthreads();
@@ -2868,8 +2849,8 @@ __global__ void __launch_bounds__(512) k_fullopt(const FullGroup* __restrict__ g
         atomicAdd(&stats[kStFullSweeps], sweeps_total);
         atomicAdd(&stats[kStNonconv], nonconv);
     }
-    if (K > 1 && threadIdx.x == 0 && sm.ns.abort_) atomicAdd(&stats[kStTimeout], 1ull);
-    if constexpr (K > 1) cooperative_groups::this_cluster().sync();  // no CTA leaves while others may read it
+    if (kClus && threadIdx.x == 0 && sm.ns.abort_) atomicAdd(&stats[kStTimeout], 1ull);
+    if constexpr (kClus) cooperative_groups::this_cluster().sync();  // no CTA leaves while others may read it
 }
 
 inline int blocks_for(long long n, int t) { return (int)((n + t - 1) / t); }
@@ -3082,49 +3063,41 @@ void launch_lengths_to_input(cudaStream_t s, int n, int count, TreeSet ts, doubl
     ++g_launches;
 }
 
-size_t sumtable_bytes(int prec, int C, int P) {
-    size_t rs = prec == 0 ? 8 : 4;
-    size_t pcap = (size_t)((P + 3) & ~3);
-    return (4 * (size_t)C + 2) * rs * pcap + 16;
+// Sum-table of ld local sites: 4C values, the weight and (FP64) the exponent of each.
+size_t sumtable_bytes(int prec, int C, int ld) {
+    const size_t pcap = (size_t)((ld + 3) & ~3);
+    return prec == 0 ? (4 * (size_t)C + 2) * 8 * pcap : (4 * (size_t)C + 1) * 4 * pcap;
 }
 
 namespace {
-template <typename R, int C>
-size_t propose_fixed() { return (sizeof(ProposeSmem<R, C>) + 15) & ~size_t(15); }
-template <typename R, int C>
-size_t full_fixed(int n) {
-    const int NN = 2 * n - 2;
-    return ((sizeof(FullSmem<R, C>) + 15) & ~size_t(15)) + (((size_t)NN * 8 + 15) & ~size_t(15));
+constexpr size_t kSmemPerCta = 227 * 1024, kSmemPerCta2 = 233472 / 2 - 1024;  // one CTA per SM, two CTAs per SM
+template <typename F>
+size_t by_kind(int prec, int C, F f) {
+    if (prec == 0) return C == 1 ? f(double(), std::integral_constant<int, 1>()) : f(double(), std::integral_constant<int, 4>());
+    return C == 1 ? f(float(), std::integral_constant<int, 1>()) : f(float(), std::integral_constant<int, 4>());
+}
+size_t propose_fixed(int prec, int C) {
+    return by_kind(prec, C, [](auto r, auto c) { return (sizeof(ProposeSmem<decltype(r), decltype(c)::value>) + 15) & ~size_t(15); });
+}
+size_t full_fixed(int prec, int C, int n) {
+    return by_kind(prec, C, [](auto r, auto c) { return (sizeof(FullSmem<decltype(r), decltype(c)::value>) + 15) & ~size_t(15); }) +
+           full_meta_bytes(2 * n - 2);
+}
+// Where a full optimisation keeps the P matrices of a tree's edges: in shared
+// memory where that does not cost a resident CTA (512 threads take the SM's whole
+// register file, smaller CTAs run two to an SM), otherwise in the CTA's slab.
+bool full_p_smem(int prec, int C, int n, size_t f, int threads) {
+    const size_t pb = (size_t)(2 * n - 2) * C * 16 * (prec == 0 ? 8 : 4);
+    return f + pb <= (threads < 512 && f <= kSmemPerCta2 ? kSmemPerCta2 : kSmemPerCta);
 }
 }  // namespace
 
-size_t propose_smem_bytes(int prec, int C, int P, bool table_in_smem, int threads) {
-    (void)threads;
-    size_t f = prec == 0 ? (C == 1 ? propose_fixed<double, 1>() : propose_fixed<double, 4>())
-                         : (C == 1 ? propose_fixed<float, 1>() : propose_fixed<float, 4>());
-    return f + (table_in_smem ? sumtable_bytes(prec, C, P) : 0);
+size_t propose_smem_bytes(int prec, int C, int ld) {
+    return propose_fixed(prec, C) + (ld ? sumtable_bytes(prec, C, ld) : 0);
 }
-
-// Where a full optimisation keeps the P matrices of a tree's edges: in shared
-// memory when the CTA already takes the SM's whole register file (512 threads x
-// 128 registers, so one CTA per SM and no other taker for the shared memory) and
-// they fit beside the rest; otherwise in the CTA's slab, read through L1, which
-// leaves the shared memory to the sum-table share so that two smaller CTAs fit.
-static bool full_p_smem(int prec, int C, int n, int P, bool table_in_smem, int threads) {
-    const size_t f = (prec == 0 ? (C == 1 ? full_fixed<double, 1>(n) : full_fixed<double, 4>(n))
-                                : (C == 1 ? full_fixed<float, 1>(n) : full_fixed<float, 4>(n))) +
-                     (table_in_smem ? sumtable_bytes(prec, C, P) : 0);
-    const size_t pb = ((size_t)(2 * n - 2) * C * 16 * (prec == 0 ? 8 : 4) + 15) & ~size_t(15);
-    return threads >= 512 && f + pb <= (size_t)227 * 1024;
-}
-
-size_t fullopt_smem_bytes(int prec, int C, int n, int P, bool table_in_smem, int threads) {
-    size_t f = prec == 0 ? (C == 1 ? full_fixed<double, 1>(n) : full_fixed<double, 4>(n))
-                         : (C == 1 ? full_fixed<float, 1>(n) : full_fixed<float, 4>(n));
-    f += table_in_smem ? sumtable_bytes(prec, C, P) : 0;
-    if (full_p_smem(prec, C, n, P, table_in_smem, threads))
-        f += ((size_t)(2 * n - 2) * C * 16 * (prec == 0 ? 8 : 4) + 15) & ~size_t(15);
-    return f;
+size_t fullopt_smem_bytes(int prec, int C, int n, int ld, int threads) {
+    const size_t f = full_fixed(prec, C, n) + (ld ? sumtable_bytes(prec, C, ld) : 0);
+    return f + (full_p_smem(prec, C, n, f, threads) ? (size_t)(2 * n - 2) * C * 16 * (prec == 0 ? 8 : 4) : 0);
 }
 
 namespace {
@@ -3139,20 +3112,17 @@ void partials_t(cudaStream_t s, const Model& M, Aln A, TreeSet ts, int first, DC
                                                                                    lo);
     ++g_launches;
     if constexpr (sizeof(R) == 4) {
-        if (g.clv_lo) {
-            const size_t sm2 = (size_t)NN * C * 16 * 8;
-            cudaFuncSetAttribute(k_partials_f2<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2);
-            dim3 grid(count.cap, blocks_for(A.P, threads));
-            k_partials_f2<C><<<grid, threads, sm2, s>>>(M, A, ts, first, count, g, reinterpret_cast<float*>(pm), lo,
-                                                        with_up ? 1 : 0);
-            ++g_launches;
-            return;
-        }
+        const size_t sm2 = (size_t)NN * C * 16 * 8;
+        cudaFuncSetAttribute(k_partials_f2<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2);
+        dim3 grid(count.cap, blocks_for(A.P, threads));
+        k_partials_f2<C><<<grid, threads, sm2, s>>>(M, A, ts, first, count, g, reinterpret_cast<float*>(pm), lo,
+                                                    with_up ? 1 : 0);
+    } else {
+        const size_t smem = (size_t)NN * C * 16 * sizeof(R);
+        cudaFuncSetAttribute(k_partials<R, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        dim3 grid(count.cap, blocks_for(A.P, threads));
+        k_partials<R, C><<<grid, threads, smem, s>>>(M, A, ts, first, count, g, pm, with_up ? 1 : 0);
     }
-    size_t smem = (size_t)NN * C * 16 * sizeof(R);
-    cudaFuncSetAttribute(k_partials<R, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    dim3 grid(count.cap, blocks_for(A.P, threads));
-    k_partials<R, C><<<grid, threads, smem, s>>>(M, A, ts, first, count, g, pm, with_up ? 1 : 0);
     ++g_launches;
 }
 }  // namespace
@@ -3177,271 +3147,113 @@ void launch_partials(cudaStream_t s, int prec, const Model& M, Aln A, TreeSet ts
 }
 
 namespace {
+using PropKernel = void (*)(const PropGroup*, const int*, int, int*, Cfg, unsigned long long*, unsigned char*, size_t,
+                            Geo, int, int);
+using FullKernel = void (*)(const FullGroup*, const int*, int, int*, int, Cfg, unsigned long long*, unsigned char*,
+                            size_t, unsigned char*, size_t, int, Geo, int, int);
+// A kernel's form for a launch shape: clusters, one CTA with its table in shared
+// memory, or one CTA with its table in global scratch.
 template <typename R, int C>
-void propose_t(cudaStream_t s, const PropGroup* groups, const int* gstart, int ngroups, int* counter, Cfg cfg,
-               unsigned long long* stats, int threads, int grid, void* scratch, size_t spc, int maxP) {
-    const int prec = sizeof(R) == 8 ? 0 : 1;
-    if (scratch) {
-        const size_t smem = propose_smem_bytes(prec, C, maxP, false, threads);
-        cudaFuncSetAttribute(k_propose<R, C, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k_propose<R, C, false><<<grid, threads, smem, s>>>(groups, gstart, ngroups, counter, cfg, stats,
-                                                           reinterpret_cast<unsigned char*>(scratch), spc);
-    } else {
-        const size_t smem = propose_smem_bytes(prec, C, maxP, true, threads);
-        cudaFuncSetAttribute(k_propose<R, C, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k_propose<R, C, true><<<grid, threads, smem, s>>>(groups, gstart, ngroups, counter, cfg, stats, nullptr, 0);
-    }
-    ++g_launches;
+PropKernel prop_kernel(bool clus, bool smem_tab) {
+    return clus ? k_propose<R, C, true, true> : smem_tab ? k_propose<R, C, true, false> : k_propose<R, C, false, false>;
 }
-// Sites per CTA of a cluster of K CTAs sharing P sites (a multiple of 4).
-inline int cluster_share(int P, int K) { return ((P + K - 1) / K + 3) & ~3; }
+PropKernel prop_kernel(int prec, int C, bool clus, bool smem_tab) {
+    if (prec == 0) return C == 1 ? prop_kernel<double, 1>(clus, smem_tab) : prop_kernel<double, 4>(clus, smem_tab);
+    return C == 1 ? prop_kernel<float, 1>(clus, smem_tab) : prop_kernel<float, 4>(clus, smem_tab);
+}
+template <typename R, int C>
+FullKernel full_kernel(bool clus, bool smem_tab) {
+    return clus ? k_fullopt<R, C, true, true> : smem_tab ? k_fullopt<R, C, true, false> : k_fullopt<R, C, false, false>;
+}
+FullKernel full_kernel(int prec, int C, bool clus, bool smem_tab) {
+    if (prec == 0) return C == 1 ? full_kernel<double, 1>(clus, smem_tab) : full_kernel<double, 4>(clus, smem_tab);
+    return C == 1 ? full_kernel<float, 1>(clus, smem_tab) : full_kernel<float, 4>(clus, smem_tab);
+}
 
-// The proposal kernel as clusters of K (2, 4 or 8) CTAs, FP32 partials, 4
-// categories, sum-tables of maxP / K sites in shared memory.  grid: a multiple
-// of K.  Returns false when the configuration cannot be launched.
-template <int K>
-bool propose_cluster_t(cudaStream_t s, const PropGroup* groups, const int* gstart, int ngroups, int* counter, Cfg cfg,
-                       unsigned long long* stats, int threads, int grid, int maxP) {
-    if (K * ((threads + 31) / 32) > kMaxClusterWarps) return false;
-    const size_t smem = propose_smem_bytes(1, 4, cluster_share(maxP, K), true, threads);
-    auto kern = k_propose<float, 4, true, K>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
+// Resident CTAs of a kernel on the whole GPU as clusters of kp (a multiple of kp; 0:
+// cannot run), or as single CTAs (kp = 1).
+template <typename K>
+int resident(K kern, int kp, int threads, size_t smem, int sms) {
+    if (smem > kSmemPerCta || kp * ((threads + 31) / 32) > kMaxTeamWarps) return 0;
+    int nb = 0;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess && kp == 1) {
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, threads, smem);
+        nb *= sms;
+    } else if (e == cudaSuccess) {
+        cudaLaunchConfig_t lc = {};
+        lc.gridDim = dim3(kp * 1024);
+        lc.blockDim = dim3(threads);
+        lc.dynamicSmemBytes = smem;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = kp;
+        at[0].val.clusterDim.y = 1;
+        at[0].val.clusterDim.z = 1;
+        lc.attrs = at;
+        lc.numAttrs = 1;
+        e = cudaOccupancyMaxActiveClusters(&nb, kern, &lc);
+        nb *= kp;
     }
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return nb;
+}
+
+template <typename K, typename... A>
+void launch_shape(K kern, cudaStream_t s, int kp, int threads, int grid, size_t smem, A... args) {
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     cudaLaunchConfig_t lc = {};
-    lc.gridDim = dim3((grid / K) * K);
+    lc.gridDim = dim3(grid / kp * kp);
     lc.blockDim = dim3(threads);
     lc.dynamicSmemBytes = smem;
     lc.stream = s;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = K;
+    at[0].val.clusterDim.x = kp;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
     lc.attrs = at;
-    lc.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&lc, kern, groups, gstart, ngroups, counter, cfg, stats,
-                                             (unsigned char*)nullptr, (size_t)0);
-    ++g_launches;
-    return e == cudaSuccess;
-}
-
-// Resident clusters of K CTAs of the proposal kernel on the whole GPU (0: cannot run).
-template <int K>
-int propose_cluster_occ(int threads, int maxP) {
-    if (K * ((threads + 31) / 32) > kMaxClusterWarps) return 0;
-    const size_t smem = propose_smem_bytes(1, 4, cluster_share(maxP, K), true, threads);
-    auto kern = k_propose<float, 4, true, K>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
-        cudaGetLastError();
-        return 0;
-    }
-    cudaLaunchConfig_t lc = {};
-    lc.gridDim = dim3(K * 1024);
-    lc.blockDim = dim3(threads);
-    lc.dynamicSmemBytes = smem;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = K;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    lc.attrs = at;
-    lc.numAttrs = 1;
-    int nc = 0;
-    if (cudaOccupancyMaxActiveClusters(&nc, kern, &lc) != cudaSuccess) {
-        cudaGetLastError();
-        return 0;
-    }
-    return nc;
-}
-
-template <typename R, int C>
-void fullopt_t(cudaStream_t s, const FullGroup* groups, const int* gstart, int ngroups, int* counter, int maxN,
-               int maxP, Cfg cfg, unsigned long long* stats, int threads, int grid, void* scratch, size_t spc,
-               void* slab, size_t slab_per_cta) {
-    const int prec = sizeof(R) == 8 ? 0 : 1;
-    const int nn = 2 * maxN - 2;
-    unsigned char* sl = reinterpret_cast<unsigned char*>(slab);
-    if (scratch) {
-        const size_t smem = fullopt_smem_bytes(prec, C, maxN, maxP, false, threads);
-        const int ps = full_p_smem(prec, C, maxN, maxP, false, threads);
-        cudaFuncSetAttribute(k_fullopt<R, C, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k_fullopt<R, C, false><<<grid, threads, smem, s>>>(groups, gstart, ngroups, counter, nn, cfg, stats,
-                                                           reinterpret_cast<unsigned char*>(scratch), spc, sl,
-                                                           slab_per_cta, ps);
-    } else {
-        const size_t smem = fullopt_smem_bytes(prec, C, maxN, maxP, true, threads);
-        const int ps = full_p_smem(prec, C, maxN, maxP, true, threads);
-        cudaFuncSetAttribute(k_fullopt<R, C, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k_fullopt<R, C, true><<<grid, threads, smem, s>>>(groups, gstart, ngroups, counter, nn, cfg, stats, nullptr, 0,
-                                                          sl, slab_per_cta, ps);
-    }
+    lc.numAttrs = kp > 1 ? 1 : 0;
+    cudaLaunchKernelEx(&lc, kern, args...);
     ++g_launches;
 }
 }  // namespace
 
-namespace {
-template <typename R, int C>
-int prop_occ(int threads, bool smem_tab, int maxP) {
-    const int prec = sizeof(R) == 8 ? 0 : 1;
-    const size_t smem = propose_smem_bytes(prec, C, maxP, smem_tab, threads);
-    int nb = 0;
-    if (smem_tab) {
-        cudaFuncSetAttribute(k_propose<R, C, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_propose<R, C, true>, threads, smem);
-    } else {
-        cudaFuncSetAttribute(k_propose<R, C, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_propose<R, C, false>, threads, smem);
-    }
-    cudaGetLastError();
-    return nb;
+int propose_resident(int prec, int C, const Shape& h, int maxP, int sms) {
+    return resident(prop_kernel(prec, C, h.kp > 1, h.smem_tab), h.kp, h.geo.vt,
+                    propose_smem_bytes(prec, C, h.smem_tab ? geo_local(maxP, h.geo, h.geo.vt) : 0), sms);
 }
-// The full optimisation as clusters of K CTAs (FP32, 4 categories): each CTA
-// a 1/K share of the sites, sum-table share in shared memory, its own slab of
-// slab_per_cta bytes (fullopt_slab_bytes of the share).  Returns false when
-// the configuration cannot be launched.
-template <int K>
-bool fullopt_cluster_t(cudaStream_t s, const FullGroup* groups, const int* gstart, int ngroups, int* counter, int maxN,
-                       int maxP, Cfg cfg, unsigned long long* stats, int threads, int grid, void* slab,
-                       size_t slab_per_cta) {
-    if (K * ((threads + 31) / 32) > kMaxClusterWarps) return false;
-    const size_t smem = fullopt_smem_bytes(1, 4, maxN, cluster_share(maxP, K), true, threads);
-    const int ps = full_p_smem(1, 4, maxN, cluster_share(maxP, K), true, threads);
-    auto kern = k_fullopt<float, 4, true, K>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    cudaLaunchConfig_t lc = {};
-    lc.gridDim = dim3((grid / K) * K);
-    lc.blockDim = dim3(threads);
-    lc.dynamicSmemBytes = smem;
-    lc.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = K;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    lc.attrs = at;
-    lc.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&lc, kern, groups, gstart, ngroups, counter, 2 * maxN - 2, cfg, stats,
-                                             (unsigned char*)nullptr, (size_t)0,
-                                             reinterpret_cast<unsigned char*>(slab), slab_per_cta, ps);
-    ++g_launches;
-    return e == cudaSuccess;
+int fullopt_resident(int prec, int C, const Shape& h, int maxN, int maxP, int sms) {
+    return resident(full_kernel(prec, C, h.kp > 1, h.smem_tab), h.kp, h.geo.vt,
+                    fullopt_smem_bytes(prec, C, maxN, h.smem_tab ? geo_local(maxP, h.geo, h.geo.vt) : 0, h.geo.vt), sms);
 }
-
-template <int K>
-int fullopt_cluster_occ(int threads, int maxN, int maxP) {
-    if (K * ((threads + 31) / 32) > kMaxClusterWarps) return 0;
-    const size_t smem = fullopt_smem_bytes(1, 4, maxN, cluster_share(maxP, K), true, threads);
-    auto kern = k_fullopt<float, 4, true, K>;
-    if (smem > 227 * 1024 ||
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
-        cudaGetLastError();
-        return 0;
-    }
-    cudaLaunchConfig_t lc = {};
-    lc.gridDim = dim3(K * 1024);
-    lc.blockDim = dim3(threads);
-    lc.dynamicSmemBytes = smem;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = K;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    lc.attrs = at;
-    lc.numAttrs = 1;
-    int nc = 0;
-    if (cudaOccupancyMaxActiveClusters(&nc, kern, &lc) != cudaSuccess) {
-        cudaGetLastError();
-        return 0;
-    }
-    return nc;
-}
-
-template <typename R, int C>
-int full_occ(int threads, bool smem_tab, int maxN, int maxP) {
-    const int prec = sizeof(R) == 8 ? 0 : 1;
-    const size_t smem = fullopt_smem_bytes(prec, C, maxN, maxP, smem_tab, threads);
-    int nb = 0;
-    if (smem_tab) {
-        cudaFuncSetAttribute(k_fullopt<R, C, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_fullopt<R, C, true>, threads, smem);
-    } else {
-        cudaFuncSetAttribute(k_fullopt<R, C, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_fullopt<R, C, false>, threads, smem);
-    }
-    cudaGetLastError();
-    return nb;
-}
-}  // namespace
-
-int propose_blocks_per_sm(int prec, int C, int threads, bool smem_tab, int maxP) {
-    if (prec == 0) return C == 1 ? prop_occ<double, 1>(threads, smem_tab, maxP) : prop_occ<double, 4>(threads, smem_tab, maxP);
-    return C == 1 ? prop_occ<float, 1>(threads, smem_tab, maxP) : prop_occ<float, 4>(threads, smem_tab, maxP);
-}
-
-int fullopt_blocks_per_sm(int prec, int C, int threads, bool smem_tab, int maxN, int maxP) {
-    if (prec == 0)
-        return C == 1 ? full_occ<double, 1>(threads, smem_tab, maxN, maxP) : full_occ<double, 4>(threads, smem_tab, maxN, maxP);
-    return C == 1 ? full_occ<float, 1>(threads, smem_tab, maxN, maxP) : full_occ<float, 4>(threads, smem_tab, maxN, maxP);
-}
-
-bool propose_cluster_ok(int prec, int C, int K) { return prec == 1 && C == 4 && (K == 2 || K == 4 || K == 8); }
-
-int propose_cluster_grid(int prec, int C, int K, int threads, int maxP) {
-    if (!propose_cluster_ok(prec, C, K)) return 0;
-    const int nc = K == 2 ? propose_cluster_occ<2>(threads, maxP)
-                          : K == 4 ? propose_cluster_occ<4>(threads, maxP) : propose_cluster_occ<8>(threads, maxP);
-    return nc * K;
+int geometry_resident(int prec, int C, bool full, int K, int threads, size_t smem, int sms) {
+    if (prec != 1 || C != 4) return 0;
+    return full ? resident(full_kernel(prec, C, true, true), K, threads, smem, sms)
+                : resident(prop_kernel(prec, C, true, true), K, threads, smem, sms);
 }
 
 void launch_propose(cudaStream_t s, int prec, int C, const PropGroup* groups, const int* gstart, int ngroups,
-                    int* counter, Cfg cfg, unsigned long long* stats, int threads, int grid, void* scratch,
-                    size_t scratch_per_cta, int maxP, int cluster) {
-    if (cluster > 1 && propose_cluster_ok(prec, C, cluster)) {
-        const bool ok = cluster == 2 ? propose_cluster_t<2>(s, groups, gstart, ngroups, counter, cfg, stats, threads, grid, maxP)
-                        : cluster == 4 ? propose_cluster_t<4>(s, groups, gstart, ngroups, counter, cfg, stats, threads, grid, maxP)
-                                       : propose_cluster_t<8>(s, groups, gstart, ngroups, counter, cfg, stats, threads, grid, maxP);
-        if (ok) return;
-        cudaGetLastError();  // not launchable here: the single-CTA form below
-    }
-    if (prec == 0) {
-        if (C == 1) propose_t<double, 1>(s, groups, gstart, ngroups, counter, cfg, stats, threads, grid, scratch, scratch_per_cta, maxP);
-        else propose_t<double, 4>(s, groups, gstart, ngroups, counter, cfg, stats, threads, grid, scratch, scratch_per_cta, maxP);
-    } else {
-        if (C == 1) propose_t<float, 1>(s, groups, gstart, ngroups, counter, cfg, stats, threads, grid, scratch, scratch_per_cta, maxP);
-        else propose_t<float, 4>(s, groups, gstart, ngroups, counter, cfg, stats, threads, grid, scratch, scratch_per_cta, maxP);
-    }
-}
-
-int fullopt_cluster_grid(int prec, int C, int K, int threads, int maxN, int maxP) {
-    if (!propose_cluster_ok(prec, C, K)) return 0;
-    const int nc = K == 2 ? fullopt_cluster_occ<2>(threads, maxN, maxP)
-                          : K == 4 ? fullopt_cluster_occ<4>(threads, maxN, maxP) : fullopt_cluster_occ<8>(threads, maxN, maxP);
-    return nc * K;
+                    int* counter, Cfg cfg, unsigned long long* stats, const Shape& h, int grid, void* scratch,
+                    size_t scratch_per_cta, int maxP, int lo, int hi) {
+    launch_shape(prop_kernel(prec, C, h.kp > 1, h.smem_tab), s, h.kp, h.geo.vt, grid,
+                 propose_smem_bytes(prec, C, h.smem_tab ? geo_local(maxP, h.geo, h.geo.vt) : 0), groups, gstart, ngroups,
+                 counter, cfg, stats, reinterpret_cast<unsigned char*>(scratch), scratch_per_cta, h.geo, lo, hi);
 }
 
 void launch_fullopt(cudaStream_t s, int prec, int C, const FullGroup* groups, const int* gstart, int ngroups,
-                    int* counter, int maxN, int maxP, Cfg cfg, unsigned long long* stats, int threads, int grid,
-                    void* scratch, size_t scratch_per_cta, void* slab, size_t slab_per_cta, int cluster) {
-    if (cluster > 1 && slab && propose_cluster_ok(prec, C, cluster)) {
-        const bool ok =
-            cluster == 2 ? fullopt_cluster_t<2>(s, groups, gstart, ngroups, counter, maxN, maxP, cfg, stats, threads, grid, slab, slab_per_cta)
-            : cluster == 4 ? fullopt_cluster_t<4>(s, groups, gstart, ngroups, counter, maxN, maxP, cfg, stats, threads, grid, slab, slab_per_cta)
-                           : fullopt_cluster_t<8>(s, groups, gstart, ngroups, counter, maxN, maxP, cfg, stats, threads, grid, slab, slab_per_cta);
-        if (ok) return;
-        cudaGetLastError();  // not launchable here: the single-CTA form below
-    }
-    if (prec == 0) {
-        if (C == 1) fullopt_t<double, 1>(s, groups, gstart, ngroups, counter, maxN, maxP, cfg, stats, threads, grid, scratch, scratch_per_cta, slab, slab_per_cta);
-        else fullopt_t<double, 4>(s, groups, gstart, ngroups, counter, maxN, maxP, cfg, stats, threads, grid, scratch, scratch_per_cta, slab, slab_per_cta);
-    } else {
-        if (C == 1) fullopt_t<float, 1>(s, groups, gstart, ngroups, counter, maxN, maxP, cfg, stats, threads, grid, scratch, scratch_per_cta, slab, slab_per_cta);
-        else fullopt_t<float, 4>(s, groups, gstart, ngroups, counter, maxN, maxP, cfg, stats, threads, grid, scratch, scratch_per_cta, slab, slab_per_cta);
-    }
+                    int* counter, int maxN, int maxP, Cfg cfg, unsigned long long* stats, const Shape& h, int grid,
+                    void* scratch, size_t scratch_per_cta, void* slab, size_t slab_per_cta, int lo, int hi) {
+    const int ld = h.smem_tab ? geo_local(maxP, h.geo, h.geo.vt) : 0;
+    const size_t f = full_fixed(prec, C, maxN) + (ld ? sumtable_bytes(prec, C, ld) : 0);
+    launch_shape(full_kernel(prec, C, h.kp > 1, h.smem_tab), s, h.kp, h.geo.vt, grid,
+                 fullopt_smem_bytes(prec, C, maxN, ld, h.geo.vt), groups, gstart, ngroups, counter, 2 * maxN - 2, cfg,
+                 stats, reinterpret_cast<unsigned char*>(scratch), scratch_per_cta,
+                 reinterpret_cast<unsigned char*>(slab), slab_per_cta, full_p_smem(prec, C, maxN, f, h.geo.vt) ? 1 : 0,
+                 h.geo, lo, hi);
 }
 
 size_t fullopt_slab_bytes(int prec, int C, int n, int P) {

@@ -81,7 +81,8 @@ extern "C" pt_status pt_score_topologies_noalloc(int n_taxa, int n_patterns, con
 
     const int n = n_taxa, NN = 2 * n - 2, E = 2 * n - 3, P = n_patterns, prec = cfg.precision;
     const int threads = cfg.threads > 0 ? cfg.threads : (P <= 128 ? 128 : 256);
-    const bool smem_tab = fullopt_smem_bytes(prec, M.C, n, P, true, threads) <= (size_t)optin;
+    const bool smem_tab = fullopt_smem_bytes(prec, M.C, n, P, threads) <= (size_t)optin;
+    const Shape shape{Geo{threads, 1, 1}, 1, smem_tab ? 1 : 0};
     // layout: flags | stats | canonical trees | launch table | per-CTA partials slabs | per-CTA sum-tables
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off += up256(bytes); return o; };
@@ -163,7 +164,7 @@ extern "C" pt_status pt_score_topologies_noalloc(int n_taxa, int n_patterns, con
         cudaGetLastError();
         return PT_ERR_CUDA;
     }
-    launch_fullopt(stream, prec, M.C, d_group, d_gstart, 1, d_counter, n, P, k, stats, threads, grid,
+    launch_fullopt(stream, prec, M.C, d_group, d_gstart, 1, d_counter, n, P, k, stats, shape, grid,
                    smem_tab ? nullptr : base + o_tab, spc, base + o_slab, slab);
     launch_lengths_to_input(stream, n, n_trees, ts, lengths_out_dev);
     if (cudaGetLastError() != cudaSuccess) return PT_ERR_CUDA;
