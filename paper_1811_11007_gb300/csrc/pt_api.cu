@@ -485,10 +485,10 @@ int default_shares(Ctx& c, bool full, int prec, int C, int n, int P, int threads
     return any ? any : 1;
 }
 
-// A launch shape and the CTAs of it that are resident at once.
+// A launch shape, the CTAs of it that are resident at once, and the sites of a thread.
 struct ShapeFit {
     Shape h;
-    int resident;
+    int resident, sites;
 };
 // The shapes of a summation geometry (vt virtual threads, vk shares), by increasing
 // cluster size: vk CTAs per item, then 2, 4, 8 as long as the lanes of a virtual
@@ -496,40 +496,45 @@ struct ShapeFit {
 std::vector<ShapeFit> shapes_of(Ctx& c, bool full, int prec, int C, int maxN, int maxP, int vt, int vk) {
     std::vector<ShapeFit> v;
     auto fit = [&](const Shape& h) {
-        return occupancy(c, {full, prec, C, maxN, maxP, h.geo.vt, h.geo.vk * 64 + h.kp, h.smem_tab}, [&] {
+        return occupancy(c, {full, prec, C, maxN, maxP, h.geo.vt, (h.geo.vk * 64 + h.kp) * 1024 + h.pt, h.smem_tab}, [&] {
             return full ? fullopt_resident(prec, C, h, maxN, maxP, c.sm_count)
                         : propose_resident(prec, C, h, maxP, c.sm_count);
         });
     };
     const int J = (cluster_sites(maxP, vk) + vt - 1) / vt;  // sites per virtual thread
-    for (int lanes = 1; vk * lanes <= 8 && (lanes == 1 || lanes < 2 * J); lanes *= 2) {
-        const Shape h{Geo{vt, vk, lanes}, vk * lanes, 1};
-        const int r = fit(h);
-        if (r > 0) v.push_back({h, r});
-    }
+    for (int kp : {1, 2, 4, 8})
+        for (int pt : {vt, vt / 2}) {
+            const int lanes = kp * pt / (vk * vt);
+            if (pt < 128 && pt != vt) continue;
+            if (lanes < 1 || kp * pt != vk * vt * lanes || (lanes > 1 && lanes >= 2 * J) || (kp == 1 && pt != vt)) continue;
+            const Shape h{Geo{vt, vk, lanes}, kp, pt, 1};
+            const int r = fit(h);
+            if (r >= kp) v.push_back({h, r, (J + lanes - 1) / lanes});
+        }
     if (v.empty() && vk > 1) return shapes_of(c, full, prec, C, maxN, maxP, vt, 1);  // not launchable as clusters
     if (v.empty()) {  // a sum-table too large for shared memory in every form
-        const Shape h{Geo{vt, 1, 1}, 1, 0};
-        v.push_back({h, std::max(fit(h), c.sm_count)});
+        const Shape h{Geo{vt, 1, 1}, 1, vt, 0};
+        v.push_back({h, std::max(fit(h), c.sm_count), J});
     }
     return v;
 }
-// The shape for more items than are resident at once: the smallest cluster with
-// (nearly) the most resident threads.
-const ShapeFit& full_load(const std::vector<ShapeFit>& v) {
-    int most = 0;
-    for (const ShapeFit& x : v) most = std::max(most, x.resident);
-    for (const ShapeFit& x : v)
-        if (10 * x.resident >= 9 * most) return x;
-    return v.back();
-}
-// The shape for `total` items: the largest clusters that are all resident at once
-// (an item's time falls with the lanes and SMs it gets while the rest of the GPU
-// would idle), else full_load.
+// The shape for `total` items: the least (rounds of resident items) x (time of an
+// item), an item's time being the fixed chain of a Newton evaluation (reduction,
+// exchange, step), worth about 5 sites of a thread, plus the thread's sites.
+// Measured on visits of 81 trees at 12 sites per virtual thread: 26.0 ms on one CTA
+// each, 19.1 on 2, 13.1 on 4 (1.1 rounds), 18.2 on 8 (2.3 rounds); on 5697 neighbours
+// at 7 sites: 84.8 ms as 8 CTAs of 256 (36 resident), 69.1 as 8 of 128 (51 resident).
 const ShapeFit& pick_shape(const std::vector<ShapeFit>& v, long long total) {
-    for (size_t i = v.size(); i-- > 0;)
-        if (total * v[i].h.kp <= v[i].resident) return v[i];
-    return full_load(v);
+    size_t best = 0;
+    double cost = 1e300;
+    for (size_t i = 0; i < v.size(); ++i) {
+        const double x = std::max(1.0, (double)total * v[i].h.kp / v[i].resident) * (5 + v[i].sites);
+        if (x < 0.999 * cost) {
+            cost = x;
+            best = i;
+        }
+    }
+    return v[best];
 }
 // The shapes of a launch whose number of items is only known on the device (at
 // most cap): each with the counts (lo, hi] it is launched for, as pick_shape picks.
@@ -539,15 +544,15 @@ struct ShapeRange {
 };
 std::vector<ShapeRange> shape_ranges(const std::vector<ShapeFit>& v, int cap) {
     std::vector<ShapeRange> out;
-    int lo = 0;
-    for (size_t i = v.size(); i-- > 0 && lo < cap;) {
-        const int hi = v[i].resident / v[i].h.kp;
-        if (hi > lo) {
-            out.push_back({v[i], lo, hi});
-            lo = hi;
-        }
+    long long most = 0;  // past this count every shape has more than one round: the choice is settled
+    for (const ShapeFit& x : v) most = std::max<long long>(most, x.resident / x.h.kp + 1);
+    for (int n = 1; n <= std::min<long long>(cap, most); ++n) {
+        const ShapeFit& f = pick_shape(v, n);
+        const bool same = !out.empty() && out.back().f.h.kp == f.h.kp && out.back().f.h.pt == f.h.pt;
+        if (same) out.back().hi = n;
+        else out.push_back({f, n - 1, n});
     }
-    if (lo < cap) out.push_back({full_load(v), lo, INT_MAX});
+    if (!out.empty()) out.back().hi = INT_MAX;
     return out;
 }
 
@@ -694,7 +699,7 @@ void run_full_jobs(Ctx& c, std::vector<FullJob> jobs, bool allow_tune = true) {
                 scratch = buf<unsigned char>(c, "full.scratch", spc * grid);
             }
             for (const FullJob& j : jobs)
-                sl = std::max(sl, fullopt_slab_bytes(prec, C, j.a->n, geo_local(j.a->P, f.h.geo, threads)));
+                sl = std::max(sl, fullopt_slab_bytes(prec, C, j.a->n, geo_local(j.a->P, f.h.geo, f.h.pt)));
             unsigned char* slab = buf<unsigned char>(c, "full.slab", sl * grid);
             ck(c, cudaMemsetAsync(counter, 0, sizeof(int), c.stream), "counter");
             size_t e0 = timed ? ev_record(c) : 0;
@@ -1677,7 +1682,7 @@ int range_grid(const ShapeRange& x) {
 size_t graph_slab(const Ctx& c, const GraphRound& g, const ShapeRange& x) {
     size_t b = 0;
     for (const GraphAln& a : g.a)
-        b = std::max(b, fullopt_slab_bytes(c.cfg.precision, c.alns[a.aln].M.C, a.n, geo_local(a.P, x.f.h.geo, x.f.h.geo.vt)));
+        b = std::max(b, fullopt_slab_bytes(c.cfg.precision, c.alns[a.aln].M.C, a.n, geo_local(a.P, x.f.h.geo, x.f.h.pt)));
     return b;
 }
 

@@ -133,16 +133,17 @@ PT_INLINE int cluster_sites(int P, int K) { return K > 1 ? ((P + K - 1) / K + 3)
 struct Geo {
     int vt, vk, lanes;
 };
-// A launch shape of the persistent kernels: clusters of kp = vk * lanes CTAs of
-// geo.vt threads per item; smem_tab 0: one CTA with its sum-table in global scratch.
+// A launch shape of the persistent kernels: clusters of kp CTAs of pt threads per
+// item (kp * pt = vk * vt * lanes); smem_tab 0: one CTA with its sum-table in global
+// scratch.
 struct Shape {
     Geo geo;
-    int kp, smem_tab;
+    int kp, pt, smem_tab;
 };
 // Local sites of one CTA of `threads` threads (its sum-table's and slab's capacity).
 PT_INLINE int geo_local(int P, const Geo& g, int threads) {
     const int Ps = cluster_sites(P, g.vk), step = g.vt * g.lanes;
-    return g.lanes == 1 ? Ps : (Ps + step - 1) / step * threads;
+    return g.lanes == 1 && threads == g.vt ? Ps : (Ps + step - 1) / step * threads;
 }
 // Warps of a cluster whose Newton sums one CTA receives: shapes above it are not offered.
 constexpr int kMaxTeamWarps = 128;

@@ -18,6 +18,7 @@
 // without barriers.
 #include "pt_internal.h"
 #include "pt_gamma.h"
+#include "pt_math.h"
 
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
@@ -46,7 +47,7 @@ template <> struct Prec<float> {
     __device__ static float mult() { return 4294967296.0f; }                // 2^32
     __device__ static float ex(float x) { return expf(x); }
     __device__ static float lg(float x) { return logf(x); }
-    __device__ static float rcp(float x) { return __frcp_rn(x); }
+    __device__ static float rcp(float x) { return rcp_rn(x); }
     __device__ static float mul(float x, float y) { return __fmul_rn(x, y); }  // never part of an FMA
 };
 template <> struct Prec<double> {
@@ -1449,11 +1450,11 @@ __device__ __forceinline__ void mbar_arrive(unsigned long long* bar) {
         "mbarrier.arrive.release.cta.shared::cta.b64 st, [%0];\n\t}" ::"r"(smem_addr(bar))
         : "memory");
 }
-__device__ __forceinline__ bool mbar_try_wait(unsigned long long* bar, unsigned parity) {
+__device__ __forceinline__ bool mbar_test_wait(unsigned long long* bar, unsigned parity) {
     uint32_t ok;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "mbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
         "selp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(ok)
         : "r"(smem_addr(bar)), "r"(parity)
@@ -1490,6 +1491,19 @@ __device__ __forceinline__ void cluster_exchange_init(NS& ns) {
     mbar_fence_init();
 }
 
+// A branch length between the solves: an FP32 pair in mixed precision (the steps
+// are taken on pairs; every FP64 instruction costs its warp some 60 cycles and the
+// SM's one FP64 pipe 16, whoever issues it), FP64 in the FP64 path.
+template <typename R> struct LenOf { using T = double; };
+template <> struct LenOf<float> { using T = F2; };
+template <typename R> using Len = typename LenOf<R>::T;
+template <typename R> __device__ __forceinline__ Len<R> len_of(double x) {
+    if constexpr (sizeof(R) == 4) return f2_of(x);
+    else return x;
+}
+__device__ __forceinline__ double len_dbl(F2 x) { return (double)x.h + (double)x.l; }
+__device__ __forceinline__ double len_dbl(double x) { return x; }
+
 // Block-wide context for the Newton machinery.
 template <typename R, int C>
 struct NewtonSmem {
@@ -1499,10 +1513,11 @@ struct NewtonSmem {
     float lrf[4 * C];      // the same in FP32 (coefficients of the Newton derivatives)
     double ex[4 * C];      // exp(lam_k r t) for a P-matrix refresh
     double W[64];          // W[(i*4+j)*4+k] = isqpi_i sqpi_j R_ik R_jk: P_ij = sum_k W_ijk exp(lam_k r t)
-    double tb;             // broadcast of the current length
+    Len<R> tmin, tmax, tol, sweep_tol, prior;  // the solver's constants
+    int moved_at;          // last sweep (from 1) of the item that moved a length by more than sweep_tol
     int done;
     int leader;            // the warp that takes the Newton steps
-    // Newton sums: each warp's (d1 h, l, d2 h, l) in FP32 or (d1, d2) in FP64; in a
+    // Newton sums: each warp's (d1 h, d2 h, d1 l, d2 l) in FP32 or (d1, d2) in FP64; in a
     // cluster every warp of every CTA pushes its entry into entry rank * nw + warp of
     // every CTA's slot, two alternating slots, each with an mbarrier that counts the
     // bytes it received
@@ -1523,23 +1538,28 @@ struct Team {
 // the lanes are added neighbours first (entries past ne count as zero, exactly).
 __device__ __forceinline__ int tree_per(int ne) { return ne > 64 ? 4 : ne > 32 ? 2 : 1; }
 
+// Two sums at once as FP32 pairs (h, l) x (d1, d2), added by packed two-sums.
+struct Sum2 {
+    f32x2 h, l;
+};
+__device__ __forceinline__ Sum2 sum2_add(Sum2 a, Sum2 b) {
+    const f32x2 t = padd(a.h, b.h), bb = psub(t, a.h);
+    const f32x2 err = padd(psub(a.h, psub(t, bb)), psub(b.h, bb));
+    return Sum2{t, padd(padd(a.l, b.l), err)};
+}
+__device__ __forceinline__ Sum2 sum2_xor(Sum2 a, int o) {
+    return Sum2{make_float2(__shfl_xor_sync(0xffffffffu, a.h.x, o), __shfl_xor_sync(0xffffffffu, a.h.y, o)),
+                make_float2(__shfl_xor_sync(0xffffffffu, a.l.x, o), __shfl_xor_sync(0xffffffffu, a.l.y, o))};
+}
 // Compensated warp sums of two FP32 partials (two-sums over the virtual threads of
 // the warp, which lie `lanes` apart; neighbours first): every lane ends with both
-// sums as unevaluated pairs (d1 h, l, d2 h, l), with no FP64 instruction.
-__device__ __forceinline__ float4 warp_sum_comp(float x, float y, int lanes) {
-    float s = x, c = 0.f, s2 = y, c2 = 0.f;
+// sums as unevaluated pairs, with no FP64 instruction.
+__device__ __forceinline__ Sum2 warp_sum_comp(float x, float y, int lanes) {
+    Sum2 a{make_float2(x, y), make_float2(0.f, 0.f)};
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        if (o < lanes) continue;
-        const float os = __shfl_xor_sync(0xffffffffu, s, o), oc = __shfl_xor_sync(0xffffffffu, c, o);
-        const float os2 = __shfl_xor_sync(0xffffffffu, s2, o), oc2 = __shfl_xor_sync(0xffffffffu, c2, o);
-        const F2 u = f2_two_sum(s, os), v = f2_two_sum(s2, os2);
-        s = u.h;
-        c = __fadd_rn(__fadd_rn(c, oc), u.l);
-        s2 = v.h;
-        c2 = __fadd_rn(__fadd_rn(c2, oc2), v.l);
-    }
-    return make_float4(s, c, s2, c2);
+    for (int o = 1; o < 32; o <<= 1)
+        if (o >= lanes) a = sum2_add(a, sum2_xor(a, o));
+    return a;
 }
 __device__ __forceinline__ double warp_sum(double x, int lanes) {
 #pragma unroll
@@ -1549,7 +1569,8 @@ __device__ __forceinline__ double warp_sum(double x, int lanes) {
 }
 
 template <typename R, int C>
-__device__ __forceinline__ void init_newton_smem(const Model& M, NewtonSmem<R, C>& ns, const double* rates) {
+__device__ __forceinline__ void init_newton_smem(const Model& M, const Cfg& cfg, NewtonSmem<R, C>& ns,
+                                                 const double* rates) {
     for (int x = threadIdx.x; x < 64; x += blockDim.x) {
         int k = x & 3, ij = x >> 2, i = ij >> 2, j = ij & 3;
         ns.W[x] = M.isqpi[i] * M.sqpi[j] * M.R[i * 4 + k] * M.R[j * 4 + k];
@@ -1567,6 +1588,17 @@ __device__ __forceinline__ void init_newton_smem(const Model& M, NewtonSmem<R, C
         for (int w = 0; w < nw && w < 4; ++w)
             if ((int)((slot + w) & 3) == want) { lead = w; break; }
         ns.leader = lead;
+        ns.moved_at = 0;
+        ns.tmin = len_of<R>(cfg.tmin);
+        ns.tmax = len_of<R>(cfg.tmax);
+        ns.tol = len_of<R>(cfg.newton_tol);
+        ns.sweep_tol = len_of<R>(cfg.sweep_tol);
+        ns.prior = len_of<R>(cfg.prior_rate);
+    }
+    if (threadIdx.x < C) {  // the stationary slots' coefficients never change
+        ns.egh[0][threadIdx.x] = (R)(1.0f / C);
+        ns.egh[1][threadIdx.x] = R(0);
+        ns.egh[2][threadIdx.x] = R(0);
     }
     for (int q = threadIdx.x; q < 4 * C; q += blockDim.x) {
         ns.lr[q] = M.lam[q / C] * rates[q % C];
@@ -1576,48 +1608,26 @@ __device__ __forceinline__ void init_newton_smem(const Model& M, NewtonSmem<R, C
 
 // Coefficients at branch length t on the sum-table (see sumtable()): egh[0]
 // gives L (1 for the stationary slot, expm1(lam r t) otherwise), egh[1] and
-// egh[2] give dL/dt and d2L/dt2; all divided by C.  Called by the first 4C
-// threads (or the lanes q of one warp).  exact = FP64 exponentials rounded once (for lnL), otherwise the
-// working precision's own (for Newton derivatives).
-template <typename R, int C>
-__device__ __forceinline__ void put_egh(const Model& M, double t, NewtonSmem<R, C>& ns, bool exact,
-                                        int q = threadIdx.x) {
-    if (q < 4 * C) {
-        if (q < C) {
-            ns.egh[0][q] = (R)(1.0 / C);
-            ns.egh[1][q] = R(0);
-            ns.egh[2][q] = R(0);
-        } else {
-            const double lr = ns.lr[q];
-            if (exact || sizeof(R) == 8) {
-                ns.egh[0][q] = (R)(expm1(lr * t) / C);
-                double e = exp(lr * t) / C;
-                ns.egh[1][q] = (R)(lr * e);
-                ns.egh[2][q] = (R)(lr * lr * e);
-            } else {
-                const float l = ns.lrf[q], x = l * (float)t, e = expf(x) * (1.0f / C);
-                ns.egh[0][q] = (R)(expm1f(x) * (1.0f / C));
-                ns.egh[1][q] = (R)(l * e);
-                ns.egh[2][q] = (R)(l * l * e);
-            }
-        }
+// egh[2] give dL/dt and d2L/dt2; all divided by C.  Called by the lanes q of one
+// warp (the stationary slots q < C are set once, init_newton_smem), in the working
+// precision's own exponentials; no FP64 instruction in FP32.
+template <int C>
+__device__ __forceinline__ void put_egh(F2 t, NewtonSmem<float, C>& ns, int q) {
+    if (q >= C && q < 4 * C) {
+        const float l = ns.lrf[q], x = l * t.h, e = expf(x) * (1.0f / C);
+        ns.egh[0][q] = expm1f(x) * (1.0f / C);
+        ns.egh[1][q] = l * e;
+        ns.egh[2][q] = l * l * e;
     }
 }
-
-// put_egh's FP32 branch for a length given as FP32 (no FP64 instruction).
-template <typename R, int C>
-__device__ __forceinline__ void put_egh_f(float t, NewtonSmem<R, C>& ns, int q) {
-    if (q < 4 * C) {
-        if (q < C) {
-            ns.egh[0][q] = (R)(1.0f / C);
-            ns.egh[1][q] = R(0);
-            ns.egh[2][q] = R(0);
-        } else {
-            const float l = ns.lrf[q], x = l * t, e = expf(x) * (1.0f / C);
-            ns.egh[0][q] = (R)(expm1f(x) * (1.0f / C));
-            ns.egh[1][q] = (R)(l * e);
-            ns.egh[2][q] = (R)(l * l * e);
-        }
+template <int C>
+__device__ __forceinline__ void put_egh(double t, NewtonSmem<double, C>& ns, int q) {
+    if (q >= C && q < 4 * C) {
+        const double lr = ns.lr[q];
+        ns.egh[0][q] = expm1(lr * t) / C;
+        const double e = exp(lr * t) / C;
+        ns.egh[1][q] = lr * e;
+        ns.egh[2][q] = lr * lr * e;
     }
 }
 
@@ -1683,7 +1693,7 @@ __device__ __forceinline__ F2 f2_sub(F2 a, F2 b) {
     return f2_norm(d.h, __fadd_rn(d.l, __fsub_rn(a.l, b.l)));
 }
 __device__ __forceinline__ F2 f2_div(F2 a, F2 b) {
-    const float rc = __frcp_rn(b.h);
+    const float rc = rcp_rn(b.h);
     const float q0 = __fmul_rn(a.h, rc);
     const float p = __fmul_rn(q0, b.h), pe = __fmaf_rn(q0, b.h, -p);
     // a - q0 b: a.h - p is exact (p lies within a factor 2 of a.h)
@@ -1695,7 +1705,7 @@ __device__ __forceinline__ F2 f2_sqrt(F2 x) {
     if (!(s0 > 0.f)) return F2{s0, 0.f};
     const float p = __fmul_rn(s0, s0), pe = __fmaf_rn(s0, s0, -p);
     const float r = __fadd_rn(__fsub_rn(__fsub_rn(x.h, p), pe), x.l);
-    return f2_norm(s0, __fmul_rn(r, __fmul_rn(0.5f, __frcp_rn(s0))));
+    return f2_norm(s0, __fmul_rn(r, __fmul_rn(0.5f, rcp_rn(s0))));
 }
 __device__ __forceinline__ bool newton_step_f2(F2& t, F2& lo, F2& hi, F2 d1, F2 d2, F2 tol) {
     if (d1.h == 0.f) return true;  // d1 == 0 (a pair is zero iff its high part is)
@@ -1750,9 +1760,9 @@ __device__ __forceinline__ void add_score(double& acc, double term, int lanes) {
 // lnL of the current sum-table at length t: sum_p w_p (ln L_p + E_p ln 2) (FP64;
 // the mixed path scores from pairs).
 template <int C, bool kClus>
-__device__ double eval_lnl(const Model& M, const STab<double, C>& st, const Sites& sx, double t,
+__device__ double eval_lnl(const STab<double, C>& st, const Sites& sx, double t,
                            NewtonSmem<double, C>& ns, Team& tm) {
-    put_egh<double, C>(M, t, ns, true);
+    put_egh<C>(t, ns, threadIdx.x);
     __syncthreads();
     double e[4 * C];
 #pragma unroll
@@ -1803,37 +1813,44 @@ __device__ __forceinline__ void newton_site(const STab<R, C>& st, int p, const R
     wt = st.w[p];
 }
 
-// Newton solve on the current sum-table from t0.  Per evaluation: every
-// thread sums w L'/L and w (L''/L - (L'/L)^2) over its sites, the warps
-// reduce, and one warp alone takes the step and writes the coefficients
-// of the next length; after the last step it also writes P_r(t) of the
-// final length into Pdst [16][C] (visible when the call returns).  Returns
-// the final length (in every thread).
+// Sets up a solve from length t0 (the coefficients of its first evaluation) and
+// returns t0 within the bounds; called before the sum-table is built, by every
+// thread, after the last barrier of the solve before.
+template <int C>
+__device__ __forceinline__ F2 newton_begin(F2 t0, NewtonSmem<float, C>& ns) {
+    F2 t = f2_lt(t0, ns.tmin) ? ns.tmin : t0;
+    if (f2_lt(ns.tmax, t)) t = ns.tmax;
+    put_egh<C>(t, ns, threadIdx.x);
+    return t;
+}
+template <int C>
+__device__ __forceinline__ double newton_begin(double t0, NewtonSmem<double, C>& ns) {
+    const double t = fmin(fmax(t0, ns.tmin), ns.tmax);
+    put_egh<C>(t, ns, threadIdx.x);
+    return t;
+}
+
+// Newton solve on the current sum-table from t (as newton_begin returned it).  Per
+// evaluation: every thread sums w L'/L and w (L''/L - (L'/L)^2) over its sites, the
+// warps reduce, and one warp alone takes the step and writes the coefficients of
+// the next length.  After the last step that warp stores the length in *dst, notes
+// in ns.moved_at whether it is more than sweep_tol from told (sweep number sweep),
+// and P_r of the final length goes to Pdst [16][C]; all visible when the call
+// returns.  Everything but the sums over sites is that warp's: what one warp does in
+// FP64 or in a long chain holds up one scheduler, what every warp does, all of them.
 // kClus: the sum-table holds this CTA's share of a cluster's sites; each
 // evaluation's derivative sums are exchanged over the cluster, and every CTA
 // takes the same step.
 template <typename R, int C, bool kClus>
-__device__ double newton_solve(const Model& M, const Cfg& cfg, const STab<R, C>& st, const Sites& sx, double t0,
-                               NewtonSmem<R, C>& ns, int& evals, bool& converged, R* Pdst, Team& tm) {
-    double lo = cfg.tmin, hi = cfg.tmax;
-    double t = fmin(fmax(t0, lo), hi);
+__device__ __forceinline__ void newton_solve(const Cfg& cfg, const STab<R, C>& st, const Sites& sx, Len<R> t,
+                                             Len<R> told, Len<R>* dst, int sweep, NewtonSmem<R, C>& ns, int& evals,
+                                             bool& converged, R* Pdst, Team& tm) {
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5;
-    const bool prior = __double_as_longlong(cfg.prior_rate) != 0;
-    put_egh<R, C>(M, t, ns, false);
-    if (threadIdx.x == 0) ns.tb = t;
-    __syncthreads();
+    __syncthreads();  // the coefficients of newton_begin
     const int ld = ns.leader;
+    Len<R> lo = ns.tmin, hi = ns.tmax;
     converged = false;
     evals = 0;
-    // mixed precision: the leader's step on pairs (t, bracket, tolerance, prior slope)
-    F2 tp{0.f, 0.f}, lop{0.f, 0.f}, hip{0.f, 0.f}, tolp{0.f, 0.f}, prp{0.f, 0.f};
-    if (sizeof(R) == 4 && w == ld) {
-        tp = f2_of(t);
-        lop = f2_of(lo);
-        hip = f2_of(hi);
-        tolp = f2_of(cfg.newton_tol);
-        prp = f2_of(cfg.prior_rate);
-    }
     for (int it = 0; it < cfg.newton_maxit; ++it) {
         R e[4 * C], g[4 * C], h[4 * C];
 #pragma unroll
@@ -1879,7 +1896,8 @@ __device__ double newton_solve(const Model& M, const Cfg& cfg, const STab<R, C>&
         const int xe = tm.nseq++, cs = kClus ? xe & 1 : 0;
         float4 v;
         if constexpr (sizeof(R) == 4) {
-            v = warp_sum_comp(a1, a2, sx.lanes);
+            const Sum2 a = warp_sum_comp(a1, a2, sx.lanes);
+            v = make_float4(a.h.x, a.h.y, a.l.x, a.l.y);
         } else {
             const double2 d = make_double2(warp_sum(a1, sx.lanes), warp_sum(a2, sx.lanes));
             v = reinterpret_cast<const float4&>(d);
@@ -1888,12 +1906,13 @@ __device__ double newton_solve(const Model& M, const Cfg& cfg, const STab<R, C>&
             // Slot cs is free in every CTA: a warp pushes exchange xe only after its
             // CTA's leader received all of exchange xe - 1, which every CTA pushed
             // after its own leader had read exchange xe - 2 (the last use of cs).
-            if (lane == 0) {
-                float* slot = &ns.cxr[cs][tm.rank * nw + w][0];
-                for (int r = 0; r < tm.kp; ++r)
-                    if (r != tm.rank) cluster_push16(slot, &ns.mbx[cs], (unsigned)r, v);
+            // Every lane holds the warp's sums: lane r pushes them to CTA r.
+            float* slot = &ns.cxr[cs][tm.rank * nw + w][0];
+            if (lane == tm.rank) {
                 *reinterpret_cast<float4*>(slot) = v;  // this CTA's own copy
                 mbar_arrive(&ns.mbx[cs]);
+            } else if (lane < tm.kp) {
+                cluster_push16(slot, &ns.mbx[cs], (unsigned)lane, v);
             }
             // no block barrier here: only the leader needs the sums
         } else {
@@ -1908,7 +1927,7 @@ __device__ double newton_solve(const Model& M, const Cfg& cfg, const STab<R, C>&
                 bool ok = ns.abort_ != 0;  // after a wait ran out, none is waited for again
                 const long long tw = clock64();
                 while (!ok) {
-                    ok = mbar_try_wait(&ns.mbx[cs], (unsigned)(xe >> 1) & 1u);
+                    ok = mbar_test_wait(&ns.mbx[cs], (unsigned)(xe >> 1) & 1u);
                     if (!ok && clock64() - tw > kExchangeWaitCycles) break;
                 }
                 if (__any_sync(0xffffffffu, !ok) && lane == 0) ns.abort_ = 1;
@@ -1921,30 +1940,26 @@ __device__ double newton_solve(const Model& M, const Cfg& cfg, const STab<R, C>&
                 // FP32 pairs, added by two-sums (~48 bits)
                 auto entry = [&](int k) {
                     const int i = lane * per + k;
-                    return k < per && i < ne ? *reinterpret_cast<const float4*>(&ns.cxr[cs][i][0])
-                                             : make_float4(0.f, 0.f, 0.f, 0.f);
+                    const float4 q = k < per && i < ne ? *reinterpret_cast<const float4*>(&ns.cxr[cs][i][0])
+                                                       : make_float4(0.f, 0.f, 0.f, 0.f);
+                    return Sum2{make_float2(q.x, q.y), make_float2(q.z, q.w)};
                 };
-                auto add = [](float4 x, float4 y) {
-                    const F2 u = f2_two_sum(x.x, y.x), z = f2_two_sum(x.z, y.z);
-                    return make_float4(u.h, __fadd_rn(__fadd_rn(x.y, y.y), u.l), z.h,
-                                       __fadd_rn(__fadd_rn(x.w, y.w), z.l));
-                };
-                float4 q = entry(0);
-                if (per > 1) q = add(q, entry(1));
-                if (per > 2) q = add(q, add(entry(2), entry(3)));
+                Sum2 q = entry(0);
+                if (per > 1) q = sum2_add(q, entry(1));
+                if (per > 2) q = sum2_add(q, sum2_add(entry(2), entry(3)));
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) {
                     if (o >= ne) break;  // only zeros from here on
-                    q = add(q, make_float4(__shfl_xor_sync(0xffffffffu, q.x, o), __shfl_xor_sync(0xffffffffu, q.y, o),
-                                           __shfl_xor_sync(0xffffffffu, q.z, o), __shfl_xor_sync(0xffffffffu, q.w, o)));
+                    q = sum2_add(q, sum2_xor(q, o));
                 }
                 // the butterfly leaves (h, l) unnormalised (l can reach a sizeable
                 // fraction of h after cancellation): renormalise, so that the
                 // quotient's reciprocal seed is taken from the rounded total
-                F2 d1p = f2_two_sum(__shfl_sync(0xffffffffu, q.x, 0), __shfl_sync(0xffffffffu, q.y, 0));
-                const F2 d2p = f2_two_sum(__shfl_sync(0xffffffffu, q.z, 0), __shfl_sync(0xffffffffu, q.w, 0));
-                if (prior) d1p = f2_sub(d1p, prp);  // MAP: the prior's slope
-                done = newton_step_f2(tp, lop, hip, d1p, d2p, tolp);
+                // (lanes past ne hold partial sums: lane 0's are taken)
+                F2 d1p = f2_two_sum(__shfl_sync(0xffffffffu, q.h.x, 0), __shfl_sync(0xffffffffu, q.l.x, 0));
+                const F2 d2p = f2_two_sum(__shfl_sync(0xffffffffu, q.h.y, 0), __shfl_sync(0xffffffffu, q.l.y, 0));
+                if (ns.prior.h != 0.f) d1p = f2_sub(d1p, ns.prior);  // MAP: the prior's slope
+                done = newton_step_f2(t, lo, hi, d1p, d2p, ns.tol);
             } else {
                 auto entry = [&](int k) {
                     const int i = lane * per + k;
@@ -1963,21 +1978,23 @@ __device__ double newton_solve(const Model& M, const Cfg& cfg, const STab<R, C>&
                 }
                 double D1 = __shfl_sync(0xffffffffu, q.x, 0);
                 const double D2 = __shfl_sync(0xffffffffu, q.y, 0);
-                if (prior) D1 -= cfg.prior_rate;  // MAP: the prior's slope
-                done = newton_step(t, lo, hi, D1, D2, (float)D2, cfg.newton_tol);
+                if (__double_as_longlong(ns.prior) != 0) D1 -= ns.prior;  // MAP: the prior's slope
+                done = newton_step(t, lo, hi, D1, D2, (float)D2, ns.tol);
             }
             const bool last = done || it + 1 == cfg.newton_maxit;
             if (!last) {
-                if constexpr (sizeof(R) == 4) put_egh_f<R, C>(tp.h, ns, lane);
-                else put_egh<R, C>(M, t, ns, false, lane);
+                put_egh<C>(t, ns, lane);
             } else {
-                if (sizeof(R) == 4) t = (double)tp.h + (double)tp.l;
-                if (lane < 4 * C) ns.ex[lane] = exp(ns.lr[lane] * t);  // for the P matrices below
+                if (lane < 4 * C) ns.ex[lane] = exp(ns.lr[lane] * len_dbl(t));  // for the P matrices below
+                if (lane == 0) {
+                    bool moved;
+                    if constexpr (sizeof(R) == 4) moved = f2_lt(ns.sweep_tol, f2_abs(f2_sub(t, told)));
+                    else moved = fabs(t - told) > ns.sweep_tol;
+                    if (moved) ns.moved_at = sweep;
+                    *dst = t;
+                }
             }
-            if (lane == 0) {
-                if (last) ns.tb = t;
-                ns.done = last ? (done ? 1 : 2) : 0;
-            }
+            if (lane == 0) ns.done = last ? (done ? 1 : 2) : 0;
         }
         __syncthreads();
         if (ns.done) {
@@ -1986,17 +2003,17 @@ __device__ double newton_solve(const Model& M, const Cfg& cfg, const STab<R, C>&
             converged = ns.done == 1;
             for (int x = threadIdx.x; x < 16 * C; x += blockDim.x) {
                 const int r = x % C, ij = x / C;
-                double acc = 0.0;
+                double acc = ns.W[ij * 4];  // lam_0 = 0
 #pragma unroll
-                for (int k = 0; k < 4; ++k) acc += ns.W[ij * 4 + k] * ns.ex[k * C + r];
+                for (int k = 1; k < 4; ++k) acc = fma(ns.W[ij * 4 + k], ns.ex[k * C + r], acc);
                 Pdst[x] = (R)acc;
             }
             __syncthreads();
             break;
         }
     }
-    return ns.tb;
 }
+
 
 // ---------------------------------------------------------------- pair scores (mixed precision)
 // Scores of the mixed path, computed from pair partials (F2) category by
@@ -2288,7 +2305,8 @@ struct ProposeSmem {
     R Pm[5][C * 16];
     R Mt[16];
     R pi[4];
-    double T[5];
+    double T[5];         // the five lengths: inherited or learned, then the final ones
+    Len<R> Tl[5];        // the same between the solves
     Src<R, C> msrc[4];   // members in post-swap position order: A, X2 (at u), B, Y2 (at v)
     int mbr[4];          // branch of each member
     int bmem[5];         // member of each branch (-1: central)
@@ -2370,7 +2388,7 @@ __global__ void __launch_bounds__(512) k_propose(const PropGroup* __restrict__ g
             if (threadIdx.x < 4) sm.pi[threadIdx.x] = (R)M.pi[threadIdx.x];
         }
         const double* rr = G.rates ? G.rates + (size_t)it.tree * kMaxCat : M.rates;  // the parent's shape
-        init_newton_smem<R, C>(M, sm.ns, rr);
+        init_newton_smem<R, C>(M, cfg, sm.ns, rr);
         if (threadIdx.x == 0) {
             const int node[4] = {u, it.swap == 0 ? c0 : c1, sib, it.swap == 0 ? c1 : c0};
             const int brn[4] = {1, it.swap == 0 ? 3 : 4, 2, it.swap == 0 ? 4 : 3};
@@ -2410,6 +2428,7 @@ __global__ void __launch_bounds__(512) k_propose(const PropGroup* __restrict__ g
                 if (y == y) { t0 = y; warm = 1; }
             }
             sm.T[threadIdx.x] = t0;
+            sm.Tl[threadIdx.x] = len_of<R>(t0);
             sm.warm[threadIdx.x] = warm;
         }
         __syncthreads();
@@ -2429,11 +2448,9 @@ __global__ void __launch_bounds__(512) k_propose(const PropGroup* __restrict__ g
             }
             __syncthreads();
         }
-        double tlast = 0.0;  // length of the last branch solved (every thread)
         int sweeps = 0, item_evals = 0;
         for (int sw = 0; sw < cfg.prop_max_sweeps; ++sw) {
             ++sweeps;
-            double moved = 0.0;
             for (int b = 0; b < nb; ++b) {
                 // Central branch: X = P0 a0 * P1 a1 (at u), Y = P2 a2 * P3 a3 (at v).
                 // Branch of member mb: X = mb itself; Y = P2 partner * Pcentral (P0 o1 * P1 o2).
@@ -2448,6 +2465,7 @@ __global__ void __launch_bounds__(512) k_propose(const PropGroup* __restrict__ g
                 const R* P1 = sm.Pm[sm.mbr[i1m]];
                 const R* P2 = sm.Pm[sm.mbr[i2m]];
                 const R* P3 = sm.Pm[sm.mbr[i3m]];
+                const Len<R> told = sm.Tl[b], tbeg = newton_begin<C>(told, sm.ns);
                 for (int m = 0; m < sx.cnt; ++m) {
                     const int pl = sx.pl0 + m * sx.pstep, p = sx.p0 + m * sx.step;
                     R X[4 * C], Y[4 * C], t0[4 * C], t1[4 * C];
@@ -2476,25 +2494,22 @@ __global__ void __launch_bounds__(512) k_propose(const PropGroup* __restrict__ g
                     sumtable<R, C>(sm.Mt, sm.pi, X, Y, s4);
                     st.put(pl, s4, ex + ey - Prec<R>::kScaleExp * (k0 + k1 + k2 + k3));
                 }
-                const double told = sm.T[b];
                 int ev;
                 bool conv;
                 // new length; the solve leaves P matrices of branch b at it in sm.Pm[b]
-                const double t = newton_solve<R, C, kClus>(M, cfg, st, sx, told, sm.ns, ev, conv, sm.Pm[b], tm);
-                moved = fmax(moved, fabs(t - told));
+                newton_solve<R, C, kClus>(cfg, st, sx, tbeg, told, &sm.Tl[b], sw + 1, sm.ns, ev, conv, sm.Pm[b], tm);
                 evals_total += ev;
                 item_evals += ev;
                 if (!conv) ++nonconv;
-                if (threadIdx.x == 0) sm.T[b] = t;  // read again only after later barriers
-                tlast = t;
             }
-            if (moved <= cfg.sweep_tol) break;
+            if (sm.ns.moved_at != sw + 1) break;
         }
+        if (threadIdx.x < nb) sm.T[threadIdx.x] = len_dbl(sm.Tl[threadIdx.x]);
+        __syncthreads();
         // exact lnL at the final lengths: the last sum-table at its new length, or,
         // in mixed precision, the pair form of the four members around the new edge
         double f1;
         if constexpr (sizeof(R) == 4) {
-            __syncthreads();  // the last solve is done with sm.Pm
             for (int z = threadIdx.x; z < 5 * 4 * C; z += blockDim.x) {
                 const int b = z / (4 * C), q = z % (4 * C);
                 sm.ex5[b][q] = exp(sm.ns.lr[q] * sm.T[b]);
@@ -2513,7 +2528,7 @@ __global__ void __launch_bounds__(512) k_propose(const PropGroup* __restrict__ g
             f1 = propose_score_f2<C, kClus>(mem, sm.mbr, reinterpret_cast<const float*>(sm.Pm), &sm.Plo[0][0], M.pi,
                                             G.A.w, P, sx, sm.ns.red, tm);
         } else {
-            f1 = eval_lnl<C, kClus>(M, st, sx, tlast, sm.ns, tm);
+            f1 = eval_lnl<C, kClus>(st, sx, sm.T[nb - 1], sm.ns, tm);
         }
         sweeps_total += sweeps;
         if (threadIdx.x == 0 && rank == 0) {
@@ -2593,7 +2608,8 @@ __global__ void __launch_bounds__(512) k_fullopt(const FullGroup* __restrict__ g
     if (total <= lo || total > hi) return;  // another launch shape's number of trees
     FullSmem<R, C>& sm = *reinterpret_cast<FullSmem<R, C>*>(smraw);
     size_t off = (sizeof(FullSmem<R, C>) + 15) & ~size_t(15);
-    double* len = reinterpret_cast<double*>(smraw + off);
+    double* len = reinterpret_cast<double*>(smraw + off);         // the lengths before and after the sweeps,
+    Len<R>* const lens = reinterpret_cast<Len<R>*>(smraw + off);  // and between the solves
     uint16_t* const sched = reinterpret_cast<uint16_t*>(len + nn_max);
     uint8_t* const up = reinterpret_cast<uint8_t*>(sched + 3 * ((nn_max + 2) / 2));
     uint8_t* const ch = up + nn_max;
@@ -2666,9 +2682,10 @@ __global__ void __launch_bounds__(512) k_fullopt(const FullGroup* __restrict__ g
         }
         // per-tree category rates (a visit that re-optimises the Gamma shape), else the model's
         const double* rr = G.rates ? G.rates + (size_t)gi * kMaxCat : M.rates;
-        init_newton_smem<R, C>(M, sm.ns, rr);
+        init_newton_smem<R, C>(M, cfg, sm.ns, rr);
         for (int v = threadIdx.x; v < NN; v += blockDim.x) {
-            len[v] = glen[v];
+            if (G.max_sweeps > 0) lens[v] = len_of<R>(glen[v]);
+            else len[v] = glen[v];
             up[v] = (uint8_t)G.ts.up[(size_t)tree * NN + v];
             ch[2 * v] = (uint8_t)G.ts.ch[((size_t)tree * NN + v) * 2];
             ch[2 * v + 1] = (uint8_t)G.ts.ch[((size_t)tree * NN + v) * 2 + 1];
@@ -2680,7 +2697,7 @@ __global__ void __launch_bounds__(512) k_fullopt(const FullGroup* __restrict__ g
         __syncthreads();
         for (int z = threadIdx.x; z < NN * C * 4; z += blockDim.x) {
             const int v = z / (C * 4), r = (z / 4) % C, i = z & 3;
-            if (v > 0) pmat_row<R>(M, len[v] * rr[r], i, Pm + (size_t)v * C * 16 + i * 4 * C + r, C);
+            if (v > 0) pmat_row<R>(M, glen[v] * rr[r], i, Pm + (size_t)v * C * 16 + i * 4 * C + r, C);
         }
         __syncthreads();
         auto srcD = [&](int v) {
@@ -2790,12 +2807,10 @@ __global__ void __launch_bounds__(512) k_fullopt(const FullGroup* __restrict__ g
         // bottom-up D pass
         if (!(pair_score && G.max_sweeps == 0))
             for (int v = NN - 1; v >= n; --v) refreshD(v);
-        int sweeps = 0;
-        double tlast = 0.0;
+        int sweeps = 0, last = n;
         if (G.max_sweeps == 0 && !pair_score) visit_build(n);
         for (int sw = 0; sw < G.max_sweeps; ++sw) {
             ++sweeps;
-            double moved = 0.0;
             for (int k = 0; k < nsched; ++k) {
                 const int op = sched[k];
                 if (op & kUpd16) {
@@ -2804,22 +2819,24 @@ __global__ void __launch_bounds__(512) k_fullopt(const FullGroup* __restrict__ g
                     continue;
                 }
                 const int v = op;
+                const Len<R> told = lens[v], tbeg = newton_begin<C>(told, sm.ns);
                 visit_build(v);
                 if (threadIdx.x == 0 && k + 1 < nsched) prefetch_op(sched[k + 1]);
-                const double told = len[v];
                 int ev;
                 bool conv;
                 // the solve leaves the P matrices of edge v at its new length in Pm
-                const double t = newton_solve<R, C, kClus>(M, cfg, st, sx, told, sm.ns, ev, conv,
-                                                           Pm + (size_t)v * C * 16, tm);
-                moved = fmax(moved, fabs(t - told));
+                newton_solve<R, C, kClus>(cfg, st, sx, tbeg, told, &lens[v], sw + 1, sm.ns, ev, conv,
+                                          Pm + (size_t)v * C * 16, tm);
                 evals_total += ev;
                 if (!conv) ++nonconv;
-                if (threadIdx.x == 0) len[v] = t;  // read again only after later barriers
-                tlast = t;
+                last = v;
             }
-            if (moved <= cfg.sweep_tol) break;
+            if (sm.ns.moved_at != sw + 1) break;
         }
+        __syncthreads();
+        if (sweeps > 0)
+            for (int v = threadIdx.x; v < NN; v += blockDim.x) len[v] = len_dbl(lens[v]);
+        __syncthreads();
         // exact lnL at the final lengths: the last visited edge's sum-table (FP64),
         // or, in mixed precision, a pruning pass in pair arithmetic: D_v of every
         // inner node bottom-up (h over the FP32 D slot, l in the U slot of v,
@@ -2829,7 +2846,7 @@ __global__ void __launch_bounds__(512) k_fullopt(const FullGroup* __restrict__ g
             f1 = fullopt_score_f2<C, kClus>(n, ch, len, A, sx, reinterpret_cast<float*>(clv), scl, sm.ns.W, sm.ns.lr,
                                             &sm.Pf[0][0], &sm.Pfl[0][0], &sm.exf[0][0], M.pi, sm.ns.red, tm);
         } else {
-            f1 = eval_lnl<C, kClus>(M, st, sx, G.max_sweeps == 0 ? len[n] : tlast, sm.ns, tm);
+            f1 = eval_lnl<C, kClus>(st, sx, len[last], sm.ns, tm);
         }
         sweeps_total += sweeps;
         __syncthreads();
@@ -3223,12 +3240,12 @@ void launch_shape(K kern, cudaStream_t s, int kp, int threads, int grid, size_t 
 }  // namespace
 
 int propose_resident(int prec, int C, const Shape& h, int maxP, int sms) {
-    return resident(prop_kernel(prec, C, h.kp > 1, h.smem_tab), h.kp, h.geo.vt,
-                    propose_smem_bytes(prec, C, h.smem_tab ? geo_local(maxP, h.geo, h.geo.vt) : 0), sms);
+    return resident(prop_kernel(prec, C, h.kp > 1, h.smem_tab), h.kp, h.pt,
+                    propose_smem_bytes(prec, C, h.smem_tab ? geo_local(maxP, h.geo, h.pt) : 0), sms);
 }
 int fullopt_resident(int prec, int C, const Shape& h, int maxN, int maxP, int sms) {
-    return resident(full_kernel(prec, C, h.kp > 1, h.smem_tab), h.kp, h.geo.vt,
-                    fullopt_smem_bytes(prec, C, maxN, h.smem_tab ? geo_local(maxP, h.geo, h.geo.vt) : 0, h.geo.vt), sms);
+    return resident(full_kernel(prec, C, h.kp > 1, h.smem_tab), h.kp, h.pt,
+                    fullopt_smem_bytes(prec, C, maxN, h.smem_tab ? geo_local(maxP, h.geo, h.pt) : 0, h.pt), sms);
 }
 int geometry_resident(int prec, int C, bool full, int K, int threads, size_t smem, int sms) {
     if (prec != 1 || C != 4) return 0;
@@ -3239,20 +3256,20 @@ int geometry_resident(int prec, int C, bool full, int K, int threads, size_t sme
 void launch_propose(cudaStream_t s, int prec, int C, const PropGroup* groups, const int* gstart, int ngroups,
                     int* counter, Cfg cfg, unsigned long long* stats, const Shape& h, int grid, void* scratch,
                     size_t scratch_per_cta, int maxP, int lo, int hi) {
-    launch_shape(prop_kernel(prec, C, h.kp > 1, h.smem_tab), s, h.kp, h.geo.vt, grid,
-                 propose_smem_bytes(prec, C, h.smem_tab ? geo_local(maxP, h.geo, h.geo.vt) : 0), groups, gstart, ngroups,
+    launch_shape(prop_kernel(prec, C, h.kp > 1, h.smem_tab), s, h.kp, h.pt, grid,
+                 propose_smem_bytes(prec, C, h.smem_tab ? geo_local(maxP, h.geo, h.pt) : 0), groups, gstart, ngroups,
                  counter, cfg, stats, reinterpret_cast<unsigned char*>(scratch), scratch_per_cta, h.geo, lo, hi);
 }
 
 void launch_fullopt(cudaStream_t s, int prec, int C, const FullGroup* groups, const int* gstart, int ngroups,
                     int* counter, int maxN, int maxP, Cfg cfg, unsigned long long* stats, const Shape& h, int grid,
                     void* scratch, size_t scratch_per_cta, void* slab, size_t slab_per_cta, int lo, int hi) {
-    const int ld = h.smem_tab ? geo_local(maxP, h.geo, h.geo.vt) : 0;
+    const int ld = h.smem_tab ? geo_local(maxP, h.geo, h.pt) : 0;
     const size_t f = full_fixed(prec, C, maxN) + (ld ? sumtable_bytes(prec, C, ld) : 0);
-    launch_shape(full_kernel(prec, C, h.kp > 1, h.smem_tab), s, h.kp, h.geo.vt, grid,
-                 fullopt_smem_bytes(prec, C, maxN, ld, h.geo.vt), groups, gstart, ngroups, counter, 2 * maxN - 2, cfg,
+    launch_shape(full_kernel(prec, C, h.kp > 1, h.smem_tab), s, h.kp, h.pt, grid,
+                 fullopt_smem_bytes(prec, C, maxN, ld, h.pt), groups, gstart, ngroups, counter, 2 * maxN - 2, cfg,
                  stats, reinterpret_cast<unsigned char*>(scratch), scratch_per_cta,
-                 reinterpret_cast<unsigned char*>(slab), slab_per_cta, full_p_smem(prec, C, maxN, f, h.geo.vt) ? 1 : 0,
+                 reinterpret_cast<unsigned char*>(slab), slab_per_cta, full_p_smem(prec, C, maxN, f, h.pt) ? 1 : 0,
                  h.geo, lo, hi);
 }
 

@@ -82,7 +82,7 @@ extern "C" pt_status pt_score_topologies_noalloc(int n_taxa, int n_patterns, con
     const int n = n_taxa, NN = 2 * n - 2, E = 2 * n - 3, P = n_patterns, prec = cfg.precision;
     const int threads = cfg.threads > 0 ? cfg.threads : (P <= 128 ? 128 : 256);
     const bool smem_tab = fullopt_smem_bytes(prec, M.C, n, P, threads) <= (size_t)optin;
-    const Shape shape{Geo{threads, 1, 1}, 1, smem_tab ? 1 : 0};
+    const Shape shape{Geo{threads, 1, 1}, 1, threads, smem_tab ? 1 : 0};
     // layout: flags | stats | canonical trees | launch table | per-CTA partials slabs | per-CTA sum-tables
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off += up256(bytes); return o; };
