@@ -1554,11 +1554,18 @@ __device__ __forceinline__ Sum2 sum2_xor(Sum2 a, int o) {
 // Compensated warp sums of two FP32 partials (two-sums over the virtual threads of
 // the warp, which lie `lanes` apart; neighbours first): every lane ends with both
 // sums as unevaluated pairs, with no FP64 instruction.
-__device__ __forceinline__ Sum2 warp_sum_comp(float x, float y, int lanes) {
+template <int kLanes>
+__device__ __forceinline__ Sum2 warp_sum_comp(float x, float y) {
     Sum2 a{make_float2(x, y), make_float2(0.f, 0.f)};
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1)
-        if (o >= lanes) a = sum2_add(a, sum2_xor(a, o));
+    for (int o = kLanes; o < 32; o <<= 1) a = sum2_add(a, sum2_xor(a, o));
+    return a;
+}
+// The last levels of the tree: n lanes' sums (a power of two) into each of them.
+template <int n>
+__device__ __forceinline__ Sum2 sum2_lanes(Sum2 a) {
+#pragma unroll
+    for (int o = 1; o < n; o <<= 1) a = sum2_add(a, sum2_xor(a, o));
     return a;
 }
 __device__ __forceinline__ double warp_sum(double x, int lanes) {
@@ -1830,6 +1837,60 @@ __device__ __forceinline__ double newton_begin(double t0, NewtonSmem<double, C>&
     return t;
 }
 
+// The warp's Newton sums at the coefficients in ns, in every lane: (d1 h, d2 h, d1 l,
+// d2 l) in FP32, (d1, d2) in FP64.  One form per number of lanes: with the number a
+// variable, its loops' branches were a tenth of an evaluation's chain.
+template <typename R, int C, int kLanes>
+__device__ __forceinline__ float4 site_sums(const STab<R, C>& st, const Sites& sx, const NewtonSmem<R, C>& ns) {
+    R e[4 * C], g[4 * C], h[4 * C];
+#pragma unroll
+    for (int q = 0; q < 4 * C; ++q) { e[q] = ns.egh[0][q]; g[q] = ns.egh[1][q]; h[q] = ns.egh[2][q]; }
+    R a1 = R(0), a2 = R(0);
+    if constexpr (kLanes == 1) {
+        // two sites per pass (their chains interleave), added in site order
+        int m = 0, p = sx.pl0;
+        for (; m + 1 < sx.cnt; m += 2, p += 2 * sx.pstep) {
+            R a, c, wt, a_, c_, wt_;
+            newton_site<R, C>(st, p, e, g, h, true, a, c, wt);
+            newton_site<R, C>(st, p + sx.pstep, e, g, h, false, a_, c_, wt_);
+            a1 = fma(wt, a, a1);
+            a2 = fma(wt, c, a2);
+            a1 = fma(wt_, a_, a1);
+            a2 = fma(wt_, c_, a2);
+        }
+        if (m < sx.cnt) {
+            R a, c, wt;
+            newton_site<R, C>(st, p, e, g, h, false, a, c, wt);
+            a1 = fma(wt, a, a1);
+            a2 = fma(wt, c, a2);
+        }
+    } else {
+        // the virtual thread's sites of this round lie in its lanes, in order:
+        // every lane of the group adds all of them (the same sum as one thread's)
+        const int base = (threadIdx.x & 31) & ~(kLanes - 1);
+        for (int m = 0; m < sx.M; ++m) {
+            R a = R(0), c = R(0), wt = R(0);
+            const int k = sx.jj + m * kLanes;  // this lane's site among the virtual thread's
+            if (m < sx.cnt)
+                newton_site<R, C>(st, sx.pl0 + m * sx.pstep, e, g, h, !(k & 1) && k + 1 < sx.nt, a, c, wt);
+#pragma unroll
+            for (int j = 0; j < kLanes; ++j) {
+                const R aj = __shfl_sync(0xffffffffu, a, base + j), cj = __shfl_sync(0xffffffffu, c, base + j),
+                        wj = __shfl_sync(0xffffffffu, wt, base + j);
+                a1 = fma(wj, aj, a1);
+                a2 = fma(wj, cj, a2);
+            }
+        }
+    }
+    if constexpr (sizeof(R) == 4) {
+        const Sum2 a = warp_sum_comp<kLanes>(a1, a2);
+        return make_float4(a.h.x, a.h.y, a.l.x, a.l.y);
+    } else {
+        const double2 d = make_double2(warp_sum(a1, kLanes), warp_sum(a2, kLanes));
+        return reinterpret_cast<const float4&>(d);
+    }
+}
+
 // Newton solve on the current sum-table from t (as newton_begin returned it).  Per
 // evaluation: every thread sums w L'/L and w (L''/L - (L'/L)^2) over its sites, the
 // warps reduce, and one warp alone takes the step and writes the coefficients of
@@ -1852,56 +1913,11 @@ __device__ __forceinline__ void newton_solve(const Cfg& cfg, const STab<R, C>& s
     converged = false;
     evals = 0;
     for (int it = 0; it < cfg.newton_maxit; ++it) {
-        R e[4 * C], g[4 * C], h[4 * C];
-#pragma unroll
-        for (int q = 0; q < 4 * C; ++q) { e[q] = ns.egh[0][q]; g[q] = ns.egh[1][q]; h[q] = ns.egh[2][q]; }
-        R a1 = R(0), a2 = R(0);
-        if (sx.lanes == 1) {
-            // two sites per pass (their chains interleave), added in site order
-            int m = 0, p = sx.pl0;
-            for (; m + 1 < sx.cnt; m += 2, p += 2 * sx.pstep) {
-                R a, c, wt, a_, c_, wt_;
-                newton_site<R, C>(st, p, e, g, h, true, a, c, wt);
-                newton_site<R, C>(st, p + sx.pstep, e, g, h, false, a_, c_, wt_);
-                a1 = fma(wt, a, a1);
-                a2 = fma(wt, c, a2);
-                a1 = fma(wt_, a_, a1);
-                a2 = fma(wt_, c_, a2);
-            }
-            if (m < sx.cnt) {
-                R a, c, wt;
-                newton_site<R, C>(st, p, e, g, h, false, a, c, wt);
-                a1 = fma(wt, a, a1);
-                a2 = fma(wt, c, a2);
-            }
-        } else {
-            // the virtual thread's sites of this round lie in its lanes, in order:
-            // every lane of the group adds all of them (the same sum as one thread's)
-            const int base = lane & ~(sx.lanes - 1);
-            for (int m = 0; m < sx.M; ++m) {
-                R a = R(0), c = R(0), wt = R(0);
-                const int k = sx.jj + m * sx.lanes;  // this lane's site among the virtual thread's
-                if (m < sx.cnt)
-                    newton_site<R, C>(st, sx.pl0 + m * sx.pstep, e, g, h, !(k & 1) && k + 1 < sx.nt, a, c, wt);
-                for (int j = 0; j < sx.lanes; ++j) {
-                    const R aj = __shfl_sync(0xffffffffu, a, base + j), cj = __shfl_sync(0xffffffffu, c, base + j),
-                            wj = __shfl_sync(0xffffffffu, wt, base + j);
-                    a1 = fma(wj, aj, a1);
-                    a2 = fma(wj, cj, a2);
-                }
-            }
-        }
-        // the per-warp sums, one 16-byte entry each: to this CTA's shared memory, or
-        // pushed into every CTA of the cluster, where the leader waits for them
+        const float4 v = sx.lanes == 1   ? site_sums<R, C, 1>(st, sx, ns)
+                         : sx.lanes == 2 ? site_sums<R, C, 2>(st, sx, ns)
+                         : sx.lanes == 4 ? site_sums<R, C, 4>(st, sx, ns)
+                                         : site_sums<R, C, 8>(st, sx, ns);
         const int xe = tm.nseq++, cs = kClus ? xe & 1 : 0;
-        float4 v;
-        if constexpr (sizeof(R) == 4) {
-            const Sum2 a = warp_sum_comp(a1, a2, sx.lanes);
-            v = make_float4(a.h.x, a.h.y, a.l.x, a.l.y);
-        } else {
-            const double2 d = make_double2(warp_sum(a1, sx.lanes), warp_sum(a2, sx.lanes));
-            v = reinterpret_cast<const float4&>(d);
-        }
         if constexpr (kClus) {
             // Slot cs is free in every CTA: a warp pushes exchange xe only after its
             // CTA's leader received all of exchange xe - 1, which every CTA pushed
@@ -1947,11 +1963,7 @@ __device__ __forceinline__ void newton_solve(const Cfg& cfg, const STab<R, C>& s
                 Sum2 q = entry(0);
                 if (per > 1) q = sum2_add(q, entry(1));
                 if (per > 2) q = sum2_add(q, sum2_add(entry(2), entry(3)));
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    if (o >= ne) break;  // only zeros from here on
-                    q = sum2_add(q, sum2_xor(q, o));
-                }
+                q = ne > 16 ? sum2_lanes<32>(q) : ne > 8 ? sum2_lanes<16>(q) : ne > 4 ? sum2_lanes<8>(q) : sum2_lanes<4>(q);
                 // the butterfly leaves (h, l) unnormalised (l can reach a sizeable
                 // fraction of h after cancellation): renormalise, so that the
                 // quotient's reciprocal seed is taken from the rounded total
