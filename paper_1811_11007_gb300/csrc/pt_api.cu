@@ -686,9 +686,10 @@ void run_full_jobs(Ctx& c, std::vector<FullJob> jobs, bool allow_tune = true) {
         const int* gstart;
         int* counter;
         const FullGroup* dg = upload_groups(c, "full", groups, counts, &gstart, &counter);
-        // one launch of a summation geometry (threads, K shares per tree) in the shape
-        // that suits the number of trees; returns its device time when timed
-        auto run = [&](int threads, int K, unsigned long long* stats, bool timed) {
+        // FP64 scores in the optimisation kernel; mixed precision in k_score, which is all
+        // that fixed lengths need
+        const bool optimise = prec == PT_PREC_FP64 || jobs[0].max_sweeps > 0;
+        auto launch = [&](int threads, int K, unsigned long long* stats) {
             const std::vector<ShapeFit> shapes = shapes_of(c, true, prec, C, maxN, maxP, threads, K);
             const ShapeFit& f = pick_shape(shapes, total);
             const int grid = (int)std::min<long long>((long long)total * f.h.kp, f.resident) / f.h.kp * f.h.kp;
@@ -702,10 +703,20 @@ void run_full_jobs(Ctx& c, std::vector<FullJob> jobs, bool allow_tune = true) {
                 sl = std::max(sl, fullopt_slab_bytes(prec, C, j.a->n, geo_local(j.a->P, f.h.geo, f.h.pt)));
             unsigned char* slab = buf<unsigned char>(c, "full.slab", sl * grid);
             ck(c, cudaMemsetAsync(counter, 0, sizeof(int), c.stream), "counter");
-            size_t e0 = timed ? ev_record(c) : 0;
             launch_fullopt(c.stream, prec, C, dg, gstart, (int)groups.size(), counter, maxN, maxP, kcfg(c), stats, f.h,
                            grid, scratch, spc, slab, sl);
             ck(c, cudaGetLastError(), "full optimisation launch");
+        };
+        // one launch of a summation geometry (threads, K shares per tree) in the shape
+        // that suits the number of trees, and the scores; returns its device time when timed
+        auto run = [&](int threads, int K, unsigned long long* stats, bool timed) {
+            size_t e0 = timed ? ev_record(c) : 0;
+            if (optimise) launch(threads, K, stats);
+            if (prec == PT_PREC_MIXED) {
+                double* part = buf<double>(c, "full.part", (size_t)total * score_units(maxP));
+                launch_score(c.stream, C, dg, gstart, (int)groups.size(), maxN, maxP, kcfg(c), 0, total, part, c.sm_count);
+                ck(c, cudaGetLastError(), "score launch");
+            }
             float ms = 0.f;
             if (timed) {
                 size_t e1 = ev_record(c);
@@ -1603,6 +1614,7 @@ struct GraphRound {
     void* prop_scratch = nullptr;
     void* full_scratch = nullptr;
     unsigned char* slab = nullptr;
+    double* part = nullptr;  // unit sums of the scores
     cudaStream_t cs = nullptr;
     cudaGraphExec_t exec = nullptr;
     long long kernels = 0;      // kernel nodes per replay
@@ -1688,7 +1700,8 @@ size_t graph_slab(const Ctx& c, const GraphRound& g, const ShapeRange& x) {
 
 // The launch sequence of one graph round on stream s (recorded under capture).
 void graph_record(Ctx& c, GraphRound& g, cudaStream_t s, int C, int maxN, int maxP,
-                  const std::vector<ShapeRange>& ps, size_t pspc, const std::vector<ShapeRange>& fs, size_t fspc) {
+                  const std::vector<ShapeRange>& ps, size_t pspc, const std::vector<ShapeRange>& fs, size_t fspc,
+                  int totCap) {
     const int na = g.na, prec = c.cfg.precision;
     int* di = g.di;
     for (GraphAln& x : g.a) {  // flags past the device counts must read as zero in the scans
@@ -1749,6 +1762,8 @@ void graph_record(Ctx& c, GraphRound& g, cudaStream_t s, int C, int maxN, int ma
     for (const ShapeRange& x : fs)
         launch_fullopt(s, prec, C, g.dfg, di + g.oGSF(), na, di + g.oCF(), maxN, maxP, kcfg(c), c.d_stats, x.f.h,
                        range_grid(x), g.full_scratch, fspc, g.slab, graph_slab(c, g, x), x.lo, x.hi);
+    if (prec == PT_PREC_MIXED)
+        launch_score(s, C, g.dfg, di + g.oGSF(), na, maxN, maxP, kcfg(c), 0, totCap, g.part, c.sm_count);
     for (int k = 0; k < na; ++k) {
         GraphAln& x = g.a[k];
         AlnState& A = c.alns[x.aln];
@@ -1887,6 +1902,8 @@ GraphRound* graph_create(Ctx& c, const std::vector<int>& ids, const std::vector<
     if (pscratch) ar.addv(g.prop_scratch, pscratch);
     if (fscratch) ar.addv(g.full_scratch, fscratch);
     ar.add(g.slab, slab);
+    g.part = nullptr;
+    if (prec == PT_PREC_MIXED) ar.add(g.part, (size_t)totCap * score_units(maxP));
     dev_alloc(c, &g.mem, ar.total(), "allocating the graph round's buffers");
     ar.carve(g.mem);
     ck(c, cudaHostAlloc(reinterpret_cast<void**>(&g.hi), sizeof(int) * g.nints(), cudaHostAllocDefault), "pinned");
@@ -1957,7 +1974,7 @@ GraphRound* graph_create(Ctx& c, const std::vector<int>& ids, const std::vector<
     ck(c, cudaStreamCreateWithFlags(&g.cs, cudaStreamNonBlocking), "graph stream");
     ck(c, cudaStreamBeginCapture(g.cs, cudaStreamCaptureModeRelaxed), "begin capture");
     const long long k0 = launch_count();
-    graph_record(c, g, g.cs, C, maxN, maxP, ps, tabb, fs, tabb);
+    graph_record(c, g, g.cs, C, maxN, maxP, ps, tabb, fs, tabb, totCap);
     g.kernels = launch_count() - k0;
     cudaGraph_t graph = nullptr;
     ck(c, cudaStreamEndCapture(g.cs, &graph), "end capture");

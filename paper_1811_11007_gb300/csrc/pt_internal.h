@@ -324,6 +324,12 @@ void launch_fullopt(cudaStream_t s, int prec, int C, const FullGroup* groups, co
                     int* counter, int maxN, int maxP, Cfg cfg, unsigned long long* stats, const Shape& h, int grid,
                     void* scratch, size_t scratch_per_cta, void* slab, size_t slab_per_cta, int lo = 0,
                     int hi = 0x7fffffff);
+// Scores (mixed precision) of items t0 .. t1 - 1 of the groups (fewer when gstart says
+// so on the device) at their lengths, into lnl_out; part: score_units(maxP) doubles
+// per item of the range.  A full optimisation in mixed precision is followed by it.
+void launch_score(cudaStream_t s, int C, const FullGroup* groups, const int* gstart, int ngroups, int maxN, int maxP,
+                  Cfg cfg, int t0, int t1, double* part, int sms);
+int score_units(int P);
 // Resident CTAs of a shape on a GPU of sms SMs (a multiple of h.kp; 0: cannot run).
 int propose_resident(int prec, int C, const Shape& h, int maxP, int sms);
 int fullopt_resident(int prec, int C, const Shape& h, int maxN, int maxP, int sms);

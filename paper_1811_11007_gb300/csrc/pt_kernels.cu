@@ -2087,87 +2087,223 @@ __device__ __noinline__ double propose_score_f2(const Src2<C>* mem, const int* m
     return team_sum<kClus>(acc, red, tm, sx.lanes);
 }
 
-// Visit: a pruning pass in pairs over one tree's partials buffer.  D_v of
-// every inner node v > n bottom-up (h over the FP32 D slot of v, l in the U
-// slot of v; the FP32 vectors are no longer needed), then node n's vector
-// combined with leaf 0 across the edge of n.  The block computes each node's
-// P pairs (its two children, and n's own edge at the root) into Pf/Pfl from
-// W and lr (as NewtonSmem) at the lengths len.
-// Stored vectors are indexed by the local site (sx.ld per slot), tips and
-// weights by the site; in a cluster the result is summed over it.
-template <int C, bool kClus>
-__device__ __noinline__ double fullopt_score_f2(int n, const uint8_t* ch, const double* len, const Aln& A,
-                                                const Sites& sx, float* clv, int32_t* scl, const double* W,
-                                                const double* lr, float* Pf, float* Pfl, double* exf, const double* pi,
-                                                double (*red)[32], Team& tm) {
-    const int NN = 2 * n - 2, Ps = sx.ld;
-    const size_t sstride = (size_t)Ps * 4 * C;
-    float pih[4], pil[4];
+// ---------------------------------------------------------------- tree scores (mixed precision)
+// Scores of trees at their lengths: one pruning pass in pair arithmetic, nothing
+// stored but the sums.  A thread owns one site and one lane group of its categories
+// and walks the tree's inner nodes in post-order, the subtree that needs more of the
+// stack first, so that at most log2(n) vectors wait (local memory); the node just
+// made stays in registers.  The categories' groups are scaled apart and merged with
+// their exponents at the root.  Sites are summed in units of kScoreUnit (a fixed
+// tree), the units in order by k_score_sum: a score does not depend on the launch.
+// Bound by FP32 issue (about 270 packed instructions per node, site and group) and,
+// for few sites, by the FP64 exponentials of the P matrices, which each CTA makes
+// once per tree, in parallel over edges and categories.  One tree of 27 taxa x 816
+// patterns took 157 us as the last step of the full optimisation, whose nodes each
+// waited for their own P matrices.
+constexpr int kScoreUnit = 64, kScoreStack = 9;
+struct ScoreProg {
+    uint8_t kind, a, b;  // kind 0: two tips, 1: tip a and the last result (edge b), 2: waiting result (edge a) and last (edge b)
+};
+__host__ __device__ inline size_t score_smem(int C, int nn) {
+    return ((size_t)nn * 32 * C * 4 + (size_t)nn * (3 + 8) + 15) & ~size_t(15);
+}
+template <int C>
+__global__ void __launch_bounds__(512) k_score(const FullGroup* __restrict__ groups, const int* __restrict__ gstart,
+                                               int ngroups, int nn_max, int t0, int t1, int chunks, int units_max,
+                                               double* __restrict__ part) {
+    extern __shared__ __align__(16) unsigned char smraw[];
+    using T = typename Lanes<C>::T;
+    constexpr int S = Lanes<C>::n;  // threads per site
+    float* const Ph = reinterpret_cast<float*>(smraw);
+    float* const Pl = Ph + (size_t)nn_max * 16 * C;
+    ScoreProg* const prog = reinterpret_cast<ScoreProg*>(Pl + (size_t)nn_max * 16 * C);
+    uint8_t* const ch = reinterpret_cast<uint8_t*>(prog + nn_max);  // children; then need[] and two stacks
+    uint8_t *const need = ch + 2 * nn_max, *const stk = need + nn_max;
+    __shared__ double W[64], red[16];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int total = min(gstart[ngroups], t1) - t0;
+    for (long long work = blockIdx.x; work < (long long)total * chunks; work += gridDim.x) {
+        const int x = t0 + (int)(work / chunks), c = (int)(work % chunks);
+        int k = 0;
+        while (k + 1 < ngroups && gstart[k + 1] <= x) ++k;
+        const FullGroup& G = groups[k];
+        const int gi = G.order ? G.order[x - gstart[k]] : x - gstart[k];
+        const Model& M = G.M;
+        const Aln& A = G.A;
+        const int n = G.ts.n, NN = 2 * n - 2, P = A.P, units = (P + kScoreUnit - 1) / kScoreUnit;
+        const int u0 = (int)((long long)units * c / chunks), u1 = (int)((long long)units * (c + 1) / chunks);
+        if (u0 == u1) continue;  // uniform over the block
+        const int tree = G.first + gi;
+        __syncthreads();  // the work item before is done with shared memory
+        for (int z = threadIdx.x; z < 64; z += blockDim.x) {
+            const int q = z & 3, ij = z >> 2, i = ij >> 2, j = ij & 3;
+            W[z] = M.isqpi[i] * M.sqpi[j] * M.R[i * 4 + q] * M.R[j * 4 + q];
+        }
+        for (int v = threadIdx.x; v < 2 * NN; v += blockDim.x) ch[v] = (uint8_t)G.ts.ch[(size_t)tree * 2 * NN + v];
+        __syncthreads();
+        if (warp == 0) {
+            if (lane == 0) {
+                // post-order program; need[v]: results that wait while v's subtree is made
+                for (int v = NN - 1; v >= n; --v) {
+                    const int a = ch[2 * v], b = ch[2 * v + 1], na = a < n ? 0 : need[a], nb = b < n ? 0 : need[b];
+                    need[v] = (uint8_t)(na == nb ? na + 1 : max(na, nb));
+                }
+                int sp = 0, np = 0;
+                uint8_t* const done = stk + NN;
+                stk[0] = (uint8_t)n;
+                done[0] = 0;
+                sp = 1;
+                while (sp) {
+                    const int v = stk[sp - 1], c0 = ch[2 * v], c1 = ch[2 * v + 1];
+                    const bool swap = c1 >= n && (c0 < n || need[c1] > need[c0]);
+                    const int a = swap ? c1 : c0, b = swap ? c0 : c1;  // a first; a tip only if both are
+                    const int st = done[sp - 1]++;
+                    if (st == 0 && a >= n) { stk[sp] = (uint8_t)a; done[sp++] = 0; continue; }
+                    if (st <= 1 && b >= n) { done[sp - 1] = 2; stk[sp] = (uint8_t)b; done[sp++] = 0; continue; }
+                    prog[np++] = a < n   ? ScoreProg{0, (uint8_t)a, (uint8_t)b}
+                                 : b < n ? ScoreProg{1, (uint8_t)b, (uint8_t)a}
+                                         : ScoreProg{2, (uint8_t)a, (uint8_t)b};
+                    --sp;
+                }
+            }
+        }
+        const double* rr = G.rates ? G.rates + (size_t)gi * kMaxCat : M.rates;
+        const double* glen = G.ts.len + (size_t)tree * NN;
+        // warps other than the one with the program start on the matrices
+        for (int z = ((int)threadIdx.x + (int)blockDim.x - 32) % (int)blockDim.x; z < (NN - 1) * C; z += blockDim.x) {
+            const int v = 1 + z / C, r = z % C;
+            double e[4] = {1.0, 0.0, 0.0, 0.0};  // lam_0 = 0
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const F2 x = f2_of(pi[i]);
-        pih[i] = x.h;
-        pil[i] = x.l;
-    }
-    auto src = [&](int v) {
-        if (v < n) return Src2<C>{nullptr, nullptr, nullptr, A.tips + (size_t)v * A.P};
-        return Src2<C>{clv + (size_t)(v - n) * sstride, clv + (size_t)(n - 2 + (v - n - 1)) * sstride,
-                       scl + (size_t)(v - n) * Ps, nullptr};
-    };
-    double acc = 0.0;
-    for (int v = NN - 1; v >= n; --v) {
-        const int c0 = ch[2 * v], c1 = ch[2 * v + 1];
-        const int nm = v == n ? 3 : 2;  // matrices: child 0, child 1 (and n's own edge at the root)
-        __syncthreads();                // the previous node's sites are done with the matrices
-        for (int z = threadIdx.x; z < nm * 4 * C; z += blockDim.x) {
-            const int k = z / (4 * C), q = z % (4 * C);
-            exf[z] = exp(lr[q] * len[k == 0 ? c0 : k == 1 ? c1 : v]);
+            for (int q = 1; q < 4; ++q) e[q] = exp(M.lam[q] * rr[r] * glen[v]);
+#pragma unroll
+            for (int ij = 0; ij < 16; ++ij) {
+                double acc = 0.0;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) acc += W[ij * 4 + q] * e[q];
+                const F2 w = f2_of(acc);
+                Ph[((size_t)v * 16 + ij) * C + r] = w.h;
+                Pl[((size_t)v * 16 + ij) * C + r] = w.l;
+            }
         }
         __syncthreads();
-        for (int z = threadIdx.x; z < nm * 16 * C; z += blockDim.x) {
-            const int k = z / (16 * C), q = z % (16 * C);
-            f2_pmat_entry<C>(W, exf + k * 4 * C, q, Pf + k * 16 * C, Pfl + k * 16 * C);
-        }
-        __syncthreads();
-        const Src2<C> s0 = src(c0), s1 = src(c1);
-        if (v > n) {
-            for (int m = 0; m < sx.cnt; ++m)
-                f2_join<C>(Pf, Pfl, s0, Pf + 16 * C, Pfl + 16 * C, s1, Ps, sx.pl0 + m * sx.pstep, sx.p0 + m * sx.step,
-                           clv + (size_t)(v - n) * sstride, clv + (size_t)(n - 2 + (v - n - 1)) * sstride,
-                           scl + (size_t)(v - n) * Ps);
-            continue;
-        }
-        auto site = [&](int p, int pg) {
-            const int kk = (s0.tip ? 0 : s0.scl[p]) + (s1.tip ? 0 : s1.scl[p]);
-            const int code = A.tips[pg];  // leaf 0
+        F2 pi[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) pi[i] = f2_of(M.pi[i]);
+        const int g = (int)threadIdx.x % S, per = (int)blockDim.x / (S * kScoreUnit);  // units per pass
+        for (int ub = u0; ub < u1; ub += per) {
+            const int u = ub + (int)threadIdx.x / (S * kScoreUnit);
+            const int p = u * kScoreUnit + (int)threadIdx.x / S % kScoreUnit;
+            const bool valid = u < u1 && p < P;
+            double term = 0.0;
             F2 L{0.f, 0.f};
             int E = 0;
-            using T = typename Lanes<C>::T;
-#pragma unroll 1
-            for (int g = 0; g < Lanes<C>::n; ++g) {
-                F2T<T> d[4], t[4];
-                int e[Lanes<C>::w];
-                f2_apply_src4<C>(Pf, Pfl, s0, Ps, p, pg, g, d);
-                f2_apply_src4<C>(Pf + 16 * C, Pfl + 16 * C, s1, Ps, p, pg, g, t);
-                f2_mul4<T>(d, t);
-                f2_normalise4(d, e);
-                f2_apply4<C>(Pf + 32 * C, Pfl + 32 * C, g, d, t);
+            if (valid) {
+                F2T<T> acc[4], wait[kScoreStack][4];
+                int kk = 0, wk[kScoreStack], sp = 0;
+                auto tip = [&](int v, F2T<T>* y) {
+                    const Src2<C> s{nullptr, nullptr, nullptr, A.tips + (size_t)v * P};
+                    f2_apply_src4<C>(Ph + (size_t)v * 16 * C, Pl + (size_t)v * 16 * C, s, 0, 0, p, g, y);
+                };
+                for (int q = 0; q < n - 2; ++q) {
+                    const ScoreProg o = prog[q];
+                    F2T<T> y[4], z[4];
+                    if (o.kind == 0) {
+                        if (q > 0) {
 #pragma unroll
-                for (int k = 0; k < Lanes<C>::w; ++k) {
+                            for (int i = 0; i < 4; ++i) wait[sp][i] = acc[i];
+                            wk[sp++] = kk;
+                        }
+                        kk = 0;
+                        tip(o.a, y);
+                        tip(o.b, z);
+                    } else {
+                        f2_apply4<C>(Ph + (size_t)o.b * 16 * C, Pl + (size_t)o.b * 16 * C, g, acc, y);
+                        if (o.kind == 1) {
+                            tip(o.a, z);
+                        } else {
+                            kk += wk[--sp];
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) acc[i] = wait[sp][i];
+                            f2_apply4<C>(Ph + (size_t)o.a * 16 * C, Pl + (size_t)o.a * 16 * C, g, acc, z);
+                        }
+                    }
+                    float mx = 0.f;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        acc[i] = t2_mul<T>(y[i], z[i]);
+                        mx = fmaxf(mx, lane_max(acc[i].h));
+                    }
+                    if (mx < Prec<float>::thresh()) {
+                        const T m = lane_all<T>(Prec<float>::mult());
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            acc[i].h = pmul(acc[i].h, m);
+                            acc[i].l = pmul(acc[i].l, m);
+                        }
+                        ++kk;
+                    }
+                }
+                const int code = A.tips[p];  // leaf 0, across the edge of node n
+                F2T<T> t[4];
+                int e[Lanes<C>::w];
+                f2_normalise4(acc, e);
+                f2_apply4<C>(Ph + (size_t)n * 16 * C, Pl + (size_t)n * 16 * C, g, acc, t);
+#pragma unroll
+                for (int w = 0; w < Lanes<C>::w; ++w) {
                     F2 Lr{0.f, 0.f};
 #pragma unroll
                     for (int i = 0; i < 4; ++i)
-                        if (code >= 4 || code == i) Lr = f2_add(Lr, f2_mul(lane_of(t[i], k), F2{pih[i], pil[i]}));
-                    f2_merge(L, E, Lr, e[k]);
+                        if (code >= 4 || code == i) Lr = f2_add(Lr, f2_mul(lane_of(t[i], w), pi[i]));
+                    f2_merge(L, E, Lr, e[w] - Prec<float>::kScaleExp * kk);
                 }
             }
-            L = F2{L.h * (1.0f / C), L.l * (1.0f / C)};
-            return __dmul_rn((double)A.w[pg], f2_log(L, E - Prec<float>::kScaleExp * kk));
-        };
-        for (int m = 0; m < sx.M; ++m)
-            add_score(acc, m < sx.cnt ? site(sx.pl0 + m * sx.pstep, sx.p0 + m * sx.step) : 0.0, sx.lanes);
+            if constexpr (S == 2) {  // the site's other categories
+                const F2 o{__shfl_xor_sync(0xffffffffu, L.h, 1), __shfl_xor_sync(0xffffffffu, L.l, 1)};
+                const int oE = __shfl_xor_sync(0xffffffffu, E, 1);
+                if (o.h > 0.f) f2_merge(L, E, o, oE);
+            }
+            if (valid && g == 0) {
+                L = F2{L.h * (1.0f / C), L.l * (1.0f / C)};  // 1/C is a power of two
+                term = __dmul_rn((double)A.w[p], f2_log(L, E));
+            }
+            // the unit's sum: its S * 2 warps
+            term = warp_sum(term, 1);
+            if (lane == 0) red[warp] = term;
+            __syncthreads();
+            if (threadIdx.x < per && ub + (int)threadIdx.x < u1) {
+                double sum = 0.0;
+#pragma unroll
+                for (int w = 0; w < 2 * S; ++w) sum += red[threadIdx.x * 2 * S + w];
+                part[(size_t)(x - t0) * units_max + ub + threadIdx.x] = sum;
+            }
+            __syncthreads();
+        }
     }
-    return team_sum<kClus>(acc, red, tm, sx.lanes);
+}
+
+// Sums a tree's units in order; with a prior, adds the log prior of its lengths.
+__global__ void k_score_sum(const FullGroup* __restrict__ groups, const int* __restrict__ gstart, int ngroups, int t0,
+                            int t1, int units_max, const double* __restrict__ part, double prior_rate,
+                            double prior_log) {
+    const int x = t0 + blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (x >= min(gstart[ngroups], t1)) return;
+    int k = 0;
+    while (k + 1 < ngroups && gstart[k + 1] <= x) ++k;
+    const FullGroup& G = groups[k];
+    const int gi = G.order ? G.order[x - gstart[k]] : x - gstart[k];
+    const int units = (G.A.P + kScoreUnit - 1) / kScoreUnit, NN = 2 * G.ts.n - 2;
+    double f = 0.0;
+    for (int u = lane; u < units; u += 32) f += part[(size_t)(x - t0) * units_max + u];
+    f = warp_sum(f, 1);
+    if (lane == 0) {
+        if (prior_rate != 0.0) {  // MAP: log prior of the lengths
+            const double* len = G.ts.len + (size_t)(G.first + gi) * NN;
+            double sum = 0.0;
+            for (int w = 1; w < NN; ++w) sum += len[w];
+            f += (double)(NN - 1) * prior_log - prior_rate * sum;
+        }
+        G.lnl_out[gi] = f;
+    }
 }
 
 // ---------------------------------------------------------------- P matrices of tree sets
@@ -2587,8 +2723,6 @@ struct FullSmem {
     R pi[4];
     int next, grp;
     alignas(16) R Pst[2][C * 16];         // the current operation's P matrices, when the tree's stay in the slab
-    float Pf[3][C * 16], Pfl[3][C * 16];  // pair P matrices of the score pass (two children, the node)
-    double exf[3][4 * C];
     NewtonSmem<R, C> ns;
 };
 // Shared memory after FullSmem: lengths, the tree (parents and children as
@@ -2813,14 +2947,10 @@ __global__ void __launch_bounds__(512) k_fullopt(const FullGroup* __restrict__ g
             }
             if (op >= n) slot(op - n);
         };
-        // mixed precision scores every tree with the pair pass below, so an
-        // evaluation at fixed lengths needs no FP32 partials at all
-        const bool pair_score = sizeof(R) == 4;
         // bottom-up D pass
-        if (!(pair_score && G.max_sweeps == 0))
-            for (int v = NN - 1; v >= n; --v) refreshD(v);
+        for (int v = NN - 1; v >= n; --v) refreshD(v);
         int sweeps = 0, last = n;
-        if (G.max_sweeps == 0 && !pair_score) visit_build(n);
+        if (G.max_sweeps == 0) visit_build(n);  // FP64 (mixed precision scores fixed lengths by k_score alone)
         for (int sw = 0; sw < G.max_sweeps; ++sw) {
             ++sweeps;
             for (int k = 0; k < nsched; ++k) {
@@ -2849,22 +2979,15 @@ __global__ void __launch_bounds__(512) k_fullopt(const FullGroup* __restrict__ g
         if (sweeps > 0)
             for (int v = threadIdx.x; v < NN; v += blockDim.x) len[v] = len_dbl(lens[v]);
         __syncthreads();
-        // exact lnL at the final lengths: the last visited edge's sum-table (FP64),
-        // or, in mixed precision, a pruning pass in pair arithmetic: D_v of every
-        // inner node bottom-up (h over the FP32 D slot, l in the U slot of v,
-        // free after the sweeps), the first inner node's combined at the root
-        double f1;
-        if constexpr (sizeof(R) == 4) {
-            f1 = fullopt_score_f2<C, kClus>(n, ch, len, A, sx, reinterpret_cast<float*>(clv), scl, sm.ns.W, sm.ns.lr,
-                                            &sm.Pf[0][0], &sm.Pfl[0][0], &sm.exf[0][0], M.pi, sm.ns.red, tm);
-        } else {
-            f1 = eval_lnl<C, kClus>(st, sx, len[last], sm.ns, tm);
-        }
         sweeps_total += sweeps;
+        // exact lnL at the final lengths: the last visited edge's sum-table (FP64); in
+        // mixed precision k_score follows on the lengths written here
+        double f1 = 0.0;
+        if constexpr (sizeof(R) == 8) f1 = eval_lnl<C, kClus>(st, sx, len[last], sm.ns, tm);
         __syncthreads();
         if (rank == 0)
             for (int v = threadIdx.x; v < NN; v += blockDim.x) glen[v] = len[v];
-        if (threadIdx.x == 0 && rank == 0) {
+        if (sizeof(R) == 8 && threadIdx.x == 0 && rank == 0) {
             if (__double_as_longlong(cfg.prior_rate) != 0) {  // MAP: log prior of the lengths
                 double sum = 0.0;
                 for (int w = 1; w < NN; ++w) sum += len[w];
@@ -3283,6 +3406,29 @@ void launch_fullopt(cudaStream_t s, int prec, int C, const FullGroup* groups, co
                  stats, reinterpret_cast<unsigned char*>(scratch), scratch_per_cta,
                  reinterpret_cast<unsigned char*>(slab), slab_per_cta, full_p_smem(prec, C, maxN, f, h.pt) ? 1 : 0,
                  h.geo, lo, hi);
+}
+
+int score_units(int P) { return (P + kScoreUnit - 1) / kScoreUnit; }
+
+void launch_score(cudaStream_t s, int C, const FullGroup* groups, const int* gstart, int ngroups, int maxN, int maxP,
+                  Cfg cfg, int t0, int t1, double* part, int sms) {
+    if (t1 <= t0) return;
+    const int units = score_units(maxP), S = C == 1 ? 1 : 2;
+    // few trees: one unit per CTA; many: four units a pass, two passes per CTA (a pass
+    // costs several times the P matrices that each CTA makes)
+    const long long tt = (long long)(t1 - t0) * units;
+    const int threads = tt <= 4LL * sms ? S * kScoreUnit : tt <= 16LL * sms ? 2 * S * kScoreUnit : 4 * S * kScoreUnit;
+    const int passes = (units + threads / (S * kScoreUnit) - 1) / (threads / (S * kScoreUnit));
+    const int chunks = tt <= 16LL * sms ? passes : (passes + 1) / 2;
+    const size_t smem = score_smem(C, 2 * maxN - 2);
+    auto kern = C == 1 ? k_score<1> : k_score<4>;
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const int grid = (int)std::min<long long>((long long)(t1 - t0) * chunks, 16LL * sms);
+    kern<<<grid, threads, smem, s>>>(groups, gstart, ngroups, 2 * maxN - 2, t0, t1, chunks, units, part);
+    ++g_launches;
+    k_score_sum<<<blocks_for(t1 - t0, 4), 128, 0, s>>>(groups, gstart, ngroups, t0, t1, units, part, cfg.prior_rate,
+                                                       cfg.prior_log);
+    ++g_launches;
 }
 
 size_t fullopt_slab_bytes(int prec, int C, int n, int P) {

@@ -164,8 +164,15 @@ extern "C" pt_status pt_score_topologies_noalloc(int n_taxa, int n_patterns, con
         cudaGetLastError();
         return PT_ERR_CUDA;
     }
-    launch_fullopt(stream, prec, M.C, d_group, d_gstart, 1, d_counter, n, P, k, stats, shape, grid,
-                   smem_tab ? nullptr : base + o_tab, spc, base + o_slab, slab);
+    if (prec == PT_PREC_FP64 || gp.max_sweeps > 0)
+        launch_fullopt(stream, prec, M.C, d_group, d_gstart, 1, d_counter, n, P, k, stats, shape, grid,
+                       smem_tab ? nullptr : base + o_tab, spc, base + o_slab, slab);
+    if (prec == PT_PREC_MIXED) {  // scores; the unit sums go where the slabs were, some trees at a time
+        const int batch = (int)std::min<size_t>(T, (size_t)grid * slab / (sizeof(double) * score_units(P)));
+        for (int t0 = 0; t0 < n_trees; t0 += batch)
+            launch_score(stream, M.C, d_group, d_gstart, 1, n, P, k, t0, std::min(n_trees, t0 + batch),
+                         reinterpret_cast<double*>(base + o_slab), nsm);
+    }
     launch_lengths_to_input(stream, n, n_trees, ts, lengths_out_dev);
     if (cudaGetLastError() != cudaSuccess) return PT_ERR_CUDA;
     return PT_OK;
