@@ -978,43 +978,6 @@ __device__ __forceinline__ void store_vec(R* dst, int ld, int p, const R* y) {
 }
 
 // ---------------------------------------------------------------- compensated FP32 (scores of the mixed path)
-// The mixed path runs its Newton iterations on FP32 partials, but every score
-// it reports comes from partials carried as unevaluated sums h + l of two FP32
-// numbers (|l| <= ulp(h)/2, about 48 significant bits): FP32 rounding errors of
-// a partial repeat at every site that shares its sub-pattern (a constant
-// column below a node, say, at thousands of sites), so at 10^4 sites they add
-// up to ~1e-3 nats; the pairs bring that below 1e-6.  Error-free steps:
-// Dekker's product by FMA (a*b = p + fma(a, b, -p)) and Knuth's two-sum.
-// Explicit _rn intrinsics keep the compiler from contracting them.
-struct F2 {
-    float h, l;
-};
-__device__ __forceinline__ F2 f2_two_sum(float a, float b) {
-    const float s = __fadd_rn(a, b);
-    const float bb = __fsub_rn(s, a);
-    return F2{s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb))};
-}
-// h + l renormalised, for |h| >= |l| (Dekker's fast two-sum)
-__device__ __forceinline__ F2 f2_norm(float h, float l) {
-    const float s = __fadd_rn(h, l);
-    return F2{s, __fsub_rn(l, __fsub_rn(s, h))};
-}
-__device__ __forceinline__ F2 f2_mul(F2 a, F2 b) {
-    const float p = __fmul_rn(a.h, b.h);
-    float e = __fmaf_rn(a.h, b.h, -p);
-    e = __fmaf_rn(a.h, b.l, e);
-    e = __fmaf_rn(a.l, b.h, e);
-    return f2_norm(p, e);
-}
-__device__ __forceinline__ F2 f2_add(F2 a, F2 b) {
-    const F2 s = f2_two_sum(a.h, b.h);
-    return f2_norm(s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l)));
-}
-__device__ __forceinline__ F2 f2_of(double x) {
-    const float h = (float)x;
-    return F2{h, (float)(x - (double)h)};
-}
-
 // The pair operations on T = float, or T = f32x2: two categories at once.
 template <typename T>
 struct F2T {
@@ -1516,6 +1479,11 @@ struct NewtonSmem {
     double lr[4 * C];      // lam_k * rate_r, [k][r] (as every 4C array here)
     float lrf[4 * C];      // the same in FP32 (coefficients of the Newton derivatives)
     double ex[4 * C];      // exp(lam_k r t) for a P-matrix refresh
+    Exp2Tab et;
+    F2 lrp[4 * C];         // lr as pairs (mixed precision)
+    F2 Wp[64];             // W as pairs
+    F2 em[4 * C];          // exp(lam_k r t) - 1 for a P-matrix refresh from pairs
+    float lr_min;          // the smallest |lr| but the zero ones
     double W[64];          // W[(i*4+j)*4+k] = isqpi_i sqpi_j R_ik R_jk: P_ij = sum_k W_ijk exp(lam_k r t)
     Len<R> tmin, tmax, tol, sweep_tol, prior;  // the solver's constants
     int moved_at;          // last sweep (from 1) of the item that moved a length by more than sweep_tol
@@ -1585,6 +1553,7 @@ __device__ __forceinline__ void init_newton_smem(const Model& M, const Cfg& cfg,
     for (int x = threadIdx.x; x < 64; x += blockDim.x) {
         int k = x & 3, ij = x >> 2, i = ij >> 2, j = ij & 3;
         ns.W[x] = M.isqpi[i] * M.sqpi[j] * M.R[i * 4 + k] * M.R[j * 4 + k];
+        if (sizeof(R) == 4) ns.Wp[x] = f2_of(ns.W[x]);
     }
     if (threadIdx.x == 0) {
         // Leader warp: FP64 instructions issue slowly and only on the issuing warp's
@@ -1614,6 +1583,12 @@ __device__ __forceinline__ void init_newton_smem(const Model& M, const Cfg& cfg,
     for (int q = threadIdx.x; q < 4 * C; q += blockDim.x) {
         ns.lr[q] = M.lam[q / C] * rates[q % C];
         ns.lrf[q] = (float)ns.lr[q];
+        if (sizeof(R) == 4) ns.lrp[q] = f2_of(ns.lr[q]);
+    }
+    if (threadIdx.x == 0) {
+        double m = 1e30;
+        for (int q = C; q < 4 * C; ++q) m = fmin(m, fabs(M.lam[q / C] * rates[q % C]));
+        ns.lr_min = (float)m;
     }
 }
 
@@ -1895,6 +1870,10 @@ __device__ __forceinline__ float4 site_sums(const STab<R, C>& st, const Sites& s
     }
 }
 
+// Below this t |lam r| (so off-diagonal entries of about 2^-17) the rounding test of
+// p_entry_pair fails for one solve in ten or more, and the FP64 sum is taken at once.
+constexpr float kPairMin = 3e-5f;
+
 // Newton solve on the current sum-table from t (as newton_begin returned it).  Per
 // evaluation: every thread sums w L'/L and w (L''/L - (L'/L)^2) over its sites, the
 // warps reduce, and one warp alone takes the step and writes the coefficients of
@@ -1914,6 +1893,7 @@ __device__ __forceinline__ void newton_solve(const Cfg& cfg, const STab<R, C>& s
     __syncthreads();  // the coefficients of newton_begin
     const int ld = ns.leader;
     Len<R> lo = ns.tmin, hi = ns.tmax;
+    bool pairs = false;
     converged = false;
     evals = 0;
     for (int it = 0; it < cfg.newton_maxit; ++it) {
@@ -2001,7 +1981,16 @@ __device__ __forceinline__ void newton_solve(const Cfg& cfg, const STab<R, C>& s
             if (!last) {
                 put_egh<C>(t, ns, lane);
             } else {
-                if (lane < 4 * C) ns.ex[lane] = exp(ns.lr[lane] * len_dbl(t));  // for the P matrices below
+                // for the P matrices below: pairs where their rounding test mostly passes
+                // (off-diagonal entries not tiny), else FP64 exponentials
+                if constexpr (sizeof(R) == 4) {
+                    pairs = t.h * ns.lr_min > kPairMin;
+                    if (pairs && lane < 4 * C) {
+                        const F2 x = f2_mul(ns.lrp[lane], t);
+                        ns.em[lane] = x.h > -80.f ? expm1_pair(x, ns.et) : F2{-1.f, 0.f};
+                    }
+                }
+                if (!pairs && lane < 4 * C) ns.ex[lane] = exp(ns.lr[lane] * len_dbl(t));
                 if (lane == 0) {
                     bool moved;
                     if constexpr (sizeof(R) == 4) moved = f2_lt(ns.sweep_tol, f2_abs(f2_sub(t, told)));
@@ -2010,13 +1999,27 @@ __device__ __forceinline__ void newton_solve(const Cfg& cfg, const STab<R, C>& s
                     *dst = t;
                 }
             }
-            if (lane == 0) ns.done = last ? (done ? 1 : 2) : 0;
+            if (lane == 0) ns.done = last ? (done ? 1 : 2) | (pairs ? 4 : 0) : 0;
         }
         __syncthreads();
         if (ns.done) {
-            // P matrices of the final length (FP64 exponentials, rounded once), spread
-            // over the first warps so their FP64 work runs on several schedulers
-            converged = ns.done == 1;
+            // P matrices of the final length, rounded once from FP64 or from pairs to the
+            // same bits (a dependent FP64 instruction takes some 60 cycles, exp() a thousand;
+            // the pairs' chain a third of that)
+            converged = (ns.done & 3) == 1;
+            bool exact = !(ns.done & 4);
+            if (sizeof(R) == 4 && !exact) {
+                bool sure = true;
+                for (int x = threadIdx.x; x < 16 * C; x += blockDim.x) {
+                    const int r = x % C, ij = x / C;
+                    bool ok;
+                    Pdst[x] = p_entry_pair(ij % 5 == 0 ? 1.f : 0.f, ns.Wp + ij * 4, ns.em + r, C, ok);
+                    sure = sure && ok;
+                }
+                if (!__syncthreads_or(!sure)) break;
+                if (w == ld && lane < 4 * C) ns.ex[lane] = exp(ns.lr[lane] * len_dbl(t));
+                __syncthreads();
+            }
             for (int x = threadIdx.x; x < 16 * C; x += blockDim.x) {
                 const int r = x % C, ij = x / C;
                 double acc = ns.W[ij * 4];  // lam_0 = 0
@@ -2489,6 +2492,7 @@ __global__ void __launch_bounds__(512) k_propose(const PropGroup* __restrict__ g
     Team tm{kClus ? (int)cluster_ctas() : 1, kClus ? (int)cluster_rank() : 0, 0, 0};
     const int rank = tm.rank;
     if (kClus && threadIdx.x == 0) cluster_exchange_init(sm.ns);  // before the first cluster barrier
+    if (sizeof(R) == 4) sm.ns.et.init();
     while (true) {
         // previous item done with shared memory (in every CTA of the cluster: rank 0 writes theirs)
         if constexpr (kClus) cooperative_groups::this_cluster().sync();
@@ -2771,6 +2775,7 @@ __global__ void __launch_bounds__(512) k_fullopt(const FullGroup* __restrict__ g
     Team tm{kClus ? (int)cluster_ctas() : 1, kClus ? (int)cluster_rank() : 0, 0, 0};
     const int rank = tm.rank;
     if (kClus && threadIdx.x == 0) cluster_exchange_init(sm.ns);  // before the first cluster barrier
+    if (sizeof(R) == 4) sm.ns.et.init();
     bool first = true;  // thread 0: this CTA (cluster) has not taken a tree yet
     while (true) {
         // previous tree done with shared memory (in every CTA of the cluster: rank 0 writes theirs)
