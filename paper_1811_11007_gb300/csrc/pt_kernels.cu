@@ -320,11 +320,18 @@ __device__ long long table_find_or_claim(Slot* tab, int log2, unsigned long long
     return -1;
 }
 
+// A thread per 16 bytes, so a warp writes one run of memory (a thread per slot wrote
+// 8 bytes at a time 64 bytes apart: 175 us for 2^22 slots).
 __global__ void k_table_init(Slot* tab, size_t nslots) {
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < nslots; i += (size_t)gridDim.x * blockDim.x) {
-        tab[i].klo = 0; tab[i].khi = 0; tab[i].tag = kTagEmpty; tab[i].ahi = kTagEmpty; tab[i].alo = kTagEmpty;
-        tab[i].lnl = __longlong_as_double(0x7ff8000000000000ll);
-        tab[i].alpha = __longlong_as_double(0x7ff8000000000000ll);
+    ulonglong2* const q = reinterpret_cast<ulonglong2*>(tab);
+    const unsigned long long nan = 0x7ff8000000000000ull;
+    static_assert(sizeof(Slot) == 64, "chunks: key; tag, ahi; alo, lnl; alpha, pad");
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < 4 * nslots; i += (size_t)gridDim.x * blockDim.x) {
+        const int c = (int)(i & 3);
+        q[i] = c == 0   ? make_ulonglong2(0, 0)
+               : c == 1 ? make_ulonglong2(kTagEmpty, kTagEmpty)
+               : c == 2 ? make_ulonglong2(kTagEmpty, nan)
+                        : make_ulonglong2(nan, 0);
     }
 }
 
@@ -2114,8 +2121,8 @@ struct ScoreProg {
 __host__ __device__ inline size_t score_smem(int C, int nn) {
     return ((size_t)nn * 32 * C * 4 + (size_t)nn * (3 + 8) + 15) & ~size_t(15);
 }
-template <int C>
-__global__ void __launch_bounds__(512) k_score(const FullGroup* __restrict__ groups, const int* __restrict__ gstart,
+template <int C, int kThreads>
+__global__ void __launch_bounds__(kThreads) k_score(const FullGroup* __restrict__ groups, const int* __restrict__ gstart,
                                                int ngroups, int nn_max, int t0, int t1, int chunks, int units_max,
                                                double* __restrict__ part) {
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -2126,7 +2133,7 @@ __global__ void __launch_bounds__(512) k_score(const FullGroup* __restrict__ gro
     ScoreProg* const prog = reinterpret_cast<ScoreProg*>(Pl + (size_t)nn_max * 16 * C);
     uint8_t* const ch = reinterpret_cast<uint8_t*>(prog + nn_max);  // children; then need[] and two stacks
     uint8_t *const need = ch + 2 * nn_max, *const stk = need + nn_max;
-    __shared__ double W[64], red[16];
+    __shared__ double W[64], red[24];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int total = min(gstart[ngroups], t1) - t0;
     for (long long work = blockIdx.x; work < (long long)total * chunks; work += gridDim.x) {
@@ -3035,7 +3042,7 @@ void launch_canon(cudaStream_t s, int n, int count, const int32_t* edges, const 
 }
 
 void launch_table_init(cudaStream_t s, Slot* tab, size_t nslots) {
-    k_table_init<<<1024, 256, 0, s>>>(tab, nslots);
+    k_table_init<<<2432, 256, 0, s>>>(tab, nslots);
     ++g_launches;
 }
 
@@ -3427,14 +3434,17 @@ void launch_score(cudaStream_t s, int C, const FullGroup* groups, const int* gst
                   Cfg cfg, int t0, int t1, double* part, int sms) {
     if (t1 <= t0) return;
     const int units = score_units(maxP), S = C == 1 ? 1 : 2;
-    // few trees: one unit per CTA; many: four units a pass, two passes per CTA (a pass
-    // costs several times the P matrices that each CTA makes)
+    // few trees: one unit per CTA; many: 24 warps per SM (80 registers a thread) as three
+    // CTAs where their P matrices fit, else as one; two passes per CTA (a pass costs
+    // several times the P matrices that each CTA makes)
     const long long tt = (long long)(t1 - t0) * units;
-    const int threads = tt <= 4LL * sms ? S * kScoreUnit : tt <= 16LL * sms ? 2 * S * kScoreUnit : 4 * S * kScoreUnit;
+    const size_t smem = score_smem(C, 2 * maxN - 2);
+    const int threads = tt <= 4LL * sms ? S * kScoreUnit
+                        : 3 * (smem + 2048) <= (size_t)228 * 1024 ? 2 * S * kScoreUnit : 6 * S * kScoreUnit;
     const int passes = (units + threads / (S * kScoreUnit) - 1) / (threads / (S * kScoreUnit));
     const int chunks = tt <= 16LL * sms ? passes : (passes + 1) / 2;
-    const size_t smem = score_smem(C, 2 * maxN - 2);
-    auto kern = C == 1 ? k_score<1> : k_score<4>;
+    const bool few = threads == S * kScoreUnit;
+    auto kern = C == 1 ? (few ? k_score<1, 256> : k_score<1, 768>) : (few ? k_score<4, 256> : k_score<4, 768>);
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     const int grid = (int)std::min<long long>((long long)(t1 - t0) * chunks, 16LL * sms);
     kern<<<grid, threads, smem, s>>>(groups, gstart, ngroups, 2 * maxN - 2, t0, t1, chunks, units, part);
