@@ -59,6 +59,15 @@ struct Ctx {
     std::string err;
     std::vector<AlnState> alns;
     std::map<std::string, DevBuf> bufs;
+    // device-to-host reads of the current call that wait for the next sync_back, through a
+    // pinned block (small reads into pageable memory are one synchronous transfer each)
+    struct Back {
+        void* host;
+        size_t off, n;
+    };
+    unsigned char* pin = nullptr;
+    size_t pin_used = 0;
+    std::vector<Back> back;
     int32_t* d_err = nullptr;
     unsigned long long* d_stats = nullptr;
     double* d_lmax = nullptr;
@@ -255,14 +264,37 @@ void zero_flags(Ctx& c) {
     ck(c, cudaMemsetAsync(c.d_err, 0, sizeof(int32_t) * kErrWords, c.stream), "memset err");
 }
 
-void check_flags(Ctx& c) {
-    int32_t h[kErrWords];
-    ck(c, cudaMemcpyAsync(h, c.d_err, sizeof h, cudaMemcpyDeviceToHost, c.stream), "read flags");
+// Queues a read of n device bytes; the host bytes are valid after sync_back.
+constexpr size_t kPinBytes = 256 << 10;
+void read_back(Ctx& c, void* host, const void* dev, size_t n, const char* what) {
+    if (!n) return;
+    if (c.pin_used + n > kPinBytes) {  // large reads go straight to the caller's memory
+        ck(c, cudaMemcpyAsync(host, dev, n, cudaMemcpyDeviceToHost, c.stream), what);
+        return;
+    }
+    ck(c, cudaMemcpyAsync(c.pin + c.pin_used, dev, n, cudaMemcpyDeviceToHost, c.stream), what);
+    c.back.push_back({host, c.pin_used, n});
+    c.pin_used += (n + 15) & ~size_t(15);
+}
+void sync_back(Ctx& c) {
     ck(c, cudaStreamSynchronize(c.stream), "stream sync");
+    for (const Ctx::Back& b : c.back) std::memcpy(b.host, c.pin + b.off, b.n);
+    c.back.clear();
+    c.pin_used = 0;
+}
+
+void test_flags(Ctx& c, const int32_t* h) {
     if (h[kErrTree]) fail(c, PT_ERR_INVALID_ARG, "tree %d is not an unrooted binary tree on leaves 0..n-1", h[kErrTree] - 1);
     if (h[kErrLen]) fail(c, PT_ERR_INVALID_ARG, "tree %d has a branch length that is not finite and >= 0", h[kErrLen] - 1);
     if (h[kErrTable]) fail(c, PT_ERR_TABLE_FULL, "visited table probe limit reached (raise table_log2)");
     if (h[kErrKey]) fail(c, PT_ERR_STATE, "neighbour key mismatch (internal error)");
+}
+// Waits for the stream (and the queued reads) and raises the device's error flags.
+void check_flags(Ctx& c) {
+    int32_t h[kErrWords];
+    read_back(c, h, c.d_err, sizeof h, "read flags");
+    sync_back(c);
+    test_flags(c, h);
 }
 
 void begin_stats(Ctx& c) {
@@ -273,10 +305,14 @@ void begin_stats(Ctx& c) {
     c.launches0 = launch_count();
 }
 
+// check_flags and the call's counters in one wait.
 void end_stats(Ctx& c, const int64_t* host_counts) {
     unsigned long long h[kStWords];
-    ck(c, cudaMemcpyAsync(h, c.d_stats, sizeof h, cudaMemcpyDeviceToHost, c.stream), "read stats");
-    ck(c, cudaStreamSynchronize(c.stream), "stream sync");
+    int32_t f[kErrWords];
+    read_back(c, h, c.d_stats, sizeof h, "read stats");
+    read_back(c, f, c.d_err, sizeof f, "read flags");
+    sync_back(c);
+    test_flags(c, f);
     for (int i = 0; i < kStWords; ++i) c.stats[i] = (int64_t)h[i];
     c.stats[kStLaunches] = launch_count() - c.launches0;
     if (h[kStTimeout]) fail(c, PT_ERR_TIMEOUT, "%llu CTAs gave up waiting for their cluster's Newton sums", h[kStTimeout]);
@@ -290,9 +326,9 @@ int scan_count(Ctx& c, const int32_t* flag, int32_t* pos, int N) {
     int32_t* tmp = buf<int32_t>(c, "scan.tmp", (size_t)(N + 1023) / 1024 + 1);
     launch_scan(c.stream, flag, pos, N, tmp);
     int32_t last[2];
-    ck(c, cudaMemcpyAsync(&last[0], pos + N - 1, 4, cudaMemcpyDeviceToHost, c.stream), "scan total");
-    ck(c, cudaMemcpyAsync(&last[1], flag + N - 1, 4, cudaMemcpyDeviceToHost, c.stream), "scan total");
-    ck(c, cudaStreamSynchronize(c.stream), "stream sync");
+    read_back(c, &last[0], pos + N - 1, 4, "scan total");
+    read_back(c, &last[1], flag + N - 1, 4, "scan total");
+    sync_back(c);
     return last[0] + last[1];
 }
 
@@ -624,14 +660,18 @@ void load_tune(Ctx& c) {
 template <typename G>
 const G* upload_groups(Ctx& c, const std::string& name, const std::vector<G>& groups, const std::vector<int>& counts,
                        const int** gstart_out, int** counter_out) {
-    G* dg = buf<G>(c, name + ".groups", groups.size());
-    int* ds = buf<int>(c, name + ".gstart", groups.size() + 1);
-    int* dc = buf<int>(c, name + ".counter", 1);
-    std::vector<int> pre(groups.size() + 1, 0);
+    // one block and one copy: the groups, their prefix sums, the zeroed counter
+    const size_t gb = sizeof(G) * groups.size(), total = gb + sizeof(int) * (groups.size() + 2);
+    unsigned char* d = buf<unsigned char>(c, name + ".groups", total);
+    std::vector<unsigned char> h(total);
+    std::memcpy(h.data(), groups.data(), gb);
+    std::vector<int> pre(groups.size() + 2, 0);
     for (size_t k = 0; k < groups.size(); ++k) pre[k + 1] = pre[k] + counts[k];
-    ck(c, cudaMemcpyAsync(dg, groups.data(), sizeof(G) * groups.size(), cudaMemcpyHostToDevice, c.stream), "groups");
-    ck(c, cudaMemcpyAsync(ds, pre.data(), sizeof(int) * pre.size(), cudaMemcpyHostToDevice, c.stream), "groups");
-    ck(c, cudaMemsetAsync(dc, 0, sizeof(int), c.stream), "counter");
+    std::memcpy(h.data() + gb, pre.data(), sizeof(int) * (groups.size() + 2));
+    ck(c, cudaMemcpyAsync(d, h.data(), total, cudaMemcpyHostToDevice, c.stream), "groups");
+    G* dg = reinterpret_cast<G*>(d);
+    int* ds = reinterpret_cast<int*>(d + gb);
+    int* dc = ds + groups.size() + 1;
     *gstart_out = ds;
     *counter_out = dc;
     return dg;
@@ -954,9 +994,9 @@ void begin_core(Ctx& c, AlnState& a, int ns, const int32_t* edges_d, const doubl
     launch_finalize_trees(c.stream, a.table, hcount(ns), winner, lnl, c.d_lmax, thr, hround(0), good, c.d_stats, sal);
     // dedup starts: a start that lost its key is not GOOD
     std::vector<int32_t> w(ns), gd(ns);
-    ck(c, cudaMemcpyAsync(w.data(), winner, 4 * (size_t)ns, cudaMemcpyDeviceToHost, c.stream), "read winners");
-    ck(c, cudaMemcpyAsync(gd.data(), good, 4 * (size_t)ns, cudaMemcpyDeviceToHost, c.stream), "read good");
-    ck(c, cudaMemcpyAsync(lmax_out, c.d_lmax, 8, cudaMemcpyDeviceToHost, c.stream), "read lmax");
+    read_back(c, w.data(), winner, 4 * (size_t)ns, "read winners");
+    read_back(c, gd.data(), good, 4 * (size_t)ns, "read good");
+    read_back(c, lmax_out, c.d_lmax, 8, "read lmax");
     check_flags(c);
     std::vector<int32_t> idx;
     for (int i = 0; i < ns; ++i) if (w[i] >= 0 && gd[i]) idx.push_back(i);
@@ -1086,8 +1126,8 @@ void expand_batch(Ctx& c, const std::vector<RoundIn>& ins, std::vector<RoundOut>
         r.tpos.assign(r.F + 1, r.W);
         if (r.ncand > 0) {
             std::vector<int32_t> allpos(r.ncand);
-            ck(c, cudaMemcpyAsync(allpos.data(), r.pos, 4 * (size_t)r.ncand, cudaMemcpyDeviceToHost, c.stream), "pos");
-            ck(c, cudaStreamSynchronize(c.stream), "sync");
+            read_back(c, allpos.data(), r.pos, 4 * (size_t)r.ncand, "pos");
+            sync_back(c);
             for (int f = 0; f < r.F; ++f) r.tpos[f] = allpos[(size_t)f * r.m];
         }
     }
@@ -1330,7 +1370,6 @@ void expand_batch(Ctx& c, const std::vector<RoundIn>& ins, std::vector<RoundOut>
     if (climb) {
         total.end();
         outs.clear();
-        check_flags(c);
         end_stats(c, hc);
         return;
     }
@@ -1410,10 +1449,9 @@ void expand_batch(Ctx& c, const std::vector<RoundIn>& ins, std::vector<RoundOut>
     sp4.end();
     total.end();
     std::vector<double> lm(na);
-    ck(c, cudaMemcpyAsync(lm.data(), d_lmax, 8 * (size_t)na, cudaMemcpyDeviceToHost, c.stream), "read lmax");
-    check_flags(c);
-    for (int k = 0; k < na; ++k) outs[k].lmax = lm[k];
+    read_back(c, lm.data(), d_lmax, 8 * (size_t)na, "read lmax");
     end_stats(c, hc);
+    for (int k = 0; k < na; ++k) outs[k].lmax = lm[k];
 }
 
 void expand_core(Ctx& c, AlnState& a, int F, const int32_t* edges_d, const double* lens_d, double thr,
@@ -1462,11 +1500,11 @@ void climb_core(Ctx& c, AlnState& a, int T, const int32_t* edges_d, const double
         l.resize((size_t)cnt * E);
         x.resize(cnt);
         k.resize((size_t)cnt * 2);
-        ck(c, cudaMemcpyAsync(e.data(), ge, 4 * e.size(), cudaMemcpyDeviceToHost, c.stream), "climb copy");
-        ck(c, cudaMemcpyAsync(l.data(), gl, 8 * l.size(), cudaMemcpyDeviceToHost, c.stream), "climb copy");
-        ck(c, cudaMemcpyAsync(x.data(), gx, 8 * x.size(), cudaMemcpyDeviceToHost, c.stream), "climb copy");
-        ck(c, cudaMemcpyAsync(k.data(), gk, 8 * k.size(), cudaMemcpyDeviceToHost, c.stream), "climb copy");
-        ck(c, cudaStreamSynchronize(c.stream), "sync");
+        read_back(c, e.data(), ge, 4 * e.size(), "climb copy");
+        read_back(c, l.data(), gl, 8 * l.size(), "climb copy");
+        read_back(c, x.data(), gx, 8 * x.size(), "climb copy");
+        read_back(c, k.data(), gk, 8 * k.size(), "climb copy");
+        sync_back(c);
     };
     fetch(T, cur, clnl, he, hl, hlnl, hkey);
     end_stats(c, nullptr);
@@ -1563,11 +1601,11 @@ void write_out(Ctx& c, const AlnState& a, RoundOut& o, int cap, int32_t* e, doub
     double* dn = buf<double>(c, "out.lnl", o.count);
     uint64_t* dk = buf<uint64_t>(c, "out.k", (size_t)o.count * 2);
     launch_gather_out(c.stream, n, hcount(o.count), o.idx, o.ts, o.lnl, de, dl, dn, dk);
-    if (e) ck(c, cudaMemcpyAsync(e, de, 4 * (size_t)o.count * 2 * E, cudaMemcpyDeviceToHost, c.stream), "copy out");
-    if (l) ck(c, cudaMemcpyAsync(l, dl, 8 * (size_t)o.count * E, cudaMemcpyDeviceToHost, c.stream), "copy out");
-    if (lnl) ck(c, cudaMemcpyAsync(lnl, dn, 8 * (size_t)o.count, cudaMemcpyDeviceToHost, c.stream), "copy out");
-    if (keys) ck(c, cudaMemcpyAsync(keys, dk, 16 * (size_t)o.count, cudaMemcpyDeviceToHost, c.stream), "copy out");
-    ck(c, cudaStreamSynchronize(c.stream), "sync");
+    if (e) read_back(c, e, de, 4 * (size_t)o.count * 2 * E, "copy out");
+    if (l) read_back(c, l, dl, 8 * (size_t)o.count * E, "copy out");
+    if (lnl) read_back(c, lnl, dn, 8 * (size_t)o.count, "copy out");
+    if (keys) read_back(c, keys, dk, 16 * (size_t)o.count, "copy out");
+    sync_back(c);
 }
 
 // ---------------------------------------------------------------- graph rounds
@@ -2041,14 +2079,24 @@ namespace {
 template <typename F>
 pt_status guarded(pt_ctx* ctx, F&& f) {
     if (!ctx) return PT_ERR_INVALID_ARG;
+    // a call that fails drops its queued reads (their host buffers end with it)
+    auto drop = [&] {
+        Ctx& c = ctx->c;
+        if (c.back.empty()) return;
+        cudaStreamSynchronize(c.stream);
+        c.back.clear();
+        c.pin_used = 0;
+    };
     try {
         ck(ctx->c, cudaSetDevice(ctx->c.cfg.device), "cudaSetDevice");
         f(ctx->c);
         ctx->c.err.clear();
         return PT_OK;
     } catch (const Fail& e) {
+        drop();
         return e.st;
     } catch (...) {
+        drop();
         ctx->c.err = "unexpected host exception";
         return PT_ERR_STATE;
     }
@@ -2104,6 +2152,7 @@ pt_status pt_create(pt_ctx** out, const pt_config* cfg) {
         dev_alloc(c, &c.d_stats, sizeof(unsigned long long) * kStWords, "alloc");
         dev_alloc(c, &c.d_lmax, 8, "alloc");
         ck(c, cudaMemset(c.d_err, 0, sizeof(int32_t) * kErrWords), "memset");
+        ck(c, cudaHostAlloc(reinterpret_cast<void**>(&c.pin), kPinBytes, cudaHostAllocDefault), "pinned");
         size_t fr, tot;
         ck(c, cudaMemGetInfo(&fr, &tot), "cudaMemGetInfo");
         // frontier partials of one proposal wave: 40% of the free memory at creation, at
@@ -2135,6 +2184,7 @@ void pt_destroy(pt_ctx* ctx) {
     for (void* p : {(void*)c.mlp_w, (void*)c.mlp_g, (void*)c.mlp_m1, (void*)c.mlp_m2, c.mlp.w1t, c.mlp.w2t, c.mlp.w3t,
                     c.mlp.w2r, c.mlp.w3r, (void*)c.log_x, (void*)c.log_t, (void*)c.log_count})
         if (p) dev_free(c, p);
+    if (c.pin) cudaFreeHost(c.pin);
     if (c.d_err) dev_free(c, c.d_err);
     if (c.d_stats) dev_free(c, c.d_stats);
     if (c.d_lmax) dev_free(c, c.d_lmax);
@@ -2252,11 +2302,9 @@ pt_status pt_score_topologies(pt_ctx* ctx, int aln_id, int n_trees, const int32_
         score_core(c, a, n_trees, de, dl, mode, "sc", ts, lnl);
         launch_lengths_to_input(c.stream, a.n, n_trees, ts, dl);
         total.end();
-        ck(c, cudaMemcpyAsync(lengths, dl, 8 * (size_t)n_trees * E, cudaMemcpyDeviceToHost, c.stream), "copy out");
-        ck(c, cudaMemcpyAsync(lnl_out, lnl, 8 * (size_t)n_trees, cudaMemcpyDeviceToHost, c.stream), "copy out");
-        if (keys_out)
-            ck(c, cudaMemcpyAsync(keys_out, ts.key, 16 * (size_t)n_trees, cudaMemcpyDeviceToHost, c.stream), "copy out");
-        check_flags(c);
+        read_back(c, lengths, dl, 8 * (size_t)n_trees * E, "copy out");
+        read_back(c, lnl_out, lnl, 8 * (size_t)n_trees, "copy out");
+        if (keys_out) read_back(c, keys_out, ts.key, 16 * (size_t)n_trees, "copy out");
         end_stats(c, nullptr);
         collect_times(c);
     });
