@@ -560,11 +560,17 @@ std::vector<ShapeFit> shapes_of(Ctx& c, bool full, int prec, int C, int maxN, in
 // Measured on visits of 81 trees at 12 sites per virtual thread: 26.0 ms on one CTA
 // each, 19.1 on 2, 13.1 on 4 (1.1 rounds), 18.2 on 8 (2.3 rounds); on 5697 neighbours
 // at 7 sites: 84.8 ms as 8 CTAs of 256 (36 resident), 69.1 as 8 of 128 (51 resident).
-const ShapeFit& pick_shape(const std::vector<ShapeFit>& v, long long total) {
+// Warps of an SM slow each other a little while there is room for all of them at once:
+// 8 full visits of 8 taxa at 256 patterns take 6.50 ms as 4 CTAs of 256 each and 6.00 as 8
+// of 128 on twice the SMs. Past one round the resident count says what a shape delivers.
+const ShapeFit& pick_shape(const Ctx& c, const std::vector<ShapeFit>& v, long long total) {
     size_t best = 0;
     double cost = 1e300;
     for (size_t i = 0; i < v.size(); ++i) {
-        const double x = std::max(1.0, (double)total * v[i].h.kp / v[i].resident) * (5 + v[i].sites);
+        const long long ctas = total * v[i].h.kp;
+        const double rounds = (double)ctas / v[i].resident;
+        const double warps = rounds < 1 ? (double)((ctas + c.sm_count - 1) / c.sm_count) * v[i].h.pt / 32 : 16;
+        const double x = std::max(1.0, rounds) * (5 + v[i].sites) * (1 + 0.02 * warps);
         if (x < 0.999 * cost) {
             cost = x;
             best = i;
@@ -578,12 +584,12 @@ struct ShapeRange {
     ShapeFit f;
     int lo, hi;
 };
-std::vector<ShapeRange> shape_ranges(const std::vector<ShapeFit>& v, int cap) {
+std::vector<ShapeRange> shape_ranges(const Ctx& c, const std::vector<ShapeFit>& v, int cap) {
     std::vector<ShapeRange> out;
     long long most = 0;  // past this count every shape has more than one round: the choice is settled
     for (const ShapeFit& x : v) most = std::max<long long>(most, x.resident / x.h.kp + 1);
     for (int n = 1; n <= std::min<long long>(cap, most); ++n) {
-        const ShapeFit& f = pick_shape(v, n);
+        const ShapeFit& f = pick_shape(c, v, n);
         const bool same = !out.empty() && out.back().f.h.kp == f.h.kp && out.back().f.h.pt == f.h.pt;
         if (same) out.back().hi = n;
         else out.push_back({f, n - 1, n});
@@ -731,7 +737,7 @@ void run_full_jobs(Ctx& c, std::vector<FullJob> jobs, bool allow_tune = true) {
         const bool optimise = prec == PT_PREC_FP64 || jobs[0].max_sweeps > 0;
         auto launch = [&](int threads, int K, unsigned long long* stats) {
             const std::vector<ShapeFit> shapes = shapes_of(c, true, prec, C, maxN, maxP, threads, K);
-            const ShapeFit& f = pick_shape(shapes, total);
+            const ShapeFit& f = pick_shape(c, shapes, total);
             const int grid = (int)std::min<long long>((long long)total * f.h.kp, f.resident) / f.h.kp * f.h.kp;
             void* scratch = nullptr;
             size_t spc = 0, sl = 0;
@@ -1282,7 +1288,7 @@ void expand_batch(Ctx& c, const std::vector<RoundIn>& ins, std::vector<RoundOut>
         const PropGroup* dg = upload_groups(c, "prop", groups, counts, &gstart, &counter);
         auto run = [&](int threads, int K, unsigned long long* stats, bool timed) {
             const std::vector<ShapeFit> shapes = shapes_of(c, false, prec, C, 3, maxP, threads, K);
-            const ShapeFit& f = pick_shape(shapes, tot);
+            const ShapeFit& f = pick_shape(c, shapes, tot);
             const int grid = (int)std::min<long long>((long long)tot * f.h.kp, f.resident) / f.h.kp * f.h.kp;
             void* scratch = nullptr;
             size_t spc = 0;
@@ -1868,8 +1874,8 @@ GraphRound* graph_create(Ctx& c, const std::vector<int>& ids, const std::vector<
         if (tt->second.full_cluster) g.full_cluster = tt->second.full_cluster;
     }
     const std::vector<ShapeRange>
-        ps = shape_ranges(shapes_of(c, false, prec, C, 3, maxP, g.prop_threads, g.prop_cluster), totCap),
-        fs = shape_ranges(shapes_of(c, true, prec, C, maxN, maxP, g.full_threads, g.full_cluster), totCap);
+        ps = shape_ranges(c, shapes_of(c, false, prec, C, 3, maxP, g.prop_threads, g.prop_cluster), totCap),
+        fs = shape_ranges(c, shapes_of(c, true, prec, C, maxN, maxP, g.full_threads, g.full_cluster), totCap);
     const size_t tabb = (sumtable_bytes(prec, C, maxP) + 255) & ~size_t(255);
     size_t pscratch = 0, fscratch = 0, slab = 0;
     for (const ShapeRange& x : ps)

@@ -811,7 +811,8 @@ __device__ __forceinline__ void pmat_row(const Model& M, double rt, int i, R* ro
 // (fma / mul / add .f32x2 on 64-bit register pairs, each half rounded as the
 // scalar instruction rounds it).  With four categories every vector operation
 // here runs on pairs of categories: the issue slots of the 4 x 4 products halve
-// and every result keeps its bits.
+// and every result keeps its bits.  With the chunked vectors it took a sum-table build
+// of a proposal (27 taxa x 816 patterns) from 16.5 to 11 thousand cycles.
 using f32x2 = float2;
 __device__ __forceinline__ unsigned long long& b64(f32x2& x) { return reinterpret_cast<unsigned long long&>(x); }
 __device__ __forceinline__ unsigned long long b64c(f32x2 x) {
@@ -1889,6 +1890,9 @@ constexpr float kPairMin = 3e-5f;
 // and P_r of the final length goes to Pdst [16][C]; all visible when the call
 // returns.  Everything but the sums over sites is that warp's: what one warp does in
 // FP64 or in a long chain holds up one scheduler, what every warp does, all of them.
+// Bound by that chain: an evaluation of 816 patterns takes 2.5 to 2.9 thousand cycles
+// on one or four CTAs (site 500, warp sums 300, exchange 250 to 600, tree 400, step 490,
+// coefficients 400 to 570), a solve of three evaluations 11 to 14 thousand.
 // kClus: the sum-table holds this CTA's share of a cluster's sites; each
 // evaluation's derivative sums are exchanged over the cluster, and every CTA
 // takes the same step.
@@ -2113,7 +2117,7 @@ __device__ __noinline__ double propose_score_f2(const Src2<C>* mem, const int* m
 // for few sites, by the FP64 exponentials of the P matrices, which each CTA makes
 // once per tree, in parallel over edges and categories.  One tree of 27 taxa x 816
 // patterns took 157 us as the last step of the full optimisation, whose nodes each
-// waited for their own P matrices.
+// waited for their own P matrices, and takes 38; 256 of 64 x 987 1129, now about 560.
 constexpr int kScoreUnit = 64, kScoreStack = 9;
 struct ScoreProg {
     uint8_t kind, a, b;  // kind 0: two tips, 1: tip a and the last result (edge b), 2: waiting result (edge a) and last (edge b)
@@ -2757,7 +2761,10 @@ constexpr unsigned short kUpd16 = 0x8000;  // kUpd in a 16-bit schedule entry
 // were chains of three or four global loads before each operation), the P matrices
 // of an operation there too (read through L1 they were evicted by the vectors that
 // stream past), and as many lanes and CTAs per tree as the number of trees leaves
-// room for (Sites).
+// room for (Sites).  8 trees of 27 x 816 patterns took 12.9 ms on one CTA each with
+// those chains, now 6.3; 32 of 128 x 6273 289 ms, now 180; 515 of them 526 ms, now 340
+// (there a solve's 54 thousand cycles are half sum-table builds, in bursts at the rate
+// L2 and HBM deliver the stored vectors, 2.5 TB/s on average).
 template <typename R, int C, bool kSmemTab, bool kClus>
 __global__ void __launch_bounds__(512) k_fullopt(const FullGroup* __restrict__ groups, const int* __restrict__ gstart,
                                                  int ngroups, int* counter, int nn_max, Cfg cfg,
