@@ -521,14 +521,15 @@ int default_shares(Ctx& c, bool full, int prec, int C, int n, int P, int threads
     return any ? any : 1;
 }
 
-// A launch shape, the CTAs of it that are resident at once, and the sites of a thread.
+// A launch shape, the CTAs of it that are resident at once, and the sites of a thread
+// (weighted by their cost).
 struct ShapeFit {
     Shape h;
     int resident, sites;
 };
 // The shapes of a summation geometry (vt virtual threads, vk shares), by increasing
 // cluster size: vk CTAs per item, then 2, 4, 8 as long as the lanes of a virtual
-// thread each get a site.
+// thread each get a site; one CTA without a sum-table in shared memory where none fits.
 std::vector<ShapeFit> shapes_of(Ctx& c, bool full, int prec, int C, int maxN, int maxP, int vt, int vk) {
     std::vector<ShapeFit> v;
     auto fit = [&](const Shape& h) {
@@ -548,9 +549,13 @@ std::vector<ShapeFit> shapes_of(Ctx& c, bool full, int prec, int C, int maxN, in
             if (r >= kp) v.push_back({h, r, (J + lanes - 1) / lanes});
         }
     if (v.empty() && vk > 1) return shapes_of(c, full, prec, C, maxN, maxP, vt, 1);  // not launchable as clusters
-    if (v.empty()) {  // a sum-table too large for shared memory in every form
+    // The sum-table of one CTA in global memory, where it is too large for its shared
+    // memory: a site costs more (in FP64, whose arithmetic hides part of the reads, 1.6
+    // times, in FP32 2.5 times), but many items need no cluster each (an FP64 round at
+    // 128 taxa x 5908 patterns: 12.1 s a round against 17.0 on clusters of 8).
+    if (vk == 1 && (v.empty() || v[0].h.kp > 1)) {
         const Shape h{Geo{vt, 1, 1}, 1, vt, 0};
-        v.push_back({h, std::max(fit(h), c.sm_count), J});
+        v.insert(v.begin(), {h, std::max(fit(h), c.sm_count), prec == PT_PREC_FP64 ? (8 * J + 4) / 5 : (5 * J + 1) / 2});
     }
     return v;
 }
@@ -562,15 +567,19 @@ std::vector<ShapeFit> shapes_of(Ctx& c, bool full, int prec, int C, int maxN, in
 // at 7 sites: 84.8 ms as 8 CTAs of 256 (36 resident), 69.1 as 8 of 128 (51 resident).
 // Warps of an SM slow each other a little while there is room for all of them at once:
 // 8 full visits of 8 taxa at 256 patterns take 6.50 ms as 4 CTAs of 256 each and 6.00 as 8
-// of 128 on twice the SMs. Past one round the resident count says what a shape delivers.
+// of 128 on twice the SMs. Past one round the resident count says what a shape delivers,
+// but for FP64: its pipe is what the warps of an SM share, so a second CTA there brings
+// little (2304 proposals at 878 patterns: 63.7 ms on 8 warps, 68.5 as pairs on 16).
 const ShapeFit& pick_shape(const Ctx& c, const std::vector<ShapeFit>& v, long long total) {
     size_t best = 0;
     double cost = 1e300;
     for (size_t i = 0; i < v.size(); ++i) {
         const long long ctas = total * v[i].h.kp;
         const double rounds = (double)ctas / v[i].resident;
-        const double warps = rounds < 1 ? (double)((ctas + c.sm_count - 1) / c.sm_count) * v[i].h.pt / 32 : 16;
-        const double x = std::max(1.0, rounds) * (5 + v[i].sites) * (1 + 0.02 * warps);
+        const bool fp64 = c.cfg.precision == PT_PREC_FP64;
+        const long long on = (std::min<long long>(ctas, v[i].resident) + c.sm_count - 1) / c.sm_count;
+        const double warps = rounds < 1 || fp64 ? (double)on * v[i].h.pt / 32 : 16;
+        const double x = std::max(1.0, rounds) * (5 + v[i].sites) * (1 + (fp64 ? 0.1 : 0.02) * warps);
         if (x < 0.999 * cost) {
             cost = x;
             best = i;
