@@ -552,7 +552,7 @@ std::vector<ShapeFit> shapes_of(Ctx& c, bool full, int prec, int C, int maxN, in
     // The sum-table of one CTA in global memory, where it is too large for its shared
     // memory: a site costs more (in FP64, whose arithmetic hides part of the reads, 1.6
     // times, in FP32 2.5 times), but many items need no cluster each (an FP64 round at
-    // 128 taxa x 5908 patterns: 12.1 s a round against 17.0 on clusters of 8).
+    // 128 taxa x 5908 patterns: 11.8 s a round against 17.0 on clusters of 8).
     if (vk == 1 && (v.empty() || v[0].h.kp > 1)) {
         const Shape h{Geo{vt, 1, 1}, 1, vt, 0};
         v.insert(v.begin(), {h, std::max(fit(h), c.sm_count), prec == PT_PREC_FP64 ? (8 * J + 4) / 5 : (5 * J + 1) / 2});
@@ -566,10 +566,11 @@ std::vector<ShapeFit> shapes_of(Ctx& c, bool full, int prec, int C, int maxN, in
 // each, 19.1 on 2, 13.1 on 4 (1.1 rounds), 18.2 on 8 (2.3 rounds); on 5697 neighbours
 // at 7 sites: 84.8 ms as 8 CTAs of 256 (36 resident), 69.1 as 8 of 128 (51 resident).
 // Warps of an SM slow each other a little while there is room for all of them at once:
-// 8 full visits of 8 taxa at 256 patterns take 6.50 ms as 4 CTAs of 256 each and 6.00 as 8
+// 8 full visits of 27 taxa at 816 patterns take 6.50 ms as 4 CTAs of 256 each and 6.00 as 8
 // of 128 on twice the SMs. Past one round the resident count says what a shape delivers,
 // but for FP64: its pipe is what the warps of an SM share, so a second CTA there brings
-// little (2304 proposals at 878 patterns: 63.7 ms on 8 warps, 68.5 as pairs on 16).
+// little (2304 proposals at 878 patterns: 63.3 ms on 8 warps, 68.5 as pairs on 16). With
+// 0.1 a warp in place of 0.06, 48 full visits at 878 patterns took 21.6 ms, not 16.8.
 const ShapeFit& pick_shape(const Ctx& c, const std::vector<ShapeFit>& v, long long total) {
     size_t best = 0;
     double cost = 1e300;
@@ -579,7 +580,7 @@ const ShapeFit& pick_shape(const Ctx& c, const std::vector<ShapeFit>& v, long lo
         const bool fp64 = c.cfg.precision == PT_PREC_FP64;
         const long long on = (std::min<long long>(ctas, v[i].resident) + c.sm_count - 1) / c.sm_count;
         const double warps = rounds < 1 || fp64 ? (double)on * v[i].h.pt / 32 : 16;
-        const double x = std::max(1.0, rounds) * (5 + v[i].sites) * (1 + (fp64 ? 0.1 : 0.02) * warps);
+        const double x = std::max(1.0, rounds) * (5 + v[i].sites) * (1 + (fp64 ? 0.06 : 0.02) * warps);
         if (x < 0.999 * cost) {
             cost = x;
             best = i;

@@ -11,10 +11,10 @@
 // D_v (the subtree below inner node v, at v) for every inner v, then U_v (the
 // rest of the tree, at v's parent) for every inner v but the first.
 //
-// Parallel structure: a thread owns sites; a CTA owns a tree (partials, full
-// optimisation) or one NNI neighbour (proposal optimisation).  Cross-thread
-// traffic is only the per-Newton-iteration reduction of d lnL/dt and
-// d2 lnL/dt2 (FP64) and the per-sweep lnL, so every pass over sites runs
+// Parallel structure: a lane owns sites; a CTA or a cluster of up to eight owns a tree
+// (full optimisation) or one NNI neighbour (proposal optimisation), as the number of
+// items leaves room for.  Cross-thread traffic is only the per-evaluation reduction of
+// d lnL/dt and d2 lnL/dt2 (FP32 pairs, or FP64) and the scores, so every pass over sites runs
 // without barriers.
 #include "pt_internal.h"
 #include "pt_gamma.h"
