@@ -1358,13 +1358,13 @@ template <typename R, int C>
 struct STab {
     R* s;          // [nchunk][pcap] vec
     R* w;          // [pcap] site weights, set once per item
-    R* e;          // [pcap] exponents (FP64)
+    int* e;        // [pcap] exponents (FP64)
     int pcap;
     __device__ __forceinline__ void init(unsigned char* base, int ld) {
         pcap = (ld + 3) & ~3;
         s = reinterpret_cast<R*>(base);
         w = s + (size_t)4 * C * pcap;
-        e = w + pcap;
+        e = reinterpret_cast<int*>(w + pcap);
     }
     __device__ __forceinline__ void put(int p, const R* v, int E) const {
         if constexpr (sizeof(R) == 4) {
@@ -1375,7 +1375,7 @@ struct STab {
 #pragma unroll
             for (int q = 0; q < 2 * C; ++q)
                 reinterpret_cast<double2*>(s)[(size_t)q * pcap + p] = make_double2(v[2 * q], v[2 * q + 1]);
-            e[p] = (R)E;
+            e[p] = E;
         }
     }
     __device__ __forceinline__ void get(int p, R* v) const {
@@ -1774,7 +1774,7 @@ __device__ double eval_lnl(const STab<double, C>& st, const Sites& sx, double t,
                 const int q = (z & 3) * C + (z >> 2);  // categories outermost
                 L = fma(e[q], s[q], L);
             }
-            term = __dmul_rn(st.w[pl], log(L) + st.e[pl] * kLn2);
+            term = __dmul_rn(st.w[pl], log(L) + (double)st.e[pl] * kLn2);
         }
         add_score(acc, term, sx.lanes);
     }
@@ -3242,10 +3242,12 @@ void launch_lengths_to_input(cudaStream_t s, int n, int count, TreeSet ts, doubl
     ++g_launches;
 }
 
-// Sum-table of ld local sites: 4C values, the weight and (FP64) the exponent of each.
+// Sum-table of ld local sites: 4C values, the weight and (FP64) the exponent of each, the
+// exponent as the 32-bit integer that it is: with 8 bytes for it, the shared memory that
+// the launch takes beside the table left room for 1532 patterns of 128 taxa, now for 1576.
 size_t sumtable_bytes(int prec, int C, int ld) {
     const size_t pcap = (size_t)((ld + 3) & ~3);
-    return prec == 0 ? (4 * (size_t)C + 2) * 8 * pcap : (4 * (size_t)C + 1) * 4 * pcap;
+    return prec == 0 ? ((4 * (size_t)C + 1) * 8 + 4) * pcap : (4 * (size_t)C + 1) * 4 * pcap;
 }
 
 namespace {

@@ -6,6 +6,7 @@ from __future__ import annotations
 import numpy as np
 import pytest
 
+import oracle
 from paper_1811_11007_gb300 import pt, synth
 
 pytestmark = pytest.mark.gpu
@@ -59,3 +60,27 @@ def test_proposals_are_shape_independent(prec, n, sites, ncat):
             both = set(few) & set(many)
             assert len(both) >= len(few) // 2  # the others have another proposer in the larger round
             assert all(few[x] == many[x] for x in both)
+
+
+@pytest.mark.parametrize("P", [1545, 1555])
+def test_noalloc_at_its_array_limit(P):
+    """84 taxa in FP64: one tree's vectors fill the fixed array, so the sum-table has to fit in shared memory.
+    Tolerance: P * 2^-52 * |lnL| of summation and about 1e3 * 2^-52 a site, below 1e-12 of |lnL|."""
+    torch = pytest.importorskip("torch")
+    n, dev = 84, torch.device("cuda", 0)
+    tips = np.random.default_rng(P).integers(0, 4, (n, P)).astype(np.uint8)
+    w = np.ones(P, np.int32)
+    e, _ = synth.random_trees(n, 1, 3)
+    l = np.full((1, 2 * n - 3), 0.1)
+    exch, freqs = np.array([1.0, 2.0, 0.7, 1.1, 2.5, 1.0]), np.array([0.3, 0.2, 0.2, 0.3])
+    want = oracle.Problem(tips, w, exch, freqs, 0.5, 4).loglik(e[0], l[0])
+    cfg = pt.default_config()
+    cfg.precision = pt.PREC_FP64
+    t = [torch.from_numpy(np.ascontiguousarray(x)).to(dev) for x in (tips, w, e, l)]
+    o_len, o_lnl = torch.empty_like(t[3]), torch.empty(1, dtype=torch.float64, device=dev)
+    st = pt.score_noalloc(n, P, t[0].data_ptr(), t[1].data_ptr(), exch, freqs, 0.5, 4, 1, t[2].data_ptr(),
+                          t[3].data_ptr(), o_len.data_ptr(), o_lnl.data_ptr(), mode="fixed",
+                          stream=torch.cuda.current_stream().cuda_stream, cfg=cfg)
+    assert st == 0
+    torch.cuda.synchronize()
+    np.testing.assert_allclose(o_lnl.item(), want, rtol=1e-12)
