@@ -541,9 +541,8 @@ std::vector<ShapeFit> shapes_of(Ctx& c, bool full, int prec, int C, int maxN, in
     const int J = (cluster_sites(maxP, vk) + vt - 1) / vt;  // sites per virtual thread
     for (int kp : {1, 2, 4, 8})
         for (int pt : {vt, vt / 2}) {
-            const int lanes = kp * pt / (vk * vt);
-            if (pt < 128 && pt != vt) continue;
-            if (lanes < 1 || kp * pt != vk * vt * lanes || (lanes > 1 && lanes >= 2 * J) || (kp == 1 && pt != vt)) continue;
+            const int lanes = shape_lanes(vt, vk, kp, pt, J);
+            if (lanes == 0) continue;
             const Shape h{Geo{vt, vk, lanes}, kp, pt, 1};
             const int r = fit(h);
             if (r >= kp) v.push_back({h, r, (J + lanes - 1) / lanes});

@@ -140,6 +140,17 @@ struct Shape {
     Geo geo;
     int kp, pt, smem_tab;
 };
+// Lanes per virtual thread when kp CTAs of pt threads carry vk shares of vt virtual
+// threads with J sites each; 0 where that is no shape.  CTAs are whole warps (half of a
+// configured size of 288 is not, and a warp's sums would take values from absent lanes)
+// of at least 128 threads unless the geometry's are smaller, and on average more than
+// half of the lanes have a site.
+PT_INLINE int shape_lanes(int vt, int vk, int kp, int pt, int J) {
+    const int lanes = kp * pt / (vk * vt);
+    if (pt % 32 != 0 || (pt < 128 && pt != vt) || (kp == 1 && pt != vt)) return 0;
+    if (lanes < 1 || kp * pt != vk * vt * lanes || (lanes > 1 && lanes >= 2 * J)) return 0;
+    return lanes;
+}
 // Local sites of one CTA of `threads` threads (its sum-table's and slab's capacity).
 PT_INLINE int geo_local(int P, const Geo& g, int threads) {
     const int Ps = cluster_sites(P, g.vk), step = g.vt * g.lanes;
