@@ -66,59 +66,67 @@ __device__ __forceinline__ void canon_tree(int n, int tree, int lane, const int3
             const double x = lengths[(size_t)tree * E + e];
             if (!(x >= 0.0 && x <= 1.7976931348623157e308)) atomicCAS(&err[kErrLen], 0, tree + 1);
         }
-    bool ok = true;
-    for (int v = lane; v < NN; v += 32) {
-        s.deg[v] = 0;
-        s.par[v] = -2;
-    }
-    if (lane == 0) s.tail = 1;
-    __syncwarp();
-    for (int e = lane; e < E; e += 32) {
-        const int a = ed[2 * e], b = ed[2 * e + 1];
-        if (a < 0 || b < 0 || a >= NN || b >= NN || a == b) { ok = false; continue; }
-        const int i = atomicAdd(&s.deg[a], 1), j = atomicAdd(&s.deg[b], 1);
-        if (i < 3) s.nbr[a][i] = (int16_t)b;
-        if (j < 3) s.nbr[b][j] = (int16_t)a;
-    }
-    __syncwarp();
-    for (int v = lane; v < NN; v += 32) ok = ok && s.deg[v] == (v < n ? 1 : 3);
-    ok = __all_sync(all, ok);
-    int levels = 0;
-    if (ok) {
-        if (lane == 0) {
-            s.par[0] = -1;
-            s.order[0] = 0;
-            s.lev[0] = 0;
+    // An edge list that is no tree is flagged and gets the key 0, which no tree has; a
+    // caterpillar takes its place, as kernels queued behind this one follow its arrays
+    // before the host reads the flag.
+    bool bad = false;
+    auto edge = [&](int e, int& a, int& b) {
+        if (!bad) { a = ed[2 * e]; b = ed[2 * e + 1]; return; }
+        a = e;
+        b = e >= n ? e + 1 : e == 0 ? n : e == n - 1 ? NN - 1 : n + e - 1;
+    };
+    int levels;
+    while (true) {
+        bool ok = true;
+        for (int v = lane; v < NN; v += 32) {
+            s.deg[v] = 0;
+            s.par[v] = -2;
+        }
+        if (lane == 0) s.tail = 1;
+        __syncwarp();
+        for (int e = lane; e < E; e += 32) {
+            int a, b;
+            edge(e, a, b);
+            if (a < 0 || b < 0 || a >= NN || b >= NN || a == b) { ok = false; continue; }
+            const int i = atomicAdd(&s.deg[a], 1), j = atomicAdd(&s.deg[b], 1);
+            if (i < 3) s.nbr[a][i] = (int16_t)b;
+            if (j < 3) s.nbr[b][j] = (int16_t)a;
         }
         __syncwarp();
-        for (int lo = 0, hi = 1; lo < hi && ok; ++levels) {
-            for (int i = lo + lane; i < hi; i += 32) {
-                const int v = s.order[i], pv = s.par[v];
-                for (int k = 0; k < (v < n ? 1 : 3); ++k) {
-                    const int c = s.nbr[v][k];
-                    if (c == pv) continue;
-                    if (atomicCAS(&s.par[c], -2, v) != -2) ok = false;  // a cycle
-                    else s.order[atomicAdd(&s.tail, 1)] = (int16_t)c;
-                }
+        for (int v = lane; v < NN; v += 32) ok = ok && s.deg[v] == (v < n ? 1 : 3);
+        ok = __all_sync(all, ok);
+        levels = 0;
+        if (ok) {
+            if (lane == 0) {
+                s.par[0] = -1;
+                s.order[0] = 0;
+                s.lev[0] = 0;
             }
-            ok = __all_sync(all, ok);
             __syncwarp();
-            lo = hi;
-            hi = s.tail;
-            if (lane == 0) s.lev[levels + 1] = (int16_t)lo;
-            __syncwarp();  // every lane has read the tail before a lane of the next level moves it
+            for (int lo = 0, hi = 1; lo < hi && ok; ++levels) {
+                for (int i = lo + lane; i < hi; i += 32) {
+                    const int v = s.order[i], pv = s.par[v];
+                    for (int k = 0; k < (v < n ? 1 : 3); ++k) {
+                        const int c = s.nbr[v][k];
+                        if (c == pv) continue;
+                        if (atomicCAS(&s.par[c], -2, v) != -2) ok = false;  // a cycle
+                        else s.order[atomicAdd(&s.tail, 1)] = (int16_t)c;
+                    }
+                }
+                ok = __all_sync(all, ok);
+                __syncwarp();
+                lo = hi;
+                hi = s.tail;
+                if (lane == 0) s.lev[levels + 1] = (int16_t)lo;
+                __syncwarp();  // every lane has read the tail before a lane of the next level moves it
+            }
+            ok = ok && s.tail == NN;
         }
-        ok = ok && s.tail == NN;
+        __syncwarp();
+        if (ok || bad) break;
+        bad = true;
+        if (lane == 0) atomicCAS(&err[kErrTree], 0, tree + 1);
     }
-    if (!ok) {
-        if (lane == 0) {
-            atomicCAS(&err[kErrTree], 0, tree + 1);
-            ts.key[2 * tree] = 0;
-            ts.key[2 * tree + 1] = 0;
-        }
-        return;
-    }
-    __syncwarp();
     for (int l = levels - 1; l >= 0; --l) {  // upward
         for (int i = s.lev[l] + lane; i < s.lev[l + 1]; i += 32) {
             const int v = s.order[i];
@@ -173,8 +181,10 @@ __device__ __forceinline__ void canon_tree(int n, int tree, int lane, const int3
     }
     if (lane == 0) len[0] = 0.0;
     for (int e = lane; e < E; e += 32) {
-        const int a = ed[2 * e], b = ed[2 * e + 1], c = s.canon[s.par[a] == b ? a : b];
-        len[c] = lengths ? lengths[(size_t)tree * E + e] : 0.1;
+        int a, b;
+        edge(e, a, b);
+        const int c = s.canon[s.par[a] == b ? a : b];
+        len[c] = lengths && !bad ? lengths[(size_t)tree * E + e] : 0.1;
         if (ts.emap) ts.emap[(size_t)tree * E + e] = c;
     }
     // key = sum of split hashes over internal edges (inner nodes except the first)
@@ -192,8 +202,8 @@ __device__ __forceinline__ void canon_tree(int n, int tree, int lane, const int3
     }
     if (lane == 0) {
         if (lo == 0 && hi == 0) lo = 1;
-        ts.key[2 * tree] = lo;
-        ts.key[2 * tree + 1] = hi;
+        ts.key[2 * tree] = bad ? 0 : lo;
+        ts.key[2 * tree + 1] = bad ? 0 : hi;
     }
     // rank of every internal split among the tree's internal splits
     for (int v = lane; v < NN; v += 32) {

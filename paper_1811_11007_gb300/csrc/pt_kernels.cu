@@ -149,7 +149,9 @@ __global__ void k_cand_insert(Slot* tab, int log2, DCount nc, const uint64_t* __
     const int ncand = dcount(nc), round = dround(rd);
     int dup = 0;
     if (i >= ncand && i < nc.cap) { cslot[i] = -1; flag[i] = 0; }  // past the device count
-    if (i < ncand) {
+    if (i < ncand && !(fr.key[2 * cinfo[4 * i]] | fr.key[2 * cinfo[4 * i] + 1])) {  // a refused tree proposes nothing
+        cslot[i] = -1; flag[i] = 0;
+    } else if (i < ncand) {
         bool created;
         long long s = table_find_or_claim(tab, log2, nkey[2 * i], nkey[2 * i + 1], &created);
         if (s < 0) {
@@ -254,6 +256,7 @@ __global__ void k_insert_trees(Slot* tab, int log2, DCount cnt, TreeSet ts, cons
                                int32_t* winner, int32_t* err) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= dcount(cnt)) return;
+    if (!(ts.key[2 * i] | ts.key[2 * i + 1])) { winner[i] = -1; return; }  // a refused tree
     bool created;
     long long s = table_find_or_claim(tab, log2, ts.key[2 * i], ts.key[2 * i + 1], &created);
     if (s < 0) { atomicExch(&err[kErrTable], 1); winner[i] = -1; return; }

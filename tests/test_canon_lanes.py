@@ -95,3 +95,28 @@ def test_canonical_form_does_not_depend_on_lane_order(canon, n):
             got = canon(n, e, l, order)
             for x in want:
                 np.testing.assert_array_equal(got[x], want[x], err_msg="%s, lane order %d" % (x, order))
+
+
+# edge lists that are no trees; the last three have a tree's degrees
+BAD = {
+    "self-loop": (5, [(0, 5), (1, 5), (5, 5), (2, 6), (6, 7), (3, 7), (4, 7)]),
+    "node out of range": (4, [(0, 4), (1, 4), (4, 5), (2, 5), (3, 6)]),
+    "negative node": (4, [(0, 4), (1, 4), (4, 5), (2, 5), (3, -1)]),
+    "leaf of degree two": (5, [(0, 5), (1, 5), (5, 6), (2, 6), (6, 7), (3, 7), (3, 4)]),
+    "cycle beside leaf 0's part": (6, [(0, 6), (1, 6), (2, 6), (3, 7), (4, 8), (5, 9), (7, 8), (8, 9), (9, 7)]),
+    "cycle in leaf 0's part": (6, [(3, 6), (4, 6), (5, 6), (0, 7), (1, 8), (2, 9), (7, 8), (8, 9), (9, 7)]),
+    "double edge in leaf 0's part": (5, [(2, 5), (3, 5), (4, 5), (6, 7), (7, 6), (0, 6), (1, 7)]),
+}
+
+
+@pytest.mark.parametrize("what", sorted(BAD))
+def test_a_list_that_is_no_tree_leaves_a_tree_behind(canon, what):
+    """Flagged, with the key 0, and with arrays that every later kernel can follow: a caterpillar's."""
+    n, e = BAD[what]
+    want = _expect(n, _caterpillar(n), np.full(2 * n - 3, 0.1))
+    want["key"][:] = 0
+    want["err"][0] = 1  # tree index + 1
+    for order in (0, 1, 2, 3):
+        got = canon(n, e, np.full(2 * n - 3, 0.3), order)
+        for x in want:
+            np.testing.assert_array_equal(got[x], want[x], err_msg=x)
