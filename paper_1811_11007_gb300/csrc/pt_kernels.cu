@@ -26,6 +26,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <cfloat>
 #include <cmath>
 #include <cstdint>
 #include <type_traits>
@@ -1282,8 +1283,10 @@ __device__ __forceinline__ void cluster_exchange_init(NS& ns) {
 template <typename R> struct LenOf { using T = double; };
 template <> struct LenOf<float> { using T = F2; };
 template <typename R> using Len = typename LenOf<R>::T;
+// A length past FP32's range (accepted, as every finite one) becomes its largest number: the
+// pair of an infinity has no difference from the solved length, and the move went unnoticed.
 template <typename R> __device__ __forceinline__ Len<R> len_of(double x) {
-    if constexpr (sizeof(R) == 4) return f2_of(x);
+    if constexpr (sizeof(R) == 4) return f2_of(fmin(x, (double)FLT_MAX));
     else return x;
 }
 __device__ __forceinline__ double len_dbl(F2 x) { return (double)x.h + (double)x.l; }
