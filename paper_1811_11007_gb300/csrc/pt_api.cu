@@ -706,7 +706,7 @@ struct FullJob {
 // Runs full-optimisation jobs in one persistent launch over all of them.  The
 // partials live in per-CTA slabs (a CTA reuses its slab tree after tree), so
 // memory grows with the grid, not with the number of trees.
-void run_full_jobs(Ctx& c, std::vector<FullJob> jobs, bool allow_tune = true) {
+void run_full_jobs(Ctx& c, std::vector<FullJob> jobs) {
     const int prec = c.cfg.precision;
     jobs.erase(std::remove_if(jobs.begin(), jobs.end(), [](const FullJob& j) { return j.count <= 0; }), jobs.end());
     if (jobs.empty()) return;
@@ -790,9 +790,10 @@ void run_full_jobs(Ctx& c, std::vector<FullJob> jobs, bool allow_tune = true) {
             if (it->second.full_cluster) K = it->second.full_cluster;
         }
         // tune on launches with enough trees to fill the GPU, and again when a
-        // launch is much larger than the one the bucket was tuned on
+        // launch is much larger than the one the bucket was tuned on; scores at given
+        // lengths run no Newton solve, so they time nothing that a shape changes
         const bool big = total >= 2 * c.sm_count && (!have || total >= 4 * it->second.full_items);
-        if (allow_tune && c.autotune && big) {
+        if (c.autotune && big && jobs[0].max_sweeps > 0) {
             // the kernel writes the optimised lengths back: trials start from a saved copy
             std::vector<std::pair<double*, size_t>> ranges;
             size_t nlen = 0;
@@ -897,7 +898,7 @@ void visit_jobs(Ctx& c, std::vector<FullJob> jobs, std::vector<std::vector<doubl
     auto eval = [&](const std::vector<double>& u, std::vector<double>& f) {  // lnL at shapes exp(u), fixed lengths
         for (size_t t = 0; t < T; ++t) h_alpha[t] = std::exp(u[t]);
         set_rates(h_alpha);
-        run_full_jobs(c, fixed, false);
+        run_full_jobs(c, fixed);
         ck(c, cudaMemcpyAsync(hf.data(), d_f, 8 * T, cudaMemcpyDeviceToHost, c.stream), "lnL");
         ck(c, cudaStreamSynchronize(c.stream), "sync");
         f = hf;
