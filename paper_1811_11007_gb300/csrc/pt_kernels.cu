@@ -1302,7 +1302,7 @@ struct NewtonSmem {
     double ex[4 * C];      // exp(lam_k r t) for a P-matrix refresh
     Exp2Tab et;
     F2 lrp[4 * C];         // lr as pairs (mixed precision)
-    F2 Wp[64];             // W as pairs
+    F2 Wp[64];             // W as pairs; [.][0].h: the entry's p_entry_base
     F2 em[4 * C];          // exp(lam_k r t) - 1 for a P-matrix refresh from pairs
     float lr_min;          // the smallest |lr| but the zero ones
     double W[64];          // W[(i*4+j)*4+k] = isqpi_i sqpi_j R_ik R_jk: P_ij = sum_k W_ijk exp(lam_k r t)
@@ -1373,8 +1373,16 @@ __device__ __forceinline__ void init_newton_smem(const Model& M, const Cfg& cfg,
                                                  const double* rates) {
     for (int x = threadIdx.x; x < 64; x += blockDim.x) {
         int k = x & 3, ij = x >> 2, i = ij >> 2, j = ij & 3;
-        ns.W[x] = M.isqpi[i] * M.sqpi[j] * M.R[i * 4 + k] * M.R[j * 4 + k];
-        if (sizeof(R) == 4) ns.Wp[x] = f2_of(ns.W[x]);
+        auto W = [&](int q) { return M.isqpi[i] * M.sqpi[j] * M.R[i * 4 + q] * M.R[j * 4 + q]; };
+        ns.W[x] = W(k);
+        if (sizeof(R) == 4) {
+            if (k == 0) {
+                const double Wij[4] = {W(0), W(1), W(2), W(3)};
+                ns.Wp[x] = F2{p_entry_base(i == j ? 1.0 : 0.0, Wij), 0.f};
+            } else {
+                ns.Wp[x] = f2_of(W(k));
+            }
+        }
     }
     if (threadIdx.x == 0) {
         // Leader warp: FP64 instructions issue slowly and only on the issuing warp's
@@ -1837,7 +1845,8 @@ __device__ __forceinline__ void newton_solve(const Cfg& cfg, const STab<R, C>& s
                 for (int x = threadIdx.x; x < 16 * C; x += blockDim.x) {
                     const int r = x % C, ij = x / C;
                     bool ok;
-                    Pdst[x] = p_entry_pair(ij % 5 == 0 ? 1.f : 0.f, ns.Wp + ij * 4, ns.em + r, C, ok);
+                    const F2* const Wk = ns.Wp + ij * 4;
+                    Pdst[x] = p_entry_pair(ij % 5 == 0 ? 1.f : 0.f, Wk, ns.em + r, C, ok, Wk[0].h);
                     sure = sure && ok;
                 }
                 if (!__syncthreads_or(!sure)) break;

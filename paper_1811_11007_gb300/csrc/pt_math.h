@@ -93,9 +93,13 @@ __device__ __forceinline__ F2 expm1_pair(F2 x, const Exp2Tab& tab) {
 // One entry of P(t) = I + sum_{k=1..3} W_k (exp(lam_k r t) - 1), rounded to FP32, from
 // the pairs W_k (w[1..3]) and em_k = expm1(lam_k r t) (em[k * stride]).  certain: the
 // rounding is that of the FP64 sum W_0 + sum W_k exp(lam_k r t) (Ziv's test: both ends
-// of the error interval round alike; the pairs' error is below 2^-42 of the terms and
-// the FP64 sum's own below 2^-48).
-__device__ __forceinline__ float p_entry_pair(float delta, const F2* w, const F2* em, int stride, bool& certain) {
+// of the error interval round alike).  Half-width of the interval, with u = 2^-24 and mag
+// the sum of |W_k em_k|: the pairs W_k and em_k are good to a few 2^-47 and the sums here
+// to 33 u^2, together below 2^-42 of mag; beside delta = 1 the sums lose up to 12 u^2
+// more; and base is how far the FP64 sum may lie from the exact one (p_entry_base; the
+// default holds where the W_k miss delta by at most 2^-49 and sum to less than one).
+__device__ __forceinline__ float p_entry_pair(float delta, const F2* w, const F2* em, int stride, bool& certain,
+                                              float base = 0x1p-48f) {
     float s = delta, c = 0.f, mag = 0.f;
 #pragma unroll
     for (int k = 1; k < 4; ++k) {
@@ -107,10 +111,19 @@ __device__ __forceinline__ float p_entry_pair(float delta, const F2* w, const F2
         c = __fadd_rn(c, __fadd_rn(t.l, pe));
         mag = __fadd_rn(mag, fabsf(p));
     }
-    const float eps = __fmaf_rn(mag, 0x1p-42f, 0x1p-48f);
+    const float eps = __fmaf_rn(mag, 0x1p-42f, __fmaf_rn(delta, 0x1.8p-45f, base));
     const float a = __fadd_rn(s, __fsub_rn(c, eps)), b = __fadd_rn(s, __fadd_rn(c, eps));
     certain = a == b;
     return a;
+}
+// The base of p_entry_pair for an entry's W_0..3: what the W_k miss delta by (they are
+// rounded products of eigenvectors, scaled by sqrt(pi_j / pi_i): 6e-15 at mild
+// frequencies, 2e-13 at frequencies of 1e-3), and the rounding of the FP64 sum, of its
+// exponentials and of this difference, below 9 * 2^-53 of the sum of |W_k|.
+__device__ __forceinline__ float p_entry_base(double delta, const double* W) {
+    const double miss = fabs(((W[0] + W[1]) + W[2]) + W[3] - delta);
+    const double all = (fabs(W[0]) + fabs(W[1])) + (fabs(W[2]) + fabs(W[3]));
+    return __double2float_ru(fma(all, 0x1p-49, miss));
 }
 
 }  // namespace pt
