@@ -1883,8 +1883,10 @@ GraphRound* graph_create(Ctx& c, const std::vector<int>& ids, const std::vector<
         if (tt->second.full_threads) g.full_threads = tt->second.full_threads;
         if (tt->second.full_cluster) g.full_cluster = tt->second.full_cluster;
     }
-    const std::vector<ShapeRange>
-        ps = shape_ranges(c, shapes_of(c, false, prec, C, 3, maxP, g.prop_threads, g.prop_cluster), totCap),
+    const std::vector<ShapeRange> ps =
+        shape_ranges(c, shapes_of(c, false, prec, C, 3, maxP, g.prop_threads, g.prop_cluster), totCap);
+    std::vector<ShapeRange> fs;  // none where a visit is its score (no sweeps, mixed precision)
+    if (prec == PT_PREC_FP64 || c.cfg.full_max_sweeps > 0)
         fs = shape_ranges(c, shapes_of(c, true, prec, C, maxN, maxP, g.full_threads, g.full_cluster), totCap);
     const size_t tabb = (sumtable_bytes(prec, C, maxP) + 255) & ~size_t(255);
     size_t pscratch = 0, fscratch = 0, slab = 0;
