@@ -64,3 +64,27 @@ def test_large_problems_do_not_depend_on_the_shape(prec, threads):
         ctx.set_model(aid, a.exch, a.freqs, 0.5, 4)
         assert ctx.alignment_info(aid)[1] > 3500  # 68 bytes a pattern in FP32
         _check(ctx, aid, e, l, (1, 4, 19))
+
+
+@pytest.mark.parametrize("prec", ["mixed", "fp64"])
+def test_a_recorded_round_is_the_same_at_every_count(prec):
+    """A recorded round issues one launch per shape and the counts decide which one runs: frontiers
+    from one tree (every CTA on few items) to more neighbours than the GPU holds at once."""
+    n, most = 14, 40
+    a, e, l = _case(n, 900, most, 0.1)
+    with pt.Context(precision=prec, table_log2=16, full_max_sweeps=2, prop_max_sweeps=2) as ctx:
+        aid = ctx.load_alignment(a.codes)
+        ctx.set_model(aid, a.exch, a.freqs, 0.5, 4)
+        g = ctx.graph([aid], [most], [np.inf])  # every neighbour is kept and visited
+        try:
+            for k in (1, 2, 3, 5, 8, 13, 22, most):
+                ctx.reset_visited(aid)
+                lm, _ = g.run([g.set_frontier(0, e[:k], l[:k])], [-1e300])
+                got = {x: np.array(v) for x, v in g.next(0).items()}
+                ctx.reset_visited(aid)
+                lm2, want = ctx.expand(aid, e[:k], l[:k], np.inf, -1e300)
+                assert lm[0] == lm2 and len(want["keys"]) >= k
+                for x in want:
+                    np.testing.assert_array_equal(got[x], want[x])
+        finally:
+            g.close()
