@@ -26,7 +26,8 @@ def _stale(obj: str, deps: list[str]) -> bool:
 
 def build(force: bool = False, verbose: bool = False) -> str:
     os.makedirs(OUT_DIR, exist_ok=True)
-    headers = [os.path.join(CSRC, h) for h in ("pt_internal.h", "pt_canon.h", "pt_gamma.h", "pt_math.h")]
+    headers = [os.path.join(CSRC, h) for h in ("pt_internal.h", "pt_canon.h", "pt_exchange.h", "pt_gamma.h",
+                                                "pt_math.h")]
     headers.append(os.path.join(ROOT, "include", "pt.h"))
     procs, objs = [], []
     for src in SOURCES:

@@ -18,6 +18,7 @@
 // without barriers.
 #include "pt_internal.h"
 #include "pt_canon.h"
+#include "pt_exchange.h"
 #include "pt_gamma.h"
 #include "pt_math.h"
 
@@ -1209,52 +1210,6 @@ struct STab {
 // Warps of one thread-block cluster whose Newton sums one CTA receives (CTAs x
 // warps per CTA); launch shapes above it are not offered.
 constexpr int kMaxClusterWarps = kMaxTeamWarps;
-// A CTA gives up waiting for its cluster's Newton sums after this many cycles
-// (about 2 s); the kernel then reports PT_ERR_TIMEOUT through its statistics.
-constexpr long long kExchangeWaitCycles = 1ll << 32;
-
-// mbarrier and cluster-push primitives (PTX).  A push st.async's 16 bytes into
-// the same variable of another CTA `rank` of the cluster and completes 16 bytes
-// of the transaction count of that CTA's barrier; a CTA's own warps store their
-// entries locally and arrive on the barrier; the receiver arms its barrier with
-// the bytes it expects from the other CTAs and waits on the phase parity.
-__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void mbar_init(unsigned long long* bar, unsigned count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_fence_init() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
-__device__ __forceinline__ void mbar_arrive_expect(unsigned long long* bar, unsigned bytes) {
-    asm volatile(
-        "{\n\t.reg .b64 st;\n\t"
-        "mbarrier.arrive.expect_tx.release.cta.shared::cta.b64 st, [%0], %1;\n\t}" ::"r"(smem_addr(bar)),
-        "r"(bytes)
-        : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(unsigned long long* bar) {
-    asm volatile(
-        "{\n\t.reg .b64 st;\n\t"
-        "mbarrier.arrive.release.cta.shared::cta.b64 st, [%0];\n\t}" ::"r"(smem_addr(bar))
-        : "memory");
-}
-__device__ __forceinline__ bool mbar_test_wait(unsigned long long* bar, unsigned parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(smem_addr(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-__device__ __forceinline__ void cluster_push16(float* dst, unsigned long long* bar, unsigned rank, float4 v) {
-    uint32_t d, b;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(d) : "r"(smem_addr(dst)), "r"(rank));
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(b) : "r"(smem_addr(bar)), "r"(rank));
-    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(d),
-                 "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(b)
-                 : "memory");
-}
 __device__ __forceinline__ unsigned cluster_rank() {
     unsigned r;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
@@ -1316,14 +1271,7 @@ struct NewtonSmem {
     // bytes it received
     alignas(16) float cxr[2][kMaxClusterWarps][4];
     alignas(8) unsigned long long mbx[2];
-    int abort_;            // a wait on mbx ran out: later waits are skipped (reported by the kernel)
-};
-
-// A CTA's place in its cluster (the CTAs that share one item): kp CTAs, and the
-// exchanges made so far (equal in every thread of the cluster).
-struct Team {
-    int kp, rank;
-    int cseq, nseq;
+    int abort_;            // a wait on mbx ran out (reported by the kernel)
 };
 
 // The entries of the binary tree that one warp finishes: entry i of ne at
@@ -1725,145 +1673,110 @@ __device__ __forceinline__ void newton_solve(const Cfg& cfg, const STab<R, C>& s
     __syncthreads();  // the coefficients of newton_begin
     const int ld = ns.leader;
     Len<R> lo = ns.tmin, hi = ns.tmax;
-    bool pairs = false;
-    converged = false;
-    evals = 0;
-    for (int it = 0; it < cfg.newton_maxit; ++it) {
-        const float4 v = sx.lanes == 1   ? site_sums<R, C, 1>(st, sx, ns)
-                         : sx.lanes == 2 ? site_sums<R, C, 2>(st, sx, ns)
-                         : sx.lanes == 4 ? site_sums<R, C, 4>(st, sx, ns)
-                                         : site_sums<R, C, 8>(st, sx, ns);
-        const int xe = tm.nseq++, cs = kClus ? xe & 1 : 0;
-        if constexpr (kClus) {
-            // Slot cs is free in every CTA: a warp pushes exchange xe only after its
-            // CTA's leader received all of exchange xe - 1, which every CTA pushed
-            // after its own leader had read exchange xe - 2 (the last use of cs).
-            // Every lane holds the warp's sums: lane r pushes them to CTA r.
-            float* slot = &ns.cxr[cs][tm.rank * nw + w][0];
-            if (lane == tm.rank) {
-                *reinterpret_cast<float4*>(slot) = v;  // this CTA's own copy
-                mbar_arrive(&ns.mbx[cs]);
-            } else if (lane < tm.kp) {
-                cluster_push16(slot, &ns.mbx[cs], (unsigned)lane, v);
-            }
-            // no block barrier here: only the leader needs the sums
+    auto sums = [&] {
+        return sx.lanes == 1   ? site_sums<R, C, 1>(st, sx, ns)
+               : sx.lanes == 2 ? site_sums<R, C, 2>(st, sx, ns)
+               : sx.lanes == 4 ? site_sums<R, C, 4>(st, sx, ns)
+                               : site_sums<R, C, 8>(st, sx, ns);
+    };
+    auto step = [&](int cs, bool last) {
+        // the rest of the tree over the kp x nw warp entries: every CTA adds the same
+        // numbers in the same order
+        const int ne = tm.kp * nw, per = tree_per(ne);
+        bool done;
+        if constexpr (sizeof(R) == 4) {
+            // FP32 pairs, added by two-sums (~48 bits)
+            auto entry = [&](int k) {
+                const int i = lane * per + k;
+                const float4 q = k < per && i < ne ? *reinterpret_cast<const float4*>(&ns.cxr[cs][i][0])
+                                                   : make_float4(0.f, 0.f, 0.f, 0.f);
+                return Sum2{make_float2(q.x, q.y), make_float2(q.z, q.w)};
+            };
+            Sum2 q = entry(0);
+            if (per > 1) q = sum2_add(q, entry(1));
+            if (per > 2) q = sum2_add(q, sum2_add(entry(2), entry(3)));
+            q = ne > 16 ? sum2_lanes<32>(q) : ne > 8 ? sum2_lanes<16>(q) : ne > 4 ? sum2_lanes<8>(q) : sum2_lanes<4>(q);
+            // the butterfly leaves (h, l) unnormalised (l can reach a sizeable
+            // fraction of h after cancellation): renormalise, so that the
+            // quotient's reciprocal seed is taken from the rounded total
+            // (lanes past ne hold partial sums: lane 0's are taken)
+            F2 d1p = f2_two_sum(__shfl_sync(0xffffffffu, q.h.x, 0), __shfl_sync(0xffffffffu, q.l.x, 0));
+            const F2 d2p = f2_two_sum(__shfl_sync(0xffffffffu, q.h.y, 0), __shfl_sync(0xffffffffu, q.l.y, 0));
+            if (ns.prior.h != 0.f) d1p = f2_sub(d1p, ns.prior);  // MAP: the prior's slope
+            done = newton_step_f2(t, lo, hi, d1p, d2p, ns.tol);
         } else {
-            if (lane == 0) *reinterpret_cast<float4*>(&ns.cxr[0][w][0]) = v;
-            __syncthreads();
-        }
-        ++evals;
-        if (w == ld) {
-            if constexpr (kClus) {
-                // wait (bounded) until the slot holds all kp x nw pushes of this exchange
-                if (lane == 0) mbar_arrive_expect(&ns.mbx[cs], (unsigned)((tm.kp - 1) * nw * 16));
-                bool ok = ns.abort_ != 0;  // after a wait ran out, none is waited for again
-                const long long tw = clock64();
-                while (!ok) {
-                    ok = mbar_test_wait(&ns.mbx[cs], (unsigned)(xe >> 1) & 1u);
-                    if (!ok && clock64() - tw > kExchangeWaitCycles) break;
-                }
-                if (__any_sync(0xffffffffu, !ok) && lane == 0) ns.abort_ = 1;
+            auto entry = [&](int k) {
+                const int i = lane * per + k;
+                return k < per && i < ne ? *reinterpret_cast<const double2*>(&ns.cxr[cs][i][0]) : make_double2(0.0, 0.0);
+            };
+            double2 q = entry(0);
+            if (per > 1) {
+                const double2 x = entry(1), y = entry(2), z = entry(3);
+                q = make_double2((q.x + x.x) + (y.x + z.x), (q.y + x.y) + (y.y + z.y));
             }
-            // the rest of the tree over the kp x nw warp entries: every CTA adds the same
-            // numbers in the same order
-            const int ne = tm.kp * nw, per = tree_per(ne);
-            bool done;
-            if constexpr (sizeof(R) == 4) {
-                // FP32 pairs, added by two-sums (~48 bits)
-                auto entry = [&](int k) {
-                    const int i = lane * per + k;
-                    const float4 q = k < per && i < ne ? *reinterpret_cast<const float4*>(&ns.cxr[cs][i][0])
-                                                       : make_float4(0.f, 0.f, 0.f, 0.f);
-                    return Sum2{make_float2(q.x, q.y), make_float2(q.z, q.w)};
-                };
-                Sum2 q = entry(0);
-                if (per > 1) q = sum2_add(q, entry(1));
-                if (per > 2) q = sum2_add(q, sum2_add(entry(2), entry(3)));
-                q = ne > 16 ? sum2_lanes<32>(q) : ne > 8 ? sum2_lanes<16>(q) : ne > 4 ? sum2_lanes<8>(q) : sum2_lanes<4>(q);
-                // the butterfly leaves (h, l) unnormalised (l can reach a sizeable
-                // fraction of h after cancellation): renormalise, so that the
-                // quotient's reciprocal seed is taken from the rounded total
-                // (lanes past ne hold partial sums: lane 0's are taken)
-                F2 d1p = f2_two_sum(__shfl_sync(0xffffffffu, q.h.x, 0), __shfl_sync(0xffffffffu, q.l.x, 0));
-                const F2 d2p = f2_two_sum(__shfl_sync(0xffffffffu, q.h.y, 0), __shfl_sync(0xffffffffu, q.l.y, 0));
-                if (ns.prior.h != 0.f) d1p = f2_sub(d1p, ns.prior);  // MAP: the prior's slope
-                done = newton_step_f2(t, lo, hi, d1p, d2p, ns.tol);
-            } else {
-                auto entry = [&](int k) {
-                    const int i = lane * per + k;
-                    return k < per && i < ne ? *reinterpret_cast<const double2*>(&ns.cxr[cs][i][0]) : make_double2(0.0, 0.0);
-                };
-                double2 q = entry(0);
-                if (per > 1) {
-                    const double2 x = entry(1), y = entry(2), z = entry(3);
-                    q = make_double2((q.x + x.x) + (y.x + z.x), (q.y + x.y) + (y.y + z.y));
-                }
 #pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    if (o >= ne) break;
-                    q.x += __shfl_xor_sync(0xffffffffu, q.x, o);
-                    q.y += __shfl_xor_sync(0xffffffffu, q.y, o);
-                }
-                double D1 = __shfl_sync(0xffffffffu, q.x, 0);
-                const double D2 = __shfl_sync(0xffffffffu, q.y, 0);
-                if (__double_as_longlong(ns.prior) != 0) D1 -= ns.prior;  // MAP: the prior's slope
-                done = newton_step(t, lo, hi, D1, D2, (float)D2, ns.tol);
+            for (int o = 1; o < 32; o <<= 1) {
+                if (o >= ne) break;
+                q.x += __shfl_xor_sync(0xffffffffu, q.x, o);
+                q.y += __shfl_xor_sync(0xffffffffu, q.y, o);
             }
-            const bool last = done || it + 1 == cfg.newton_maxit;
-            if (!last) {
-                put_egh<C>(t, ns, lane);
-            } else {
-                // for the P matrices below: pairs where their rounding test mostly passes
-                // (off-diagonal entries not tiny), else FP64 exponentials
-                if constexpr (sizeof(R) == 4) {
-                    pairs = t.h * ns.lr_min > kPairMin;
-                    if (pairs && lane < 4 * C) {
-                        const F2 x = f2_mul(ns.lrp[lane], t);
-                        ns.em[lane] = x.h > -80.f ? expm1_pair(x, ns.et) : F2{-1.f, 0.f};
-                    }
-                }
-                if (!pairs && lane < 4 * C) ns.ex[lane] = exp(ns.lr[lane] * len_dbl(t));
-                if (lane == 0) {
-                    bool moved;
-                    if constexpr (sizeof(R) == 4) moved = f2_lt(ns.sweep_tol, f2_abs(f2_sub(t, told)));
-                    else moved = fabs(t - told) > ns.sweep_tol;
-                    if (moved) ns.moved_at = sweep;
-                    *dst = t;
-                }
-            }
-            if (lane == 0) ns.done = last ? (done ? 1 : 2) | (pairs ? 4 : 0) : 0;
+            double D1 = __shfl_sync(0xffffffffu, q.x, 0);
+            const double D2 = __shfl_sync(0xffffffffu, q.y, 0);
+            if (__double_as_longlong(ns.prior) != 0) D1 -= ns.prior;  // MAP: the prior's slope
+            done = newton_step(t, lo, hi, D1, D2, (float)D2, ns.tol);
         }
+        if (!done && !last) {
+            put_egh<C>(t, ns, lane);
+            return 0;
+        }
+        // for the P matrices below: pairs where their rounding test mostly passes
+        // (off-diagonal entries not tiny), else FP64 exponentials
+        bool pairs = false;
+        if constexpr (sizeof(R) == 4) {
+            pairs = t.h * ns.lr_min > kPairMin;
+            if (pairs && lane < 4 * C) {
+                const F2 x = f2_mul(ns.lrp[lane], t);
+                ns.em[lane] = x.h > -80.f ? expm1_pair(x, ns.et) : F2{-1.f, 0.f};
+            }
+        }
+        if (!pairs && lane < 4 * C) ns.ex[lane] = exp(ns.lr[lane] * len_dbl(t));
+        if (lane == 0) {
+            bool moved;
+            if constexpr (sizeof(R) == 4) moved = f2_lt(ns.sweep_tol, f2_abs(f2_sub(t, told)));
+            else moved = fabs(t - told) > ns.sweep_tol;
+            if (moved) ns.moved_at = sweep;
+            *dst = t;
+        }
+        return (done ? 1 : 2) | (pairs ? 4 : 0);
+    };
+    converged = false;
+    evals = newton_evaluations<kClus>(cfg.newton_maxit, w, lane, nw, ld, ns, tm, sums, step);
+    if (kClus && evals == 0) return;  // given up: the length stays
+    // P matrices of the final length, rounded once from FP64 or from pairs to the
+    // same bits (a dependent FP64 instruction takes some 60 cycles, exp() a thousand;
+    // the pairs' chain a third of that)
+    converged = (ns.done & 3) == 1;
+    if (sizeof(R) == 4 && (ns.done & 4)) {
+        bool sure = true;
+        for (int x = threadIdx.x; x < 16 * C; x += blockDim.x) {
+            const int r = x % C, ij = x / C;
+            bool ok;
+            const F2* const Wk = ns.Wp + ij * 4;
+            Pdst[x] = p_entry_pair(ij % 5 == 0 ? 1.f : 0.f, Wk, ns.em + r, C, ok, Wk[0].h);
+            sure = sure && ok;
+        }
+        if (!__syncthreads_or(!sure)) return;
+        if (w == ld && lane < 4 * C) ns.ex[lane] = exp(ns.lr[lane] * len_dbl(t));
         __syncthreads();
-        if (ns.done) {
-            // P matrices of the final length, rounded once from FP64 or from pairs to the
-            // same bits (a dependent FP64 instruction takes some 60 cycles, exp() a thousand;
-            // the pairs' chain a third of that)
-            converged = (ns.done & 3) == 1;
-            bool exact = !(ns.done & 4);
-            if (sizeof(R) == 4 && !exact) {
-                bool sure = true;
-                for (int x = threadIdx.x; x < 16 * C; x += blockDim.x) {
-                    const int r = x % C, ij = x / C;
-                    bool ok;
-                    const F2* const Wk = ns.Wp + ij * 4;
-                    Pdst[x] = p_entry_pair(ij % 5 == 0 ? 1.f : 0.f, Wk, ns.em + r, C, ok, Wk[0].h);
-                    sure = sure && ok;
-                }
-                if (!__syncthreads_or(!sure)) break;
-                if (w == ld && lane < 4 * C) ns.ex[lane] = exp(ns.lr[lane] * len_dbl(t));
-                __syncthreads();
-            }
-            for (int x = threadIdx.x; x < 16 * C; x += blockDim.x) {
-                const int r = x % C, ij = x / C;
-                double acc = ns.W[ij * 4];  // lam_0 = 0
-#pragma unroll
-                for (int k = 1; k < 4; ++k) acc = fma(ns.W[ij * 4 + k], ns.ex[k * C + r], acc);
-                Pdst[x] = (R)acc;
-            }
-            __syncthreads();
-            break;
-        }
     }
+    for (int x = threadIdx.x; x < 16 * C; x += blockDim.x) {
+        const int r = x % C, ij = x / C;
+        double acc = ns.W[ij * 4];  // lam_0 = 0
+#pragma unroll
+        for (int k = 1; k < 4; ++k) acc = fma(ns.W[ij * 4 + k], ns.ex[k * C + r], acc);
+        Pdst[x] = (R)acc;
+    }
+    __syncthreads();
 }
 
 
