@@ -48,8 +48,6 @@ template <> struct Prec<float> {
     static constexpr int kScaleExp = 32;
     __device__ static float thresh() { return 2.3283064365386963e-10f; }   // 2^-32
     __device__ static float mult() { return 4294967296.0f; }                // 2^32
-    __device__ static float ex(float x) { return expf(x); }
-    __device__ static float lg(float x) { return logf(x); }
     __device__ static float rcp(float x) { return rcp_rn(x); }
     __device__ static float mul(float x, float y) { return __fmul_rn(x, y); }  // never part of an FMA
 };
@@ -57,8 +55,6 @@ template <> struct Prec<double> {
     static constexpr int kScaleExp = 256;
     __device__ static double thresh() { return 8.636168555094445e-78; }      // 2^-256
     __device__ static double mult() { return 1.157920892373162e+77; }        // 2^256
-    __device__ static double ex(double x) { return exp(x); }
-    __device__ static double lg(double x) { return log(x); }
     __device__ static double rcp(double x) { return 1.0 / x; }
     __device__ static double mul(double x, double y) { return __dmul_rn(x, y); }
 };
@@ -1207,9 +1203,6 @@ struct STab {
     }
 };
 
-// Warps of one thread-block cluster whose Newton sums one CTA receives (CTAs x
-// warps per CTA); launch shapes above it are not offered.
-constexpr int kMaxClusterWarps = kMaxTeamWarps;
 __device__ __forceinline__ unsigned cluster_rank() {
     unsigned r;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
@@ -1269,7 +1262,7 @@ struct NewtonSmem {
     // cluster every warp of every CTA pushes its entry into entry rank * nw + warp of
     // every CTA's slot, two alternating slots, each with an mbarrier that counts the
     // bytes it received
-    alignas(16) float cxr[2][kMaxClusterWarps][4];
+    alignas(16) float cxr[2][kMaxTeamWarps][4];
     alignas(8) unsigned long long mbx[2];
     int abort_;            // a wait on mbx ran out (reported by the kernel)
 };
@@ -1553,8 +1546,10 @@ __device__ double eval_lnl(const STab<double, C>& st, const Sites& sx, double t,
 // One site's terms of the Newton sums: a = L'/L, c = L''/L - (L'/L)^2 and the site
 // weight, from the sum-table at the coefficients e, g, h (the stationary slots,
 // k = 0, have zero derivative coefficients).  A virtual thread takes its sites in
-// pairs; the two of a pair (and a last single one) round c in the forms they have
-// always had: first of a pair fma(-a, a, L''/L), else fma(L'', 1/L, -a a).
+// pairs; the two of a pair (and a last single one) round c in two forms: first of a pair
+// fma(-a, a, L''/L), else fma(L'', 1/L, -a a).  Neither is the better one: an earlier
+// source left the contraction to the compiler, which chose these, and results that are
+// stored or compared keep their bits only if they stay.
 template <typename R, int C>
 __device__ __forceinline__ void newton_site(const STab<R, C>& st, int p, const R* e, const R* g, const R* h, bool first,
                                             R& a, R& c, R& wt) {
@@ -1847,7 +1842,7 @@ __device__ __noinline__ double propose_score_f2(const Src2<C>* mem, const int* m
 // stack first, so that at most log2(n) vectors wait (local memory); the node just
 // made stays in registers.  The categories' groups are scaled apart and merged with
 // their exponents at the root.  Sites are summed in units of kScoreUnit (a fixed
-// tree), the units in order by k_score_sum: a score does not depend on the launch.
+// tree), the units in a fixed order by k_score_sum: a score does not depend on the launch.
 // Bound by FP32 issue (about 270 packed instructions per node, site and group) and,
 // for few sites, by the FP64 exponentials of the P matrices, which each CTA makes
 // once per tree, in parallel over edges and categories.  One tree of 27 taxa x 816
@@ -2034,7 +2029,8 @@ __global__ void __launch_bounds__(kThreads) k_score(const FullGroup* __restrict_
     }
 }
 
-// Sums a tree's units in order; with a prior, adds the log prior of its lengths.
+// Sums a tree's units (lane l takes units l, l + 32, ..., then the lanes by a butterfly);
+// with a prior, adds the log prior of its lengths.
 __global__ void k_score_sum(const FullGroup* __restrict__ groups, const int* __restrict__ gstart, int ngroups, int t0,
                             int t1, int units_max, const double* __restrict__ part, double prior_rate,
                             double prior_log) {
@@ -2195,7 +2191,7 @@ __global__ void k_partials_f2(Model M, Aln A, TreeSet ts, int first, DCount cnt,
 }
 
 // ---------------------------------------------------------------- proposal optimisation (K4)
-// One CTA per NNI neighbour (persistent loop).  The quartet around internal
+// One CTA or cluster per NNI neighbour (persistent loop).  The quartet around internal
 // edge (u, v): A = the side of u towards leaf 0 (U_u, or leaf 0 itself when u
 // is the first inner node), B = v's sibling, C < D = v's children.  After the
 // swap u holds A and X2, v holds B and Y2 (swap 0: X2 = C, Y2 = D; swap 1:
@@ -2467,10 +2463,11 @@ __global__ void __launch_bounds__(512) k_propose(const PropGroup* __restrict__ g
 }
 
 // ---------------------------------------------------------------- full optimisation (K7)
-// One CTA per tree (persistent loop).  Bottom-up D pass, then sweeps over the
+// One CTA or cluster per tree (persistent loop).  Bottom-up D pass, then sweeps over the
 // schedule: visit edge v = compute U_v (stored for inner v), sum-table of
-// (U_v, D_v), Newton on the length; refresh D_v after its subtree.  With
-// max_sweeps = 0 it only evaluates lnL at the given lengths.
+// (U_v, D_v), Newton on the length; refresh D_v after its subtree.  In FP64
+// the lnL at the final lengths follows (with max_sweeps = 0: at the given ones); in
+// mixed precision k_score makes it, and a launch has max_sweeps > 0.
 template <typename R, int C>
 struct FullSmem {
     R Mt[16];
@@ -2497,9 +2494,10 @@ constexpr unsigned short kUpd16 = 0x8000;  // kUpd in a 16-bit schedule entry
 // of an operation there too (read through L1 they were evicted by the vectors that
 // stream past), and as many lanes and CTAs per tree as the number of trees leaves
 // room for (Sites).  8 trees of 27 x 816 patterns took 12.9 ms on one CTA each with
-// those chains, now 6.3; 32 of 128 x 6273 289 ms, now 180; 515 of them 526 ms, now 340
-// (there a solve's 54 thousand cycles are half sum-table builds, in bursts at the rate
-// L2 and HBM deliver the stored vectors, 2.5 TB/s on average).
+// those chains, now 6.0; 32 of 128 x 6273 289 ms, now 165; 515 of them 526 ms, now 340
+// (there a solve's 54 thousand cycles are half sum-table builds, which wait for their
+// stored vectors: 2.5 TB/s on average, of 6.8 that a copy reaches, with long scoreboard the
+// first stall, so it is the latency of too few bytes in flight and not their rate).
 template <typename R, int C, bool kSmemTab, bool kClus>
 __global__ void __launch_bounds__(512) k_fullopt(const FullGroup* __restrict__ groups, const int* __restrict__ gstart,
                                                  int ngroups, int* counter, int nn_max, Cfg cfg,
@@ -3178,6 +3176,7 @@ void launch_score(cudaStream_t s, int C, const FullGroup* groups, const int* gst
                   Cfg cfg, int t0, int t1, double* part, int sms) {
     if (t1 <= t0) return;
     const int units = score_units(maxP), S = C == 1 ? 1 : 2;
+    // (in a recorded round, whose count only the device knows, by the capacity t1 - t0)
     // few trees: one unit per CTA; many: 24 warps per SM (80 registers a thread) as three
     // CTAs where their P matrices fit, else as one; two passes per CTA (a pass costs
     // several times the P matrices that each CTA makes)
