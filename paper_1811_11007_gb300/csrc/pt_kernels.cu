@@ -2985,6 +2985,13 @@ size_t sumtable_bytes(int prec, int C, int ld) {
 
 namespace {
 constexpr size_t kSmemPerCta = 227 * 1024, kSmemPerCta2 = 233472 / 2 - 1024;  // one CTA per SM, two CTAs per SM
+// Lets a kernel's launches take any amount of dynamic shared memory that a CTA can have
+// beside the kernel's own (kOwn bytes at most): the limit belongs to the kernel, so one that
+// followed each launch's size could be lowered by another thread before the launch it was for.
+template <size_t kOwn = 0, typename K>
+cudaError_t allow_smem(K kern) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kSmemPerCta - kOwn));
+}
 template <typename F>
 size_t by_kind(int prec, int C, F f) {
     if (prec == 0) return C == 1 ? f(double(), std::integral_constant<int, 1>()) : f(double(), std::integral_constant<int, 4>());
@@ -3027,13 +3034,13 @@ void partials_t(cudaStream_t s, const Model& M, Aln A, TreeSet ts, int first, DC
     ++g_launches;
     if constexpr (sizeof(R) == 4) {
         const size_t sm2 = (size_t)NN * C * 16 * 8;
-        cudaFuncSetAttribute(k_partials_f2<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2);
+        allow_smem(k_partials_f2<C>);
         dim3 grid(count.cap, blocks_for(A.P, threads));
         k_partials_f2<C><<<grid, threads, sm2, s>>>(M, A, ts, first, count, g, reinterpret_cast<float*>(pm), lo,
                                                     with_up ? 1 : 0);
     } else {
         const size_t smem = (size_t)NN * C * 16 * sizeof(R);
-        cudaFuncSetAttribute(k_partials<R, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        allow_smem(k_partials<R, C>);
         dim3 grid(count.cap, blocks_for(A.P, threads));
         k_partials<R, C><<<grid, threads, smem, s>>>(M, A, ts, first, count, g, pm, with_up ? 1 : 0);
     }
@@ -3090,7 +3097,7 @@ template <typename K>
 int resident(K kern, int kp, int threads, size_t smem, int sms) {
     if (smem > kSmemPerCta || kp * ((threads + 31) / 32) > kMaxTeamWarps) return 0;
     int nb = 0;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(kern);
     if (e == cudaSuccess && kp == 1) {
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, threads, smem);
         nb *= sms;
@@ -3118,7 +3125,7 @@ int resident(K kern, int kp, int threads, size_t smem, int sms) {
 
 template <typename K, typename... A>
 void launch_shape(K kern, cudaStream_t s, int kp, int threads, int grid, size_t smem, A... args) {
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem(kern);
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3(grid / kp * kp);
     lc.blockDim = dim3(threads);
@@ -3188,7 +3195,7 @@ void launch_score(cudaStream_t s, int C, const FullGroup* groups, const int* gst
     const int chunks = tt <= 16LL * sms ? passes : (passes + 1) / 2;
     const bool few = threads == S * kScoreUnit;
     auto kern = C == 1 ? (few ? k_score<1, 256> : k_score<1, 768>) : (few ? k_score<4, 256> : k_score<4, 768>);
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem<1024>(kern);
     const int grid = (int)std::min<long long>((long long)(t1 - t0) * chunks, 16LL * sms);
     kern<<<grid, threads, smem, s>>>(groups, gstart, ngroups, 2 * maxN - 2, t0, t1, chunks, units, part);
     ++g_launches;
