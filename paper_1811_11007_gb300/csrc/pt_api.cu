@@ -705,7 +705,10 @@ struct FullJob {
 
 // Runs full-optimisation jobs in one persistent launch over all of them.  The
 // partials live in per-CTA slabs (a CTA reuses its slab tree after tree), so
-// memory grows with the grid, not with the number of trees.
+// memory grows with the grid, not with the number of trees; nor does it with the
+// scores' unit sums, 8 bytes per tree and 64 patterns, which are made for as many trees
+// at a time as kPartBytes hold (40000 trees of 6000 patterns).
+constexpr size_t kPartBytes = 32 << 20;
 void run_full_jobs(Ctx& c, std::vector<FullJob> jobs) {
     const int prec = c.cfg.precision;
     jobs.erase(std::remove_if(jobs.begin(), jobs.end(), [](const FullJob& j) { return j.count <= 0; }), jobs.end());
@@ -768,8 +771,12 @@ void run_full_jobs(Ctx& c, std::vector<FullJob> jobs) {
             size_t e0 = timed ? ev_record(c) : 0;
             if (optimise) launch(threads, K, stats);
             if (prec == PT_PREC_MIXED) {
-                double* part = buf<double>(c, "full.part", (size_t)total * score_units(maxP));
-                launch_score(c.stream, C, dg, gstart, (int)groups.size(), maxN, maxP, kcfg(c), 0, total, part, c.sm_count);
+                const size_t units = score_units(maxP);
+                const int batch = (int)std::min<size_t>(total, std::max<size_t>(1, kPartBytes / (sizeof(double) * units)));
+                double* part = buf<double>(c, "full.part", batch * units);
+                for (int t0 = 0; t0 < total; t0 += batch)
+                    launch_score(c.stream, C, dg, gstart, (int)groups.size(), maxN, maxP, kcfg(c), t0,
+                                 std::min(total, t0 + batch), part, c.sm_count);
                 ck(c, cudaGetLastError(), "score launch");
             }
             float ms = 0.f;

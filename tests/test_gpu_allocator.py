@@ -96,3 +96,30 @@ def test_allocator_without_memory_reports_oom():
         e, l = synth.random_trees(8, 1, 1)
         lnl, _, _ = ctx.score(aid, e, l, mode="fixed")
         assert np.isfinite(lnl[0])
+
+
+def test_scores_of_many_trees_take_bounded_memory():
+    """The sums that a score is made of (8 bytes per tree and 64 patterns, 60 MB here) are held for some
+    trees at a time, 32 MiB and a quarter; the trees' own largest array takes 22 MB."""
+    import torch
+    n, trees = 8, 80000
+    a = synth.simulate(n, 9000, 61, model="gtr", alpha=2.0, mean_branch=1.5)
+    alloc_t, free_t = pt.torch_allocator(0, torch.cuda.current_stream())
+    sizes = []
+
+    def alloc(b):
+        sizes.append(b)
+        return alloc_t(b)
+    rng = np.random.default_rng(5)
+    few, _ = synth.random_trees(n, 50, 23)
+    e = np.ascontiguousarray(few[rng.integers(0, 50, trees)], np.int32)
+    l = rng.exponential(0.3, (trees, 2 * n - 3)) + 1e-3
+    with pt.Context(precision="mixed", table_log2=12, stream=torch.cuda.current_stream()) as ctx:
+        ctx.set_allocator(alloc, free_t)
+        aid = ctx.load_alignment(a.codes)
+        ctx.set_model(aid, a.exch, a.freqs, 0.5, 4)
+        assert ctx.alignment_info(aid)[1] > 5600
+        lnl = ctx.score(aid, e, l, "fixed")[0]
+        assert max(sizes) <= 42 << 20
+        for k in (slice(0, 700), slice(44500, 46000), slice(trees - 3, trees)):  # both sides of the cut, and the end
+            np.testing.assert_array_equal(ctx.score(aid, e[k], l[k], "fixed")[0], lnl[k])
